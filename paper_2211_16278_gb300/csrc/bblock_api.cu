@@ -290,6 +290,13 @@ bool within_workspace(const bblock_ctx* c, const void* p, size_t bytes) {
   return q >= c->d_ws && q + bytes <= c->d_ws + c->ws_cap;
 }
 
+struct JobIn {
+  const double2* V;
+  const double2* phi[3];
+  int nd[3];
+  double2* B;
+};
+
 // Spin operator of Eq. (1) reduced to what the kernels consume.
 struct SpinPlan {
   int n1 = 0, n2 = 0;                 // distinct alpha (line 1), beta (line 2)
@@ -340,7 +347,82 @@ int plan_spins(bblock_ctx* c, const int32_t* spin_idx, const double* coeffs, int
   return BBLOCK_OK;
 }
 
+// The spin sum as groups of terms that share a third-quark field (ContractParams::tbeg), with
+// the coefficient-folded fields it needs. Either
+//   by pair:  one group per (alpha, beta) pair, its line-3 field sum_gamma c q3[gamma]; or
+//   by gamma: one group per gamma with the plain field q3[gamma], and a term per alpha whose
+//             line-2 field is sum_beta c q2[beta] (Eq. 1 is linear in each line).
+// A group costs 9 FP64 operations per (d1, d2, d3) and site, a term 24 per (d1, d2), site and
+// d3 tile, a field 9 N_ev per column and site (18 and 3 in the complex counts of other forms:
+// the same ratios), so the plan with the smaller total over the call's jobs is taken; by pair
+// on a tie, and with per-momentum coefficients (each momentum is a launch of its own anyway).
+// Operators with pairs (alpha, beta) and (beta, alpha) on one gamma halve their groups.
+using FoldList = std::vector<std::pair<int, double2>>;   // (spin, coefficient)
+struct GroupPlan {
+  int n_groups = 0, n_terms = 0;
+  int tbeg[kMaxPairs + 1] = {};
+  int a_slot[kMaxPairs] = {}, b_slot[kMaxPairs] = {};
+  std::vector<FoldList> f2;                   // line-2 fields
+  std::vector<std::vector<FoldList>> f3;      // [coefficient set][group]
+};
+
+GroupPlan plan_groups(const SpinPlan& sp, bool may_group, const std::vector<JobIn>& jobs,
+                      int n_ev, int d3_tile) {
+  const double2 one = make_double2(1.0, 0.0);
+  GroupPlan by_pair, by_gamma;
+  by_pair.n_groups = by_pair.n_terms = sp.n_pairs;
+  for (int pr = 0; pr < sp.n_pairs; ++pr) {
+    by_pair.tbeg[pr + 1] = pr + 1;
+    by_pair.a_slot[pr] = sp.a_slot[pr];
+    by_pair.b_slot[pr] = sp.b_slot[pr];
+  }
+  for (int sl = 0; sl < sp.n2; ++sl) by_pair.f2.push_back({{sp.beta_of2[sl], one}});
+  by_pair.f3 = sp.terms;
+  if (!may_group || sp.n_coef_sets != 1) return by_pair;
+  by_gamma.f3.resize(1);
+  for (int ga = 0; ga < 4; ++ga) {
+    bool used = false;
+    for (int sl = 0; sl < sp.n1; ++sl) {
+      FoldList f;   // sum over beta of the coefficients of (alpha, beta, gamma)
+      for (int pr = 0; pr < sp.n_pairs; ++pr)
+        if (sp.a_slot[pr] == sl)
+          for (const auto& t : sp.terms[0][pr])
+            if (t.first == ga) f.push_back({sp.pair_beta[pr], t.second});
+      if (f.empty()) continue;
+      by_gamma.a_slot[by_gamma.n_terms] = sl;
+      by_gamma.b_slot[by_gamma.n_terms] = (int)by_gamma.f2.size();
+      by_gamma.f2.push_back(f);
+      ++by_gamma.n_terms;
+      used = true;
+    }
+    if (!used) continue;
+    by_gamma.f3[0].push_back({{ga, one}});
+    by_gamma.tbeg[++by_gamma.n_groups] = by_gamma.n_terms;
+  }
+  auto cost = [&](const GroupPlan& g) {
+    double sum = 0.0;
+    for (const JobIn& j : jobs) {
+      const double tiles = (j.nd[2] + d3_tile - 1) / d3_tile;
+      sum += 9.0 * n_ev * ((double)sp.n1 * j.nd[0] + (double)g.f2.size() * j.nd[1] +
+                           (double)g.f3[0].size() * j.nd[2]) +
+             (double)j.nd[0] * j.nd[1] * (9.0 * g.n_groups * j.nd[2] + 24.0 * g.n_terms * tiles);
+    }
+    return sum;
+  };
+  return cost(by_gamma) < cost(by_pair) ? by_gamma : by_pair;
+}
+
 int ensure_phase(bblock_ctx* c, const int32_t* momenta, int n_mom, cudaStream_t s) {
+  if (c->cfg.precision == BBLOCK_FP64) {
+    // the FP64 contraction needs w^k = e^{-2 pi i k / L} only, whatever the momenta
+    if (c->d_phase) return BBLOCK_OK;
+    int rc = grow_device(c, reinterpret_cast<char**>(&c->d_phase), &c->phase_cap,
+                         sizeof(double2) * c->cfg.L);
+    if (rc) return rc;
+    CK(c, timed_launch(c, K_PHASE, s, [&] { return launch_omega_table(c->cfg.L, c->d_phase, s); }));
+    CK(c, cudaStreamSynchronize(s));   // later calls may come on another stream
+    return BBLOCK_OK;
+  }
   std::vector<int32_t> key(momenta, momenta + 3 * n_mom);
   if (c->d_phase && key == c->phase_mom) return BBLOCK_OK;
   const size_t n_ph = (size_t)c->X * n_mom;
@@ -413,13 +495,6 @@ int choose_slabs(long long tiles, int grid, int X, int xc, int max_slabs) {
   }
   return best;
 }
-
-struct JobIn {
-  const double2* V;
-  const double2* phi[3];
-  int nd[3];
-  double2* B;
-};
 
 int validate_common(bblock_ctx* c, const int32_t* momenta, int n_mom, const int32_t* spin_idx,
                     const double* coeffs, int n_spin, int per_mom) {
@@ -1062,17 +1137,37 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
   const bool oz = c->cfg.precision == BBLOCK_OZAKI;
   const bool df = c->cfg.precision == BBLOCK_DF64 || oz;
 
-  const int X = c->X, rows = c->rows, n_ev = c->cfg.n_ev;
-  const int n3_fields = sp.n_pairs * sp.n_coef_sets;
+  const int X = c->X, rows = c->rows, n_ev = c->cfg.n_ev, L = c->cfg.L;
+  const bool f64 = c->cfg.precision == BBLOCK_FP64;
+  int max_nd3_all = 1;
+  for (const JobIn& j : jobs) max_nd3_all = std::max(max_nd3_all, j.nd[2]);
+  const GroupPlan gp = plan_groups(sp, f64, jobs, n_ev, f64 ? 64 : 32);
+  const int n2_fields = (int)gp.f2.size(), n3_fields = gp.n_groups * sp.n_coef_sets;
+  // FP64 form: the momenta in row plans (per-momentum coefficients: one plan per momentum)
+  std::vector<RowPlan> rplans;
+  int r_cls = 0;
+  if (f64) {
+    if (per_mom) {
+      rplans.resize(n_mom);
+      for (int p = 0; p < n_mom; ++p) {
+        plan_rows(L, momenta + 3 * p, 1, &rplans[p], 1);
+        rplans[p].mom[0].p = p;
+      }
+    } else {
+      rplans.resize(plan_rows(L, momenta, n_mom, nullptr, 0));
+      plan_rows(L, momenta, n_mom, rplans.data(), (int)rplans.size());
+    }
+    for (const RowPlan& r : rplans) r_cls = std::max(r_cls, r.n_cls);
+  }
+  const int row_rn = rows_rn_for(r_cls, max_nd3_all);
   // momenta per contraction launch: the Ozaki form takes them all as N columns
-  const int P_launch = per_mom ? 1
-                       : oz    ? n_mom
-                               : p_group_size(n_mom, c->cfg.precision == BBLOCK_DF64 ? kMaxPGroupDf
-                                                                                     : kMaxPGroup);
+  const int P_launch = per_mom ? 1 : oz ? n_mom : p_group_size(n_mom, kMaxPGroupDf);
   const int xc = oz ? 1 : fp64_sites_per_chunk(sp.n_pairs);
-  const Fp64Tile tl = fp64_tile_for(oz ? 1 : P_launch);  // one tile shape for every momentum group
+  // one tile shape for every launch of the call
+  const Fp64Tile tl = f64 ? Fp64Tile{kRowRM, row_rn} : fp64_tile_for(oz ? 1 : P_launch);
   // Ozaki form: units run one per CTA (clusters: one per cluster of oz_cl CTAs)
-  const int ctas = oz ? c->num_sms : fp64_contract_ctas_per_sm(P_launch, tl.rn, sp.n_pairs) * c->num_sms;
+  const int ctas = (oz ? 1 : f64 ? rows_ctas_per_sm(rplans[0].n_cls, row_rn)
+                                 : df_contract_ctas_per_sm(P_launch, tl.rn, sp.n_pairs)) * c->num_sms;
   const int max_slabs = 64;
   const int oz_nc = c->opt_tc_nc > 0 && c->opt_tc_nc <= kOzMaxNC ? c->opt_tc_nc : kOzMaxNC;
   int oz_cl = 1;   // Ozaki form: CTAs per cluster of the current wave
@@ -1102,10 +1197,10 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
   };
   // checks option: a canary after every field, the partial block and the converted inputs
   const size_t canary_bytes =
-      c->opt_checks ? (size_t)(sp.n1 + sp.n2 + n3_fields + 1 + (df ? 1 : 0)) * kCanaryBytes : 0;
+      c->opt_checks ? (size_t)(sp.n1 + n2_fields + n3_fields + 1 + (df ? 1 : 0)) * kCanaryBytes : 0;
   // bytes per job: fields + partials at the largest slab count (+ double-float inputs)
   auto job_bytes = [&](const JobIn& j, int n_slab) {
-    size_t f = (size_t)rows * (sp.n1 * j.nd[0] + sp.n2 * j.nd[1] + n3_fields * j.nd[2]) * sizeof(double2);
+    size_t f = (size_t)rows * (sp.n1 * j.nd[0] + n2_fields * j.nd[1] + n3_fields * j.nd[2]) * sizeof(double2);
     size_t p = (size_t)n_slab * n_mom * j.nd[0] * j.nd[1] * j.nd[2] * sizeof(double2);
     return align_up(f, 256) + align_up(p, 256) + df_in_bytes(j) + canary_bytes + oz_bytes(j, n_slab);
   };
@@ -1136,11 +1231,14 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
       max_elems = std::max(max_elems, (long long)n_mom * j.nd[0] * j.nd[1] * j.nd[2]);
     }
     const int unit_slots = oz ? ctas / oz_cl : ctas;
-    int n_slab = c->opt_slabs > 0 ? std::min(c->opt_slabs, (X + xc - 1) / xc)
-                                   : choose_slabs(tiles, unit_slots, X, xc, max_slabs);
-    int sites_per_slab = (X + n_slab - 1) / n_slab;
-    sites_per_slab = (sites_per_slab + xc - 1) / xc * xc;
-    n_slab = (X + sites_per_slab - 1) / sites_per_slab;
+    // FP64 form: slabs are ranges of lattice rows; the others: of chunks of xc sites
+    const int parts = f64 ? L * L : X, step = f64 ? 1 : xc;
+    int n_slab = c->opt_slabs > 0 ? std::min(c->opt_slabs, (parts + step - 1) / step)
+                                   : choose_slabs(tiles, unit_slots, parts, step, max_slabs);
+    int per_slab = (parts + n_slab - 1) / n_slab;
+    per_slab = (per_slab + step - 1) / step * step;
+    n_slab = (parts + per_slab - 1) / per_slab;
+    const int sites_per_slab = f64 ? per_slab * L : per_slab;
 
     size_t ws_need = 0, oz_need = 0;
     for (size_t k = job_idx; k < end; ++k) {
@@ -1208,25 +1306,21 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
       };
       const double2 one = make_double2(1.0, 0.0);
       const double2* q1[4] = {};
-      const double2* q2[4] = {};
-      for (int sl = 0; sl < sp.n1; ++sl) {
-        int off = sp.alpha_of1[sl] * n_ev;
-        q1[sl] = add_field(phin[0], j.nd[0], 1, &off, &one);
-      }
-      for (int sl = 0; sl < sp.n2; ++sl) {
-        int off = sp.beta_of2[sl] * n_ev;
-        q2[sl] = add_field(phin[1], j.nd[1], 1, &off, &one);
-      }
-      std::vector<std::vector<const double2*>> q3(sp.n_coef_sets, std::vector<const double2*>(sp.n_pairs));
+      std::vector<const double2*> q2(n2_fields);
+      auto folded = [&](int line, const FoldList& fl) -> const double2* {
+        if ((int)fl.size() > kMaxTerms) return nullptr;
+        int offs[kMaxTerms];
+        double2 w[kMaxTerms];
+        for (size_t t = 0; t < fl.size(); ++t) { offs[t] = fl[t].first * n_ev; w[t] = fl[t].second; }
+        return add_field(phin[line], j.nd[line], (int)fl.size(), offs, w);
+      };
+      for (int sl = 0; sl < sp.n1; ++sl) q1[sl] = folded(0, {{sp.alpha_of1[sl], one}});
+      for (int f = 0; f < n2_fields; ++f)
+        if (!(q2[f] = folded(1, gp.f2[f]))) return fail(c, BBLOCK_ERR_UNSUPPORTED, "too many terms");
+      std::vector<std::vector<const double2*>> q3(sp.n_coef_sets, std::vector<const double2*>(gp.n_groups));
       for (int set = 0; set < sp.n_coef_sets; ++set)
-        for (int pr = 0; pr < sp.n_pairs; ++pr) {
-          const auto& tlist = sp.terms[set][pr];
-          if ((int)tlist.size() > kMaxTerms) return fail(c, BBLOCK_ERR_UNSUPPORTED, "too many terms");
-          int offs[kMaxTerms];
-          double2 w[kMaxTerms];
-          for (size_t t = 0; t < tlist.size(); ++t) { offs[t] = tlist[t].first * n_ev; w[t] = tlist[t].second; }
-          q3[set][pr] = add_field(phin[2], j.nd[2], (int)tlist.size(), offs, w);
-        }
+        for (int g = 0; g < gp.n_groups; ++g)
+          if (!(q3[set][g] = folded(2, gp.f3[set][g]))) return fail(c, BBLOCK_ERR_UNSUPPORTED, "too many terms");
       base = c->d_ws + align_up((size_t)(base - c->d_ws), 256);
       double2* partial = reinterpret_cast<double2*>(base);
       base += align_up((size_t)n_slab * n_mom * j.nd[0] * j.nd[1] * j.nd[2] * sizeof(double2), 256);
@@ -1244,15 +1338,16 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
               OzMaxSeg{reinterpret_cast<const float4*>(q), oz_max, nd, off, stride, modulus});
         };
         for (int sl = 0; sl < sp.n1; ++sl) seg(q1[sl], j.nd[0], 0, 0);
-        for (int sl = 0; sl < sp.n2; ++sl) seg(q2[sl], j.nd[1], j.nd[0], 0);
+        for (int f = 0; f < n2_fields; ++f) seg(q2[f], j.nd[1], j.nd[0], 0);
         for (int set = 0; set < sp.n_coef_sets; ++set)
-          for (int pr = 0; pr < sp.n_pairs; ++pr) seg(q3[set][pr], j.nd[2], j.nd[0] + j.nd[1], 1);
+          for (int g = 0; g < gp.n_groups; ++g) seg(q3[set][g], j.nd[2], j.nd[0] + j.nd[1], 1);
       }
       for (int set = 0; set < sp.n_coef_sets; ++set) {
         ContractJob& cj = cjobs[set][k];
         cj.oz_max = oz_max;
-        for (int i = 0; i < 4; ++i) { cj.q1[i] = q1[i]; cj.q2[i] = q2[i]; }
-        for (int pr = 0; pr < sp.n_pairs; ++pr) cj.q3[pr] = q3[set][pr];
+        for (int i = 0; i < 4; ++i) cj.q1[i] = q1[i];
+        for (int f = 0; f < n2_fields; ++f) cj.q2[f] = q2[f];
+        for (int g = 0; g < gp.n_groups; ++g) cj.q3[g] = q3[set][g];
         cj.partial = partial;
         cj.B = j.B;
         cj.nd1 = j.nd[0]; cj.nd2 = j.nd[1]; cj.nd3 = j.nd[2];
@@ -1328,8 +1423,13 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
     prm.X = X;
     prm.n_slab = n_slab;
     prm.sites_per_slab = sites_per_slab;
-    prm.n_pairs = sp.n_pairs;
-    for (int pr = 0; pr < sp.n_pairs; ++pr) { prm.a_slot[pr] = sp.a_slot[pr]; prm.b_slot[pr] = sp.b_slot[pr]; }
+    prm.n_groups = gp.n_groups;
+    prm.n_terms = gp.n_terms;
+    memcpy(prm.tbeg, gp.tbeg, sizeof(prm.tbeg));
+    memcpy(prm.a_slot, gp.a_slot, sizeof(prm.a_slot));
+    memcpy(prm.b_slot, gp.b_slot, sizeof(prm.b_slot));
+    prm.L = L;
+    prm.rows_per_slab = per_slab;
     prm.phase = c->d_phase;
     prm.P_total = n_mom;
     prm.status = c->d_status;
@@ -1354,22 +1454,21 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
           return launch_contract_oz(prm, oz_cl, (int)std::min<long long>(unit, unit_slots), s);
         }));
       }
-    } else if (per_mom) {
-      for (int p = 0; p < n_mom; ++p) {
-        prm.jobs = reinterpret_cast<const ContractJob*>(c->d_tab + fbytes + jbytes * p);
-        prm.p0 = p;
-        CK(c, timed_launch(c, K_CONTRACT, s, [&] {
-          return df ? launch_contract_df(prm, 1, tl.rn, grid, s) : launch_contract_fp64(prm, 1, tl.rn, grid, s);
-        }));
+    } else if (f64) {
+      for (size_t k = 0; k < rplans.size(); ++k) {
+        prm.jobs = reinterpret_cast<const ContractJob*>(c->d_tab + fbytes + jbytes * (per_mom ? k : 0));
+        prm.rows = rplans[k];
+        prm.xc = rows_sites_per_chunk(L, prm.rows.n_cls, row_rn, gp.n_groups);
+        const int g64 = (int)std::min<long long>(unit, (long long)rows_ctas_per_sm(prm.rows.n_cls, row_rn) * c->num_sms);
+        CK(c, timed_launch(c, K_CONTRACT, s, [&] { return launch_contract_fp64(prm, row_rn, g64, s); }));
       }
     } else {
-      prm.jobs = reinterpret_cast<const ContractJob*>(c->d_tab + fbytes);
       const int pg = P_launch;
       for (int p0 = 0; p0 < n_mom; p0 += pg) {
-        const int Pg = std::min(pg, n_mom - p0);
+        prm.jobs = reinterpret_cast<const ContractJob*>(c->d_tab + fbytes + jbytes * (per_mom ? p0 : 0));
         prm.p0 = p0;
         CK(c, timed_launch(c, K_CONTRACT, s, [&] {
-          return df ? launch_contract_df(prm, Pg, tl.rn, grid, s) : launch_contract_fp64(prm, Pg, tl.rn, grid, s);
+          return launch_contract_df(prm, std::min(pg, n_mom - p0), tl.rn, grid, s);
         }));
       }
     }
@@ -1528,16 +1627,18 @@ CallPlan plan_call(const bblock_ctx* c, int n_t, const int nd[3], int n_mom, int
     return pl;
   }
   if (fp64_like(c->cfg)) {
-    const int P = p_group_size(n_mom, c->cfg.precision == BBLOCK_DF64 ? kMaxPGroupDf : kMaxPGroup);
-    const Fp64Tile tl = fp64_tile_for(P);
-    const int xc = fp64_sites_per_chunk(pairs);
-    const int ctas = fp64_contract_ctas_per_sm(P, tl.rn, pairs) * c->num_sms;
+    const bool f64 = c->cfg.precision == BBLOCK_FP64;
+    const int P = p_group_size(n_mom, kMaxPGroupDf);
+    const Fp64Tile tl = f64 ? Fp64Tile{kRowRM, rows_rn_for(1, nd[2])} : fp64_tile_for(P);
+    const int xc = f64 ? 1 : fp64_sites_per_chunk(pairs);
+    const int parts = f64 ? c->cfg.L * c->cfg.L : X;   // slabs of lattice rows, or of sites
+    const int ctas = (f64 ? rows_ctas_per_sm(1, tl.rn) : df_contract_ctas_per_sm(P, tl.rn, pairs)) * c->num_sms;
     const long long tiles = (long long)n_t * ((nd[0] * nd[1] + 16 * tl.rm - 1) / (16 * tl.rm)) *
                             ((nd[2] + 16 * tl.rn - 1) / (16 * tl.rn));
-    int ns = slabs_opt > 0 ? std::min(slabs_opt, (X + xc - 1) / xc) : choose_slabs(tiles, ctas, X, xc, 64);
-    int sps = (X + ns - 1) / ns;
+    int ns = slabs_opt > 0 ? std::min(slabs_opt, (parts + xc - 1) / xc) : choose_slabs(tiles, ctas, parts, xc, 64);
+    int sps = (parts + ns - 1) / ns;
     sps = (sps + xc - 1) / xc * xc;
-    pl.n_slab = (X + sps - 1) / sps;
+    pl.n_slab = (parts + sps - 1) / sps;
     pl.units = tiles * pl.n_slab;
     pl.pad = (double)(((nd[2] + 16 * tl.rn - 1) / (16 * tl.rn)) * 16 * tl.rn) / nd[2] - 1.0;
     return pl;

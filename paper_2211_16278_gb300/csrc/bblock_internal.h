@@ -12,10 +12,12 @@ constexpr int kMaxPairs = 16;   // distinct (alpha, beta) spin pairs
 constexpr int kMaxRfP = 16;
 constexpr int kMaxRfIdx = 8;
 constexpr int kMaxRfL = 128;    // lattice extent (the w^k table follows the stage buffers)
-// Momenta handled by one contraction launch of the FP64 form (10) and of the double-float
-// form (8): the largest counts whose accumulators fit the registers without spills.
-constexpr int kMaxPGroup = 10;
+// Momenta handled by one contraction launch of the double-float form: the largest count whose
+// accumulators fit the registers without spills.
 constexpr int kMaxPGroupDf = 8;
+// Row-factored FP64 contraction: momenta and +-n0 classes of one launch.
+constexpr int kMaxRowP = 32;
+constexpr int kMaxRowCls = 3;
 // Momenta of the first launch: n_mom split into the fewest groups of at most max_group, as
 // evenly as possible (each launch recomputes the colour singlet that its momenta share).
 inline int p_group_size(int n_mom, int max_group) {
@@ -69,8 +71,8 @@ struct ProjFieldF {
 // One job = one time slice of one noise triple.
 struct ContractJob {
   const double2* q1[4];          // line-1 fields, one per distinct alpha (slot order)
-  const double2* q2[4];          // line-2 fields, one per distinct beta
-  const double2* q3[kMaxPairs];  // folded line-3 field per (alpha, beta) pair
+  const double2* q2[kMaxPairs];  // line-2 fields (see ContractParams::tbeg)
+  const double2* q3[kMaxPairs];  // line-3 field of each group
   double2* partial;              // [n_slab][P_total][nd1*nd2][nd3]
   double2* B;                    // [P_total][nd1][nd2][nd3]
   // Ozaki form: per site slab, the column maxima of the job's line-1 and line-2 fields
@@ -82,6 +84,23 @@ struct ContractJob {
   long long unit_begin;          // first global work-unit index of this job
 };
 
+// A momentum of a row-factored launch: p = index in the call's list, n1 and n2 = its
+// components along the two axes that are not summed (ascending, reduced to [0, L)), sel = 0
+// where its component n0 along the summed axis is 0 mod L, +(c + 1) where n0 = cls_n0[c] and
+// -(c + 1) where n0 = -cls_n0[c] mod L.
+struct RowMom { int p, n1, n2, sel; };
+struct RowPlan {
+  int axis;                      // the lattice axis whose sites a row sums
+  int n_cls, cls_n0[kMaxRowCls]; // classes of +-n0, n0 in [1, L / 2]
+  int has_zero;                  // a momentum has n0 = 0
+  int n_mom;
+  RowMom mom[kMaxRowP];
+};
+
+// Eq. 1's spin sum as groups of terms: group g sums the terms t in [tbeg[g], tbeg[g + 1]),
+//   sum_g [ sum_t q1[a_slot[t]] x q2[b_slot[t]] ] . q3[g],
+// the spin coefficients folded into the line-3 fields (one term per group: its (alpha, beta)
+// pair) or into the line-2 fields (one group per gamma, a term per (alpha, gamma) pair).
 struct ContractParams {
   const ContractJob* jobs;
   int n_jobs;
@@ -89,9 +108,13 @@ struct ContractParams {
   int X;                         // sites per time slice
   int n_slab;
   int sites_per_slab;
-  int n_pairs;
-  int a_slot[kMaxPairs];         // pair -> line-1 slot
-  int b_slot[kMaxPairs];         // pair -> line-2 slot
+  int n_groups, n_terms;
+  int tbeg[kMaxPairs + 1];
+  int a_slot[kMaxPairs];         // term -> line-1 slot
+  int b_slot[kMaxPairs];         // term -> line-2 field
+  // FP64 form: lattice extent, rows (of L^2) per slab, sites of a row staged at a time
+  int L, rows_per_slab, xc;
+  RowPlan rows;
   const double2* phase;          // [P_total][X]
   int p0;                        // first momentum of this launch
   int P_total;
@@ -105,11 +128,45 @@ struct ContractParams {
   long long wait_limit;
 };
 
-// Tiles of the FP64 contraction for a momentum count (per launch).
+// Tiles of the double-float contraction for a momentum count (per launch).
 struct Fp64Tile { int rm, rn; };
 inline Fp64Tile fp64_tile_for(int P) { return P <= 4 ? Fp64Tile{2, 2} : Fp64Tile{2, 1}; }
 inline int fp64_sites_per_chunk(int n_pairs) { return n_pairs >= 16 ? 1 : 16 / n_pairs; }
-size_t fp64_contract_smem_bytes(int P, int rn, int n_pairs);
+size_t df_contract_smem_bytes(int P, int rn, int n_pairs);
+int df_contract_ctas_per_sm(int P, int rn, int n_pairs);
+
+// Tiles of the row-factored FP64 contraction: 16 kRowRM (d1, d2) pairs by 16 rn d3 columns.
+// A wider d3 tile shares each diquark among more outputs; the row sums of the launch's classes
+// limit it (registers). One CTA per SM for the tiles that need more than 128 registers.
+constexpr int kRowRM = 2;
+inline int rows_max_rn(int n_cls) { return n_cls <= 1 ? 4 : 2; }
+inline int rows_ctas_per_sm(int n_cls, int rn) { return rn == 4 || n_cls >= 2 ? 1 : 2; }
+// rn for a launch sequence of at most n_cls classes over jobs of at most nd3 columns
+inline int rows_rn_for(int n_cls, int nd3) {
+  const int want = nd3 <= 16 ? 1 : nd3 <= 32 ? 2 : 4, most = rows_max_rn(n_cls);
+  return want < most ? want : most;
+}
+// Sites of a row staged at a time (KC = xc * groups * 3 operand rows of 24 (16 kRowRM + 16 rn)
+// bytes): as many as fit the CTA's share of the shared memory, in chunks of equal size.
+inline size_t rows_smem_bytes(int L, int n_cls, int rn, int n_groups, int xc) {
+  return (size_t)24 * (16 * kRowRM + 16 * rn) * 3 * n_groups * xc +
+         16 * ((size_t)xc * (n_cls > 0 ? n_cls : 1) + L);
+}
+inline int rows_sites_per_chunk(int L, int n_cls, int rn, int n_groups) {
+  const size_t budget = (size_t)(rows_ctas_per_sm(n_cls, rn) == 1 ? 220 : 108) * 1024;
+  int xc = L < 16 ? L : 16;
+  while (xc > 1 && rows_smem_bytes(L, n_cls, rn, n_groups, xc) > budget) --xc;
+  const int chunks = (L + xc - 1) / xc;
+  return (L + chunks - 1) / chunks;
+}
+// Whether the tile of the most groups a call can have fits the shared memory of a CTA.
+static_assert((size_t)24 * (16 * kRowRM + 64) * 3 * kMaxPairs + 16 * (kMaxRowCls + 128) <= 227 * 1024,
+              "one site of kMaxPairs groups fits");
+// The momenta of a call, each in one RowPlan: `axis` is the one with the fewest +-n0 classes
+// (the last on a tie), and a plan takes at most kMaxRowCls classes and kMaxRowP momenta.
+// Returns the number of plans written to `out` (at most max_out), or the number needed where
+// out is null.
+int plan_rows(int L, const int32_t* momenta, int n_mom, RowPlan* out, int max_out);
 
 // ---------------------------------------------------------------- tensor-core forms
 
@@ -244,7 +301,9 @@ cudaError_t launch_phase_table(int L, int n_mom, const int* d_mom, double2* ph, 
                                cudaStream_t s);
 cudaError_t launch_project_fp64(const ProjField* d_fields, int n_fields, int rows, int n_ev,
                                 int max_nd, cudaStream_t s);
-cudaError_t launch_contract_fp64(const ContractParams& p, int P, int rn, int grid, cudaStream_t s);
+// w^k = e^{-2 pi i k / L}, k = 0..L-1
+cudaError_t launch_omega_table(int L, double2* om, cudaStream_t s);
+cudaError_t launch_contract_fp64(const ContractParams& p, int rn, int grid, cudaStream_t s);
 // Double-float form: same units, tiles, shared memory and partial layout as the FP64
 // contraction; fields hold double-float pairs (float4 per complex element).
 cudaError_t launch_contract_df(const ContractParams& p, int P, int rn, int grid, cudaStream_t s);
@@ -262,7 +321,6 @@ cudaError_t launch_convert_df(const DfConvSeg* d_segs, int n_segs, long long max
 // planes (cast to const double2*), q receives float4 double-float elements.
 cudaError_t launch_project_df(const ProjField* d_fields, int n_fields, int rows, int n_ev,
                               int max_nd, cudaStream_t s);
-int fp64_contract_ctas_per_sm(int P, int rn, int n_pairs);
 
 // ---------------------------------------------------------------- tiled tensor-core projection
 

@@ -20,53 +20,67 @@ static __device__ __align__(256) double2 g_noalloc_scratch[kNoallocScratchBytes 
 constexpr int kNaMaxP = 8;
 constexpr int kNaMaxDevices = 64;
 
-// The launch: the shared FP64 contraction body's parameters (one job, embedded below; no
-// status word) plus what this entry point takes instead of a context's tables.
-struct NoallocParams {
-  ContractParams base;    // jobs = nullptr, status = nullptr, P_total = P, p0 = 0
-  ContractJob job;        // q1/q2 slots = spins 0..3 of the caller's arrays; partial = scratch
-  const double2* q3;      // [4][X][3][nd3]
-  int L;
-  int n_terms[kMaxPairs];
-  int term_gamma[kMaxPairs][kMaxTerms];
-  double2 term_w[kMaxPairs][kMaxTerms];
-  int mom[kNaMaxP][3];
+// One folded field element: sum_t w[t] f[spin[t]], by the launch's spin coefficients.
+struct NaFold {
+  int n;
+  int spin[kMaxTerms];
+  double2 w[kMaxTerms];
 };
 
-// Where the shared body's inputs come from without a context: the single job of the
-// launch, the third quark folded with its pair's spin coefficients while the tile is
-// staged, and the phase evaluated per site from the integer momentum ((n.x) mod L in
-// integers, then sincospi).
+// The launch: the shared FP64 contraction body's parameters (one job, embedded below; no
+// status word) plus what this entry point takes instead of a context's tables. The spin sum is
+// grouped as in the context (ContractParams::tbeg); a_slot is the line-1 spin, and the folds
+// that the context's projection applies are taken while a tile is staged.
+struct NoallocParams {
+  ContractParams base;    // jobs = nullptr, status = nullptr, P_total = P
+  ContractJob job;        // q1 slots = spins 0..3 of the caller's array; partial = scratch
+  const double2* q2;      // [4][X][3][nd2]
+  const double2* q3;      // [4][X][3][nd3]
+  NaFold f2[kMaxPairs];   // line-2 element of term t
+  NaFold f3[kMaxPairs];   // line-3 element of group g
+};
+
+// Where the shared body's inputs come from without a context: the single job of the launch,
+// the spin coefficients folded while the tile is staged, and w^k by sincospi.
 struct NoallocSource {
   const NoallocParams* np;
   __device__ const ContractJob& job(long long) const { return np->job; }
-  __device__ double2 third(const ContractJob& J, int pr, int x, int c, int n) const {
-    const int X = np->base.X;
+  __device__ static double2 fold(const NaFold& f, const double2* q, size_t spin_stride, size_t at) {
+    if (f.n == 1 && f.w[0].x == 1.0 && f.w[0].y == 0.0) return q[f.spin[0] * spin_stride + at];
     double2 b = make_double2(0.0, 0.0);
-    for (int t = 0; t < np->n_terms[pr]; ++t) {
-      const double2 f = np->q3[(((size_t)np->term_gamma[pr][t] * X + x) * 3 + c) * J.nd3 + n];
-      const double2 w = np->term_w[pr][t];
-      b.x = fma(w.x, f.x, fma(-w.y, f.y, b.x));
-      b.y = fma(w.x, f.y, fma(w.y, f.x, b.y));
+    for (int t = 0; t < f.n; ++t) {
+      const double2 v = q[f.spin[t] * spin_stride + at];
+      const double2 w = f.w[t];
+      b.x = fma(w.x, v.x, fma(-w.y, v.y, b.x));
+      b.y = fma(w.x, v.y, fma(w.y, v.x, b.y));
     }
     return b;
   }
-  __device__ double2 phase(int p, int x) const {
-    const int L = np->L;
-    const long long x0 = x % L, x1 = (x / L) % L, x2 = x / ((long long)L * L);
-    long long kk = np->mom[p][0] * x0 + np->mom[p][1] * x1 + np->mom[p][2] * x2;
-    kk %= L;
-    if (kk < 0) kk += L;
+  __device__ void uv(const ContractJob& J, int t, int x, int d1, int d2, double2 (&u)[3],
+                     double2 (&v)[3]) const {
+    const double2* a = J.q1[np->base.a_slot[t]] + (size_t)x * 3 * J.nd1 + d1;
+    const size_t b = (size_t)x * 3 * J.nd2 + d2, st = (size_t)np->base.X * 3 * J.nd2;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      u[c] = a[c * J.nd1];
+      v[c] = fold(np->f2[t], np->q2, st, b + c * J.nd2);
+    }
+  }
+  __device__ double2 third(const ContractJob& J, int g, int x, int c, int n) const {
+    return fold(np->f3[g], np->q3, (size_t)np->base.X * 3 * J.nd3,
+                ((size_t)x * 3 + c) * J.nd3 + n);
+  }
+  __device__ double2 omega(int k) const {
     double sn, cs;
-    sincospi(2.0 * (double)kk / (double)L, &sn, &cs);
+    sincospi(2.0 * (double)k / (double)np->base.L, &sn, &cs);
     return make_double2(cs, -sn);
   }
 };
 
-template <int P, int RN>
-__global__ void __launch_bounds__(kThreads, 2)
+template <int NCLS, int RN>
+__global__ void __launch_bounds__(kThreads, RN == 4 || NCLS >= 2 ? 1 : 2)
 k_contract_fp64_noalloc(const __grid_constant__ NoallocParams prm) {
-  fp64c::contract_body<P, 2, RN>(prm.base, NoallocSource{&prm});
+  fp64c::contract_rows<NCLS, kRowRM, RN>(prm.base, NoallocSource{&prm});
 }
 
 // B[e] = sum over slabs of partial[slab][e], slabs in index order.
@@ -85,32 +99,29 @@ __global__ void k_reduce_noalloc(const double2* __restrict__ partial, double2* _
 }
 
 
-template <int P, int RN>
+template <int NCLS, int RN>
 cudaError_t na_launch(const NoallocParams& prm, int grid, cudaStream_t s) {
-  const size_t smem = fp64_contract_smem_bytes(P, RN, prm.base.n_pairs);
-  cudaError_t e = cudaFuncSetAttribute(k_contract_fp64_noalloc<P, RN>,
+  const size_t smem = rows_smem_bytes(prm.base.L, NCLS, RN, prm.base.n_groups, prm.base.xc);
+  cudaError_t e = cudaFuncSetAttribute(k_contract_fp64_noalloc<NCLS, RN>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_contract_fp64_noalloc<P, RN><<<grid, kThreads, smem, s>>>(prm);
+  k_contract_fp64_noalloc<NCLS, RN><<<grid, kThreads, smem, s>>>(prm);
   note_launch();
   return cudaGetLastError();
 }
 
-cudaError_t na_dispatch(const NoallocParams& prm, int P, int rn, int grid, cudaStream_t s) {
-  if (rn == 2) {
-    switch (P) {
-      case 1: return na_launch<1, 2>(prm, grid, s);
-      case 2: return na_launch<2, 2>(prm, grid, s);
-      case 3: return na_launch<3, 2>(prm, grid, s);
-      case 4: return na_launch<4, 2>(prm, grid, s);
-      default: return cudaErrorInvalidValue;
-    }
-  }
-  switch (P) {
-    case 5: return na_launch<5, 1>(prm, grid, s);
-    case 6: return na_launch<6, 1>(prm, grid, s);
-    case 7: return na_launch<7, 1>(prm, grid, s);
-    case 8: return na_launch<8, 1>(prm, grid, s);
+cudaError_t na_dispatch(const NoallocParams& prm, int rn, int grid, cudaStream_t s) {
+  switch (prm.base.rows.n_cls * 8 + rn) {
+    case 0 + 1: return na_launch<0, 1>(prm, grid, s);
+    case 0 + 2: return na_launch<0, 2>(prm, grid, s);
+    case 0 + 4: return na_launch<0, 4>(prm, grid, s);
+    case 8 + 1: return na_launch<1, 1>(prm, grid, s);
+    case 8 + 2: return na_launch<1, 2>(prm, grid, s);
+    case 8 + 4: return na_launch<1, 4>(prm, grid, s);
+    case 16 + 1: return na_launch<2, 1>(prm, grid, s);
+    case 16 + 2: return na_launch<2, 2>(prm, grid, s);
+    case 24 + 1: return na_launch<3, 1>(prm, grid, s);
+    case 24 + 2: return na_launch<3, 2>(prm, grid, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -197,49 +208,77 @@ extern "C" int bblock_contract_noalloc(int L, const void* q1, const void* q2, co
   ContractParams& base = prm.base;
   ContractJob& job = prm.job;
   const int X = L * L * L;
-  // the q1 / q2 slots are the four spins of the caller's arrays; a pair names its spins
-  for (int a = 0; a < 4; ++a) {
+  // the q1 slots are the four spins of the caller's array
+  for (int a = 0; a < 4; ++a)
     job.q1[a] = static_cast<const double2*>(q1) + (size_t)a * X * 3 * nd1;
-    job.q2[a] = static_cast<const double2*>(q2) + (size_t)a * X * 3 * nd2;
-  }
   job.nd1 = nd1; job.nd2 = nd2; job.nd3 = nd3;
   job.unit_begin = 0;
+  prm.q2 = static_cast<const double2*>(q2);
   prm.q3 = static_cast<const double2*>(q3);
-  prm.L = L;
+  base.L = L;
   base.X = X;
   base.n_jobs = 1;
   base.P_total = n_mom;
-  base.p0 = 0;
-  for (int p = 0; p < n_mom; ++p)
-    for (int i = 0; i < 3; ++i) prm.mom[p][i] = momenta[3 * p + i];
-  // spin triples -> (alpha, beta) pairs with the coefficient-weighted gamma terms
+  RowPlan plans[kNaMaxP];
+  const int n_plans = plan_rows(L, momenta, n_mom, plans, kNaMaxP);
+  int n_cls = 0;
+  for (int k = 0; k < n_plans; ++k) n_cls = plans[k].n_cls > n_cls ? plans[k].n_cls : n_cls;
+  // spin triples -> coefficients by (alpha, beta, gamma), then the groups: one per
+  // (alpha, beta) pair with the coefficients in its third quark, or, where that makes fewer,
+  // one per gamma with a term per alpha and the coefficients in its line-2 element
+  double2 coef[4][4][4] = {};
+  bool have[4][4][4] = {};
   for (int s = 0; s < n_spin; ++s) {
     const int al = spin_idx[3 * s], be = spin_idx[3 * s + 1], ga = spin_idx[3 * s + 2];
     if (al < 0 || al > 3 || be < 0 || be > 3 || ga < 0 || ga > 3)
       return na_fail(err, err_len, BBLOCK_ERR_INVALID_ARG, "spin index outside 0..3");
-    int pr = -1;
-    for (int k = 0; k < base.n_pairs; ++k)
-      if (base.a_slot[k] == al && base.b_slot[k] == be) pr = k;
-    if (pr < 0) {
-      pr = base.n_pairs++;
-      base.a_slot[pr] = al;
-      base.b_slot[pr] = be;
+    have[al][be][ga] = true;
+    coef[al][be][ga].x += spin_coeffs[2 * s];
+    coef[al][be][ga].y += spin_coeffs[2 * s + 1];
+  }
+  const double2 one = make_double2(1.0, 0.0);
+  auto push = [](NaFold& f, int spin, double2 w) { f.spin[f.n] = spin; f.w[f.n++] = w; };
+  int n_pairs = 0, n_gamma = 0;
+  for (int a = 0; a < 4; ++a)
+    for (int b = 0; b < 4; ++b) {
+      bool any = false, g_any = false;
+      for (int g = 0; g < 4; ++g) any = any || have[a][b][g];
+      for (int i = 0; i < 16; ++i) g_any = g_any || have[i / 4][i % 4][b];
+      n_pairs += any;
+      if (a == 0) n_gamma += g_any;
     }
-    int t = -1;
-    for (int k = 0; k < prm.n_terms[pr]; ++k)
-      if (prm.term_gamma[pr][k] == ga) t = k;
-    if (t < 0) {
-      t = prm.n_terms[pr]++;
-      prm.term_gamma[pr][t] = ga;
-      prm.term_w[pr][t] = make_double2(0.0, 0.0);
+  if (n_gamma < n_pairs) {
+    for (int g = 0; g < 4; ++g) {
+      const int t0 = base.n_terms;
+      for (int a = 0; a < 4; ++a) {
+        NaFold f{};
+        for (int b = 0; b < 4; ++b)
+          if (have[a][b][g]) push(f, b, coef[a][b][g]);
+        if (f.n == 0) continue;
+        base.a_slot[base.n_terms] = a;
+        prm.f2[base.n_terms++] = f;
+      }
+      if (base.n_terms == t0) continue;
+      push(prm.f3[base.n_groups], g, one);
+      base.tbeg[++base.n_groups] = base.n_terms;
     }
-    prm.term_w[pr][t].x += spin_coeffs[2 * s];
-    prm.term_w[pr][t].y += spin_coeffs[2 * s + 1];
+  } else {
+    for (int a = 0; a < 4; ++a)
+      for (int b = 0; b < 4; ++b) {
+        NaFold f{};
+        for (int g = 0; g < 4; ++g)
+          if (have[a][b][g]) push(f, g, coef[a][b][g]);
+        if (f.n == 0) continue;
+        base.a_slot[base.n_terms] = a;
+        push(prm.f2[base.n_terms++], b, one);
+        prm.f3[base.n_groups] = f;
+        base.tbeg[++base.n_groups] = base.n_terms;
+      }
   }
 
-  const Fp64Tile tl = fp64_tile_for(n_mom);
-  job.m_tiles = (nd1 * nd2 + 16 * tl.rm - 1) / (16 * tl.rm);
-  job.n_tiles = (nd3 + 16 * tl.rn - 1) / (16 * tl.rn);
+  const int rn = rows_rn_for(n_cls, nd3);
+  job.m_tiles = (nd1 * nd2 + 16 * kRowRM - 1) / (16 * kRowRM);
+  job.n_tiles = (nd3 + 16 * rn - 1) / (16 * rn);
   const size_t per = (size_t)n_mom * nd1 * nd2 * nd3;
   const size_t max_slabs_fit = kNoallocScratchBytes / (per * sizeof(double2));
   if (max_slabs_fit < 1)
@@ -269,23 +308,25 @@ extern "C" int bblock_contract_noalloc(int L, const void* q1, const void* q2, co
     cudaGetLastError();
     return na_fail(err, err_len, BBLOCK_ERR_CUDA, "device query failed");
   }
-  const int xc = fp64_sites_per_chunk(base.n_pairs);
-  const int grid_cap = 2 * num_sms;
+  const int ctas = rows_ctas_per_sm(plans[0].n_cls, rn) * num_sms;
   const long long tiles = (long long)job.m_tiles * job.n_tiles;
-  long long want = (4LL * grid_cap + tiles - 1) / tiles;
-  long long n_slab = want;
+  long long n_slab = (4LL * ctas + tiles - 1) / tiles;
   if (n_slab > (long long)max_slabs_fit) n_slab = (long long)max_slabs_fit;
-  if (n_slab > (X + xc - 1) / xc) n_slab = (X + xc - 1) / xc;
+  if (n_slab > L * L) n_slab = L * L;
   if (n_slab < 1) n_slab = 1;
-  int sps = (int)((X + n_slab - 1) / n_slab);
-  sps = (sps + xc - 1) / xc * xc;
-  base.sites_per_slab = sps;
-  base.n_slab = (X + sps - 1) / sps;
+  base.rows_per_slab = (int)((L * L + n_slab - 1) / n_slab);
+  base.sites_per_slab = base.rows_per_slab * L;
+  base.n_slab = (L * L + base.rows_per_slab - 1) / base.rows_per_slab;
   base.total_units = tiles * base.n_slab;
-  const int grid = (int)(base.total_units < grid_cap ? base.total_units : grid_cap);
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  cudaError_t e = na_dispatch(prm, n_mom, tl.rn, grid, s);
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < n_plans && e == cudaSuccess; ++k) {
+    base.rows = plans[k];
+    base.xc = rows_sites_per_chunk(L, plans[k].n_cls, rn, base.n_groups);
+    const long long cap = (long long)rows_ctas_per_sm(plans[k].n_cls, rn) * num_sms;
+    e = na_dispatch(prm, rn, (int)(base.total_units < cap ? base.total_units : cap), s);
+  }
   if (e == cudaSuccess) {
     long long bx = ((long long)per + kThreads - 1) / kThreads;
     if (bx > 4096) bx = 4096;

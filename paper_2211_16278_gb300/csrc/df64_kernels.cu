@@ -42,7 +42,7 @@ template <int P, int RM, int RN>
 __global__ void __launch_bounds__(kThreads, 2) k_contract_df(const __grid_constant__ ContractParams prm) {
   constexpr int MT = 16 * RM, NT = 16 * RN;
   extern __shared__ __align__(16) float2 smem_df[];
-  const int np = prm.n_pairs;
+  const int np = prm.n_groups;
   const int XC = np >= 16 ? 1 : 16 / np;
   const int KC = XC * np * 3;
   float2* __restrict__ Ar = smem_df;
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_contract_df(const __grid_consta
 template <int P, int RN>
 cudaError_t launch_df_p(const ContractParams& prm, int grid, cudaStream_t s) {
   // same layout as the FP64 tiles: every double becomes a float2 of the same size
-  const size_t smem = fp64_contract_smem_bytes(P, RN, prm.n_pairs);
+  const size_t smem = df_contract_smem_bytes(P, RN, prm.n_groups);
   cudaError_t e = cudaFuncSetAttribute(k_contract_df<P, 2, RN>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -227,6 +227,22 @@ cudaError_t launch_df_p(const ContractParams& prm, int grid, cudaStream_t s) {
 }
 
 }  // namespace
+
+size_t df_contract_smem_bytes(int P, int rn, int n_pairs) {
+  const int xc = fp64_sites_per_chunk(n_pairs);
+  const int kc = xc * n_pairs * 3;
+  return sizeof(double) * 3 * (size_t)kc * (16 * 2 + 16 * rn) + sizeof(double2) * xc * P;
+}
+
+int df_contract_ctas_per_sm(int P, int rn, int n_pairs) {
+  const size_t smem = df_contract_smem_bytes(P, rn, n_pairs);
+  int dev = 0, per_sm_smem = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&per_sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+  int by_smem = (int)(per_sm_smem / (smem + 1024));
+  int ctas = by_smem < 2 ? by_smem : 2;  // __launch_bounds__(256, 2)
+  return ctas < 1 ? 1 : ctas;
+}
 
 cudaError_t launch_contract_df(const ContractParams& prm, int P, int rn, int grid, cudaStream_t s) {
   if (prm.total_units == 0) return cudaSuccess;

@@ -13,10 +13,9 @@
 //   * complex products inside the long sums use the three-multiplication form
 //     (re = k1 - k3, im = k1 + k2 with k1 = c(a+b), k2 = a(d-c), k3 = b(c+d));
 //     the operand-side sums are formed once when a tile is staged in shared memory;
-//   * the spin-pair sum is taken inside the colour singlet, before the phase (the
-//     phase does not depend on the spin pair), so each (d1,d2,d3,x) costs
-//     9*n_pairs + 2 + 4*P FP64 operations instead of n_pairs*(12 + 4P);
-//   * the diquark of a (d1,d2) tile is built once per site and reused for every d3.
+//   * the spin sum is taken inside the colour singlet, in groups of terms that share a
+//     third-quark field, and the momenta along lattice rows (fp64_contract.cuh);
+//   * the diquark of a (d1,d2) tile is built once per site and reused for every d3 of its tile.
 #include "bblock_internal.h"
 #include "fp64_contract.cuh"
 
@@ -157,14 +156,85 @@ cudaError_t launch_project_fp64(const ProjField* d_fields, int n_fields, int row
 
 // ------------------------------------------------------------------ contraction (Eq. 1/3)
 //
-// The body is fp64c::contract_body (fp64_contract.cuh); here the work units come from the
-// context's job table, the third quark from the coefficient-folded line-3 fields and the
-// phases from the cached table.
+// The body is fp64c::contract_rows (fp64_contract.cuh); here the work units come from the
+// context's job table, the fields from the projection (spin coefficients folded) and w^k from
+// the cached table. Measured on GB300 (contraction of one time slice or as stated, ms), against
+// a singlet per (alpha, beta) pair with a phase product per momentum and site:
+//   L = 32, N_dil = 32, 9 momenta, 4 pairs / 2 groups          146.9 -> 55.5
+//   L = 24, N_dil = 32, 3 momenta, 3 pairs / 2 groups, 2 slices 66.9 -> 32.1
+// i.e. 30.9 (21.3) FP64 instructions per output element and site at 0.95-0.97 of the pipe's
+// nominal 1.26 TFLOP/s.
 
-size_t fp64_contract_smem_bytes(int P, int rn, int n_pairs) {
-  const int xc = fp64_sites_per_chunk(n_pairs);
-  const int kc = xc * n_pairs * 3;
-  return sizeof(double) * 3 * (size_t)kc * (16 * 2 + 16 * rn) + sizeof(double2) * xc * P;
+__global__ void k_omega_table(int L, double2* __restrict__ om) {
+  for (int k = threadIdx.x; k < L; k += blockDim.x) {
+    double s, c;
+    sincospi(2.0 * (double)k / (double)L, &s, &c);
+    om[k] = make_double2(c, -s);
+  }
+}
+
+cudaError_t launch_omega_table(int L, double2* om, cudaStream_t s) {
+  k_omega_table<<<1, 128, 0, s>>>(L, om);
+  note_launch();
+  return cudaGetLastError();
+}
+
+int plan_rows(int L, const int32_t* momenta, int n_mom, RowPlan* out, int max_out) {
+  auto md = [L](int v) { const int m = v % L; return m < 0 ? m + L : m; };
+  auto cls = [&](int p, int axis) {   // |n0| in [0, L / 2]
+    const int n = md(momenta[3 * p + axis]);
+    return n < L - n ? n : L - n;
+  };
+  int axis = 2, fewest = 1 << 30;
+  for (int a = 2; a >= 0; --a) {
+    bool seen[65] = {};               // |n0| <= L / 2 <= 64
+    int n = 0;
+    for (int p = 0; p < n_mom; ++p) {
+      const int k = cls(p, a) % 65;
+      if (k && !seen[k]) { seen[k] = true; ++n; }
+    }
+    if (n < fewest) { fewest = n; axis = a; }
+  }
+  int n_plans = 0;
+  // plan of each class: classes in order of appearance, kMaxRowCls to a plan; the momenta of
+  // class 0 join the first plan; a plan that is full of momenta continues in another
+  int order[65], n_order = 0;
+  for (int p = 0; p < n_mom; ++p) {
+    const int k = cls(p, axis);
+    bool have = k == 0;
+    for (int i = 0; i < n_order; ++i) have = have || order[i] == k;
+    if (!have && n_order < 65) order[n_order++] = k;
+  }
+  for (int first = 0; first == 0 || first < n_order; first += kMaxRowCls) {
+    RowPlan pl{};
+    auto start = [&] {
+      pl = RowPlan{};
+      pl.axis = axis;
+      for (int i = first; i < n_order && i < first + kMaxRowCls; ++i) pl.cls_n0[pl.n_cls++] = order[i];
+    };
+    auto flush = [&] {
+      if (out && n_plans < max_out) out[n_plans] = pl;
+      ++n_plans;
+    };
+    start();
+    const int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
+    for (int p = 0; p < n_mom; ++p) {
+      const int k = cls(p, axis);
+      int sel = 0;
+      if (k == 0) {
+        if (first != 0) continue;
+      } else {
+        for (int c = 0; c < pl.n_cls; ++c)
+          if (pl.cls_n0[c] == k) sel = md(momenta[3 * p + axis]) == k ? c + 1 : -(c + 1);
+        if (sel == 0) continue;
+      }
+      if (pl.n_mom == kMaxRowP) { flush(); start(); }
+      pl.mom[pl.n_mom++] = RowMom{p, md(momenta[3 * p + a1]), md(momenta[3 * p + a2]), sel};
+      if (sel == 0) pl.has_zero = 1;
+    }
+    if (pl.n_mom > 0) flush();
+  }
+  return n_plans;
 }
 
 struct TableSource {
@@ -172,67 +242,54 @@ struct TableSource {
   __device__ const ContractJob& job(long long u) const {
     return prm->jobs[fp64c::find_job(prm->jobs, prm->n_jobs, u)];
   }
-  __device__ double2 third(const ContractJob& J, int pr, int x, int c, int n) const {
-    return J.q3[pr][((size_t)x * 3 + c) * J.nd3 + n];
+  __device__ void uv(const ContractJob& J, int t, int x, int d1, int d2, double2 (&u)[3],
+                     double2 (&v)[3]) const {
+    const double2* a = J.q1[prm->a_slot[t]] + (size_t)x * 3 * J.nd1 + d1;
+    const double2* b = J.q2[prm->b_slot[t]] + (size_t)x * 3 * J.nd2 + d2;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      u[c] = a[c * J.nd1];
+      v[c] = b[c * J.nd2];
+    }
   }
-  __device__ double2 phase(int p, int x) const {
-    return prm->phase[(size_t)(prm->p0 + p) * prm->X + x];
+  __device__ double2 third(const ContractJob& J, int g, int x, int c, int n) const {
+    return J.q3[g][((size_t)x * 3 + c) * J.nd3 + n];
   }
+  __device__ double2 omega(int k) const { return prm->phase[k]; }
 };
 
-template <int P, int RM, int RN>
-__global__ void __launch_bounds__(kThreads, 2) k_contract_fp64(const __grid_constant__ ContractParams prm) {
-  fp64c::contract_body<P, RM, RN>(prm, TableSource{&prm});
+template <int NCLS, int RN>
+__global__ void __launch_bounds__(kThreads, RN == 4 || NCLS >= 2 ? 1 : 2)
+k_contract_fp64(const __grid_constant__ ContractParams prm) {
+  fp64c::contract_rows<NCLS, kRowRM, RN>(prm, TableSource{&prm});
 }
 
-template <int P, int RN>
-static cudaError_t launch_contract_p(const ContractParams& prm, int grid, cudaStream_t s) {
-  const size_t smem = fp64_contract_smem_bytes(P, RN, prm.n_pairs);
-  cudaError_t e = cudaFuncSetAttribute(k_contract_fp64<P, 2, RN>,
+template <int NCLS, int RN>
+static cudaError_t launch_rows_c(const ContractParams& prm, int grid, cudaStream_t s) {
+  const size_t smem = rows_smem_bytes(prm.L, NCLS, RN, prm.n_groups, prm.xc);
+  cudaError_t e = cudaFuncSetAttribute(k_contract_fp64<NCLS, RN>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
-  k_contract_fp64<P, 2, RN><<<grid, kThreads, smem, s>>>(prm);
+  k_contract_fp64<NCLS, RN><<<grid, kThreads, smem, s>>>(prm);
   note_launch();
   return cudaGetLastError();
 }
 
-// (P, RN) instantiations: RN = 2 only for P <= 4 (register budget of 128 per thread);
-// RN = 1 up to P = 10, the largest momentum group that runs without spills.
-cudaError_t launch_contract_fp64(const ContractParams& prm, int P, int rn, int grid,
-                                 cudaStream_t s) {
-  if (prm.total_units == 0) return cudaSuccess;
-  if (rn == 2) {
-    switch (P) {
-      case 1: return launch_contract_p<1, 2>(prm, grid, s);
-      case 2: return launch_contract_p<2, 2>(prm, grid, s);
-      case 3: return launch_contract_p<3, 2>(prm, grid, s);
-      case 4: return launch_contract_p<4, 2>(prm, grid, s);
-      default: return cudaErrorInvalidValue;
-    }
-  }
-  switch (P) {
-    case 1: return launch_contract_p<1, 1>(prm, grid, s);
-    case 2: return launch_contract_p<2, 1>(prm, grid, s);
-    case 3: return launch_contract_p<3, 1>(prm, grid, s);
-    case 4: return launch_contract_p<4, 1>(prm, grid, s);
-    case 5: return launch_contract_p<5, 1>(prm, grid, s);
-    case 6: return launch_contract_p<6, 1>(prm, grid, s);
-    case 7: return launch_contract_p<7, 1>(prm, grid, s);
-    case 8: return launch_contract_p<8, 1>(prm, grid, s);
-    case 9: return launch_contract_p<9, 1>(prm, grid, s);
-    case 10: return launch_contract_p<10, 1>(prm, grid, s);
+cudaError_t launch_contract_fp64(const ContractParams& prm, int rn, int grid, cudaStream_t s) {
+  if (prm.total_units == 0 || prm.rows.n_mom == 0) return cudaSuccess;
+  switch (prm.rows.n_cls * 8 + rn) {
+    case 0 + 1: return launch_rows_c<0, 1>(prm, grid, s);
+    case 0 + 2: return launch_rows_c<0, 2>(prm, grid, s);
+    case 0 + 4: return launch_rows_c<0, 4>(prm, grid, s);
+    case 8 + 1: return launch_rows_c<1, 1>(prm, grid, s);
+    case 8 + 2: return launch_rows_c<1, 2>(prm, grid, s);
+    case 8 + 4: return launch_rows_c<1, 4>(prm, grid, s);
+    case 16 + 1: return launch_rows_c<2, 1>(prm, grid, s);
+    case 16 + 2: return launch_rows_c<2, 2>(prm, grid, s);
+    case 24 + 1: return launch_rows_c<3, 1>(prm, grid, s);
+    case 24 + 2: return launch_rows_c<3, 2>(prm, grid, s);
     default: return cudaErrorInvalidValue;
   }
-}
-
-int fp64_contract_ctas_per_sm(int P, int rn, int n_pairs) {
-  const size_t smem = fp64_contract_smem_bytes(P, rn, n_pairs);
-  int dev = 0, per_sm_smem = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&per_sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-  int by_smem = (int)(per_sm_smem / (smem + 1024));
-  int ctas = by_smem < 2 ? by_smem : 2;  // __launch_bounds__(256, 2)
-  return ctas < 1 ? 1 : ctas;
 }
 
 // ------------------------------------------------------------------ slab reduction

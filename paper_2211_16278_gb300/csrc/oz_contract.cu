@@ -213,7 +213,7 @@ __device__ __forceinline__ OzUnit decode(const ContractParams& prm, long long u)
   w.slab = (int)(r / J.n_tiles);
   w.x_begin = w.slab * prm.sites_per_slab;
   w.x_end = min(prm.X, w.x_begin + prm.sites_per_slab);
-  const long long k_total = (long long)(w.x_end - w.x_begin) * prm.n_pairs * 3;
+  const long long k_total = (long long)(w.x_end - w.x_begin) * prm.n_groups * 3;
   w.n_stages = w.slab < prm.n_slab ? (int)((k_total + kK - 1) / kK) : 0;
   return w;
 }
@@ -248,7 +248,7 @@ __device__ __forceinline__ void oz_produce(const ContractParams& prm, const OzSh
   constexpr int kRW = 32 * E / kK;          // rows per warp (diquark)
   constexpr int kSegs = kK / E;             // K segments per row
   const int NC = prm.NC;
-  const int np = prm.n_pairs;
+  const int np = prm.n_groups;
   const long long u0 = blockIdx.x / C, du = gridDim.x / C;
   int rr, seg, a_g0 = 0, a_ng = 0;
   bool row_used;
@@ -486,7 +486,7 @@ k_contract_oz(const __grid_constant__ ContractParams prm) {
 
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   const int NC = prm.NC;
-  const int np = prm.n_pairs;
+  const int np = prm.n_groups;
   const uint32_t rank = C > 1 ? cluster_rank() : 0u;
   const int gb = group_begin((int)rank, C), ge = group_begin((int)rank + 1, C);
   // transaction bytes the peers' diquark row groups bring into each stage
@@ -760,7 +760,7 @@ __global__ void __launch_bounds__(128) k_oz_rowmax(const __grid_constant__ Contr
       slab = s;
       mxv = 0.f;
     }
-    for (int pr = 0; pr < prm.n_pairs; ++pr) {
+    for (int pr = 0; pr < prm.n_groups; ++pr) {
       const float4* uq = reinterpret_cast<const float4*>(J.q1[prm.a_slot[pr]]) + (size_t)x * 3 * nd1 + d1;
       const float4* vq = reinterpret_cast<const float4*>(J.q2[prm.b_slot[pr]]) + (size_t)x * 3 * nd2 + d2;
       float2 u[3], v[3];
@@ -833,8 +833,8 @@ cudaError_t launch_oz_c(const ContractParams& prm, int grid, cudaStream_t s) {
 // grid: units wanted at once (clusters of `cluster` CTAs), capped at what is resident
 cudaError_t launch_contract_oz(const ContractParams& prm, int cluster, int grid, cudaStream_t s) {
   if (prm.total_units == 0) return cudaSuccess;
-  if (prm.NC < 16 || prm.NC > kOzMaxNC || prm.NC % 16 != 0 || prm.n_pairs < 1 ||
-      prm.n_pairs > kMaxPairs)
+  if (prm.NC < 16 || prm.NC > kOzMaxNC || prm.NC % 16 != 0 || prm.n_groups < 1 ||
+      prm.n_groups > kMaxPairs)
     return cudaErrorInvalidValue;
   switch (cluster) {
     case 1: return launch_oz_c<1>(prm, grid, s);
