@@ -413,8 +413,8 @@ GroupPlan plan_groups(const SpinPlan& sp, bool may_group, const std::vector<JobI
 }
 
 int ensure_phase(bblock_ctx* c, const int32_t* momenta, int n_mom, cudaStream_t s) {
-  if (c->cfg.precision == BBLOCK_FP64) {
-    // the FP64 contraction needs w^k = e^{-2 pi i k / L} only, whatever the momenta
+  if (c->cfg.precision == BBLOCK_FP64 || c->cfg.precision == BBLOCK_DF64) {
+    // these contractions need w^k = e^{-2 pi i k / L} only, whatever the momenta
     if (c->d_phase) return BBLOCK_OK;
     int rc = grow_device(c, reinterpret_cast<char**>(&c->d_phase), &c->phase_cap,
                          sizeof(double2) * c->cfg.L);
@@ -1138,15 +1138,15 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
   const bool df = c->cfg.precision == BBLOCK_DF64 || oz;
 
   const int X = c->X, rows = c->rows, n_ev = c->cfg.n_ev, L = c->cfg.L;
-  const bool f64 = c->cfg.precision == BBLOCK_FP64;
+  const bool rowf = !oz;   // FP64 and double-float: the row-factored contraction
   int max_nd3_all = 1;
   for (const JobIn& j : jobs) max_nd3_all = std::max(max_nd3_all, j.nd[2]);
-  const GroupPlan gp = plan_groups(sp, f64, jobs, n_ev, f64 ? 64 : 32);
+  const GroupPlan gp = plan_groups(sp, rowf, jobs, n_ev, rowf ? 64 : 32);
   const int n2_fields = (int)gp.f2.size(), n3_fields = gp.n_groups * sp.n_coef_sets;
-  // FP64 form: the momenta in row plans (per-momentum coefficients: one plan per momentum)
+  // the momenta in row plans (per-momentum coefficients: one plan per momentum)
   std::vector<RowPlan> rplans;
   int r_cls = 0;
-  if (f64) {
+  if (rowf) {
     if (per_mom) {
       rplans.resize(n_mom);
       for (int p = 0; p < n_mom; ++p) {
@@ -1160,14 +1160,10 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
     for (const RowPlan& r : rplans) r_cls = std::max(r_cls, r.n_cls);
   }
   const int row_rn = rows_rn_for(r_cls, max_nd3_all);
-  // momenta per contraction launch: the Ozaki form takes them all as N columns
-  const int P_launch = per_mom ? 1 : oz ? n_mom : p_group_size(n_mom, kMaxPGroupDf);
-  const int xc = oz ? 1 : fp64_sites_per_chunk(sp.n_pairs);
-  // one tile shape for every launch of the call
-  const Fp64Tile tl = f64 ? Fp64Tile{kRowRM, row_rn} : fp64_tile_for(oz ? 1 : P_launch);
+  // Ozaki form: every momentum of a launch as N columns
+  const int P_launch = per_mom ? 1 : n_mom;
   // Ozaki form: units run one per CTA (clusters: one per cluster of oz_cl CTAs)
-  const int ctas = (oz ? 1 : f64 ? rows_ctas_per_sm(rplans[0].n_cls, row_rn)
-                                 : df_contract_ctas_per_sm(P_launch, tl.rn, sp.n_pairs)) * c->num_sms;
+  const int ctas = (oz ? 1 : rows_ctas_per_sm(rplans[0].n_cls, row_rn)) * c->num_sms;
   const int max_slabs = 64;
   const int oz_nc = c->opt_tc_nc > 0 && c->opt_tc_nc <= kOzMaxNC ? c->opt_tc_nc : kOzMaxNC;
   int oz_cl = 1;   // Ozaki form: CTAs per cluster of the current wave
@@ -1177,8 +1173,8 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
       mt = (j.nd[0] * j.nd[1] + kOzM - 1) / kOzM;
       nt = ((P_launch * j.nd[2] + oz_nc - 1) / oz_nc + oz_cl - 1) / oz_cl;
     } else {
-      mt = (j.nd[0] * j.nd[1] + 16 * tl.rm - 1) / (16 * tl.rm);
-      nt = (j.nd[2] + 16 * tl.rn - 1) / (16 * tl.rn);
+      mt = (j.nd[0] * j.nd[1] + 16 * kRowRM - 1) / (16 * kRowRM);
+      nt = (j.nd[2] + 16 * row_rn - 1) / (16 * row_rn);
     }
   };
   // Ozaki form: the column and row maxima of every job, [n_slab][nd1 + nd2 + nd3] and
@@ -1231,14 +1227,13 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
       max_elems = std::max(max_elems, (long long)n_mom * j.nd[0] * j.nd[1] * j.nd[2]);
     }
     const int unit_slots = oz ? ctas / oz_cl : ctas;
-    // FP64 form: slabs are ranges of lattice rows; the others: of chunks of xc sites
-    const int parts = f64 ? L * L : X, step = f64 ? 1 : xc;
-    int n_slab = c->opt_slabs > 0 ? std::min(c->opt_slabs, (parts + step - 1) / step)
-                                   : choose_slabs(tiles, unit_slots, parts, step, max_slabs);
-    int per_slab = (parts + n_slab - 1) / n_slab;
-    per_slab = (per_slab + step - 1) / step * step;
+    // slabs are ranges of lattice rows (Ozaki form: of sites)
+    const int parts = oz ? X : L * L;
+    int n_slab = c->opt_slabs > 0 ? std::min(c->opt_slabs, parts)
+                                   : choose_slabs(tiles, unit_slots, parts, 1, max_slabs);
+    const int per_slab = (parts + n_slab - 1) / n_slab;
     n_slab = (parts + per_slab - 1) / per_slab;
-    const int sites_per_slab = f64 ? per_slab * L : per_slab;
+    const int sites_per_slab = oz ? per_slab : per_slab * L;
 
     size_t ws_need = 0, oz_need = 0;
     for (size_t k = job_idx; k < end; ++k) {
@@ -1437,7 +1432,6 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
     prm.NC = oz_nc;
     prm.wait_limit = c->opt_wait_us > 0 ? (long long)c->opt_wait_us * c->cycles_per_us
                                         : 4000000000LL;
-    const int grid = (int)std::min<long long>(unit, ctas);
     if (oz) {
       // the diquark's row maxima (from the line-1 and line-2 fields of any coefficient set)
       int max_mt = 0;
@@ -1454,21 +1448,15 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
           return launch_contract_oz(prm, oz_cl, (int)std::min<long long>(unit, unit_slots), s);
         }));
       }
-    } else if (f64) {
+    } else {
       for (size_t k = 0; k < rplans.size(); ++k) {
         prm.jobs = reinterpret_cast<const ContractJob*>(c->d_tab + fbytes + jbytes * (per_mom ? k : 0));
         prm.rows = rplans[k];
         prm.xc = rows_sites_per_chunk(L, prm.rows.n_cls, row_rn, gp.n_groups);
-        const int g64 = (int)std::min<long long>(unit, (long long)rows_ctas_per_sm(prm.rows.n_cls, row_rn) * c->num_sms);
-        CK(c, timed_launch(c, K_CONTRACT, s, [&] { return launch_contract_fp64(prm, row_rn, g64, s); }));
-      }
-    } else {
-      const int pg = P_launch;
-      for (int p0 = 0; p0 < n_mom; p0 += pg) {
-        prm.jobs = reinterpret_cast<const ContractJob*>(c->d_tab + fbytes + jbytes * (per_mom ? p0 : 0));
-        prm.p0 = p0;
+        const int grid = (int)std::min<long long>(
+            unit, (long long)rows_ctas_per_sm(prm.rows.n_cls, row_rn) * c->num_sms);
         CK(c, timed_launch(c, K_CONTRACT, s, [&] {
-          return launch_contract_df(prm, std::min(pg, n_mom - p0), tl.rn, grid, s);
+          return df ? launch_contract_df(prm, row_rn, grid, s) : launch_contract_fp64(prm, row_rn, grid, s);
         }));
       }
     }
@@ -1627,20 +1615,16 @@ CallPlan plan_call(const bblock_ctx* c, int n_t, const int nd[3], int n_mom, int
     return pl;
   }
   if (fp64_like(c->cfg)) {
-    const bool f64 = c->cfg.precision == BBLOCK_FP64;
-    const int P = p_group_size(n_mom, kMaxPGroupDf);
-    const Fp64Tile tl = f64 ? Fp64Tile{kRowRM, rows_rn_for(1, nd[2])} : fp64_tile_for(P);
-    const int xc = f64 ? 1 : fp64_sites_per_chunk(pairs);
-    const int parts = f64 ? c->cfg.L * c->cfg.L : X;   // slabs of lattice rows, or of sites
-    const int ctas = (f64 ? rows_ctas_per_sm(1, tl.rn) : df_contract_ctas_per_sm(P, tl.rn, pairs)) * c->num_sms;
-    const long long tiles = (long long)n_t * ((nd[0] * nd[1] + 16 * tl.rm - 1) / (16 * tl.rm)) *
-                            ((nd[2] + 16 * tl.rn - 1) / (16 * tl.rn));
-    int ns = slabs_opt > 0 ? std::min(slabs_opt, (parts + xc - 1) / xc) : choose_slabs(tiles, ctas, parts, xc, 64);
-    int sps = (parts + ns - 1) / ns;
-    sps = (sps + xc - 1) / xc * xc;
+    const int rn = rows_rn_for(1, nd[2]);
+    const int parts = c->cfg.L * c->cfg.L;   // slabs of lattice rows
+    const long long tiles = (long long)n_t * ((nd[0] * nd[1] + 16 * kRowRM - 1) / (16 * kRowRM)) *
+                            ((nd[2] + 16 * rn - 1) / (16 * rn));
+    const int ns = slabs_opt > 0 ? std::min(slabs_opt, parts)
+                                 : choose_slabs(tiles, rows_ctas_per_sm(1, rn) * c->num_sms, parts, 1, 64);
+    const int sps = (parts + ns - 1) / ns;
     pl.n_slab = (parts + sps - 1) / sps;
     pl.units = tiles * pl.n_slab;
-    pl.pad = (double)(((nd[2] + 16 * tl.rn - 1) / (16 * tl.rn)) * 16 * tl.rn) / nd[2] - 1.0;
+    pl.pad = (double)((nd[2] + 15) / 16 * 16) / nd[2] - 1.0;   // idle 16-column blocks are skipped
     return pl;
   }
   const int G = tc_groups_per_stage(tc_form_of(c->cfg));

@@ -12,18 +12,9 @@ constexpr int kMaxPairs = 16;   // distinct (alpha, beta) spin pairs
 constexpr int kMaxRfP = 16;
 constexpr int kMaxRfIdx = 8;
 constexpr int kMaxRfL = 128;    // lattice extent (the w^k table follows the stage buffers)
-// Momenta handled by one contraction launch of the double-float form: the largest count whose
-// accumulators fit the registers without spills.
-constexpr int kMaxPGroupDf = 8;
-// Row-factored FP64 contraction: momenta and +-n0 classes of one launch.
+// Row-factored FP64 and double-float contractions: momenta and +-n0 classes of one launch.
 constexpr int kMaxRowP = 32;
 constexpr int kMaxRowCls = 3;
-// Momenta of the first launch: n_mom split into the fewest groups of at most max_group, as
-// evenly as possible (each launch recomputes the colour singlet that its momenta share).
-inline int p_group_size(int n_mom, int max_group) {
-  const int groups = (n_mom + max_group - 1) / max_group;
-  return groups > 0 ? (n_mom + groups - 1) / groups : 0;
-}
 constexpr int kThreads = 256;   // threads per CTA of the FP64 kernels
 
 // Kernel launches made by the calling host thread, counted at every launch site of the
@@ -112,11 +103,11 @@ struct ContractParams {
   int tbeg[kMaxPairs + 1];
   int a_slot[kMaxPairs];         // term -> line-1 slot
   int b_slot[kMaxPairs];         // term -> line-2 field
-  // FP64 form: lattice extent, rows (of L^2) per slab, sites of a row staged at a time
+  // FP64 and double-float forms: lattice extent, rows (of L^2) per slab, sites of a row staged at a time
   int L, rows_per_slab, xc;
   RowPlan rows;
-  const double2* phase;          // [P_total][X]
-  int p0;                        // first momentum of this launch
+  const double2* phase;          // w^k = e^{-2 pi i k / L}, k = 0..L-1
+  int p0;                        // Ozaki form: first momentum of this launch
   int P_total;
   int* status;
   // Ozaki form: the phases as double-float float4 (re.h, re.l, im.h, im.l), [P_total][X];
@@ -128,14 +119,7 @@ struct ContractParams {
   long long wait_limit;
 };
 
-// Tiles of the double-float contraction for a momentum count (per launch).
-struct Fp64Tile { int rm, rn; };
-inline Fp64Tile fp64_tile_for(int P) { return P <= 4 ? Fp64Tile{2, 2} : Fp64Tile{2, 1}; }
-inline int fp64_sites_per_chunk(int n_pairs) { return n_pairs >= 16 ? 1 : 16 / n_pairs; }
-size_t df_contract_smem_bytes(int P, int rn, int n_pairs);
-int df_contract_ctas_per_sm(int P, int rn, int n_pairs);
-
-// Tiles of the row-factored FP64 contraction: 16 kRowRM (d1, d2) pairs by 16 rn d3 columns.
+// Tiles of the row-factored FP64 and double-float contractions: 16 kRowRM (d1, d2) pairs by 16 rn d3 columns.
 // A wider d3 tile shares each diquark among more outputs; the row sums of the launch's classes
 // limit it (registers). One CTA per SM for the tiles that need more than 128 registers.
 constexpr int kRowRM = 2;
@@ -306,7 +290,7 @@ cudaError_t launch_omega_table(int L, double2* om, cudaStream_t s);
 cudaError_t launch_contract_fp64(const ContractParams& p, int rn, int grid, cudaStream_t s);
 // Double-float form: same units, tiles, shared memory and partial layout as the FP64
 // contraction; fields hold double-float pairs (float4 per complex element).
-cudaError_t launch_contract_df(const ContractParams& p, int P, int rn, int grid, cudaStream_t s);
+cudaError_t launch_contract_df(const ContractParams& p, int rn, int grid, cudaStream_t s);
 
 // One input array of a call converted to double-float planes: n complex128 elements
 // from src to float4 (re.h, re.l, im.h, im.l) at dst.

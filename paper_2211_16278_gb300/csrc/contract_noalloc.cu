@@ -7,7 +7,7 @@
 
 #include "../../include/bblock.h"
 #include "bblock_internal.h"
-#include "fp64_contract.cuh"
+#include "rows_contract.cuh"
 
 namespace bb {
 namespace {
@@ -43,6 +43,7 @@ struct NoallocParams {
 // Where the shared body's inputs come from without a context: the single job of the launch,
 // the spin coefficients folded while the tile is staged, and w^k by sincospi.
 struct NoallocSource {
+  using Cx = rowsc::ArithF64::Cx;
   const NoallocParams* np;
   __device__ const ContractJob& job(long long) const { return np->job; }
   __device__ static double2 fold(const NaFold& f, const double2* q, size_t spin_stride, size_t at) {
@@ -56,31 +57,31 @@ struct NoallocSource {
     }
     return b;
   }
-  __device__ void uv(const ContractJob& J, int t, int x, int d1, int d2, double2 (&u)[3],
-                     double2 (&v)[3]) const {
+  __device__ void uv(const ContractJob& J, int t, int x, int d1, int d2, Cx (&u)[3],
+                     Cx (&v)[3]) const {
     const double2* a = J.q1[np->base.a_slot[t]] + (size_t)x * 3 * J.nd1 + d1;
     const size_t b = (size_t)x * 3 * J.nd2 + d2, st = (size_t)np->base.X * 3 * J.nd2;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      u[c] = a[c * J.nd1];
-      v[c] = fold(np->f2[t], np->q2, st, b + c * J.nd2);
+      u[c] = rowsc::ArithF64::load(a + c * J.nd1);
+      v[c] = rowsc::ArithF64::cx(fold(np->f2[t], np->q2, st, b + c * J.nd2));
     }
   }
-  __device__ double2 third(const ContractJob& J, int g, int x, int c, int n) const {
-    return fold(np->f3[g], np->q3, (size_t)np->base.X * 3 * J.nd3,
-                ((size_t)x * 3 + c) * J.nd3 + n);
+  __device__ Cx third(const ContractJob& J, int g, int x, int c, int n) const {
+    return rowsc::ArithF64::cx(fold(np->f3[g], np->q3, (size_t)np->base.X * 3 * J.nd3,
+                                    ((size_t)x * 3 + c) * J.nd3 + n));
   }
-  __device__ double2 omega(int k) const {
+  __device__ Cx omega(int k) const {
     double sn, cs;
     sincospi(2.0 * (double)k / (double)np->base.L, &sn, &cs);
-    return make_double2(cs, -sn);
+    return Cx{cs, -sn};
   }
 };
 
 template <int NCLS, int RN>
 __global__ void __launch_bounds__(kThreads, RN == 4 || NCLS >= 2 ? 1 : 2)
 k_contract_fp64_noalloc(const __grid_constant__ NoallocParams prm) {
-  fp64c::contract_rows<NCLS, kRowRM, RN>(prm.base, NoallocSource{&prm});
+  rowsc::contract_rows<rowsc::ArithF64, NCLS, kRowRM, RN>(prm.base, NoallocSource{&prm});
 }
 
 // B[e] = sum over slabs of partial[slab][e], slabs in index order.

@@ -14,10 +14,10 @@
 //     (re = k1 - k3, im = k1 + k2 with k1 = c(a+b), k2 = a(d-c), k3 = b(c+d));
 //     the operand-side sums are formed once when a tile is staged in shared memory;
 //   * the spin sum is taken inside the colour singlet, in groups of terms that share a
-//     third-quark field, and the momenta along lattice rows (fp64_contract.cuh);
+//     third-quark field, and the momenta along lattice rows (rows_contract.cuh);
 //   * the diquark of a (d1,d2) tile is built once per site and reused for every d3 of its tile.
 #include "bblock_internal.h"
-#include "fp64_contract.cuh"
+#include "rows_contract.cuh"
 
 namespace bb {
 
@@ -156,7 +156,7 @@ cudaError_t launch_project_fp64(const ProjField* d_fields, int n_fields, int row
 
 // ------------------------------------------------------------------ contraction (Eq. 1/3)
 //
-// The body is fp64c::contract_rows (fp64_contract.cuh); here the work units come from the
+// The body is rowsc::contract_rows (rows_contract.cuh); here the work units come from the
 // context's job table, the fields from the projection (spin coefficients folded) and w^k from
 // the cached table. Measured on GB300 (contraction of one time slice or as stated, ms), against
 // a singlet per (alpha, beta) pair with a phase product per momentum and site:
@@ -237,31 +237,10 @@ int plan_rows(int L, const int32_t* momenta, int n_mom, RowPlan* out, int max_ou
   return n_plans;
 }
 
-struct TableSource {
-  const ContractParams* prm;
-  __device__ const ContractJob& job(long long u) const {
-    return prm->jobs[fp64c::find_job(prm->jobs, prm->n_jobs, u)];
-  }
-  __device__ void uv(const ContractJob& J, int t, int x, int d1, int d2, double2 (&u)[3],
-                     double2 (&v)[3]) const {
-    const double2* a = J.q1[prm->a_slot[t]] + (size_t)x * 3 * J.nd1 + d1;
-    const double2* b = J.q2[prm->b_slot[t]] + (size_t)x * 3 * J.nd2 + d2;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      u[c] = a[c * J.nd1];
-      v[c] = b[c * J.nd2];
-    }
-  }
-  __device__ double2 third(const ContractJob& J, int g, int x, int c, int n) const {
-    return J.q3[g][((size_t)x * 3 + c) * J.nd3 + n];
-  }
-  __device__ double2 omega(int k) const { return prm->phase[k]; }
-};
-
 template <int NCLS, int RN>
 __global__ void __launch_bounds__(kThreads, RN == 4 || NCLS >= 2 ? 1 : 2)
 k_contract_fp64(const __grid_constant__ ContractParams prm) {
-  fp64c::contract_rows<NCLS, kRowRM, RN>(prm, TableSource{&prm});
+  rowsc::contract_rows<rowsc::ArithF64, NCLS, kRowRM, RN>(prm, rowsc::TableSource<rowsc::ArithF64>{&prm});
 }
 
 template <int NCLS, int RN>

@@ -62,7 +62,7 @@ def rel(a, b):
 
 @pytest.mark.parametrize("slabs", [0, 1])
 @pytest.mark.parametrize("name", CASES)
-@pytest.mark.parametrize("form", ["fp64"])
+@pytest.mark.parametrize("form", ["fp64", "df64"])
 def test_matches_oracle(env, form, name, slabs):
     torch, bb = env
     L, n_ev, nd, mom, spins, coeffs = CASES[name]
