@@ -295,6 +295,7 @@ struct JobIn {
   const double2* phi[3];
   int nd[3];
   double2* B;
+  bool tri = false;   // mode triplet of V in a row-factored form: antisymmetric, phi not read
 };
 
 // Spin operator of Eq. (1) reduced to what the kernels consume.
@@ -1114,6 +1115,107 @@ int oz_cluster_for(const bblock_ctx* c, const std::vector<JobIn>& jobs, size_t b
   return tiles > 0 && (double)(padded - tiles) / tiles <= 0.2 ? 2 : 1;
 }
 
+// The mode triplet of every job's V in the FP64 or double-float form: the ordered elements
+// l1 < l2 < l3 by the row-factored contraction, then T by its antisymmetry.
+int run_triplet(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momenta, int n_mom,
+                cudaStream_t s) {
+  const int L = c->cfg.L, rows = c->rows, n = c->cfg.n_ev, X = c->X;
+  const bool df = c->cfg.precision == BBLOCK_DF64;
+  const int M = n * (n - 1) / 2;
+  std::vector<RowPlan> rplans(plan_rows(L, momenta, n_mom, nullptr, 0));
+  plan_rows(L, momenta, n_mom, rplans.data(), (int)rplans.size());
+  int r_cls = 0;
+  for (const RowPlan& r : rplans) r_cls = std::max(r_cls, r.n_cls);
+  const int rn = rows_rn_for(r_cls, n);
+  const int m_tiles = (M + 16 * kRowRM - 1) / (16 * kRowRM), n_tiles = (n + 16 * rn - 1) / (16 * rn);
+  const int max_slabs = 64;
+  const size_t f_bytes = align_up((size_t)rows * n * sizeof(double2), 256);
+  const size_t c_bytes = align_up((size_t)n_mom * M * n * sizeof(double2), 256);
+  const size_t b_bytes = align_up((size_t)n * sizeof(int), 256);
+  auto job_bytes = [&](int n_slab) {
+    return f_bytes + b_bytes + c_bytes + align_up((size_t)n_slab * n_mom * M * n * sizeof(double2), 256);
+  };
+  for (size_t job_idx = 0; job_idx < jobs.size();) {
+    const size_t fit = std::max<size_t>(1, wave_budget(c) / job_bytes(max_slabs));
+    const size_t end = std::min(jobs.size(), job_idx + fit);
+    const int nj = (int)(end - job_idx);
+    ++c->last_waves;
+    const long long tiles = std::max(1LL, (long long)nj * m_tiles * n_tiles);
+    int n_slab = c->opt_slabs > 0 ? std::min(c->opt_slabs, L * L)
+                                  : choose_slabs(tiles, rows_ctas_per_sm(rplans[0].n_cls, rn) * c->num_sms,
+                                                 L * L, 1, max_slabs);
+    const int per_slab = (L * L + n_slab - 1) / n_slab;
+    n_slab = (L * L + per_slab - 1) / per_slab;
+    int rc = grow_device(c, &c->d_ws, &c->ws_cap, nj * job_bytes(n_slab));
+    if (rc) return rc;
+    std::vector<ContractJob> cjobs(nj);
+    std::vector<TriSlice> slices(nj);
+    // the flags of every slice first (one memset), then each slice's blocks
+    char* base = c->d_ws + nj * b_bytes;
+    for (int k = 0; k < nj; ++k) {
+      TriSlice& sl = slices[k];
+      ContractJob& cj = cjobs[k];
+      sl.V = jobs[job_idx + k].V;
+      sl.T = jobs[job_idx + k].B;
+      sl.bad = reinterpret_cast<int*>(c->d_ws + k * b_bytes);
+      sl.field = reinterpret_cast<double2*>(base);
+      base += f_bytes;
+      cj.B = reinterpret_cast<double2*>(base);
+      sl.compact = cj.B;
+      base += c_bytes;
+      cj.partial = reinterpret_cast<double2*>(base);
+      base += align_up((size_t)n_slab * n_mom * M * n * sizeof(double2), 256);
+      cj.q1[0] = cj.q2[0] = cj.q3[0] = sl.field;
+      cj.nd1 = cj.nd2 = cj.nd3 = n;
+      cj.tri = 1;
+      cj.m_tiles = m_tiles;
+      cj.n_tiles = n_tiles;
+      cj.unit_begin = (long long)k * m_tiles * n_tiles * n_slab;
+    }
+    if (!within_workspace(c, c->d_ws, base - c->d_ws))
+      return fail(c, BBLOCK_ERR_INVALID_ARG, "internal: triplet blocks outside the workspace");
+    const size_t sofs = align_up((size_t)nj * sizeof(ContractJob), 256);
+    std::vector<char> tab(sofs + (size_t)nj * sizeof(TriSlice));
+    memcpy(tab.data(), cjobs.data(), (size_t)nj * sizeof(ContractJob));
+    memcpy(tab.data() + sofs, slices.data(), (size_t)nj * sizeof(TriSlice));
+    rc = upload_tables(c, tab.data(), tab.size(), s);
+    if (rc) return rc;
+    const ContractJob* d_jobs = reinterpret_cast<const ContractJob*>(c->d_tab);
+    const TriSlice* d_slices = reinterpret_cast<const TriSlice*>(c->d_tab + sofs);
+    CK(c, cudaMemsetAsync(c->d_ws, 0, nj * b_bytes, s));
+    CK(c, timed_launch(c, K_PROJECT, s, [&] { return launch_tri_field(d_slices, nj, n, rows, df, s); }));
+    ContractParams prm{};
+    prm.jobs = d_jobs;
+    prm.n_jobs = nj;
+    prm.total_units = (long long)nj * m_tiles * n_tiles * n_slab;
+    prm.X = X;
+    prm.n_slab = n_slab;
+    prm.sites_per_slab = per_slab * L;
+    prm.n_groups = prm.n_terms = 1;
+    prm.tbeg[1] = 1;
+    prm.L = L;
+    prm.rows_per_slab = per_slab;
+    prm.phase = c->d_phase;
+    prm.P_total = n_mom;
+    prm.status = c->d_status;
+    for (const RowPlan& r : rplans) {
+      prm.rows = r;
+      prm.xc = rows_sites_per_chunk(L, r.n_cls, rn, 1);
+      const int grid = (int)std::min<long long>(prm.total_units,
+                                                (long long)rows_ctas_per_sm(r.n_cls, rn) * c->num_sms);
+      CK(c, timed_launch(c, K_CONTRACT, s, [&] {
+        return df ? launch_contract_df(prm, rn, grid, s) : launch_contract_fp64(prm, rn, grid, s);
+      }));
+    }
+    CK(c, timed_launch(c, K_REDUCE, s, [&] {
+      const cudaError_t e = launch_reduce_slabs(d_jobs, nj, n_slab, n_mom, (long long)n_mom * M * n, s);
+      return e != cudaSuccess ? e : launch_tri_fill(d_slices, nj, n, n_mom, s);
+    }));
+    job_idx = end;
+  }
+  return BBLOCK_OK;
+}
+
 int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momenta, int n_mom,
              const int32_t* spin_idx, const double* coeffs, int n_spin, int per_mom,
              cudaStream_t s) {
@@ -1133,6 +1235,7 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
   rc = ensure_phase(c, momenta, n_mom, s);
   if (rc) return rc;
   if (!fp64_like(c->cfg)) return run_jobs_tc(c, jobs, sp, n_mom, per_mom, s);
+  if (jobs[0].tri) return run_triplet(c, jobs, momenta, n_mom, s);
   // the Ozaki form runs on the double-float form's converted inputs and fields
   const bool oz = c->cfg.precision == BBLOCK_OZAKI;
   const bool df = c->cfg.precision == BBLOCK_DF64 || oz;
@@ -1498,7 +1601,8 @@ std::vector<uint64_t> call_signature(const bblock_ctx* c, const std::vector<JobI
     k.push_back(reinterpret_cast<uint64_t>(j.V));
     for (int i = 0; i < 3; ++i) k.push_back(reinterpret_cast<uint64_t>(j.phi[i]));
     k.push_back(reinterpret_cast<uint64_t>(j.B));
-    k.push_back((uint64_t)j.nd[0] | ((uint64_t)j.nd[1] << 20) | ((uint64_t)j.nd[2] << 40));
+    k.push_back((uint64_t)j.nd[0] | ((uint64_t)j.nd[1] << 20) | ((uint64_t)j.nd[2] << 40) |
+                ((uint64_t)j.tri << 60));
   }
   return k;
 }
@@ -1892,6 +1996,7 @@ int bblock_mode_triplet(bblock_ctx* c, int n_t, const void* V, const int32_t* mo
     j.phi[0] = j.phi[1] = j.phi[2] = c->d_ident;
     j.nd[0] = j.nd[1] = j.nd[2] = n_ev;
     j.B = static_cast<double2*>(T_out) + t * tstride;
+    j.tri = !c->opt_checks && (c->cfg.precision == BBLOCK_FP64 || c->cfg.precision == BBLOCK_DF64);
     rc = validate_job(c, j, t, true, n_mom);
     if (rc) return rc;
   }

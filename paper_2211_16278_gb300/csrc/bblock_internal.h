@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <cmath>
 #include <cstdint>
 
 namespace bb {
@@ -73,7 +74,21 @@ struct ContractJob {
   int nd1, nd2, nd3;
   int m_tiles, n_tiles;
   long long unit_begin;          // first global work-unit index of this job
+  // row-factored contractions: 1 where the rows are the pairs l1 < l2 of nd1 = nd2 = nd3 equal
+  // lines (the mode triplet), ordered by l2: m = l2 (l2 - 1) / 2 + l1
+  int tri;
 };
+// (d1, d2) rows of a job's block
+__host__ __device__ inline int job_rows(const ContractJob& j) {
+  return j.tri ? j.nd1 * (j.nd1 - 1) / 2 : j.nd1 * j.nd2;
+}
+// l2 of the triangular row m: the largest l2 with l2 (l2 - 1) / 2 <= m (m < 2^15)
+__host__ __device__ inline int tri_l2(int m) {
+  int l = (int)((1.f + sqrtf(1.f + 8.f * (float)m)) * 0.5f);
+  while (l * (l - 1) / 2 > m) --l;
+  while ((l + 1) * l / 2 <= m) ++l;
+  return l;
+}
 
 // A momentum of a row-factored launch: p = index in the call's list, n1 and n2 = its
 // components along the two axes that are not summed (ascending, reduced to [0, L)), sel = 0
@@ -272,6 +287,21 @@ struct ZgemmParams {
 };
 
 cudaError_t launch_fill_identity(double2* id, int n_ev, cudaStream_t s);
+
+// One time slice of the antisymmetric mode triplet: field[r][l] = V[l][r] (FP64, or
+// double-float float4), bad[l] != 0 where V[l] holds an infinity or a NaN; then T from the
+// compact sums of its l1 < l2 < l3, compact[p][l2 (l2 - 1) / 2 + l1][l3].
+struct TriSlice {
+  const double2* V;              // [n][rows]
+  double2* field;                // [rows][n]
+  int* bad;                      // [n], zeroed before
+  const double2* compact;
+  double2* T;                    // [n_mom][n][n][n]
+};
+cudaError_t launch_tri_field(const TriSlice* d_slices, int n_slices, int n, int rows, bool df,
+                             cudaStream_t s);
+cudaError_t launch_tri_fill(const TriSlice* d_slices, int n_slices, int n, int n_mom,
+                            cudaStream_t s);
 cudaError_t launch_fold_phi(const double2* phi, int n_ev, int nd, const FoldTerms& terms,
                             double2* out, cudaStream_t s);
 cudaError_t launch_zgemm(const ZgemmParams& p, cudaStream_t s);

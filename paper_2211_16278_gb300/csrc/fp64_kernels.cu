@@ -275,7 +275,7 @@ cudaError_t launch_contract_fp64(const ContractParams& prm, int rn, int grid, cu
 
 __global__ void k_reduce_slabs(const ContractJob* __restrict__ jobs, int n_slab, int P_total) {
   const ContractJob& J = jobs[blockIdx.y];
-  const long long per = (long long)P_total * J.nd1 * J.nd2 * J.nd3;
+  const long long per = (long long)P_total * job_rows(J) * J.nd3;
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < per;
        e += (long long)gridDim.x * blockDim.x) {
     double2 s = J.partial[e];

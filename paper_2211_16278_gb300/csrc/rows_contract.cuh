@@ -32,6 +32,8 @@
 // diquark costs 24 operations per term, pair and site for all of the tile's columns.
 #pragma once
 
+#include <type_traits>
+
 #include "bblock_internal.h"
 #include "dfloat.cuh"
 
@@ -163,8 +165,8 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
 
   for (long long u = blockIdx.x; u < prm.total_units; u += gridDim.x) {
     const ContractJob& J = src.job(u);
-    const int nd1 = J.nd1, nd2 = J.nd2, nd3 = J.nd3;
-    const int M = nd1 * nd2;
+    const int nd2 = J.nd2, nd3 = J.nd3;
+    const int M = job_rows(J);
     long long r = u - J.unit_begin;
     const int mt = (int)(r % J.m_tiles);
     r /= J.m_tiles;
@@ -174,14 +176,24 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
       if (tid == 0 && prm.status) atomicOr(prm.status, kStatusBadJob);
       continue;
     }
+    // the tile's first column: with triangular rows (m = (l1, l2), l1 < l2, ordered by l2) only
+    // the 16-column blocks that hold an l3 > l2 of the tile's first row are needed
+    const int col0 = (J.tri ? (tri_l2(mt * MT) + 1) / 16 * 16 : 0) + nt * NT;
+    if (col0 >= nd3) continue;
     const int row_begin = slab * prm.rows_per_slab;
     const int row_end = min(L * L, row_begin + prm.rows_per_slab);
     const int ms = mt * MT + ml;
     const bool m_ok = ms < M;
-    const int d1 = m_ok ? ms / nd2 : 0, d2 = m_ok ? ms - d1 * nd2 : 0;
-    // 16-row and 16-column blocks of the tile that hold outputs: the others are skipped
-    const int act_m = min(RM, (M - mt * MT + 15) / 16);
-    const int act_n = min(RN, (nd3 - nt * NT + 15) / 16);
+    int d1 = 0, d2 = 0;
+    if (m_ok && J.tri) {
+      d2 = tri_l2(ms);
+      d1 = ms - d2 * (d2 - 1) / 2;
+    } else if (m_ok) {
+      d1 = ms / nd2;
+      d2 = ms - d1 * nd2;
+    }
+    // 16-column blocks of the tile that hold outputs
+    const int act_n = min(RN, (nd3 - col0 + 15) / 16);
     const int n_cols = act_n * 16;
 
     for (int row = row_begin; row < row_end; ++row) {
@@ -198,6 +210,60 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
 #pragma unroll
           for (int c = 0; c < NC; ++c) cr[i][j][c] = si_[i][j][c] = ci[i][j][c] = sr_[i][j][c] = A::zero();
         }
+
+      auto add_sites = [&](auto act, int nx) {
+        constexpr int ACT = decltype(act)::value;
+        for (int xc = 0; xc < nx; ++xc) {
+          const int kbeg = xc * G * 3, kend = kbeg + G * 3;
+#pragma unroll 3
+          for (int k = kbeg; k < kend; ++k) {
+            T ar[RM], ai[RM], as[RM], bc[RN], bd[RN], be[RN];
+#pragma unroll
+            for (int i = 0; i < RM; ++i) {
+              ar[i] = Ar[k * MT + tm + 16 * i];
+              ai[i] = Ai[k * MT + tm + 16 * i];
+              as[i] = As[k * MT + tm + 16 * i];
+            }
+#pragma unroll
+            for (int j = 0; j < ACT; ++j) {
+              bc[j] = Bc[k * NT + tn + 16 * j];
+              bd[j] = Bd[k * NT + tn + 16 * j];
+              be[j] = Be[k * NT + tn + 16 * j];
+            }
+#pragma unroll
+            for (int i = 0; i < RM; ++i)
+#pragma unroll
+              for (int j = 0; j < ACT; ++j) {
+                A::fma_add(k1[i][j], bc[j], as[i]);
+                A::fma_add(k2[i][j], ar[i], bd[j]);
+                A::fma_add(k3[i][j], ai[i], be[j]);
+              }
+          }
+          if (NCLS > 0) {
+            Cx e[NC];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) e[c] = A::load(ph + xc * NC + c);
+#pragma unroll
+            for (int i = 0; i < RM; ++i)
+#pragma unroll
+              for (int j = 0; j < ACT; ++j) {
+                  const T sr = A::sub(k1[i][j], k3[i][j]), si = A::add(k1[i][j], k2[i][j]);
+                  k1[i][j] = k2[i][j] = k3[i][j] = A::zero();
+                  if (rp.has_zero) {
+                    zr[i][j] = A::add(zr[i][j], sr);
+                    zi[i][j] = A::add(zi[i][j], si);
+                  }
+#pragma unroll
+                  for (int c = 0; c < NC; ++c) {
+                    A::fma_add(cr[i][j][c], e[c].re, sr);
+                    A::fma_add(si_[i][j][c], e[c].im, si);
+                    A::fma_add(ci[i][j][c], e[c].re, si);
+                    A::fma_add(sr_[i][j][c], e[c].im, sr);
+                  }
+                }
+          }
+        }
+      };
 
       for (int x0 = 0; x0 < L; x0 += XC) {
         const int nx = min(XC, L - x0);
@@ -233,7 +299,7 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
           const int k = idx / n_cols;
           const int c = k % 3, t2 = k / 3;
           const int g = t2 % G, xc = t2 / G;
-          const int n = nt * NT + nl;
+          const int n = col0 + nl;
           Cx b{A::zero(), A::zero()};
           if (n < nd3) b = src.third(J, g, base + (x0 + xc) * sx, c, n);
           Bc[k * NT + nl] = b.re;
@@ -247,57 +313,13 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
           }
         __syncthreads();
 
-        for (int xc = 0; xc < nx; ++xc) {
-          const int kbeg = xc * G * 3, kend = kbeg + G * 3;
-#pragma unroll 3
-          for (int k = kbeg; k < kend; ++k) {
-            T ar[RM], ai[RM], as[RM], bc[RN], bd[RN], be[RN];
-#pragma unroll
-            for (int i = 0; i < RM; ++i) {
-              ar[i] = Ar[k * MT + tm + 16 * i];
-              ai[i] = Ai[k * MT + tm + 16 * i];
-              as[i] = As[k * MT + tm + 16 * i];
-            }
-#pragma unroll
-            for (int j = 0; j < RN; ++j) {
-              bc[j] = Bc[k * NT + tn + 16 * j];
-              bd[j] = Bd[k * NT + tn + 16 * j];
-              be[j] = Be[k * NT + tn + 16 * j];
-            }
-#pragma unroll
-            for (int i = 0; i < RM; ++i)
-#pragma unroll
-              for (int j = 0; j < RN; ++j)
-                if (i < act_m && j < act_n) {
-                  A::fma_add(k1[i][j], bc[j], as[i]);
-                  A::fma_add(k2[i][j], ar[i], bd[j]);
-                  A::fma_add(k3[i][j], ai[i], be[j]);
-                }
-          }
-          if (NCLS > 0) {
-            Cx e[NC];
-#pragma unroll
-            for (int c = 0; c < NC; ++c) e[c] = A::load(ph + xc * NC + c);
-#pragma unroll
-            for (int i = 0; i < RM; ++i)
-#pragma unroll
-              for (int j = 0; j < RN; ++j)
-                if (i < act_m && j < act_n) {
-                  const T sr = A::sub(k1[i][j], k3[i][j]), si = A::add(k1[i][j], k2[i][j]);
-                  k1[i][j] = k2[i][j] = k3[i][j] = A::zero();
-                  if (rp.has_zero) {
-                    zr[i][j] = A::add(zr[i][j], sr);
-                    zi[i][j] = A::add(zi[i][j], si);
-                  }
-#pragma unroll
-                  for (int c = 0; c < NC; ++c) {
-                    A::fma_add(cr[i][j][c], e[c].re, sr);
-                    A::fma_add(si_[i][j][c], e[c].im, si);
-                    A::fma_add(ci[i][j][c], e[c].re, si);
-                    A::fma_add(sr_[i][j][c], e[c].im, sr);
-                  }
-                }
-          }
+        // the staged sites into the sums, by the tile's 16-column blocks in use: a block that is
+        // only predicated off still takes the FP64 pipe (measured: 96 columns cost 128)
+        switch (act_n) {
+          case 1: add_sites(std::integral_constant<int, 1>{}, nx); break;
+          case 2: add_sites(std::integral_constant<int, RN < 2 ? RN : 2>{}, nx); break;
+          case 3: add_sites(std::integral_constant<int, RN < 3 ? RN : 3>{}, nx); break;
+          default: add_sites(std::integral_constant<int, RN>{}, nx); break;
         }
         // renormalise once per chunk of sites
 #pragma unroll
@@ -342,7 +364,7 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
           const int m = mt * MT + tm + 16 * i;
 #pragma unroll
           for (int j = 0; j < RN; ++j) {
-            const int n = nt * NT + tn + 16 * j;
+            const int n = col0 + tn + 16 * j;
             if (m < M && n < nd3) {
               Cx t{zr[i][j], zi[i][j]};
 #pragma unroll
