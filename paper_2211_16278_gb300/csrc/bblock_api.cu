@@ -27,6 +27,7 @@ struct bblock_ctx {
   double2* d_phase = nullptr;     // FP64 phases [n_mom][X], then their FP32 copy
   float2* d_phase_f = nullptr;
   float4* d_phase_df = nullptr;    // Ozaki form: the phases as double-float float4
+  double2* d_omega = nullptr;      // Ozaki form: w^k, k = 0..L-1 (the FP64 forms' d_phase is that)
   size_t phase_cap = 0;
   int* d_mom = nullptr;
   size_t mom_cap = 0;
@@ -429,9 +430,11 @@ int ensure_phase(bblock_ctx* c, const int32_t* momenta, int n_mom, cudaStream_t 
   const size_t n_ph = (size_t)c->X * n_mom;
   const bool oz = c->cfg.precision == BBLOCK_OZAKI;
   const size_t df_ofs = align_up((sizeof(double2) + sizeof(float2)) * n_ph, 256);
+  const size_t om_ofs = df_ofs + sizeof(float4) * n_ph;   // Ozaki form: w^k after its phases
   int rc = grow_device(c, reinterpret_cast<char**>(&c->d_phase), &c->phase_cap,
-                       df_ofs + (oz ? sizeof(float4) * n_ph : 0));
+                       oz ? om_ofs + sizeof(double2) * c->cfg.L : df_ofs);
   if (rc) return rc;
+  c->d_omega = oz ? reinterpret_cast<double2*>(reinterpret_cast<char*>(c->d_phase) + om_ofs) : nullptr;
   c->d_phase_f = reinterpret_cast<float2*>(c->d_phase + n_ph);
   c->d_phase_df = oz ? reinterpret_cast<float4*>(reinterpret_cast<char*>(c->d_phase) + df_ofs)
                      : nullptr;
@@ -440,7 +443,10 @@ int ensure_phase(bblock_ctx* c, const int32_t* momenta, int n_mom, cudaStream_t 
   CK(c, cudaMemcpyAsync(c->d_mom, momenta, sizeof(int) * 3 * n_mom, cudaMemcpyHostToDevice, s));
   CK(c, timed_launch(c, K_PHASE, s, [&] { return launch_phase_table(c->cfg.L, n_mom, c->d_mom, c->d_phase, c->d_phase_f, s); }));
   if (oz)
-    CK(c, timed_launch(c, K_PHASE, s, [&] { return launch_phase_df(c->d_phase, c->d_phase_df, (long long)n_ph, s); }));
+    CK(c, timed_launch(c, K_PHASE, s, [&] {
+      const cudaError_t e = launch_phase_df(c->d_phase, c->d_phase_df, (long long)n_ph, s);
+      return e != cudaSuccess ? e : launch_omega_table(c->cfg.L, c->d_omega, s);
+    }));
   // the host momentum array may be reused by the caller right after return
   CK(c, cudaStreamSynchronize(s));
   c->phase_mom = key;
@@ -1095,6 +1101,48 @@ int run_jobs_tc(bblock_ctx* c, const std::vector<JobIn>& jobs, const SpinPlan& s
   return BBLOCK_OK;
 }
 
+// Ozaki form: the row-factored phase, e^{-ip.x} = w^{n0 x0} w^{n1 x1 + n2 x2} along the axis
+// with the fewest distinct n0. The tensor cores then run nidx instead of n_mom phase columns
+// per d3, a row's last stage is padded with zeros, and the epilogue adds each row's sums into
+// the running sums of all momenta. Taken where the model of a row says it is faster: stages of
+// about 10 kcycles, an epilogue of 6 kcycles plus 0.18 per column and momentum beside them
+// (measured at L = 32, 9 momenta, N_dil = 48: 12 stages a row). BBLOCK_OPT_TC_ROWS 1: wherever
+// it fits, 2: never.
+OzRows plan_oz_rows(const bblock_ctx* c, const int32_t* momenta, int n_mom, int per_mom, int n_groups) {
+  OzRows r{};
+  const int L = c->cfg.L;
+  r.slabs.axis = -1;
+  r.slabs.L = L;
+  if (per_mom || n_mom < 1 || n_mom > kMaxRowP || c->opt_tc_rows == 2) return r;
+  auto md = [L](int v) { const int m = v % L; return m < 0 ? m + L : m; };
+  int axis = 2, fewest = 1 << 30;
+  for (int a = 2; a >= 0; --a) {
+    std::vector<int> seen;
+    for (int p = 0; p < n_mom; ++p) {
+      const int n0 = md(momenta[3 * p + a]);
+      if (std::find(seen.begin(), seen.end(), n0) == seen.end()) seen.push_back(n0);
+    }
+    if ((int)seen.size() < fewest) { fewest = (int)seen.size(); axis = a; }
+  }
+  if (fewest > kOzMaxIdx) return r;
+  const double k_row = 3.0 * n_groups * L, spr = std::ceil(k_row / 16.0), stage = 10.0;
+  const double row_rf = std::max(spr * stage, 6.0 + 0.18 * kOzMaxNC * n_mom / fewest);
+  if (c->opt_tc_rows == 0 && fewest * row_rf >= n_mom * (k_row / 16.0) * stage) return r;
+  const int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
+  for (int p = 0; p < n_mom; ++p) {
+    const int n0 = md(momenta[3 * p + axis]);
+    int idx = 0;
+    while (idx < r.nidx && r.n0[idx] != n0) ++idx;
+    if (idx == r.nidx) r.n0[r.nidx++] = n0;
+    r.mask[idx] |= 1u << p;
+    r.mom[p] = RowMom{p, md(momenta[3 * p + a1]), md(momenta[3 * p + a2]), idx};
+  }
+  r.n_mom = n_mom;
+  r.on = 1;
+  r.axis = r.slabs.axis = axis;
+  return r;
+}
+
 // The whole launch sequence for a list of jobs sharing momenta and spin operator.
 // Ozaki form: clusters of C CTAs share each diquark tile across C adjacent N tiles; each
 // builds 1/C of the tile's rows, with shorter per-thread chains, which sets the stage time.
@@ -1244,7 +1292,13 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
   const bool rowf = !oz;   // FP64 and double-float: the row-factored contraction
   int max_nd3_all = 1;
   for (const JobIn& j : jobs) max_nd3_all = std::max(max_nd3_all, j.nd[2]);
-  const GroupPlan gp = plan_groups(sp, rowf, jobs, n_ev, rowf ? 64 : 32);
+  const GroupPlan gp = plan_groups(sp, true, jobs, n_ev, rowf ? 64 : 32);
+  OzRows ozr{};
+  if (oz) ozr = plan_oz_rows(c, momenta, n_mom, per_mom, gp.n_groups);
+  for (int g = 0; g < gp.n_groups; ++g)
+    ozr.max_terms_i = std::max(ozr.max_terms_i, gp.tbeg[g + 1] - gp.tbeg[g]);
+  ozr.max_terms = (float)ozr.max_terms_i;
+  const size_t oz_scratch = ozr.on ? (size_t)c->num_sms * kOzMaxNC * kOzM * sizeof(float4) : 0;
   const int n2_fields = (int)gp.f2.size(), n3_fields = gp.n_groups * sp.n_coef_sets;
   // the momenta in row plans (per-momentum coefficients: one plan per momentum)
   std::vector<RowPlan> rplans;
@@ -1263,8 +1317,8 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
     for (const RowPlan& r : rplans) r_cls = std::max(r_cls, r.n_cls);
   }
   const int row_rn = rows_rn_for(r_cls, max_nd3_all);
-  // Ozaki form: every momentum of a launch as N columns
-  const int P_launch = per_mom ? 1 : n_mom;
+  // Ozaki form: N columns per d3 of a launch, the momenta or their distinct n0
+  const int P_cols = ozr.on ? ozr.nidx : per_mom ? 1 : n_mom;
   // Ozaki form: units run one per CTA (clusters: one per cluster of oz_cl CTAs)
   const int ctas = (oz ? 1 : rows_ctas_per_sm(rplans[0].n_cls, row_rn)) * c->num_sms;
   const int max_slabs = 64;
@@ -1274,7 +1328,7 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
   auto job_tiles = [&](const JobIn& j, int& mt, int& nt) {
     if (oz) {
       mt = (j.nd[0] * j.nd[1] + kOzM - 1) / kOzM;
-      nt = ((P_launch * j.nd[2] + oz_nc - 1) / oz_nc + oz_cl - 1) / oz_cl;
+      nt = ((P_cols * j.nd[2] + oz_nc - 1) / oz_nc + oz_cl - 1) / oz_cl;
     } else {
       mt = (j.nd[0] * j.nd[1] + 16 * kRowRM - 1) / (16 * kRowRM);
       nt = (j.nd[2] + 16 * row_rn - 1) / (16 * row_rn);
@@ -1316,7 +1370,7 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
     }
     ++c->last_waves;
     const int nj = (int)(end - job_idx);
-    if (oz) oz_cl = oz_cluster_for(c, jobs, job_idx, end, P_launch, oz_nc);
+    if (oz) oz_cl = oz_cluster_for(c, jobs, job_idx, end, P_cols, oz_nc);
     long long tiles = 0;
     int max_nd3 = 0, max_ndf = 0;
     long long max_elems = 0;
@@ -1330,15 +1384,17 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
       max_elems = std::max(max_elems, (long long)n_mom * j.nd[0] * j.nd[1] * j.nd[2]);
     }
     const int unit_slots = oz ? ctas / oz_cl : ctas;
-    // slabs are ranges of lattice rows (Ozaki form: of sites)
-    const int parts = oz ? X : L * L;
+    // slabs are ranges of lattice rows (Ozaki form with momentum columns: of sites)
+    const bool row_slabs = rowf || ozr.on;
+    const int parts = row_slabs ? L * L : X;
     int n_slab = c->opt_slabs > 0 ? std::min(c->opt_slabs, parts)
                                    : choose_slabs(tiles, unit_slots, parts, 1, max_slabs);
     const int per_slab = (parts + n_slab - 1) / n_slab;
     n_slab = (parts + per_slab - 1) / per_slab;
-    const int sites_per_slab = oz ? per_slab : per_slab * L;
+    const int sites_per_slab = row_slabs ? per_slab * L : per_slab;
+    ozr.slabs.per_slab = per_slab;
 
-    size_t ws_need = 0, oz_need = 0;
+    size_t ws_need = oz_scratch, oz_need = 0;
     for (size_t k = job_idx; k < end; ++k) {
       ws_need += job_bytes(jobs[k], n_slab);
       oz_need += oz_bytes(jobs[k], n_slab);
@@ -1355,7 +1411,8 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
     std::vector<DfConvSeg> segs;
     std::vector<uint32_t*> canaries;
     long long max_seg = 0;
-    char* ws = c->d_ws;
+    char* ws = c->d_ws + oz_scratch;
+    ozr.scratch = ozr.on ? reinterpret_cast<float4*>(c->d_ws) : nullptr;
     long long unit = 0;
     for (int k = 0; k < nj; ++k) {
       const JobIn& j = jobs[job_idx + k];
@@ -1511,7 +1568,7 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
       CK(c, cudaMemsetAsync(c->d_ws + (ws_need - oz_need), 0, oz_need, s));
       CK(c, timed_launch(c, K_PROJECT, s, [&] {
         return launch_oz_colmax(reinterpret_cast<const OzMaxSeg*>(c->d_tab + zofs),
-                                (int)ozsegs.size(), X, sites_per_slab, s);
+                                (int)ozsegs.size(), X, ozr.slabs, s);
       }));
     }
 
@@ -1532,6 +1589,8 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
     prm.P_total = n_mom;
     prm.status = c->d_status;
     prm.phase_df = c->d_phase_df;
+    prm.oz = ozr;
+    if (oz) prm.phase = c->d_omega;
     prm.NC = oz_nc;
     prm.wait_limit = c->opt_wait_us > 0 ? (long long)c->opt_wait_us * c->cycles_per_us
                                         : 4000000000LL;
@@ -1564,8 +1623,9 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
       }
     }
     CK(c, timed_launch(c, K_REDUCE, s, [&] {
-      return launch_reduce_slabs(reinterpret_cast<const ContractJob*>(c->d_tab + fbytes), nj,
-                                 n_slab, n_mom, max_elems, s);
+      const ContractJob* d_jobs = reinterpret_cast<const ContractJob*>(c->d_tab + fbytes);
+      return ozr.on ? launch_reduce_slabs_oz(d_jobs, nj, n_slab, n_mom, max_elems, s)
+                    : launch_reduce_slabs(d_jobs, nj, n_slab, n_mom, max_elems, s);
     }));
     if (!canaries.empty())
       CK(c, timed_launch(c, K_CANARY, s, [&] {
@@ -1708,14 +1768,18 @@ CallPlan plan_call(const bblock_ctx* c, int n_t, const int nd[3], int n_mom, int
   if (c->cfg.precision == BBLOCK_OZAKI) {
     // units (job, 128-row tile, N tile over every momentum's columns, slab)
     const int nc = nc_opt > 0 && nc_opt <= kOzMaxNC ? nc_opt : kOzMaxNC;
-    const long long nt = ((long long)n_mom * nd[2] + nc - 1) / nc;
+    OzRows ozr{};   // (the momenta of the last call, as for the FP16 form)
+    if (c->phase_mom.size() == (size_t)3 * n_mom)
+      ozr = plan_oz_rows(c, c->phase_mom.data(), n_mom, 0, pairs);
+    const int cols = ozr.on ? ozr.nidx : n_mom, parts = ozr.on ? c->cfg.L * c->cfg.L : X;
+    const long long nt = ((long long)cols * nd[2] + nc - 1) / nc;
     const long long tiles = (long long)n_t * ((nd[0] * nd[1] + kOzM - 1) / kOzM) * nt;
     pl.nc = nc;
-    pl.n_slab = slabs_opt > 0 ? std::min(slabs_opt, X) : choose_slabs(tiles, c->num_sms, X, 1, 64);
-    const int sps = (X + pl.n_slab - 1) / pl.n_slab;
-    pl.n_slab = (X + sps - 1) / sps;
+    pl.n_slab = slabs_opt > 0 ? std::min(slabs_opt, parts) : choose_slabs(tiles, c->num_sms, parts, 1, 64);
+    const int sps = (parts + pl.n_slab - 1) / pl.n_slab;
+    pl.n_slab = (parts + sps - 1) / sps;
     pl.units = tiles * pl.n_slab;
-    pl.pad = (double)(nt * nc) / ((double)n_mom * nd[2]) - 1.0;
+    pl.pad = (double)(nt * nc) / ((double)cols * nd[2]) - 1.0;
     return pl;
   }
   if (fp64_like(c->cfg)) {

@@ -103,6 +103,24 @@ struct RowPlan {
   RowMom mom[kMaxRowP];
 };
 
+// Ozaki form. Site slabs: of consecutive sites (axis < 0) or of lattice rows along `axis`.
+struct OzSlabs { int axis, L, per_slab; };
+constexpr int kOzMaxIdx = 8;
+// Row-factored units (on = 1): the N columns are n = d3 nidx + idx0 with the factor
+// w^{n0[idx0] x0} along `axis` of the nidx distinct n0 of the momenta; each row's sums, times
+// w^{n1 x1 + n2 x2}, go into the running sum of every momentum of mask[idx0] (bits over mom,
+// whose sel is its idx0). scratch: kOzMaxNC x kOzM float4 per CTA of the grid.
+struct OzRows {
+  int on, axis, nidx, n_mom;
+  int n0[kOzMaxIdx];
+  uint32_t mask[kOzMaxIdx];
+  RowMom mom[kMaxRowP];
+  float4* scratch;
+  OzSlabs slabs;
+  int max_terms_i;               // most terms of a group, and the same as a factor of the
+  float max_terms;               // diquark's rounding bound
+};
+
 // Eq. 1's spin sum as groups of terms: group g sums the terms t in [tbeg[g], tbeg[g + 1]),
 //   sum_g [ sum_t q1[a_slot[t]] x q2[b_slot[t]] ] . q3[g],
 // the spin coefficients folded into the line-3 fields (one term per group: its (alpha, beta)
@@ -125,6 +143,7 @@ struct ContractParams {
   int p0;                        // Ozaki form: first momentum of this launch
   int P_total;
   int* status;
+  OzRows oz;
   // Ozaki form: the phases as double-float float4 (re.h, re.l, im.h, im.l), [P_total][X];
   // P momenta per launch (columns n = p * nd3 + d3, p < P), NC complex columns per N tile,
   // and the limit of every bounded wait in SM cycles
@@ -405,8 +424,11 @@ struct OzMaxSeg {
   int stride;
   int modulus;                   // 1: the modulus, 0: |Re| + |Im|
 };
-cudaError_t launch_oz_colmax(const OzMaxSeg* d_segs, int n_segs, int X, int sites_per_slab,
+cudaError_t launch_oz_colmax(const OzMaxSeg* d_segs, int n_segs, int X, const OzSlabs& slabs,
                              cudaStream_t s);
+// B from row-factored partial blocks ([slab][p][d3][m])
+cudaError_t launch_reduce_slabs_oz(const ContractJob* d_jobs, int n_jobs, int n_slab, int P_total,
+                                   long long max_elems, cudaStream_t s);
 // The diquark's row maxima (see ContractJob::oz_max) of every job of p.jobs; max_m_tiles:
 // the largest job's 128-row tiles
 cudaError_t launch_oz_rowmax(const ContractParams& p, int max_m_tiles, cudaStream_t s);

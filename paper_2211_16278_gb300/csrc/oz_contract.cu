@@ -199,9 +199,12 @@ __device__ __forceinline__ int find_job(const ContractJob* jobs, int n_jobs, lon
   return lo;
 }
 
+// A unit's K elements come in `n_rows` runs of `k_row` elements, each run padded with zeros to
+// `spr` stages: the lattice rows [row0, row0 + n_rows) of the slab (RF), or its sites as one run.
 struct OzUnit {
-  int job, mt, nt, slab, x_begin, x_end, n_stages;
+  int job, mt, nt, slab, row0, n_rows, k_row, spr, n_stages;
 };
+template <bool RF>
 __device__ __forceinline__ OzUnit decode(const ContractParams& prm, long long u) {
   OzUnit w;
   w.job = find_job(prm.jobs, prm.n_jobs, u);
@@ -211,11 +214,29 @@ __device__ __forceinline__ OzUnit decode(const ContractParams& prm, long long u)
   r /= J.m_tiles;
   w.nt = (int)(r % J.n_tiles);
   w.slab = (int)(r / J.n_tiles);
-  w.x_begin = w.slab * prm.sites_per_slab;
-  w.x_end = min(prm.X, w.x_begin + prm.sites_per_slab);
-  const long long k_total = (long long)(w.x_end - w.x_begin) * prm.n_groups * 3;
-  w.n_stages = w.slab < prm.n_slab ? (int)((k_total + kK - 1) / kK) : 0;
+  if (RF) {
+    w.row0 = w.slab * prm.rows_per_slab;
+    w.n_rows = min(prm.L * prm.L, w.row0 + prm.rows_per_slab) - w.row0;
+    w.k_row = prm.L * prm.n_groups * 3;
+  } else {
+    w.row0 = w.slab * prm.sites_per_slab;   // the run's first site
+    w.n_rows = 1;
+    w.k_row = (min(prm.X, w.row0 + prm.sites_per_slab) - w.row0) * prm.n_groups * 3;
+  }
+  w.spr = (w.k_row + kK - 1) / kK;
+  w.n_stages = w.slab < prm.n_slab ? w.n_rows * w.spr : 0;
   return w;
+}
+// stages between drains: at most kChunk, a row's chunks of equal length
+__device__ __forceinline__ int chunk_stages(int spr) {
+  const int chunks = (spr + kChunk - 1) / kChunk;
+  return chunks > 0 ? (spr + chunks - 1) / chunks : 1;
+}
+// the first site of a run: x = base + xl * stride for its xl-th site
+template <bool RF> __device__ __forceinline__ int run_base(const ContractParams& prm, int row) {
+  if (!RF) return row;
+  const int ra = row % prm.L, rb = row / prm.L;
+  return prm.oz.axis == 0 ? prm.L * row : prm.oz.axis == 1 ? ra + prm.L * prm.L * rb : row;
 }
 
 // Shared-memory state the producer roles use.
@@ -225,9 +246,10 @@ struct OzShared {
   uint64_t* bar_full;
   uint64_t* bar_empty;
   volatile int* abort_flag;
-  const float4** s_q1;
+  const float4** s_q1;   // per term
   const float4** s_q2;
-  const float4** s_q3;
+  const float4** s_q3;   // per group
+  const float4* s_om;    // RF: w^k, double-float
 };
 
 // Stores of one K run of E BF16 digits (E = 8: 16 bytes, E = 4: 8 bytes).
@@ -240,7 +262,7 @@ template <int E> __device__ __forceinline__ void store_run(uint8_t* dst, const u
 // segments of 32 kEA / 16 rows); A = false: the third-quark rows (48 rows x 16 / E segments).
 // Each thread builds E consecutive K elements of its row per stage, splits them into digits
 // and stores every digit's run; a diquark warp then pushes its row groups to the peers.
-template <int C, int E, bool A>
+template <int C, int E, bool A, bool RF>
 __device__ __forceinline__ void oz_produce(const ContractParams& prm, const OzShared& sh, int pt,
                                            int lane, uint32_t rank, int gb, int ge,
                                            uint32_t peer_tx) {
@@ -248,8 +270,9 @@ __device__ __forceinline__ void oz_produce(const ContractParams& prm, const OzSh
   constexpr int kRW = 32 * E / kK;          // rows per warp (diquark)
   constexpr int kSegs = kK / E;             // K segments per row
   const int NC = prm.NC;
-  const int np = prm.n_groups;
+  const int ng = prm.n_groups;
   const long long u0 = blockIdx.x / C, du = gridDim.x / C;
+  const int sx = !RF ? 1 : prm.oz.axis == 0 ? 1 : prm.oz.axis == 1 ? prm.L : prm.L * prm.L;
   int rr, seg, a_g0 = 0, a_ng = 0;
   bool row_used;
   if (A) {
@@ -273,7 +296,7 @@ __device__ __forceinline__ void oz_produce(const ContractParams& prm, const OzSh
   (void)kSegs;
   long long s_g = 0;
   for (long long u = u0; u < prm.total_units; u += du) {
-    const OzUnit w = decode(prm, u);
+    const OzUnit w = decode<RF>(prm, u);
     const ContractJob& J = prm.jobs[w.job];
     const int nd1 = J.nd1, nd2 = J.nd2, nd3 = J.nd3;
     const int stride = nd1 + nd2 + nd3;
@@ -282,48 +305,66 @@ __device__ __forceinline__ void oz_produce(const ContractParams& prm, const OzSh
     // the slab's row maxima follow every slab's column maxima
     const float* rmx = J.oz_max + (size_t)prm.n_slab * stride + (size_t)slab * nd1 * nd2;
     bool row_ok;
-    int o1 = 0, o2 = 0, s1 = 0, s2 = 0, p = 0;
+    int o1 = 0, o2 = 0, s1 = 0, s2 = 0, p = 0, n0 = 0;
     float sc = 1.f;
     if (A) {
       const int m = w.mt * kOzM + rr;
       row_ok = row_used && m < nd1 * nd2;
       const int d1 = row_ok ? m / nd2 : 0, d2 = row_ok ? m - d1 * nd2 : 0;
       o1 = d1; o2 = d2; s1 = nd1; s2 = nd2;
-      if (row_ok) sc = pow2(-exp_a(rmx[m], mx[d1], mx[nd1 + d2]));
+      if (row_ok) sc = pow2(-exp_a(rmx[m], prm.oz.max_terms * mx[d1], mx[nd1 + d2]));
     } else {
+      // column n = p nd3 + d3, or (RF) n = d3 nidx + idx0
       const int n = (w.nt * C + (int)rank) * NC + rr;
-      row_ok = row_used && n < prm.P * nd3;
-      p = row_ok ? n / nd3 : 0;
-      const int d3 = row_ok ? n - p * nd3 : 0;
+      int d3 = 0;
+      if (RF) {
+        d3 = n / prm.oz.nidx;
+        row_ok = row_used && d3 < nd3;
+        if (row_ok) n0 = prm.oz.n0[n - d3 * prm.oz.nidx];
+        else d3 = 0;
+      } else {
+        row_ok = row_used && n < prm.P * nd3;
+        p = row_ok ? n / nd3 : 0;
+        d3 = row_ok ? n - p * nd3 : 0;
+      }
       o1 = d3; s1 = nd3;
       if (row_ok) sc = pow2(-exp_b(mx[nd1 + nd2 + d3]));
     }
-    const float4* ph = prm.phase_df + (size_t)(prm.p0 + p) * prm.X;
+    const float4* ph = RF ? nullptr : prm.phase_df + (size_t)(prm.p0 + p) * prm.X;
     // the unit's field table (producer warps meet before and after rewriting it)
     __syncwarp();
     named_bar(kBarProd, R::kProdThreads);
-    if (pt < np) {
+    if (pt < prm.n_terms) {
       sh.s_q1[pt] = reinterpret_cast<const float4*>(J.q1[prm.a_slot[pt]]);
       sh.s_q2[pt] = reinterpret_cast<const float4*>(J.q2[prm.b_slot[pt]]);
-      sh.s_q3[pt] = reinterpret_cast<const float4*>(J.q3[pt]);
     }
+    if (pt < ng) sh.s_q3[pt] = reinterpret_cast<const float4*>(J.q3[pt]);
     __syncwarp();
     named_bar(kBarProd, R::kProdThreads);
-    // K elements of the unit (< 2^31: at most 3 L^3 kMaxPairs) and the (site, pair, colour)
-    // of this thread's first element of the current stage; field offsets fit in 32 bits
+    // The (site of the run, group, colour) of this thread's first element of the current stage;
+    // K elements of a run < 2^31 (at most 3 L^3 kMaxPairs) and field offsets fit in 32 bits
     // (3 L^3 nd < 2^31 for L <= 128, nd <= 256)
-    const int k_total = (w.x_end - w.x_begin) * np * 3;
+    int row = w.row0, base = run_base<RF>(prm, row), sr = 0;
     int kk0 = seg * E;
-    int c0 = kk0 % 3, pr0 = (kk0 / 3) % np, x0 = w.x_begin + (kk0 / 3) / np;
+    const int cs = kk0 % 3, gs = (kk0 / 3) % ng, xs = (kk0 / 3) / ng;
+    int c0 = cs, g0 = gs, x0 = xs;
 
     for (int st = 0; st < w.n_stages; ++st, ++s_g) {
       if (st > 0) {
-        // advance the state by one stage: 16 = 5 groups of 3 + 1 colour
-        int groups = 5;
-        if (++c0 == 3) { c0 = 0; ++groups; }
-        pr0 += groups;
-        while (pr0 >= np) { pr0 -= np; ++x0; }
-        kk0 += kK;
+        if (++sr == w.spr) {
+          // the next run
+          sr = 0;
+          base = run_base<RF>(prm, ++row);
+          kk0 = seg * E;
+          c0 = cs; g0 = gs; x0 = xs;
+        } else {
+          // advance the state by one stage: 16 = 5 groups of 3 + 1 colour
+          int groups = 5;
+          if (++c0 == 3) { c0 = 0; ++groups; }
+          g0 += groups;
+          while (g0 >= ng) { g0 -= ng; ++x0; }
+          kk0 += kK;
+        }
       }
       const int slot = (int)(s_g % kStages);
       bool ok = !*sh.abort_flag;
@@ -332,85 +373,107 @@ __device__ __forceinline__ void oz_produce(const ContractParams& prm, const OzSh
                           sh.abort_flag, prm.status, prm.wait_limit);
       ok = __all_sync(0xffffffffu, ok);
       if (ok && row_used) {
-        // this thread's E K elements: k = 16 st + E seg + j = ((x - x_begin) np + pair) 3 + c,
-        // from the (site, pair, colour) state of its first element. They span at most
-        // G = (E + 4) / 3 (site, pair) groups, whose field pointers are read once; the loads
-        // of a batch of elements (4 diquark elements, 8 third-quark ones) are all issued
-        // before its arithmetic, so that their latencies overlap.
+        // this thread's E K elements: k = 16 sr + E seg + j = (xl n_groups + group) 3 + c, from
+        // the (site, group, colour) state of its first element. They span at most
+        // G = (E + 4) / 3 (site, group) pairs; the loads of a batch of elements (4 diquark
+        // elements of one term, 8 third-quark ones) are all issued before its arithmetic, so
+        // that their latencies overlap.
         constexpr int G = (E + 4) / 3;
         constexpr int LB = A ? 4 : 8;
-        const float4* pa[G];
-        const float4* pb[G];
-        int xg[G];
+        int gg[G], xg[G];
 #pragma unroll
         for (int k = 0; k < G; ++k) {
-          int pr = pr0 + k, xx = x0;
-          while (pr >= np) { pr -= np; ++xx; }
-          pa[k] = A ? sh.s_q1[pr] : sh.s_q3[pr];
-          pb[k] = A ? sh.s_q2[pr] : nullptr;
+          int g = g0 + k, xx = x0;
+          while (g >= ng) { g -= ng; ++xx; }
+          gg[k] = g;
           xg[k] = xx;
         }
         float2 va[E], vb[E];   // scaled entries (re, im): high parts, low parts
         int c = c0, gi = 0, kk = kk0;
 #pragma unroll
         for (int b0 = 0; b0 < E; b0 += LB) {
-          float4 ld[LB][A ? 4 : 2];
           bool vld[LB];
+          int eg[LB], ex[LB], ec[LB];   // group, site and colour of the batch's elements
 #pragma unroll
           for (int jj = 0; jj < LB; ++jj) {
-            vld[jj] = row_ok && kk < k_total;
-            const float4* fa = pa[0];
-            const float4* fb = pb[0];
+            vld[jj] = row_ok && kk < w.k_row;
+            eg[jj] = gg[0];
             int x = xg[0];
 #pragma unroll
             for (int k = 1; k < G; ++k)
-              if (gi == k) { fa = pa[k]; fb = pb[k]; x = xg[k]; }
-            if (!vld[jj]) x = w.x_begin;   // zero elements read a valid site
-            if (A) {
-              const int c1 = c == 2 ? 0 : c + 1, c2 = c == 0 ? 2 : c - 1;
-              const float4* uq = fa + (x * 3 * s1 + o1);
-              const float4* vq = fb + (x * 3 * s2 + o2);
-              ld[jj][0] = __ldg(uq + c1 * s1);
-              ld[jj][1] = __ldg(uq + c2 * s1);
-              ld[jj][2] = __ldg(vq + c1 * s2);
-              ld[jj][3] = __ldg(vq + c2 * s2);
-            } else {
-              ld[jj][0] = __ldg(fa + ((x * 3 + c) * s1 + o1));
-              ld[jj][1] = __ldg(ph + x);
-            }
+              if (gi == k) { eg[jj] = gg[k]; x = xg[k]; }
+            ex[jj] = vld[jj] ? x : 0;   // zero elements read a valid site
+            ec[jj] = c;
             ++kk;
             if (++c == 3) { c = 0; ++gi; }
           }
+          df2 v[LB];
+          if (A) {
+            // the terms of each element's group, one load batch per term
+            for (int tt = 0; tt < prm.oz.max_terms_i; ++tt) {
+              float4 ld[LB][4];
+              bool has[LB];
 #pragma unroll
-          for (int jj = 0; jj < LB; ++jj) {
-            const int j = b0 + jj;
-            df2 v;
-            if (A) {
-              // colour c of the diquark: D = u_c1 v_c2 - u_c2 v_c1, (c, c1, c2) cyclic;
-              // lanes (Re D, Im D):
-              //   Re = u1r v2r - u1i v2i - u2r v1r + u2i v1i
-              //   Im = u1r v2i + u1i v2r - u2r v1i - u2i v1r
-              const float4 u1 = ld[jj][0], u2 = ld[jj][1], v1 = ld[jj][2], v2 = ld[jj][3];
-              v = df2_prod(make_float2(u1.x, u1.x), make_float2(u1.y, u1.y),
-                           make_float2(v2.x, v2.z), make_float2(v2.y, v2.w));
-              df2_fma(v, make_float2(-u1.z, u1.z), make_float2(-u1.w, u1.w),
-                      make_float2(v2.z, v2.x), make_float2(v2.w, v2.y));
-              df2_fma(v, make_float2(-u2.x, -u2.x), make_float2(-u2.y, -u2.y),
-                      make_float2(v1.x, v1.z), make_float2(v1.y, v1.w));
-              df2_fma(v, make_float2(u2.z, -u2.z), make_float2(u2.w, -u2.w),
-                      make_float2(v1.z, v1.x), make_float2(v1.w, v1.y));
-            } else {
+              for (int jj = 0; jj < LB; ++jj) {
+                int t = prm.tbeg[eg[jj]] + tt;
+                has[jj] = t < prm.tbeg[eg[jj] + 1];
+                if (!has[jj]) t = 0;
+                const int cc = ec[jj];
+                const int c1 = cc == 2 ? 0 : cc + 1, c2 = cc == 0 ? 2 : cc - 1;
+                const int x = base + ex[jj] * sx;
+                const float4* uq = sh.s_q1[t] + (x * 3 * s1 + o1);
+                const float4* vq = sh.s_q2[t] + (x * 3 * s2 + o2);
+                ld[jj][0] = __ldg(uq + c1 * s1);
+                ld[jj][1] = __ldg(uq + c2 * s1);
+                ld[jj][2] = __ldg(vq + c1 * s2);
+                ld[jj][3] = __ldg(vq + c2 * s2);
+              }
+#pragma unroll
+              for (int jj = 0; jj < LB; ++jj) {
+                // colour c of the diquark: D = u_c1 v_c2 - u_c2 v_c1, (c, c1, c2) cyclic;
+                // lanes (Re D, Im D):
+                //   Re = u1r v2r - u1i v2i - u2r v1r + u2i v1i
+                //   Im = u1r v2i + u1i v2r - u2r v1i - u2i v1r
+                if (!has[jj]) continue;
+                const float4 u1 = ld[jj][0], u2 = ld[jj][1], v1 = ld[jj][2], v2 = ld[jj][3];
+                if (tt == 0)
+                  v[jj] = df2_prod(make_float2(u1.x, u1.x), make_float2(u1.y, u1.y),
+                                   make_float2(v2.x, v2.z), make_float2(v2.y, v2.w));
+                else
+                  df2_fma(v[jj], make_float2(u1.x, u1.x), make_float2(u1.y, u1.y),
+                          make_float2(v2.x, v2.z), make_float2(v2.y, v2.w));
+                df2_fma(v[jj], make_float2(-u1.z, u1.z), make_float2(-u1.w, u1.w),
+                        make_float2(v2.z, v2.x), make_float2(v2.w, v2.y));
+                df2_fma(v[jj], make_float2(-u2.x, -u2.x), make_float2(-u2.y, -u2.y),
+                        make_float2(v1.x, v1.z), make_float2(v1.y, v1.w));
+                df2_fma(v[jj], make_float2(u2.z, -u2.z), make_float2(u2.w, -u2.w),
+                        make_float2(v1.z, v1.x), make_float2(v1.w, v1.y));
+              }
+            }
+          } else {
+            float4 ld[LB][2];
+#pragma unroll
+            for (int jj = 0; jj < LB; ++jj) {
+              const int x = base + ex[jj] * sx;
+              ld[jj][0] = __ldg(sh.s_q3[eg[jj]] + ((x * 3 + ec[jj]) * s1 + o1));
+              ld[jj][1] = RF ? sh.s_om[(n0 * ex[jj]) % prm.L] : __ldg(ph + x);
+            }
+#pragma unroll
+            for (int jj = 0; jj < LB; ++jj) {
               // e^{-ip.x} q3: Re = er qr - ei qi, Im = er qi + ei qr
               const float4 q = ld[jj][0], e = ld[jj][1];
-              v = df2_prod(make_float2(e.x, e.x), make_float2(e.y, e.y),
-                           make_float2(q.x, q.z), make_float2(q.y, q.w));
-              df2_fma(v, make_float2(-e.z, e.z), make_float2(-e.w, e.w),
+              v[jj] = df2_prod(make_float2(e.x, e.x), make_float2(e.y, e.y),
+                               make_float2(q.x, q.z), make_float2(q.y, q.w));
+              df2_fma(v[jj], make_float2(-e.z, e.z), make_float2(-e.w, e.w),
                       make_float2(q.z, q.x), make_float2(q.w, q.y));
             }
-            // elements past the unit's K or of an unused row are zero
-            const float s = vld[jj] ? sc : 0.f;
-            va[j] = __fmul2_rn(v.h, make_float2(s, s));
-            vb[j] = __fmul2_rn(v.l, make_float2(s, s));
+          }
+#pragma unroll
+          for (int jj = 0; jj < LB; ++jj) {
+            // elements past the run's K or of an unused row are zero
+            const float sv = vld[jj] ? sc : 0.f;
+            va[b0 + jj] = __fmul2_rn(v[jj].h, make_float2(sv, sv));
+            vb[b0 + jj] = __fmul2_rn(v[jj].l, make_float2(sv, sv));
           }
         }
         // digits, most significant first; each digit's E values are one K run of the row
@@ -471,7 +534,18 @@ __device__ __forceinline__ void oz_produce(const ContractParams& prm, const OzSh
   }
 }
 
-template <int C>
+// A chunk's sum of column i: TwoSum of the exact levels, the shared level into the tail.
+__device__ __forceinline__ void chunk_sum(const float (&ar)[kAcc][4], const float (&ai)[kAcc][4],
+                                          int i, float2& h, float2& l) {
+  float2 s0, e0, s1, e1;
+  two_sum2(make_float2(ar[0][i], ai[0][i]), make_float2(ar[1][i], ai[1][i]), s0, e0);
+  two_sum2(make_float2(ar[2][i], ai[2][i]), make_float2(ar[3][i], ai[3][i]), s1, e1);
+  e1 = __fadd2_rn(e1, make_float2(ar[4][i], ai[4][i]));
+  two_sum2(s0, s1, h, l);
+  l = __fadd2_rn(l, __fadd2_rn(e0, e1));
+}
+
+template <int C, bool RF>
 __global__ void __maxnreg__(OzRoles<C>::kMaxRegs)
 k_contract_oz(const __grid_constant__ ContractParams prm) {
   using R = OzRoles<C>;
@@ -483,10 +557,14 @@ k_contract_oz(const __grid_constant__ ContractParams prm) {
   __shared__ const float4* s_q1[kMaxPairs];
   __shared__ const float4* s_q2[kMaxPairs];
   __shared__ const float4* s_q3[kMaxPairs];
+  // RF: w^k; each momentum's w^{n1 x1 + n2 x2} of the epilogue's current row and of the one
+  // before; the unit's momentum updates (column << 8 | momentum)
+  __shared__ float4 s_om[RF ? 128 : 1];
+  __shared__ float4 s_rowph[2][RF ? kMaxRowP : 1];
+  __shared__ uint16_t s_upd[RF ? kOzMaxNC * kMaxRowP : 1];
 
   const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
   const int NC = prm.NC;
-  const int np = prm.n_groups;
   const uint32_t rank = C > 1 ? cluster_rank() : 0u;
   const int gb = group_begin((int)rank, C), ge = group_begin((int)rank + 1, C);
   // transaction bytes the peers' diquark row groups bring into each stage
@@ -502,6 +580,12 @@ k_contract_oz(const __grid_constant__ ContractParams prm) {
     mbar_init(smem_u32(&bar_final), 1);
     abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if constexpr (RF) {
+    for (int k = tid; k < prm.L; k += blockDim.x) {
+      const dcomplex z = dc_from_double2(prm.phase[k]);
+      s_om[k] = make_float4(z.re.h, z.re.l, z.im.h, z.im.l);
+    }
   }
   if (warp == R::kMmaWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -519,11 +603,11 @@ k_contract_oz(const __grid_constant__ ContractParams prm) {
   if (warp >= R::kProdWarp0) {
     // ------------------------------------------------------------ producers
     const int pt = tid - R::kProdWarp0 * 32;
-    OzShared sh{smem, smem_base, bar_full, bar_empty, &abort_flag, s_q1, s_q2, s_q3};
+    OzShared sh{smem, smem_base, bar_full, bar_empty, &abort_flag, s_q1, s_q2, s_q3, s_om};
     if (pt < R::kAThreads)
-      oz_produce<C, R::kEA, true>(prm, sh, pt, lane, rank, gb, ge, peer_tx);
+      oz_produce<C, R::kEA, true, RF>(prm, sh, pt, lane, rank, gb, ge, peer_tx);
     else
-      oz_produce<C, R::kEB, false>(prm, sh, pt, lane, rank, gb, ge, peer_tx);
+      oz_produce<C, R::kEB, false, RF>(prm, sh, pt, lane, rank, gb, ge, peer_tx);
   } else if (warp == R::kMmaWarp) {
     // ------------------------------------------------------------ MMA issue (one thread)
     if (lane == 0) {
@@ -533,11 +617,15 @@ k_contract_oz(const __grid_constant__ ContractParams prm) {
       long long s_g = 0, c_g = 0;
       bool stop = false;
       for (long long u = u0; u < prm.total_units && !stop; u += du) {
-        const OzUnit w = decode(prm, u);
+        const OzUnit w = decode<RF>(prm, u);
+        const int cl = RF ? chunk_stages(w.spr) : kChunk;
+        int sr = 0, cpos = 0;   // stage within the run, stage within the chunk
         for (int st = 0; st < w.n_stages; ++st, ++s_g) {
           const int slot = (int)(s_g % kStages);
-          const bool chunk_first = st % kChunk == 0;
-          const bool chunk_last = st % kChunk == kChunk - 1 || st == w.n_stages - 1;
+          const bool chunk_first = cpos == 0;
+          const bool chunk_last = cpos == cl - 1 || sr == w.spr - 1;
+          if (++sr == w.spr) { sr = 0; cpos = 0; }
+          else if (++cpos == cl) cpos = 0;
           if (chunk_first && c_g >= 1 &&
               !wait_bounded(smem_u32(&bar_acc_empty), (uint32_t)((c_g + 1) & 1), &abort_flag,
                             prm.status, prm.wait_limit)) { stop = true; break; }
@@ -597,7 +685,7 @@ k_contract_oz(const __grid_constant__ ContractParams prm) {
     const int ncols = NC, col0 = 0;
     long long c_g = 0;
     for (long long u = u0; u < prm.total_units; u += du) {
-      const OzUnit w = decode(prm, u);
+      const OzUnit w = decode<RF>(prm, u);
       if (w.slab >= prm.n_slab && tid == 0) atomicOr(prm.status, kStatusBadJob);
       const ContractJob& J = prm.jobs[w.job];
       const int nd1 = J.nd1, nd2 = J.nd2, nd3 = J.nd3, M = nd1 * nd2;
@@ -612,15 +700,110 @@ k_contract_oz(const __grid_constant__ ContractParams prm) {
       int eA = 0;
       if (row_ok) {
         const int d1 = m / nd2, d2 = m - d1 * nd2;
-        eA = exp_a(rmx[m], mx[d1], mx[nd1 + d2]);
+        eA = exp_a(rmx[m], prm.oz.max_terms * mx[d1], mx[nd1 + d2]);
       }
-      const int n_chunks = (w.n_stages + kChunk - 1) / kChunk;
+      const int cl = RF ? chunk_stages(w.spr) : kChunk;
+      const int cpr = (w.spr + cl - 1) / cl;               // chunks per run
+      const int n_chunks = w.n_stages > 0 ? w.n_rows * cpr : 0;
+      float4* const tsum = RF ? prm.oz.scratch + (size_t)blockIdx.x * kOzMaxNC * kOzM : nullptr;
+      int n_upd = 0;
+      if constexpr (RF) {
+        // the tile's (column, momentum) updates, listed once per unit: column by column, its
+        // momenta in order (the warps may still read the last unit's list)
+        __syncwarp();
+        named_bar(kBarEpi, R::kEpiWarps * 32);
+        for (int cq = 0; cq < NC; ++cq) {
+          const int n = n_base + cq, d3 = n / prm.oz.nidx;
+          if (d3 >= nd3) break;
+          const uint32_t mask = prm.oz.mask[n - d3 * prm.oz.nidx];
+          if (row < 32 && ((mask >> row) & 1u))
+            s_upd[n_upd + __popc(mask & ((1u << row) - 1u))] = (uint16_t)(cq << 8 | row);
+          n_upd += __popc(mask);
+        }
+        __syncwarp();
+        named_bar(kBarEpi, R::kEpiWarps * 32);
+      }
       for (int ch = 0; ch < n_chunks; ++ch, ++c_g) {
         bool ok = !abort_flag;
         if (ok)
           ok = wait_bounded(smem_u32(&bar_acc_full), (uint32_t)(c_g & 1), &abort_flag,
                             prm.status, prm.wait_limit);
         ok = __all_sync(0xffffffffu, ok);
+        if constexpr (RF) {
+          // Row-factored: the chunk's sums go to the CTA's own scratch (L2), the accumulators
+          // back to the MMA thread, and then, beside the next chunk's MMAs, each column's sum
+          // times w^{n1 x1 + n2 x2} into the running sum of every momentum of its n0, kept in
+          // the unit's partial block ([p][d3][m]: a warp's accesses are 512-byte runs).
+          const int lrow = w.row0 + ch / cpr, rpar = (int)(c_g & 1);
+          if (row < prm.oz.n_mom)
+            s_rowph[rpar][row] = s_om[(prm.oz.mom[row].n1 * (lrow % prm.L) +
+                                       prm.oz.mom[row].n2 * (lrow / prm.L)) % prm.L];
+          if (ok) {
+            tc_fence_after();
+            for (int col = 0; col < NC; col += 4) {
+              float ar[kAcc][4], ai[kAcc][4];
+#pragma unroll
+              for (int t = 0; t < kAcc; ++t) {
+                tmem_ld4(lane_base + (uint32_t)(t * 2 * NC + col), ar[t]);
+                tmem_ld4(lane_base + (uint32_t)(t * 2 * NC + NC + col), ai[t]);
+              }
+              tmem_wait_ld();
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                float2 h, l;
+                chunk_sum(ar, ai, i, h, l);
+                tsum[(col + i) * kOzM + row] = make_float4(h.x, l.x, h.y, l.y);
+              }
+            }
+          }
+          tc_fence_before();
+          __syncwarp();
+          named_bar(kBarEpi, R::kEpiWarps * 32);
+          if (tid == 0) mbar_arrive(smem_u32(&bar_acc_empty));
+          __syncwarp();
+          if (ok && row_ok) {
+            const bool last = ch == n_chunks - 1;
+            float4* const part = reinterpret_cast<float4*>(J.partial) +
+                                 (size_t)w.slab * prm.P_total * nd3 * M + m;
+            constexpr int UB = 8;   // updates whose loads are in flight together
+            for (int b = 0; b < n_upd; b += UB) {
+              float4 run[UB], ts[UB], *at[UB];
+              int mom[UB], d3s[UB];
+#pragma unroll
+              for (int i = 0; i < UB; ++i) {
+                const int e = s_upd[min(b + i, n_upd - 1)];
+                mom[i] = e & 255;
+                d3s[i] = (n_base + (e >> 8)) / prm.oz.nidx;
+                at[i] = part + ((size_t)prm.oz.mom[mom[i]].p * nd3 + d3s[i]) * M;
+                run[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (ch > 0) run[i] = *at[i];
+                ts[i] = tsum[(e >> 8) * kOzM + row];
+              }
+#pragma unroll
+              for (int i = 0; i < UB; ++i) {
+                if (b + i >= n_upd) break;
+                const float4 e = s_rowph[rpar][mom[i]];
+                df2 v{make_float2(run[i].x, run[i].z), make_float2(run[i].y, run[i].w)};
+                // Re = er tr - ei ti, Im = er ti + ei tr
+                df2_fma(v, make_float2(e.x, e.x), make_float2(e.y, e.y),
+                        make_float2(ts[i].x, ts[i].z), make_float2(ts[i].y, ts[i].w));
+                df2_fma(v, make_float2(-e.z, e.z), make_float2(-e.w, e.w),
+                        make_float2(ts[i].z, ts[i].x), make_float2(ts[i].w, ts[i].y));
+                float2 h, l;
+                two_sum2(v.h, v.l, h, l);
+                if (!last) {
+                  *at[i] = make_float4(h.x, l.x, h.y, l.y);
+                } else {
+                  const double scale =
+                      __longlong_as_double((long long)(1023 + eA + exp_b(mx[nd1 + nd2 + d3s[i]])) << 52);
+                  *reinterpret_cast<double2*>(at[i]) = make_double2(
+                      ((double)h.x + (double)l.x) * scale, ((double)h.y + (double)l.y) * scale);
+                }
+              }
+            }
+          }
+          continue;
+        }
         if (ok) {
           tc_fence_after();
           const bool last = ch == n_chunks - 1;
@@ -653,14 +836,8 @@ k_contract_oz(const __grid_constant__ ContractParams prm) {
             for (int i = 0; i < 4; ++i) {
               const int n = n_base + col + i;
               if (n >= Ncols) break;
-              // the chunk's sum: TwoSum of the exact levels, the shared level into the tail
-              float2 s0, e0, s1, e1;
-              two_sum2(make_float2(ar[0][i], ai[0][i]), make_float2(ar[1][i], ai[1][i]), s0, e0);
-              two_sum2(make_float2(ar[2][i], ai[2][i]), make_float2(ar[3][i], ai[3][i]), s1, e1);
-              e1 = __fadd2_rn(e1, make_float2(ar[4][i], ai[4][i]));
               float2 h, l;
-              two_sum2(s0, s1, h, l);
-              l = __fadd2_rn(l, __fadd2_rn(e0, e1));
+              chunk_sum(ar, ai, i, h, l);
               if (ch > 0) {
                 // running sum += chunk sum (double-float)
                 float2 rh, rl;
@@ -704,8 +881,14 @@ k_contract_oz(const __grid_constant__ ContractParams prm) {
 // Column maxima of the fields per site slab (see the header): one block per (field, 64
 // sites); thread t takes column t % nd of rows t / nd + lanes * i.
 constexpr int kColmaxSites = 64;
+__device__ __forceinline__ int slab_of(const OzSlabs& sl, int x) {
+  if (sl.axis < 0) return x / sl.per_slab;
+  const int L = sl.L;
+  const int row = sl.axis == 0 ? x / L : sl.axis == 1 ? x % L + L * (x / (L * L)) : x % (L * L);
+  return row / sl.per_slab;
+}
 __global__ void __launch_bounds__(256) k_oz_colmax(const OzMaxSeg* __restrict__ segs, int X,
-                                                    int sites_per_slab) {
+                                                    const OzSlabs sl) {
   const OzMaxSeg g = segs[blockIdx.y];
   const int nd = g.nd;
   const int lanes = blockDim.x / nd;
@@ -716,7 +899,7 @@ __global__ void __launch_bounds__(256) k_oz_colmax(const OzMaxSeg* __restrict__ 
   float m = 0.f;
   int slab = -1;
   for (int x = x0 + lane; x < x1; x += lanes) {
-    const int s = x / sites_per_slab;
+    const int s = slab_of(sl, x);
     if (s != slab) {
       if (slab >= 0)
         atomicMax(reinterpret_cast<unsigned int*>(g.out + (size_t)slab * g.stride + g.col_off + d),
@@ -742,6 +925,7 @@ __global__ void __launch_bounds__(256) k_oz_colmax(const OzMaxSeg* __restrict__ 
 constexpr int kRowmaxSites = 32;
 __global__ void __launch_bounds__(128) k_oz_rowmax(const __grid_constant__ ContractParams prm,
                                                     int max_m_tiles) {
+  const OzSlabs sl = prm.oz.slabs;
   const int job = blockIdx.y / max_m_tiles, mt = blockIdx.y % max_m_tiles;
   const ContractJob& J = prm.jobs[job];
   const int M = J.nd1 * J.nd2;
@@ -753,30 +937,34 @@ __global__ void __launch_bounds__(128) k_oz_rowmax(const __grid_constant__ Contr
   float mxv = 0.f;
   int slab = -1;
   for (int x = x0; x < x1; ++x) {
-    const int s = x / prm.sites_per_slab;
+    const int s = slab_of(sl, x);
     if (s != slab) {
       if (slab >= 0)
         atomicMax(reinterpret_cast<unsigned int*>(rmx + (size_t)slab * M + m), __float_as_uint(mxv));
       slab = s;
       mxv = 0.f;
     }
-    for (int pr = 0; pr < prm.n_groups; ++pr) {
-      const float4* uq = reinterpret_cast<const float4*>(J.q1[prm.a_slot[pr]]) + (size_t)x * 3 * nd1 + d1;
-      const float4* vq = reinterpret_cast<const float4*>(J.q2[prm.b_slot[pr]]) + (size_t)x * 3 * nd2 + d2;
-      float2 u[3], v[3];
+    for (int g = 0; g < prm.n_groups; ++g) {
+      float re[3] = {0.f, 0.f, 0.f}, im[3] = {0.f, 0.f, 0.f};
+      for (int t = prm.tbeg[g]; t < prm.tbeg[g + 1]; ++t) {
+        const float4* uq = reinterpret_cast<const float4*>(J.q1[prm.a_slot[t]]) + (size_t)x * 3 * nd1 + d1;
+        const float4* vq = reinterpret_cast<const float4*>(J.q2[prm.b_slot[t]]) + (size_t)x * 3 * nd2 + d2;
+        float2 u[3], v[3];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const float4 a = __ldg(uq + (size_t)c * nd1), b = __ldg(vq + (size_t)c * nd2);
-        u[c] = make_float2(a.x, a.z);
-        v[c] = make_float2(b.x, b.z);
+        for (int c = 0; c < 3; ++c) {
+          const float4 a = __ldg(uq + (size_t)c * nd1), b = __ldg(vq + (size_t)c * nd2);
+          u[c] = make_float2(a.x, a.z);
+          v[c] = make_float2(b.x, b.z);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const int c1 = c == 2 ? 0 : c + 1, c2 = c == 0 ? 2 : c - 1;
+          re[c] += u[c1].x * v[c2].x - u[c1].y * v[c2].y - (u[c2].x * v[c1].x - u[c2].y * v[c1].y);
+          im[c] += u[c1].x * v[c2].y + u[c1].y * v[c2].x - (u[c2].x * v[c1].y + u[c2].y * v[c1].x);
+        }
       }
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const int c1 = c == 2 ? 0 : c + 1, c2 = c == 0 ? 2 : c - 1;
-        const float re = u[c1].x * v[c2].x - u[c1].y * v[c2].y - (u[c2].x * v[c1].x - u[c2].y * v[c1].y);
-        const float im = u[c1].x * v[c2].y + u[c1].y * v[c2].x - (u[c2].x * v[c1].y + u[c2].y * v[c1].x);
-        mxv = fmaxf(mxv, fmaxf(fabsf(re), fabsf(im)));
-      }
+      for (int c = 0; c < 3; ++c) mxv = fmaxf(mxv, fmaxf(fabsf(re[c]), fabsf(im[c])));
     }
   }
   if (slab >= 0)
@@ -791,11 +979,11 @@ __global__ void k_phase_df(const double2* __restrict__ ph, float4* __restrict__ 
   }
 }
 
-template <int C>
+template <int C, bool RF>
 cudaError_t launch_oz_c(const ContractParams& prm, int grid, cudaStream_t s) {
   using R = OzRoles<C>;
   const size_t smem = (size_t)kStages * kStageBytes;
-  auto kern = k_contract_oz<C>;
+  auto kern = k_contract_oz<C, RF>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
   if (C == 1) {
@@ -836,20 +1024,32 @@ cudaError_t launch_contract_oz(const ContractParams& prm, int cluster, int grid,
   if (prm.NC < 16 || prm.NC > kOzMaxNC || prm.NC % 16 != 0 || prm.n_groups < 1 ||
       prm.n_groups > kMaxPairs)
     return cudaErrorInvalidValue;
+  if (prm.oz.on) {
+    if (prm.oz.nidx < 1 || prm.oz.nidx > kOzMaxIdx || prm.oz.n_mom < 1 || prm.oz.n_mom > kMaxRowP ||
+        !prm.oz.scratch || prm.L > 128)
+      return cudaErrorInvalidValue;
+    switch (cluster) {
+      case 1: return launch_oz_c<1, true>(prm, grid, s);
+      case 2: return launch_oz_c<2, true>(prm, grid, s);
+      case 3: return launch_oz_c<3, true>(prm, grid, s);
+      case 4: return launch_oz_c<4, true>(prm, grid, s);
+      default: return cudaErrorInvalidValue;
+    }
+  }
   switch (cluster) {
-    case 1: return launch_oz_c<1>(prm, grid, s);
-    case 2: return launch_oz_c<2>(prm, grid, s);
-    case 3: return launch_oz_c<3>(prm, grid, s);
-    case 4: return launch_oz_c<4>(prm, grid, s);
+    case 1: return launch_oz_c<1, false>(prm, grid, s);
+    case 2: return launch_oz_c<2, false>(prm, grid, s);
+    case 3: return launch_oz_c<3, false>(prm, grid, s);
+    case 4: return launch_oz_c<4, false>(prm, grid, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
-cudaError_t launch_oz_colmax(const OzMaxSeg* d_segs, int n_segs, int X, int sites_per_slab,
+cudaError_t launch_oz_colmax(const OzMaxSeg* d_segs, int n_segs, int X, const OzSlabs& slabs,
                              cudaStream_t s) {
   if (n_segs == 0) return cudaSuccess;
   dim3 grid((unsigned)((X + kColmaxSites - 1) / kColmaxSites), (unsigned)n_segs);
-  k_oz_colmax<<<grid, 256, 0, s>>>(d_segs, X, sites_per_slab);
+  k_oz_colmax<<<grid, 256, 0, s>>>(d_segs, X, slabs);
   note_launch();
   return cudaGetLastError();
 }
@@ -860,6 +1060,55 @@ cudaError_t launch_oz_rowmax(const ContractParams& prm, int max_m_tiles, cudaStr
   k_oz_rowmax<<<grid, 128, 0, s>>>(prm, max_m_tiles);
   note_launch();
   return cudaGetLastError();
+}
+
+// B[p][m][d3] = sum over slabs, in order, of partial[slab][p][d3][m] (row-factored units), by
+// 32 x 32 tiles through shared memory so that both sides are 512-byte runs.
+__global__ void __launch_bounds__(256) k_reduce_slabs_oz(const ContractJob* __restrict__ jobs,
+                                                          int n_slab, int P_total) {
+  __shared__ double2 tile[32][33];
+  const ContractJob& J = jobs[blockIdx.z];
+  const int M = J.nd1 * J.nd2, nd3 = J.nd3;
+  const int mt = (M + 31) / 32, dt = (nd3 + 31) / 32;
+  const size_t per = (size_t)P_total * M * nd3;
+  const int tx = threadIdx.x % 32, ty = threadIdx.x / 32;
+  for (int b = blockIdx.x; b < P_total * mt * dt; b += gridDim.x) {
+    const int p = b / (mt * dt), m0 = b / dt % mt * 32, d0 = b % dt * 32;
+    for (int i = ty; i < 32; i += 8) {
+      const int d3 = d0 + i, m = m0 + tx;
+      double2 s = make_double2(0.0, 0.0);
+      if (d3 < nd3 && m < M) {
+        const double2* in = J.partial + ((size_t)p * nd3 + d3) * M + m;
+        s = in[0];
+        for (int sl = 1; sl < n_slab; ++sl) {
+          const double2 v = in[sl * per];
+          s.x += v.x;
+          s.y += v.y;
+        }
+      }
+      tile[i][tx] = s;
+    }
+    __syncthreads();
+    for (int i = ty; i < 32; i += 8) {
+      const int m = m0 + i, d3 = d0 + tx;
+      if (m < M && d3 < nd3) J.B[((size_t)p * M + m) * nd3 + d3] = tile[tx][i];
+    }
+    __syncthreads();
+  }
+}
+
+cudaError_t launch_reduce_slabs_oz(const ContractJob* d_jobs, int n_jobs, int n_slab, int P_total,
+                                   long long max_elems, cudaStream_t s) {
+  if (n_jobs == 0 || max_elems == 0) return cudaSuccess;
+  const long long bx = std::min<long long>((max_elems + 1023) / 1024 + 64, 8192);
+  for (int j0 = 0; j0 < n_jobs; j0 += 65535) {   // grid.z limit
+    const dim3 grid((unsigned)bx, 1, std::min(n_jobs - j0, 65535));
+    k_reduce_slabs_oz<<<grid, 256, 0, s>>>(d_jobs + j0, n_slab, P_total);
+    note_launch();
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_phase_df(const double2* ph, float4* out, long long n, cudaStream_t s) {

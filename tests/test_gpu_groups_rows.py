@@ -62,14 +62,19 @@ def rel(a, b):
 
 @pytest.mark.parametrize("slabs", [0, 1])
 @pytest.mark.parametrize("name", CASES)
-@pytest.mark.parametrize("form", ["fp64", "df64"])
-def test_matches_oracle(env, form, name, slabs):
+@pytest.mark.parametrize("form,options", [
+    ("fp64", {}), ("df64", {}), ("ozaki", {"tc_rows": 2}), ("ozaki", {"tc_rows": 1}),
+    ("ozaki", {"tc_rows": 1, "tc_cluster": 1, "tc_nc": 32}), ("ozaki", {"tc_rows": 1, "tc_cluster": 3}),
+    ("ozaki", {"tc_rows": 1, "tc_cluster": 4, "tc_nc": 16})], ids=str)
+def test_matches_oracle(env, form, options, name, slabs):
     torch, bb = env
     L, n_ev, nd, mom, spins, coeffs = CASES[name]
     inp = workloads.custom(L, n_ev, nd, 2, mom, spins, coeffs, seed=9000 + len(name))
     dev = torch.device("cuda:0")
     ctx = bb.bblock_create(L, n_ev, max(nd), form)
     bb.bblock_set_option(ctx, "slabs", slabs)
+    for k, v in options.items():
+        bb.bblock_set_option(ctx, k, v)
     B = bb.bblock_compute(ctx, torch.from_numpy(inp.V).to(dev),
                           *[torch.from_numpy(inp.phi[0][i]).to(dev) for i in range(3)],
                           inp.momenta, inp.spins, inp.coeffs)
