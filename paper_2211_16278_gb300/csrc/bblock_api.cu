@@ -368,8 +368,10 @@ struct GroupPlan {
   std::vector<std::vector<FoldList>> f3;      // [coefficient set][group]
 };
 
+// The plan by gamma, or by pair where it is no cheaper for the FP64-accurate contractions or
+// not allowed; force_gamma: by gamma wherever allowed (another caller compares the costs).
 GroupPlan plan_groups(const SpinPlan& sp, bool may_group, const std::vector<JobIn>& jobs,
-                      int n_ev, int d3_tile) {
+                      int n_ev, int d3_tile, bool force_gamma = false) {
   const double2 one = make_double2(1.0, 0.0);
   GroupPlan by_pair, by_gamma;
   by_pair.n_groups = by_pair.n_terms = sp.n_pairs;
@@ -411,7 +413,7 @@ GroupPlan plan_groups(const SpinPlan& sp, bool may_group, const std::vector<JobI
     }
     return sum;
   };
-  return cost(by_gamma) < cost(by_pair) ? by_gamma : by_pair;
+  return force_gamma || cost(by_gamma) < cost(by_pair) ? by_gamma : by_pair;
 }
 
 int ensure_phase(bblock_ctx* c, const int32_t* momenta, int n_mom, cudaStream_t s) {
@@ -2106,18 +2108,41 @@ int bblock_from_triplet(bblock_ctx* c, int n_t, const void* T, const void* phi1,
   CK(c, cudaSetDevice(c->cfg.device));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   c->last_stream = s;
-  // intermediates for the momenta of one coefficient set
+  if (sp.n_pairs > kMaxPairs) return fail(c, BBLOCK_ERR_UNSUPPORTED, "more than %d spin pairs", kMaxPairs);
+  // T x3 phi3' once per group (the dominant product), x2 phi2' once per term, and x1 phi1 summed
+  // over the terms. The plan with fewer of them: by gamma, or by pair (see plan_groups)
+  JobIn shape{};
+  for (int i = 0; i < 3; ++i) shape.nd[i] = nds[i];
+  GroupPlan gp = plan_groups(sp, false, {shape}, n_ev, 1), by_gamma = plan_groups(sp, true, {shape}, n_ev, 1, true);
+  auto products = [&](const GroupPlan& g) {
+    return (double)n_ev * n_ev * nd3 * ((double)g.n_groups * n_ev + (double)g.n_terms * nd2);
+  };
+  if (products(by_gamma) < products(gp)) gp = by_gamma;
+  std::vector<int> group_of(gp.n_terms);
+  for (int g = 0; g < gp.n_groups; ++g)
+    for (int t = gp.tbeg[g]; t < gp.tbeg[g + 1]; ++t) group_of[t] = g;
+  // intermediates for the momenta of one coefficient set, for as many terms at a time as fit
+  // 1 GiB (one at least)
   const int P_set = coeff_per_mom ? 1 : n_mom;
-  const size_t f_bytes = align_up(sizeof(double2) * (size_t)n_ev * nd3, 256);
+  const size_t f3_bytes = align_up(sizeof(double2) * (size_t)n_ev * nd3, 256);
+  const size_t f2_bytes = align_up(sizeof(double2) * (size_t)n_ev * nd2, 256);
   const size_t u1_bytes = align_up(sizeof(double2) * (size_t)P_set * n_ev * n_ev * nd3, 256);
   const size_t u2_bytes = align_up(sizeof(double2) * (size_t)P_set * n_ev * nd2 * nd3, 256);
-  rc = grow_device(c, &c->d_tri, &c->tri_cap, f_bytes + u1_bytes + u2_bytes);
+  auto groups_in = [&](int t0, int t1) { return group_of[t1 - 1] - group_of[t0] + 1; };
+  auto bytes_of = [&](int t0, int t1) {
+    return groups_in(t0, t1) * (f3_bytes + u1_bytes) + (t1 - t0) * (f2_bytes + u2_bytes);
+  };
+  std::vector<int> cut{0};   // the chunks of terms
+  size_t need = 0;
+  while (cut.back() < gp.n_terms) {
+    int t1 = cut.back() + 1;
+    while (t1 < gp.n_terms && bytes_of(cut.back(), t1 + 1) <= ((size_t)1 << 30)) ++t1;
+    need = std::max(need, bytes_of(cut.back(), t1));
+    cut.push_back(t1);
+  }
+  rc = grow_device(c, &c->d_tri, &c->tri_cap, need);
   if (rc) return rc;
-  double2* fold = reinterpret_cast<double2*>(c->d_tri);
-  double2* U1 = reinterpret_cast<double2*>(c->d_tri + f_bytes);
-  double2* U2 = reinterpret_cast<double2*>(c->d_tri + f_bytes + u1_bytes);
-  int launches = 0;
-  const double2 one = make_double2(1.0, 0.0);
+  const long long launches0 = t_kernel_launches;
   for (int t = 0; t < n_t; ++t) {
     const double2* Tt = static_cast<const double2*>(T) + t * tstride;
     const double2* p1 = static_cast<const double2*>(phi1) + t * pst[0];
@@ -2126,41 +2151,66 @@ int bblock_from_triplet(bblock_ctx* c, int n_t, const void* T, const void* phi1,
     double2* Bt = static_cast<double2*>(B_out) + t * bstride;
     for (int set = 0; set < sp.n_coef_sets; ++set) {
       const int p0 = coeff_per_mom ? set : 0;
-      for (int pr = 0; pr < sp.n_pairs; ++pr) {
-        FoldTerms ft{};
-        const auto& tl = sp.terms[set][pr];
-        ft.n = (int)tl.size();
-        for (int k = 0; k < ft.n; ++k) { ft.row[k] = tl[k].first; ft.w[k] = tl[k].second; }
-        CK(c, launch_fold_phi(p3, n_ev, nd3, ft, fold, s));
-        // U1[(p, l1, l2)][d3] = sum_l3 T[p][l1][l2][l3] phi3'[l3][d3]
-        ZgemmParams g{};
-        g.M = P_set * n_ev * n_ev; g.N = nd3; g.K = n_ev; g.batch = 1;
-        g.A = Tt + (size_t)p0 * n_ev * n_ev * n_ev; g.a_m = n_ev; g.a_k = 1;
-        g.B = fold; g.b_k = nd3; g.b_n = 1;
-        g.C = U1; g.c_m = nd3; g.c_n = 1;
-        g.alpha = one; g.accumulate = 0;
-        CK(c, launch_zgemm(g, s));
-        // U2[(p, l1)][d2][d3] = sum_l2 phi2[beta n_ev + l2][d2] U1[(p, l1, l2)][d3]
-        g = ZgemmParams{};
-        g.M = nd2; g.N = nd3; g.K = n_ev; g.batch = (long long)P_set * n_ev;
-        g.A = p2 + (size_t)sp.pair_beta[pr] * n_ev * nd2; g.a_m = 1; g.a_k = nd2; g.a_b = 0;
-        g.B = U1; g.b_k = nd3; g.b_n = 1; g.b_b = (long long)n_ev * nd3;
-        g.C = U2; g.c_m = nd3; g.c_n = 1; g.c_b = (long long)nd2 * nd3;
-        g.alpha = one; g.accumulate = 0;
-        CK(c, launch_zgemm(g, s));
-        // B[p][d1][(d2, d3)] (+)= sum_l1 phi1[alpha n_ev + l1][d1] U2[(p, l1)][(d2, d3)]
-        g = ZgemmParams{};
-        g.M = nd1; g.N = nd2 * nd3; g.K = n_ev; g.batch = P_set;
-        g.A = p1 + (size_t)sp.pair_alpha[pr] * n_ev * nd1; g.a_m = 1; g.a_k = nd1; g.a_b = 0;
-        g.B = U2; g.b_k = (long long)nd2 * nd3; g.b_n = 1; g.b_b = (long long)n_ev * nd2 * nd3;
-        g.C = Bt + (size_t)p0 * nd1 * nd2 * nd3; g.c_m = (long long)nd2 * nd3; g.c_n = 1;
-        g.c_b = (long long)nd1 * nd2 * nd3;
-        g.alpha = one; g.accumulate = pr > 0;
-        CK(c, launch_zgemm(g, s));
-        launches += 4;
+      for (size_t ch = 0; ch + 1 < cut.size(); ++ch) {
+        const int t0 = cut[ch], t1 = cut[ch + 1], g0 = group_of[t0], ngr = groups_in(t0, t1);
+        char* at = c->d_tri;
+        auto take = [&](size_t bytes) {
+          double2* p = reinterpret_cast<double2*>(at);
+          at += bytes;
+          return p;
+        };
+        FoldBatch fb{};
+        fb.n_ev = n_ev;
+        // a line's folded coefficients, or the caller's where nothing is folded
+        auto folded = [&](const double2* phi, int nd, const FoldList& fl, double2* out) -> const double2* {
+          if (fl.size() == 1 && fl[0].second.x == 1.0 && fl[0].second.y == 0.0)
+            return phi + (size_t)fl[0].first * n_ev * nd;
+          FoldTerms& f = fb.fold[fb.n++];
+          f.phi = phi;
+          f.out = out;
+          f.nd = nd;
+          f.n = (int)fl.size();
+          for (int k = 0; k < f.n; ++k) { f.row[k] = fl[k].first; f.w[k] = fl[k].second; }
+          return out;
+        };
+        // U1_g[(p, l1, l2)][d3] = sum_l3 T[p][l1][l2][l3] phi3'_g[l3][d3]
+        ZgemmParams g1{};
+        g1.M = P_set * n_ev * n_ev; g1.N = nd3; g1.K = n_ev; g1.batch = 1; g1.n_list = ngr;
+        g1.a_m = n_ev; g1.a_k = 1; g1.b_k = nd3; g1.b_n = 1; g1.c_m = nd3; g1.c_n = 1;
+        for (int g = 0; g < ngr; ++g) {
+          g1.A[g] = Tt + (size_t)p0 * n_ev * n_ev * n_ev;
+          g1.B[g] = folded(p3, nd3, gp.f3[set][g0 + g], take(f3_bytes));
+          g1.C[g] = take(u1_bytes);
+        }
+        // U2_t[(p, l1)][d2][d3] = sum_l2 phi2'_t[l2][d2] U1[(p, l1, l2)][d3]
+        ZgemmParams g2{};
+        g2.M = nd2; g2.N = nd3; g2.K = n_ev; g2.batch = (long long)P_set * n_ev; g2.n_list = t1 - t0;
+        g2.a_m = 1; g2.a_k = nd2; g2.a_b = 0;
+        g2.b_k = nd3; g2.b_n = 1; g2.b_b = (long long)n_ev * nd3;
+        g2.c_m = nd3; g2.c_n = 1; g2.c_b = (long long)nd2 * nd3;
+        // B[p][d1][(d2, d3)] = sum_t sum_l1 phi1[alpha_t n_ev + l1][d1] U2_t[(p, l1)][(d2, d3)]
+        ZgemmParams g3{};
+        g3.M = nd1; g3.N = nd2 * nd3; g3.K = n_ev; g3.batch = P_set; g3.n_list = t1 - t0; g3.sum_list = 1;
+        g3.a_m = 1; g3.a_k = nd1; g3.a_b = 0;
+        g3.b_k = (long long)nd2 * nd3; g3.b_n = 1; g3.b_b = (long long)n_ev * nd2 * nd3;
+        g3.C[0] = Bt + (size_t)p0 * nd1 * nd2 * nd3; g3.c_m = (long long)nd2 * nd3; g3.c_n = 1;
+        g3.c_b = (long long)nd1 * nd2 * nd3;
+        g3.accumulate = ch > 0;
+        for (int k = t0; k < t1; ++k) {
+          g2.A[k - t0] = folded(p2, nd2, gp.f2[gp.b_slot[k]], take(f2_bytes));
+          g2.B[k - t0] = g1.C[group_of[k] - g0];
+          g2.C[k - t0] = take(u2_bytes);
+          g3.A[k - t0] = p1 + (size_t)sp.alpha_of1[gp.a_slot[k]] * n_ev * nd1;
+          g3.B[k - t0] = g2.C[k - t0];
+        }
+        CK(c, launch_fold_phi(fb, s));
+        CK(c, launch_zgemm(g1, s));
+        CK(c, launch_zgemm(g2, s));
+        CK(c, launch_zgemm(g3, s));
       }
     }
   }
+  const int launches = (int)(t_kernel_launches - launches0);
   c->last_launches = launches;
   return BBLOCK_OK;
 }

@@ -282,26 +282,33 @@ cudaError_t launch_reduce_slabs_f32(const TcJob* d_jobs, int n_jobs, int n_slab,
 
 // ---------------------------------------------------------------- mode-triplet ordering
 
-// Line-3 coefficients of one (alpha, beta) pair: phi3' = sum_t w[t] phi3[row[t] N_ev + l][d].
+// Folded coefficients of one line: out[l][d] = sum_t w[t] phi[row[t] N_ev + l][d].
 struct FoldTerms {
-  int n;
+  const double2* phi;
+  double2* out;
+  int nd, n;
   int row[kMaxTerms];
   double2 w[kMaxTerms];
 };
+struct FoldBatch {
+  int n, n_ev;
+  FoldTerms fold[2 * kMaxPairs];
+};
 
-// Batched complex GEMM, FP64: for b < batch,
-//   C_b[m][n] = alpha * sum_k A_b[m][k] B_b[k][n]  (+ C_b[m][n] if accumulate),
-// element (m, k) of A_b at A + b * a_b + m * a_m + k * a_k (strides in elements), likewise B, C.
+// Batched complex GEMMs, FP64: for b < batch and every l < n_list,
+//   C[l]_b[m][n] = sum_k A[l]_b[m][k] B[l]_b[k][n]  (+ C[l]_b[m][n] if accumulate),
+// or with sum_list the sum over l into C[0]. Element (m, k) of A_b is at
+// A + b * a_b + m * a_m + k * a_k (strides in elements), likewise B, C.
 struct ZgemmParams {
   int M, N, K;
+  int n_list, sum_list;
   long long batch;
-  const double2* A;
+  const double2* A[kMaxPairs];
   long long a_m, a_k, a_b;
-  const double2* B;
+  const double2* B[kMaxPairs];
   long long b_k, b_n, b_b;
-  double2* C;
+  double2* C[kMaxPairs];
   long long c_m, c_n, c_b;
-  double2 alpha;
   int accumulate;
 };
 
@@ -321,8 +328,7 @@ cudaError_t launch_tri_field(const TriSlice* d_slices, int n_slices, int n, int 
                              cudaStream_t s);
 cudaError_t launch_tri_fill(const TriSlice* d_slices, int n_slices, int n, int n_mom,
                             cudaStream_t s);
-cudaError_t launch_fold_phi(const double2* phi, int n_ev, int nd, const FoldTerms& terms,
-                            double2* out, cudaStream_t s);
+cudaError_t launch_fold_phi(const FoldBatch& fb, cudaStream_t s);
 cudaError_t launch_zgemm(const ZgemmParams& p, cudaStream_t s);
 
 // Fill (check == false) or verify (check == true) the n canaries listed at d_list.

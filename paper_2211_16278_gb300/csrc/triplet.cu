@@ -15,10 +15,11 @@
 // sixth), projection 5.9 -> 0.03 ms, k_tri_fill and the slab reduction 0.07 ms.
 // For the second step:
 //   k_fill_identity   the identity coefficient matrix [4 N_ev][N_ev]
-//   k_fold_phi        phi3' = sum_t w_t phi3[gamma_t N_ev + l][d]  (line-3 coefficients of one
-//                     (alpha, beta) pair, as in the projection's fold)
+//   k_fold_phi        phi' = sum_t w_t phi[spin_t N_ev + l][d]  (the spin coefficients of a group's
+//                     third line or of a term's second line, as in the projection's fold)
 //   k_zgemm           batched complex GEMM with arbitrary strides, FP64, for the three mode
-//                     products T x3 phi3', x2 phi2, x1 phi1
+//                     products T x3 phi3' (one per group of spin terms, the dominant one),
+//                     x2 phi2' (one per term) and x1 phi1 (summed over the terms)
 #include "bblock_internal.h"
 #include "dfloat.cuh"
 
@@ -34,20 +35,21 @@ __global__ void k_fill_identity(double2* __restrict__ id, int n_ev) {
   }
 }
 
-__global__ void k_fold_phi(const double2* __restrict__ phi, int n_ev, int nd, FoldTerms terms,
-                           double2* __restrict__ out) {
-  const long long total = (long long)n_ev * nd;
+__global__ void k_fold_phi(const __grid_constant__ FoldBatch fb) {
+  const FoldTerms& terms = fb.fold[blockIdx.y];
+  const int nd = terms.nd;
+  const long long total = (long long)fb.n_ev * nd;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
        i += (long long)gridDim.x * blockDim.x) {
     const long long l = i / nd, d = i - l * nd;
     double re = 0.0, im = 0.0;
     for (int t = 0; t < terms.n; ++t) {
-      const double2 f = phi[((long long)terms.row[t] * n_ev + l) * nd + d];
+      const double2 f = terms.phi[((long long)terms.row[t] * fb.n_ev + l) * nd + d];
       const double2 w = terms.w[t];
       re = fma(w.x, f.x, fma(-w.y, f.y, re));
       im = fma(w.x, f.y, fma(w.y, f.x, im));
     }
-    out[i] = make_double2(re, im);
+    terms.out[i] = make_double2(re, im);
   }
 }
 
@@ -112,65 +114,92 @@ __global__ void k_tri_fill(const TriSlice* __restrict__ slices, int n, int n_mom
   }
 }
 
-constexpr int ZBM = 64, ZBN = 32, ZBK = 16;
+// Complex GEMMs of the three mode products, FP64. Bound by the FP64 pipe: three-multiplication
+// complex products (re = k1 - k3, im = k1 + k2; the operand sums formed once per staged element)
+// take 3 instead of 4 operations per multiply-add, and the row tile is the one that wastes fewer
+// rows: 64 (T x3 phi3, thousands of rows), or 32 (the products over N_dil rows, half of a 64-row
+// tile idle at N_dil = 32). L = 24, N_ev = 96, N_dil = 32, 3 momenta, 3 pairs / 2 gammas, all
+// products of one time slice: 3.61 -> 1.67 ms (1.4 ms of FP64 operations).
+constexpr int ZBK = 16, ZRN = 4, ZBN = 8 * ZRN;
 
-__global__ void __launch_bounds__(kThreads) k_zgemm(const ZgemmParams p) {
-  __shared__ double2 As[ZBK][ZBM];
-  __shared__ double2 Bs[ZBK][ZBN];
-  const int m0 = blockIdx.x * ZBM, n0 = blockIdx.y * ZBN;
-  const long long bt = blockIdx.z;
-  const double2* __restrict__ A = p.A + bt * p.a_b;
-  const double2* __restrict__ B = p.B + bt * p.b_b;
-  double2* __restrict__ C = p.C + bt * p.c_b;
+template <int RM>
+__global__ void __launch_bounds__(kThreads) k_zgemm(const __grid_constant__ ZgemmParams p) {
+  constexpr int BM = 32 * RM;
+  __shared__ double Ar[ZBK][BM], Ai[ZBK][BM], As[ZBK][BM];
+  __shared__ double Bc[ZBK][ZBN], Bd[ZBK][ZBN], Be[ZBK][ZBN];
+  const int m0 = blockIdx.x * BM, n0 = blockIdx.y * ZBN;
+  const long long bt = blockIdx.z % p.batch;
+  const int l0 = p.sum_list ? 0 : (int)(blockIdx.z / p.batch), l1 = p.sum_list ? p.n_list : l0 + 1;
+  double2* __restrict__ C = p.C[p.sum_list ? 0 : l0] + bt * p.c_b;
   const int tid = threadIdx.x, tn = tid % 8, tm = tid / 8;
-  double2 acc[2][4];
+  double k1[RM][ZRN], k2[RM][ZRN], k3[RM][ZRN];
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+  for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = make_double2(0.0, 0.0);
+    for (int j = 0; j < ZRN; ++j) k1[i][j] = k2[i][j] = k3[i][j] = 0.0;
 
-  for (int k0 = 0; k0 < p.K; k0 += ZBK) {
-    for (int idx = tid; idx < ZBK * ZBM; idx += kThreads) {
-      const int r = idx % ZBM, kk = idx / ZBM;
-      const int m = m0 + r, k = k0 + kk;
-      As[kk][r] = (m < p.M && k < p.K) ? A[(long long)m * p.a_m + (long long)k * p.a_k]
-                                         : make_double2(0.0, 0.0);
-    }
-    for (int idx = tid; idx < ZBK * ZBN; idx += kThreads) {
-      const int c = idx % ZBN, kk = idx / ZBN;
-      const int n = n0 + c, k = k0 + kk;
-      Bs[kk][c] = (n < p.N && k < p.K) ? B[(long long)k * p.b_k + (long long)n * p.b_n]
-                                         : make_double2(0.0, 0.0);
-    }
-    __syncthreads();
+  for (int l = l0; l < l1; ++l) {
+    const double2* __restrict__ A = p.A[l] + bt * p.a_b;
+    const double2* __restrict__ B = p.B[l] + bt * p.b_b;
+    for (int k0 = 0; k0 < p.K; k0 += ZBK) {
+      for (int idx = tid; idx < ZBK * BM; idx += kThreads) {
+        // neighbouring threads along A's unit stride
+        const int r = p.a_k == 1 ? idx / ZBK : idx % BM, kk = p.a_k == 1 ? idx % ZBK : idx / BM;
+        const int m = m0 + r, k = k0 + kk;
+        double2 v = make_double2(0.0, 0.0);
+        if (m < p.M && k < p.K) v = A[(long long)m * p.a_m + (long long)k * p.a_k];
+        Ar[kk][r] = v.x;
+        Ai[kk][r] = v.y;
+        As[kk][r] = v.x + v.y;
+      }
+      for (int idx = tid; idx < ZBK * ZBN; idx += kThreads) {
+        const int c = idx % ZBN, kk = idx / ZBN;
+        const int n = n0 + c, k = k0 + kk;
+        double2 v = make_double2(0.0, 0.0);
+        if (n < p.N && k < p.K) v = B[(long long)k * p.b_k + (long long)n * p.b_n];
+        Bc[kk][c] = v.x;
+        Bd[kk][c] = v.y - v.x;
+        Be[kk][c] = v.x + v.y;
+      }
+      __syncthreads();
+      const int kn = min(ZBK, p.K - k0);
 #pragma unroll 4
-    for (int kk = 0; kk < ZBK; ++kk) {
-      double2 a[2], b[4];
+      for (int kk = 0; kk < kn; ++kk) {
+        double ar[RM], ai[RM], as[RM], bc[ZRN], bd[ZRN], be[ZRN];
 #pragma unroll
-      for (int i = 0; i < 2; ++i) a[i] = As[kk][tm + 32 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tn + 8 * j];
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          acc[i][j].x = fma(a[i].x, b[j].x, fma(-a[i].y, b[j].y, acc[i][j].x));
-          acc[i][j].y = fma(a[i].x, b[j].y, fma(a[i].y, b[j].x, acc[i][j].y));
+        for (int i = 0; i < RM; ++i) {
+          ar[i] = Ar[kk][tm + 32 * i];
+          ai[i] = Ai[kk][tm + 32 * i];
+          as[i] = As[kk][tm + 32 * i];
         }
+#pragma unroll
+        for (int j = 0; j < ZRN; ++j) {
+          bc[j] = Bc[kk][tn + 8 * j];
+          bd[j] = Bd[kk][tn + 8 * j];
+          be[j] = Be[kk][tn + 8 * j];
+        }
+#pragma unroll
+        for (int i = 0; i < RM; ++i)
+#pragma unroll
+          for (int j = 0; j < ZRN; ++j) {
+            k1[i][j] = fma(bc[j], as[i], k1[i][j]);
+            k2[i][j] = fma(ar[i], bd[j], k2[i][j]);
+            k3[i][j] = fma(ai[i], be[j], k3[i][j]);
+          }
+      }
+      __syncthreads();
     }
-    __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
+  for (int i = 0; i < RM; ++i) {
     const int m = m0 + tm + 32 * i;
     if (m >= p.M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < ZRN; ++j) {
       const int n = n0 + tn + 8 * j;
       if (n >= p.N) continue;
       double2& c = C[(long long)m * p.c_m + (long long)n * p.c_n];
-      const double2 v = acc[i][j];
-      double2 r = make_double2(p.alpha.x * v.x - p.alpha.y * v.y, p.alpha.x * v.y + p.alpha.y * v.x);
+      double2 r = make_double2(k1[i][j] - k3[i][j], k1[i][j] + k2[i][j]);
       if (p.accumulate) { r.x += c.x; r.y += c.y; }
       c = r;
     }
@@ -216,25 +245,34 @@ cudaError_t launch_tri_fill(const TriSlice* d_slices, int n_slices, int n, int n
   return cudaSuccess;
 }
 
-cudaError_t launch_fold_phi(const double2* phi, int n_ev, int nd, const FoldTerms& terms,
-                            double2* out, cudaStream_t s) {
-  k_fold_phi<<<grid_for((long long)n_ev * nd), kThreads, 0, s>>>(phi, n_ev, nd, terms, out);
+cudaError_t launch_fold_phi(const FoldBatch& fb, cudaStream_t s) {
+  if (fb.n == 0) return cudaSuccess;
+  int nd = 1;
+  for (int k = 0; k < fb.n; ++k) nd = fb.fold[k].nd > nd ? fb.fold[k].nd : nd;
+  k_fold_phi<<<dim3(grid_for((long long)fb.n_ev * nd), fb.n), kThreads, 0, s>>>(fb);
   note_launch();
   return cudaGetLastError();
 }
 
 cudaError_t launch_zgemm(const ZgemmParams& p, cudaStream_t s) {
-  if (p.M <= 0 || p.N <= 0 || p.batch <= 0) return cudaSuccess;
-  for (long long b0 = 0; b0 < p.batch; b0 += 65535) {  // grid.z limit
+  if (p.M <= 0 || p.N <= 0 || p.batch <= 0 || p.n_list <= 0) return cudaSuccess;
+  const int per = p.sum_list ? 1 : p.n_list;
+  const long long step = 65535 / per;            // grid.z limit
+  const bool half = (p.M + 31) / 32 % 2 == 1 && p.M < 1024;
+  for (long long b0 = 0; b0 < p.batch; b0 += step) {
     ZgemmParams q = p;
-    q.A += b0 * p.a_b;
-    q.B += b0 * p.b_b;
-    q.C += b0 * p.c_b;
-    q.batch = (int)(p.batch - b0 < 65535 ? p.batch - b0 : 65535);
-    dim3 grid((p.M + ZBM - 1) / ZBM, (p.N + ZBN - 1) / ZBN, q.batch);
-    k_zgemm<<<grid, kThreads, 0, s>>>(q);
+    for (int l = 0; l < p.n_list; ++l) {
+      q.A[l] += b0 * p.a_b;
+      q.B[l] += b0 * p.b_b;
+    }
+    for (int l = 0; l < per; ++l) q.C[l] += b0 * p.c_b;
+    q.batch = (int)(p.batch - b0 < step ? p.batch - b0 : step);
+    const int bm = half ? 32 : 64;
+    const dim3 grid((p.M + bm - 1) / bm, (p.N + ZBN - 1) / ZBN, q.batch * per);
+    if (half) k_zgemm<1><<<grid, kThreads, 0, s>>>(q);
+    else k_zgemm<2><<<grid, kThreads, 0, s>>>(q);
     note_launch();
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -69,3 +69,28 @@ def test_non_finite_vectors(env, form):
     assert not np.isfinite(got[1][:, bad]).any()
     ref = oracle.mode_triplet(L, clean, MOM)
     assert np.linalg.norm((got[0] - ref)[:, ~bad]) <= TOL * np.linalg.norm(ref)
+
+
+def test_blocks_from_the_triplet_in_chunks_of_terms(env):
+    """All 64 spin triples (16 terms in 4 groups) at a size whose intermediates exceed the
+    chunk of terms taken at a time, and an operator grouped by gamma with several betas folded
+    into one term; blocks of the direct contraction as the reference."""
+    torch, bb = env
+    L, n_ev, nd = 4, 128, (64, 60, 64)
+    mom = [(a, b, c) for a in (0, 1, -1) for b in (0, 1, -1) for c in (0,)]
+    rng = np.random.default_rng(6600)
+    every = [(a, b, g) for a in range(4) for b in range(4) for g in range(4)]
+    dev = torch.device("cuda:0")
+    inp = workloads.custom(L, n_ev, nd, 1, mom, [(0, 0, 0)], [1.0], seed=6601)
+    V = torch.from_numpy(inp.V).to(dev)
+    phis = [torch.from_numpy(inp.phi[0][i]).to(dev) for i in range(3)]
+    ctx = bb.bblock_create(L, n_ev, n_ev, "fp64")
+    T = bb.bblock_mode_triplet(ctx, V, mom)
+    for spins in (every, [(0, 0, 1), (0, 1, 1), (0, 2, 1), (1, 0, 1), (2, 3, 1)]):
+        coeffs = rng.standard_normal(len(spins)) + 1j * rng.standard_normal(len(spins))
+        via = bb.bblock_from_triplet(ctx, T, *phis, spins, coeffs)
+        direct = bb.bblock_compute(ctx, V, *phis, mom, spins, coeffs)
+        bb.bblock_status(ctx)
+        err = (torch.linalg.norm(via - direct) / torch.linalg.norm(direct)).item()
+        assert err <= TOL
+    bb.bblock_destroy(ctx)
