@@ -17,6 +17,7 @@ constexpr int kMaxRfL = 128;    // lattice extent (the w^k table follows the sta
 constexpr int kMaxRowP = 32;
 constexpr int kMaxRowCls = 3;
 constexpr int kThreads = 256;   // threads per CTA of the FP64 kernels
+constexpr int kSmHint = 152;    // SMs of a GB300: where small launches take smaller tiles
 
 // Kernel launches made by the calling host thread, counted at every launch site of the
 // library (a call's launch count is the difference across it).

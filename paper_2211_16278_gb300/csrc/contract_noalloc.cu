@@ -309,15 +309,24 @@ extern "C" int bblock_contract_noalloc(int L, const void* q1, const void* q2, co
     cudaGetLastError();
     return na_fail(err, err_len, BBLOCK_ERR_CUDA, "device query failed");
   }
-  const int ctas = rows_ctas_per_sm(plans[0].n_cls, rn) * num_sms;
   const long long tiles = (long long)job.m_tiles * job.n_tiles;
-  long long n_slab = (4LL * ctas + tiles - 1) / tiles;
-  if (n_slab > (long long)max_slabs_fit) n_slab = (long long)max_slabs_fit;
-  if (n_slab > L * L) n_slab = L * L;
-  if (n_slab < 1) n_slab = 1;
-  base.rows_per_slab = (int)((L * L + n_slab - 1) / n_slab);
+  // Slabs of lattice rows, at most what the scratch holds: the count with the fewest rows on the
+  // busiest SM (the FP64 pipe is shared by an SM's CTAs, so only its units count). With 12 slabs
+  // allowed and 32 tiles (L = 16, N_dil = 32, 5 momenta) 12 would put 3 units of 22 rows on some
+  // SMs, 9 put 2 of 29: 9.64 -> 8.36 ms.
+  const int n_rows = L * L;
+  long long best = -1;
+  for (long long n = 1; n <= (long long)max_slabs_fit && n <= n_rows; ++n) {
+    const long long rps = (n_rows + n - 1) / n, slabs = (n_rows + rps - 1) / rps;
+    const long long cost = (tiles * slabs + num_sms - 1) / num_sms * rps;
+    if (best < 0 || cost < best) {
+      best = cost;
+      base.rows_per_slab = (int)rps;
+    }
+    if (slabs * tiles >= 8LL * num_sms) break;   // finer slabs gain nothing more
+  }
   base.sites_per_slab = base.rows_per_slab * L;
-  base.n_slab = (L * L + base.rows_per_slab - 1) / base.rows_per_slab;
+  base.n_slab = (n_rows + base.rows_per_slab - 1) / base.rows_per_slab;
   base.total_units = tiles * base.n_slab;
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);

@@ -9,6 +9,8 @@
 //                   three-multiplication form as the FP64 projection, each double replaced
 //                   by a double-float; writes the float4 fields the double-float
 //                   contraction reads
+#include <type_traits>
+
 #include "bblock_internal.h"
 #include "dfloat.cuh"
 
@@ -43,6 +45,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_project_df(const ProjField* __r
   const int m0 = blockIdx.x * DBM;
   const int tid = threadIdx.x, tn = tid % 8, tm = tid / 8;
   const int n_terms = F.n_terms;
+  const int act = min(4, (nd - n0 + 7) / 8);   // 8-column blocks in use: the others are skipped
   // this field's inputs are double-float planes (k_convert_df), its output too
   const float4* __restrict__ V = reinterpret_cast<const float4*>(F.V);
   const float4* __restrict__ phi = reinterpret_cast<const float4*>(F.phi);
@@ -55,7 +58,39 @@ __global__ void __launch_bounds__(kThreads, 2) k_project_df(const ProjField* __r
 #pragma unroll
     for (int j = 0; j < 4; ++j) k1[i][j] = k2[i][j] = k3[i][j] = df_zero();
 
+  auto multiply = [&](auto blocks, int kn) {
+    constexpr int ACT = decltype(blocks)::value;
+#pragma unroll 4
+    for (int kk = 0; kk < kn; ++kk) {
+      dfloat ar[2], ai[2], as[2], bc[ACT], bd[ACT], be[ACT];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float2 a = Ar[kk][tm + 32 * i], b = Ai[kk][tm + 32 * i], s = As[kk][tm + 32 * i];
+        ar[i] = dfloat{a.x, a.y};
+        ai[i] = dfloat{b.x, b.y};
+        as[i] = dfloat{s.x, s.y};
+      }
+#pragma unroll
+      for (int j = 0; j < ACT; ++j) {
+        const float2 c = Bc[kk][tn + 8 * j], d = Bd[kk][tn + 8 * j], e = Be[kk][tn + 8 * j];
+        bc[j] = dfloat{c.x, c.y};
+        bd[j] = dfloat{d.x, d.y};
+        be[j] = dfloat{e.x, e.y};
+      }
+      // three-multiplication form: re = k1 - k3, im = k1 + k2 (see the FP64 projection)
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < ACT; ++j) {
+          df_fma(k1[i][j], bc[j], as[i]);
+          df_fma(k2[i][j], ar[i], bd[j]);
+          df_fma(k3[i][j], ai[i], be[j]);
+        }
+    }
+  };
+
   for (int kb = 0; kb < n_ev; kb += DBK) {
+    const int kn = min(DBK, n_ev - kb);
     for (int idx = tid; idx < DBK * DBM; idx += kThreads) {
       const int r = idx % DBM, kk = idx / DBM;
       const int l = kb + kk, row = m0 + r;
@@ -88,32 +123,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_project_df(const ProjField* __r
       Be[kk][c] = make_float2(e.h, e.l);
     }
     __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < DBK; ++kk) {
-      dfloat ar[2], ai[2], as[2], bc[4], bd[4], be[4];
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const float2 a = Ar[kk][tm + 32 * i], b = Ai[kk][tm + 32 * i], s = As[kk][tm + 32 * i];
-        ar[i] = dfloat{a.x, a.y};
-        ai[i] = dfloat{b.x, b.y};
-        as[i] = dfloat{s.x, s.y};
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float2 c = Bc[kk][tn + 8 * j], d = Bd[kk][tn + 8 * j], e = Be[kk][tn + 8 * j];
-        bc[j] = dfloat{c.x, c.y};
-        bd[j] = dfloat{d.x, d.y};
-        be[j] = dfloat{e.x, e.y};
-      }
-      // three-multiplication form: re = k1 - k3, im = k1 + k2 (see the FP64 projection)
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          df_fma(k1[i][j], bc[j], as[i]);
-          df_fma(k2[i][j], ar[i], bd[j]);
-          df_fma(k3[i][j], ai[i], be[j]);
-        }
+    switch (act) {
+      case 1: multiply(std::integral_constant<int, 1>{}, kn); break;
+      case 2: multiply(std::integral_constant<int, 2>{}, kn); break;
+      case 3: multiply(std::integral_constant<int, 3>{}, kn); break;
+      default: multiply(std::integral_constant<int, 4>{}, kn); break;
     }
     // renormalise once per K block
 #pragma unroll

@@ -54,10 +54,17 @@ cudaError_t launch_phase_table(int L, int n_mom, const int* d_mom, double2* ph, 
 
 // ------------------------------------------------------------------ projection (Eq. 2)
 
-constexpr int PBM = 64, PBN = 32, PBK = 16;
+// Bound by the FP64 pipe; a padded column or eigenvector costs as much as a real one (a
+// predicated-off DFMA still takes the pipe), so the inner loop is instantiated for the 8-column
+// blocks of the tile in use and stops at N_ev. 64-row tiles, or 32-row ones where the launch
+// would not fill the SMs twice (small lattices: one 64-row CTA of 4 column blocks takes 24 us
+// whatever its columns). 4^3, N_ev = 8, N_dil = 8: 36 -> 8 us; the large cases are unchanged.
+constexpr int PBN = 32, PBK = 16;
 
+template <int RM>
 __global__ void __launch_bounds__(kThreads) k_project_fp64(const ProjField* __restrict__ fields,
                                                            int rows, int n_ev) {
+  constexpr int PBM = 32 * RM;
   __shared__ double Ar[PBK][PBM], Ai[PBK][PBM], As[PBK][PBM];
   __shared__ double Bc[PBK][PBN], Bd[PBK][PBN], Be[PBK][PBN];
   const ProjField& F = fields[blockIdx.z];
@@ -67,28 +74,58 @@ __global__ void __launch_bounds__(kThreads) k_project_fp64(const ProjField* __re
   const int m0 = blockIdx.x * PBM;
   const int tid = threadIdx.x, tn = tid % 8, tm = tid / 8;
   const int n_terms = F.n_terms;
+  const int act = min(4, (nd - n0 + 7) / 8);   // 8-column blocks in use
 
-  double k1[2][4], k2[2][4], k3[2][4];
+  double k1[RM][4], k2[RM][4], k3[RM][4];
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+  for (int i = 0; i < RM; ++i)
 #pragma unroll
     for (int j = 0; j < 4; ++j) k1[i][j] = k2[i][j] = k3[i][j] = 0.0;
+  auto multiply = [&](auto blocks, int kn) {
+    constexpr int ACT = decltype(blocks)::value;
+#pragma unroll 4
+    for (int kk = 0; kk < kn; ++kk) {
+      double ar[RM], ai[RM], as[RM], bc[ACT], bd[ACT], be[ACT];
+#pragma unroll
+      for (int i = 0; i < RM; ++i) {
+        ar[i] = Ar[kk][tm + 32 * i];
+        ai[i] = Ai[kk][tm + 32 * i];
+        as[i] = As[kk][tm + 32 * i];
+      }
+#pragma unroll
+      for (int j = 0; j < ACT; ++j) {
+        bc[j] = Bc[kk][tn + 8 * j];
+        bd[j] = Bd[kk][tn + 8 * j];
+        be[j] = Be[kk][tn + 8 * j];
+      }
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < ACT; ++j) {
+          k1[i][j] = fma(bc[j], as[i], k1[i][j]);
+          k2[i][j] = fma(ar[i], bd[j], k2[i][j]);
+          k3[i][j] = fma(ai[i], be[j], k3[i][j]);
+        }
+    }
+  };
 
   for (int kb = 0; kb < n_ev; kb += PBK) {
-    for (int idx = tid; idx < PBK * PBM; idx += kThreads) {
+    const int kn = min(PBK, n_ev - kb);
+    for (int idx = tid; idx < kn * PBM; idx += kThreads) {
       const int r = idx % PBM, kk = idx / PBM;
       const int l = kb + kk, row = m0 + r;
       double2 v = make_double2(0.0, 0.0);
-      if (l < n_ev && row < rows) v = F.V[(size_t)l * rows + row];
+      if (row < rows) v = F.V[(size_t)l * rows + row];
       Ar[kk][r] = v.x;
       Ai[kk][r] = v.y;
       As[kk][r] = v.x + v.y;
     }
-    for (int idx = tid; idx < PBK * PBN; idx += kThreads) {
+    for (int idx = tid; idx < kn * PBN; idx += kThreads) {
       const int c = idx % PBN, kk = idx / PBN;
+      if (c >= 8 * act) continue;
       const int l = kb + kk, col = n0 + c;
       double2 b = make_double2(0.0, 0.0);
-      if (l < n_ev && col < nd) {
+      if (col < nd) {
         for (int t = 0; t < n_terms; ++t) {
           const double2 f = F.phi[(size_t)(F.row_off[t] + l) * nd + col];
           const double2 w = F.w[t];
@@ -101,34 +138,16 @@ __global__ void __launch_bounds__(kThreads) k_project_fp64(const ProjField* __re
       Be[kk][c] = b.x + b.y;
     }
     __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < PBK; ++kk) {
-      double ar[2], ai[2], as[2], bc[4], bd[4], be[4];
-#pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        ar[i] = Ar[kk][tm + 32 * i];
-        ai[i] = Ai[kk][tm + 32 * i];
-        as[i] = As[kk][tm + 32 * i];
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        bc[j] = Bc[kk][tn + 8 * j];
-        bd[j] = Bd[kk][tn + 8 * j];
-        be[j] = Be[kk][tn + 8 * j];
-      }
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          k1[i][j] = fma(bc[j], as[i], k1[i][j]);
-          k2[i][j] = fma(ar[i], bd[j], k2[i][j]);
-          k3[i][j] = fma(ai[i], be[j], k3[i][j]);
-        }
+    switch (act) {
+      case 1: multiply(std::integral_constant<int, 1>{}, kn); break;
+      case 2: multiply(std::integral_constant<int, 2>{}, kn); break;
+      case 3: multiply(std::integral_constant<int, 3>{}, kn); break;
+      default: multiply(std::integral_constant<int, 4>{}, kn); break;
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
+  for (int i = 0; i < RM; ++i) {
     const int row = m0 + tm + 32 * i;
     if (row >= rows) continue;
 #pragma unroll
@@ -143,10 +162,13 @@ __global__ void __launch_bounds__(kThreads) k_project_fp64(const ProjField* __re
 cudaError_t launch_project_fp64(const ProjField* d_fields, int n_fields, int rows, int n_ev,
                                 int max_nd, cudaStream_t s) {
   if (n_fields == 0 || rows == 0) return cudaSuccess;
+  const long long ctas64 = (long long)((rows + 63) / 64) * ((max_nd + PBN - 1) / PBN) * n_fields;
   for (int f0 = 0; f0 < n_fields; f0 += 65535) {  // grid.z limit
     const int nf = n_fields - f0 < 65535 ? n_fields - f0 : 65535;
-    dim3 grid((rows + PBM - 1) / PBM, (max_nd + PBN - 1) / PBN, nf);
-    k_project_fp64<<<grid, kThreads, 0, s>>>(d_fields + f0, rows, n_ev);
+    const int bm = ctas64 < 2 * kSmHint ? 32 : 64;
+    dim3 grid((rows + bm - 1) / bm, (max_nd + PBN - 1) / PBN, nf);
+    if (bm == 32) k_project_fp64<1><<<grid, kThreads, 0, s>>>(d_fields + f0, rows, n_ev);
+    else k_project_fp64<2><<<grid, kThreads, 0, s>>>(d_fields + f0, rows, n_ev);
     note_launch();
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
@@ -279,7 +301,9 @@ __global__ void k_reduce_slabs(const ContractJob* __restrict__ jobs, int n_slab,
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < per;
        e += (long long)gridDim.x * blockDim.x) {
     double2 s = J.partial[e];
-    for (int sl = 1; sl < n_slab; ++sl) {   // fixed order: the result is run-to-run identical
+    // fixed order: the result is run-to-run identical; the loads of 8 slabs are in flight at once
+#pragma unroll 8
+    for (int sl = 1; sl < n_slab; ++sl) {
       const double2 v = J.partial[(size_t)sl * per + e];
       s.x += v.x;
       s.y += v.y;
