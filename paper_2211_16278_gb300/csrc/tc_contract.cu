@@ -121,6 +121,10 @@ __device__ __forceinline__ float tf32_round(float v) {
   return __uint_as_float(r);
 }
 
+__device__ __forceinline__ float2 sub2f(float2 a, float2 b) {
+  return make_float2(a.x - b.x, a.y - b.y);
+}
+
 // Split 8 FP32 values into LEVELS pieces and store each piece's 8 values as one K run of
 // a core-matrix row (16 bytes of BF16, or 32 bytes = two 16-byte rows of TF32).
 // BF16: the pieces are successive truncations to the top 8 significant bits,
@@ -212,8 +216,8 @@ __device__ __forceinline__ void split_store8_f16(const float (&v)[8], uint8_t* c
 #pragma unroll
   for (int i = 0; i < NG / 2; ++i) {
     const __half2 h = __floats2half2_rn(v[2 * i], v[2 * i + 1]);   // .x = low 16 bits
-    const float2 hf = __half22float2(h);
-    const __half2 l = __floats2half2_rn(v[2 * i] - hf.x, v[2 * i + 1] - hf.y);
+    const float2 d = sub2f(make_float2(v[2 * i], v[2 * i + 1]), __half22float2(h));
+    const __half2 l = __floats2half2_rn(d.x, d.y);
     hw[i] = *reinterpret_cast<const uint32_t*>(&h);
     lw[i] = *reinterpret_cast<const uint32_t*>(&l);
   }
@@ -371,6 +375,17 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
                 "the FP16 form: two pieces, contraction only, clusters only as CTA pairs");
   static_assert(!SHB || (F16 && C == 2 && !CHECKS), "CTA pairs: the FP16 form, unchecked");
   constexpr bool kShareA = C > 1 && !SHB;          // cluster CTAs share the diquark tile
+  // Row-factored clusters: two sets of four diquark warps take alternate stages (with two stage
+  // buffers, each set has one of its own). A thread then owns one of the CTA's 64 rows and 8
+  // groups as in the plain CTAs: a warp's loads are 32 rows of one site (2 wavefronts; 4 runs
+  // of 8 rows take 4) and its stores whole 16-byte runs. The tile's K halves lie apart, so that
+  // a warp's 4 row groups of every plane are one contiguous block, one copy to the peer (16
+  // before). Contraction of one time slice, L = 32, 9 momenta, N_dil = 64: 15.3 -> 14.6 ms; the
+  // bound is then the third quark's warps and the epilogue's read of its single accumulator.
+  constexpr bool kSets = RF && kShareA;
+  constexpr uint32_t kSetGroup = LEVELS * 2 * 384, kSetHalf = (kTcM / 8) * kSetGroup;
+  static_assert(!kSets || (C == 2 && TcLayout<TF32, LEVELS, F16, SHB, RF>::kStages == 2), "a set per stage buffer");
+  constexpr int kAG = kSets ? 8 : R::kAGroups;     // groups of a diquark thread
   constexpr int G = TF32 ? 8 : 16;                 // (site, pair) groups per stage
   // transaction bytes a stage receives from the peers: their diquark rows, every plane
   constexpr uint32_t kPeerTx = (uint32_t)((C - 1) * (R::kARows / 8) * 768 * LEVELS * 2);
@@ -381,7 +396,7 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
   constexpr int kBPlanes = Lay::kBPlanes;
   // groups whose loads a producer thread issues together before computing: all 8 in one
   // round where the registers allow it; the A-sharing cluster and checked variants would spill
-  constexpr int kLoadRun = (!kShareA && !CHECKS) ? 8 : 4;
+  constexpr int kLoadRun = ((!kShareA || kSets) && !CHECKS) ? 8 : 4;
   auto decode = [&](long long u) -> Unit {
     if constexpr (PROJ) return decode_unit_proj(prm, u, 3 * G);
     else if constexpr (RF) return decode_unit_rf(prm, u);
@@ -416,7 +431,8 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
 
   if (tid == 0) {
     for (int s = 0; s < STAGES; ++s) {
-      mbar_init(smem_u32(&bar_full[s]), R::kProdThreads / 32);   // one arrival per producer warp
+      // one arrival per producer warp (that takes the stage)
+      mbar_init(smem_u32(&bar_full[s]), R::kProdThreads / 32 - (kSets ? 4 : 0));
       mbar_init(smem_u32(&bar_empty[s]), C);   // the MMA completion of every CTA of the cluster
     }
     for (int b = 0; b < 2; ++b) {
@@ -477,7 +493,10 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
     int rr, g0;
     bool b_row_in = false;   // a third-quark row of this CTA's share
     if (is_a) {
-      if (!kShareA) {
+      if (kSets) {
+        rr = (int)rank * R::kARows + pt % 64;
+        g0 = (pt % 128 / 64) * 8;
+      } else if (!kShareA) {
         rr = pt % kTcM;
         g0 = (pt / kTcM) * 8;
       } else {
@@ -501,14 +520,57 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
         b_row_in = rr < NC;
       }
     }
-    const int NG = is_a ? R::kAGroups : R::kBGroups;
+    const int NG = is_a ? kAG : R::kBGroups;
     const bool row_used = is_a || (is_b && b_row_in);
-    // row-factored: a stage's first group (site x0 = xl of its lattice row, pair pr) and the
-    // phase index (n0 x0) mod L advance incrementally from stage to stage, with no division
-    // in the stage loop: each stage moves G groups on (G / np sites and G % np pairs)
-    const int rf_gq = RF ? G / prm.n_pairs : 0, rf_gr = RF ? G % prm.n_pairs : 0;
-    const int rf_xl0 = RF ? g0 / prm.n_pairs : 0, rf_pr0 = RF ? g0 % prm.n_pairs : 0;
-    int rf_sub = 0, rf_row = 0, rf_xl = 0, rf_pr = 0, rf_ph = 0, rf_ph0 = 0, rf_step = 0;
+    // This thread's K run in stage slot 0, plane 0 of its operand. Colour c occupies K bytes
+    // [32c, 32c + 32) (BF16; TF32: [32c, 32c + 32) of each 8-group stage as well); group g sits
+    // in 16-byte column 2c + g / 8 at 2 (g % 8).
+    const uint32_t run_ofs =
+        kSets && is_a ? (uint32_t)(g0 / 8) * kSetHalf + (uint32_t)(rr >> 3) * kSetGroup + (uint32_t)(rr & 7) * 16
+                      : row_seg(rr, g0 / 8) + (TF32 ? 0u : (uint32_t)((g0 % 8) * 2)) +
+                            (is_a ? 0u : (uint32_t)(LEVELS * 2 * kAPlaneBytes));
+    const uint32_t b_plane_bytes = (uint32_t)(NC * 96);
+    // split the NG groups' values of the 3 colours into pieces and store them. A side: planes
+    // Ar, Ai. B side: Br, Bi, and -Bi beside them (plane 0; two-MMA forms).
+    auto store_run = [&](float (&re)[3][8], float (&im)[3][8], auto kNG, auto kIsA, int slot) {
+      [[maybe_unused]] constexpr int NGc = decltype(kNG)::value;
+      constexpr bool Ac = decltype(kIsA)::value;
+      uint8_t* const run = smem + (uint32_t)(slot * STAGE_BYTES) + run_ofs;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        uint8_t* dr[LEVELS];
+        uint8_t* di[LEVELS];
+        uint8_t* dn[LEVELS];
+#pragma unroll
+        for (int l = 0; l < LEVELS; ++l) {
+          constexpr bool kS = kSets && Ac;
+          uint8_t* const q = run + c * (kS ? 128 : 256) +
+                             l * (kS ? 768 : Ac ? 2 * kAPlaneBytes : kBPlanes * Lay::kBPlaneB);
+          dr[l] = q + (Ac ? 0u : (uint32_t)Lay::kBr * b_plane_bytes);
+          di[l] = q + (kS ? 384u : Ac ? (uint32_t)kAPlaneBytes : (uint32_t)Lay::kBi * b_plane_bytes);
+          dn[l] = q;
+        }
+        uint8_t* const* neg = (Ac || !kTwoMma) ? nullptr : dn;
+        if constexpr (F16) {
+          split_store8_f16<NGc>(re[c], dr, nullptr);
+          split_store8_f16<NGc>(im[c], di, neg);
+        } else if constexpr (TF32) {
+          split_store8<TF32, LEVELS>(re[c], dr, nullptr);
+          split_store8<TF32, LEVELS>(im[c], di, neg);
+        } else {
+          split_store8<TF32, LEVELS, NGc>(re[c], dr, nullptr);
+          split_store8<TF32, LEVELS, NGc>(im[c], di, neg);
+        }
+      }
+    };
+    // a stage's first group (site g_xl of the slab or, row-factored, of the stage's lattice row,
+    // and pair g_pr) and the row-factored phase index (n0 x0) mod L advance incrementally from
+    // stage to stage, with no division in the stage loop: each stage moves G groups on
+    // (G / np sites and G % np pairs)
+    const int g_q = PROJ ? 0 : G / np, g_r = PROJ ? 0 : G % np;
+    const int g_xl0 = PROJ ? 0 : g0 / np, g_pr0 = PROJ ? 0 : g0 % np;
+    int g_xl = 0, g_pr = 0;
+    int rf_sub = 0, rf_row = 0, rf_ph = 0, rf_ph0 = 0, rf_step = 0;
     long long s_g = 0;
     for (long long u = u0; u < prm.total_units; u += du) {
       const Unit w = decode(u);
@@ -581,15 +643,17 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
         __syncwarp();
         named_bar(kBarProd, R::kProdThreads);
         if constexpr (!RF) phase_p = prm.phase + (size_t)pidx * prm.X;
+        g_xl = g_xl0; g_pr = g_pr0;
         if constexpr (RF) {
-          rf_ph0 = (pidx * rf_xl0) % prm.L;
-          rf_step = (pidx * rf_gq) % prm.L;
+          rf_ph0 = (pidx * g_xl0) % prm.L;
+          rf_step = (pidx * g_q) % prm.L;
           rf_sub = 0; rf_row = 0;
-          rf_xl = rf_xl0; rf_pr = rf_pr0; rf_ph = rf_ph0;
+          rf_ph = rf_ph0;
         }
       }
       for (int st = 0; st < w.n_stages; ++st, ++s_g) {
         const int slot = (int)(s_g % STAGES);
+        if (!kSets || !is_a || (int)(s_g & 1) == pt / 128) {
         bool ok = !abort_flag;
         if (ok && s_g >= STAGES)
           ok = wait_bounded(smem_u32(&bar_empty[slot]), (uint32_t)(((s_g / STAGES) + 1) & 1),
@@ -597,8 +661,8 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
         // a warp either fills its rows of this stage or (after an abort) none of them
         ok = __all_sync(0xffffffffu, ok);
         if (ok && row_used) {
-          float re[3][8], im[3][8];
           if constexpr (PROJ) {
+            float re[3][8], im[3][8];
             // element (colour c, group g0 + j) of this stage is eigenvector index l
             const int rows = prm.p_rows, n_ev = prm.p_n_ev;
             if (is_a) {
@@ -635,55 +699,65 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
                   im[c][j] = b.y;
                 }
             }
+            if (is_a) store_run(re, im, std::integral_constant<int, 8>{}, std::true_type{}, slot);
+            else store_run(re, im, std::integral_constant<int, 8>{}, std::false_type{}, slot);
           } else {
-            // the stage's sites [sx0, sx1) and this thread's first group of its run of NG
-            // (row-factored: the stage's row, groups counted from the row's first site)
-            int sx0 = w.x_begin, sx1 = w.x_end, xl, pr, ph = 0;
-            if constexpr (RF) {
-              sx0 = (w.x_begin + rf_row) * prm.L;
-              sx1 = sx0 + prm.L;
-              xl = rf_xl; pr = rf_pr; ph = rf_ph;
-            } else {
-              const int gi0 = st * G + g0;
-              xl = gi0 / np;
-              pr = gi0 - xl * np;
-            }
-            uint32_t vmask = 0;   // groups of this run that lie inside the slab and a used row
+            // the stage's sites [sx0, sx1): the slab's, or (row-factored) the stage's row, whose
+            // groups count from its first site; this thread's first group of its run of NG is
+            // (site sx0 + g_xl, pair g_pr)
+            const int sx0 = RF ? (w.x_begin + rf_row) * prm.L : w.x_begin;
+            const int sx1 = RF ? sx0 + prm.L : w.x_end;
             // One role's groups, with their group count and loads per group known at compile
             // time, so that each role's load buffers take only its own registers: the
             // diquark side loads 6 values per group in rounds of kLoadRun groups, the
-            // third-quark side 4 per group, all of its groups in one round (unchecked).
+            // third-quark side 4 per group, all of its groups in one round (unchecked). Then
+            // the run is split into pieces and stored. The producers' instructions bound the
+            // stage (half of its issue slots at 55 % issue activity), so offsets are 32-bit (a
+            // field has 3 X nd < 2^31 elements) and stores take one address per thread with
+            // constant plane offsets. Measured against 64-bit offsets and per-plane pointers,
+            // contraction of one time slice, L = 32, N_dil = 64: BF16 6 products, 5 momenta
+            // 34.9 -> 31.4 ms, TF32 46.7 -> 40.0, FP16 pairs, 9 momenta 38.3 -> 34.0.
+            // (Tried without gain: packed FP32 pairs; the next run's loads issued ahead of the
+            // split and the wait, 15.5 against 14.6 ms row-factored; row sums in registers with
+            // setmaxnreg, 17.4.)
             auto build = [&](auto kNG, auto kIsA) {
               constexpr int NGc = decltype(kNG)::value;
               constexpr bool Ac = decltype(kIsA)::value;
               constexpr int LR = Ac ? (kLoadRun < NGc ? kLoadRun : NGc) : (CHECKS ? 4 : NGc);
               constexpr int NV = Ac ? 6 : 4;
+              float re[3][8], im[3][8];
+              uint32_t vmask = 0;   // groups of this run that lie inside the slab and a used row
+              int xl = g_xl, pr = g_pr;
+              [[maybe_unused]] int ph = rf_ph;
+              const int s1x3 = 3 * s1, s2x3 = 3 * s2;
 #pragma unroll
               for (int half = 0; half < NGc / LR; ++half) {
                 // LR groups: issue every load first, then compute
                 float2 ld[LR][NV];
-                bool vld[LR];
 #pragma unroll
                 for (int j = 0; j < LR; ++j) {
                   const int x = sx0 + xl;
-                  vld[j] = row_ok && x < sx1;
-                  int xs = vld[j] ? x : sx0;
+                  bool vld = row_ok && x < sx1;
+                  int xs = x < sx1 ? x : sx0;
                   if (CHECKS) {
                     const long long fl = 3LL * prm.X * s1;            // elements of a field
                     bool good = idx_ok(prm, (long long)xs * 3 * s1 + off1 + 2LL * s1, fl, Ac ? 1 : 3, w.job) &&
                                 idx_ok(prm, pr, np, 6, w.job);
                     if (Ac) good = good && idx_ok(prm, (long long)xs * 3 * s2 + off2 + 2LL * s2, 3LL * prm.X * s2, 2, w.job);
                     else good = good && idx_ok(prm, (long long)pidx * prm.X + xs, (long long)prm.P * prm.X, 4, w.job);
-                    if (!good) { vld[j] = false; xs = 0; pr = 0; }
+                    if (!good) { vld = false; xs = 0; pr = 0; }
                   }
+                  vmask |= (uint32_t)vld << (half * LR + j);
+                  const uint32_t ou = (uint32_t)(xs * s1x3 + off1);
                   if constexpr (Ac) {
-                    const float2* uq = s_q1[pr] + (size_t)xs * 3 * s1 + off1;
-                    const float2* vq = s_q2[pr] + (size_t)xs * 3 * s2 + off2;
-                    ld[j][0] = uq[0]; ld[j][1] = uq[s1]; ld[j][2] = uq[2 * s1];
-                    ld[j][3] = vq[0]; ld[j][4] = vq[s2]; ld[j][5] = vq[2 * s2];
+                    const float2* const uf = s_q1[pr];
+                    const float2* const vf = s_q2[pr];
+                    const uint32_t ov = (uint32_t)(xs * s2x3 + off2);
+                    ld[j][0] = uf[ou]; ld[j][1] = uf[ou + s1]; ld[j][2] = uf[ou + 2 * s1];
+                    ld[j][3] = vf[ov]; ld[j][4] = vf[ov + s2]; ld[j][5] = vf[ov + 2 * s2];
                   } else {
-                    const float2* q = s_q3[pr] + (size_t)xs * 3 * s1 + off1;
-                    ld[j][0] = q[0]; ld[j][1] = q[s1]; ld[j][2] = q[2 * s1];
+                    const float2* const qf = s_q3[pr];
+                    ld[j][0] = qf[ou]; ld[j][1] = qf[ou + s1]; ld[j][2] = qf[ou + 2 * s1];
                     if constexpr (RF) ld[j][3] = s_omega[ph];
                     else ld[j][3] = phase_p[xs];
                   }
@@ -698,88 +772,43 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
                 }
 #pragma unroll
                 for (int j = 0; j < LR; ++j) {
-                  float2 c0, c1, c2;
+                  float2 c[3];
                   if constexpr (Ac) {
                     const float2 u0 = ld[j][0], u1 = ld[j][1], u2 = ld[j][2];
                     const float2 v0 = ld[j][3], v1 = ld[j][4], v2 = ld[j][5];
-                    const float2 a12 = cmulf(u1, v2), a21 = cmulf(u2, v1);
-                    const float2 a20 = cmulf(u2, v0), a02 = cmulf(u0, v2);
-                    const float2 a01 = cmulf(u0, v1), a10 = cmulf(u1, v0);
-                    c0 = make_float2(a12.x - a21.x, a12.y - a21.y);
-                    c1 = make_float2(a20.x - a02.x, a20.y - a02.y);
-                    c2 = make_float2(a01.x - a10.x, a01.y - a10.y);
+                    c[0] = sub2f(cmulf(u1, v2), cmulf(u2, v1));
+                    c[1] = sub2f(cmulf(u2, v0), cmulf(u0, v2));
+                    c[2] = sub2f(cmulf(u0, v1), cmulf(u1, v0));
                     if constexpr (F16) {
-                      c0.x *= f16s; c0.y *= f16s;
-                      c1.x *= f16s; c1.y *= f16s;
-                      c2.x *= f16s; c2.y *= f16s;
+#pragma unroll
+                      for (int k = 0; k < 3; ++k) { c[k].x *= f16s; c[k].y *= f16s; }
                     }
                   } else {
                     float2 phv = ld[j][3];
                     if constexpr (F16) { phv.x *= f16s; phv.y *= f16s; }
-                    c0 = cmulf(phv, ld[j][0]);
-                    c1 = cmulf(phv, ld[j][1]);
-                    c2 = cmulf(phv, ld[j][2]);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) c[k] = cmulf(phv, ld[j][k]);
                   }
                   const int jj = half * LR + j;
-                  vmask |= (uint32_t)vld[j] << jj;
-                  re[0][jj] = c0.x; im[0][jj] = c0.y;
-                  re[1][jj] = c1.x; im[1][jj] = c1.y;
-                  re[2][jj] = c2.x; im[2][jj] = c2.y;
+#pragma unroll
+                  for (int k = 0; k < 3; ++k) { re[k][jj] = c[k].x; im[k][jj] = c[k].y; }
                 }
               }
+              // groups past the slab's end or of an unused row (their loads read a valid site)
+              // contribute zeros; this branch is taken only at ragged edges
+              if (vmask != (1u << NGc) - 1u) {
+#pragma unroll
+                for (int jj = 0; jj < NGc; ++jj)
+                  if (!((vmask >> jj) & 1u)) {
+                    re[0][jj] = 0.f; im[0][jj] = 0.f;
+                    re[1][jj] = 0.f; im[1][jj] = 0.f;
+                    re[2][jj] = 0.f; im[2][jj] = 0.f;
+                  }
+              }
+              store_run(re, im, kNG, kIsA, slot);
             };
-            if (is_a) build(std::integral_constant<int, R::kAGroups>{}, std::true_type{});
+            if (is_a) build(std::integral_constant<int, kAG>{}, std::true_type{});
             else build(std::integral_constant<int, R::kBGroups>{}, std::false_type{});
-            // groups past the slab's end or of an unused row (their loads read a valid site)
-            // contribute zeros; this branch is taken only at ragged edges
-            if (vmask != (1u << NG) - 1u) {
-#pragma unroll
-              for (int jj = 0; jj < 8; ++jj)
-                if (!((vmask >> jj) & 1u)) {
-                  re[0][jj] = 0.f; im[0][jj] = 0.f;
-                  re[1][jj] = 0.f; im[1][jj] = 0.f;
-                  re[2][jj] = 0.f; im[2][jj] = 0.f;
-                }
-            }
-          }
-          // colour c occupies K bytes [32c, 32c + 32) (BF16; TF32: [32c, 32c + 32) of each
-          // 8-group stage as well); group g sits in 16-byte column 2c + g / 8 at 2 (g % 8)
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const int seg = 2 * c + g0 / 8;
-            const uint32_t in_row = TF32 ? 0u : (uint32_t)((g0 % 8) * 2);
-            // A side: planes Ar, Ai. B side: Br, Bi, and -Bi beside them (plane 0).
-            uint8_t* dr[LEVELS];
-            uint8_t* di[LEVELS];
-            uint8_t* dn[LEVELS];
-#pragma unroll
-            for (int l = 0; l < LEVELS; ++l) {
-              const uint32_t o = row_seg(rr, seg) + in_row;
-              dr[l] = smem + (is_a ? a_plane(slot, l, 0) : b_plane(slot, l, Lay::kBr)) + o;
-              di[l] = smem + (is_a ? a_plane(slot, l, 1) : b_plane(slot, l, Lay::kBi)) + o;
-              dn[l] = smem + b_plane(slot, l, 0) + o;
-            }
-            uint8_t* const* neg = (is_a || !kTwoMma) ? nullptr : dn;
-            if constexpr (F16) {
-              if (NG == 8) {
-                split_store8_f16<8>(re[c], dr, nullptr);
-                split_store8_f16<8>(im[c], di, neg);
-              } else {
-                split_store8_f16<4>(re[c], dr, nullptr);
-                split_store8_f16<4>(im[c], di, neg);
-              }
-            } else if constexpr (TF32) {
-              split_store8<TF32, LEVELS>(re[c], dr, nullptr);
-              split_store8<TF32, LEVELS>(im[c], di, neg);
-            } else {
-              if (NG == 8) {
-                split_store8<TF32, LEVELS>(re[c], dr, nullptr);
-                split_store8<TF32, LEVELS>(im[c], di, neg);
-              } else {
-                split_store8<TF32, LEVELS, 4>(re[c], dr, nullptr);
-                split_store8<TF32, LEVELS, 4>(im[c], di, neg);
-              }
-            }
           }
         }
         // every lane's core-matrix stores are made visible to the tensor core's (async)
@@ -806,7 +835,15 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
                 }
             }
           }
-          if (kShareA && is_a && ok) {
+          if (kSets && is_a && ok) {
+            // this warp's 32 diquark rows and K half of every plane go to the peer
+            const uint32_t src = smem_base + (uint32_t)(slot * STAGE_BYTES) +
+                                 (uint32_t)(g0 / 8) * kSetHalf + (uint32_t)(rr >> 3) * kSetGroup;
+            const uint32_t peer = rank ^ 1u;
+            copy_to_peer(map_to_rank(src, peer), src, 4 * kSetGroup,
+                         map_to_rank(smem_u32(&bar_full[slot]), peer));
+          }
+          if (kShareA && !kSets && is_a && ok) {
             // this warp's 8 diquark rows (one row group) of every plane go to every peer
             const uint32_t rg = (uint32_t)(rr >> 3);
             const uint32_t full_local = smem_u32(&bar_full[slot]);
@@ -822,23 +859,30 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
                 }
             }
           }
-          if (C > 1 && pt == 0)
+          if (C > 1 && (pt == 0 || (kSets && pt == 128)))
             mbar_arrive_expect_tx(smem_u32(&bar_full[slot]), peer_tx);
           else
             mbar_arrive(smem_u32(&bar_full[slot]));
         }
         __syncwarp();
-        if constexpr (RF) {
+        }
+        if constexpr (!PROJ) {
           // the next stage's first group: G groups on, or the next row's first
-          if (++rf_sub == prm.rf_spr) {
+          bool next_row = false;
+          if constexpr (RF) next_row = ++rf_sub == prm.rf_spr;
+          if (next_row) {
             rf_sub = 0; ++rf_row;
-            rf_xl = rf_xl0; rf_pr = rf_pr0; rf_ph = rf_ph0;
+            g_xl = g_xl0; g_pr = g_pr0; rf_ph = rf_ph0;
           } else {
-            rf_xl += rf_gq;
-            rf_pr += rf_gr;
-            rf_ph += rf_step;
-            if (rf_pr >= np) { rf_pr -= np; ++rf_xl; rf_ph += pidx; }
-            while (rf_ph >= prm.L) rf_ph -= prm.L;
+            g_xl += g_q;
+            g_pr += g_r;
+            const bool wrap = g_pr >= np;
+            if (wrap) { g_pr -= np; ++g_xl; }
+            if constexpr (RF) {
+              rf_ph += rf_step;
+              if (wrap) rf_ph += pidx;
+              while (rf_ph >= prm.L) rf_ph -= prm.L;
+            }
           }
         }
       }
@@ -887,8 +931,10 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
             const uint32_t first = (chunk_first && ks == 0) ? 0u : 1u;
 #pragma unroll
             for (int q = 0; q < NPROD; ++q) {
-              const uint64_t ar = smem_desc(sa + (PI[q] * 2 + 0) * kAPlaneBytes + kofs);
-              const uint64_t ai = smem_desc(sa + (PI[q] * 2 + 1) * kAPlaneBytes + kofs);
+              const uint64_t ar = kSets ? smem_desc(sa + (PI[q] * 2 + 0) * 384 + ks * 128, kSetGroup, kSetHalf)
+                                        : smem_desc(sa + (PI[q] * 2 + 0) * kAPlaneBytes + kofs);
+              const uint64_t ai = kSets ? smem_desc(sa + (PI[q] * 2 + 1) * 384 + ks * 128, kSetGroup, kSetHalf)
+                                        : smem_desc(sa + (PI[q] * 2 + 1) * kAPlaneBytes + kofs);
               const uint32_t bl = sb + (uint32_t)(PJ[q] * kBPlanes * Lay::kBPlaneB);
               const uint32_t d = q == 0 ? lead : corr;
               const uint32_t acc = (q <= 1) ? first : 1u;

@@ -46,10 +46,12 @@ __device__ __forceinline__ void tc_fence_before() {
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
-__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t sbo = 768) {
-  // K-major, no swizzle: LBO = 128 B between core matrices along K, SBO (768 B for stages of
-  // K = 48 BF16 elements, 256 B for K = 16) between 8-row groups; descriptor version 1.
-  return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)(128 >> 4) << 16) |
+__device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t sbo = 768,
+                                              uint32_t lbo = 128) {
+  // K-major, no swizzle: LBO (128 B unless the K halves are apart) between core matrices along
+  // K, SBO (768 B for stages of K = 48 BF16 elements, 256 B for K = 16) between 8-row groups;
+  // descriptor version 1.
+  return (uint64_t)((saddr >> 4) & 0x3FFF) | ((uint64_t)((lbo >> 4) & 0x3FFF) << 16) |
          ((uint64_t)((sbo >> 4) & 0x3FFF) << 32) | ((uint64_t)1 << 46);
 }
 template <bool TF32>
