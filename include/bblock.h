@@ -251,8 +251,8 @@ int bblock_last_wave_count(const bblock_ctx* ctx);
                                        Index checks and the wait-limit test hook use no
                                        clusters. BBLOCK_OZAKI: 1, 2, 3 or 4 CTAs sharing each
                                        diquark tile across adjacent N tiles (results bitwise
-                                       those of 1); 0 (default): 2 unless the ragged last
-                                       clusters pad the N tiles by more than 20 %, else 1 */
+                                       those of 1); 0 (default): chosen from the wave's N
+                                       tiles (ragged last clusters pad them) */
 #define BBLOCK_OPT_CORRUPT_CANARY 9  /* test hook (with BBLOCK_OPT_CHECKS): 1 makes the next
                                        call overwrite its first canary from the host, in
                                        stream order between the fill and the check, once */
@@ -267,7 +267,10 @@ int bblock_last_wave_count(const bblock_ctx* ctx);
                                   fit; 2: never (CTA pairs over all (p, d3) columns). With it,
                                   BBLOCK_OPT_TC_NC sets the d3 columns per tile. Not with
                                   index checks, per-momentum coefficients or the wait-limit
-                                  test hook */
+                                  test hook. BBLOCK_OZAKI has the same choice, along the lattice
+                                  axis with the fewest distinct components of the momenta:
+                                  0 (default) where it is expected to be faster, 1 wherever it
+                                  fits, 2 never (columns over all (p, d3)) */
 #define BBLOCK_OPT_TC_PROJECTION 12  /* mixed forms' projection (Eq. 2): 0 (default) on the
                                        tensor cores from pre-tiled operands (V once per
                                        distinct V of a call's wave, and every field's folded

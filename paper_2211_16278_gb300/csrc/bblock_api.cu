@@ -1164,24 +1164,27 @@ OzRows plan_oz_rows(const bblock_ctx* c, const int32_t* momenta, int n_mom, int 
   return r;
 }
 
-// The whole launch sequence for a list of jobs sharing momenta and spin operator.
-// Ozaki form: clusters of C CTAs share each diquark tile across C adjacent N tiles; each
-// builds 1/C of the tile's rows, with shorter per-thread chains, which sets the stage time.
-// Measured on GB300 (L = 32, 9 momenta, N_dil 32-64): pairs are the fastest, 1.6x the plain
-// CTA; clusters of 3 and 4 are 10 % and 3 % slower than pairs (fewer resident CTAs: 138 and
-// 144 of 152 SMs, and N tiles padded to a multiple of C). Auto: pairs unless their ragged
-// last clusters pad the N tiles by more than 20 %.
+// Ozaki form: clusters of C CTAs share each diquark tile across C adjacent N tiles; each builds
+// 1/C of the tile's rows, which sets the stage time, but the last cluster of a ragged job pads its
+// N tiles, and fewer CTAs of larger clusters are resident (138 and 144 of 152 SMs at 3 and 4).
+// Measured per N tile slot (L = 32, 9 momenta, row-factored, N_dil 32 to 64): 1.95, 1, 1.27 and
+// 1.06 for C = 1 to 4. Auto: the C with the least slots times that over the wave's jobs.
 int oz_cluster_for(const bblock_ctx* c, const std::vector<JobIn>& jobs, size_t b, size_t e,
                    int P_launch, int nc) {
   if (c->opt_tc_cluster >= 1 && c->opt_tc_cluster <= 4) return c->opt_tc_cluster;
-  long long tiles = 0, padded = 0;
-  for (size_t k = b; k < e; ++k) {
-    const long long nt = ((long long)P_launch * jobs[k].nd[2] + nc - 1) / nc;
-    const long long mt = ((long long)jobs[k].nd[0] * jobs[k].nd[1] + kOzM - 1) / kOzM;
-    tiles += mt * nt;
-    padded += mt * ((nt + 1) / 2) * 2;
+  const double slot_cost[4] = {1.95, 1.0, 1.27, 1.06};
+  int best = 1;
+  double least = 0.0;
+  for (int cl = 1; cl <= 4; ++cl) {
+    double sum = 0.0;
+    for (size_t k = b; k < e; ++k) {
+      const long long nt = ((long long)P_launch * jobs[k].nd[2] + nc - 1) / nc;
+      const long long mt = ((long long)jobs[k].nd[0] * jobs[k].nd[1] + kOzM - 1) / kOzM;
+      sum += (double)(mt * ((nt + cl - 1) / cl) * cl) * slot_cost[cl - 1];
+    }
+    if (cl == 1 || sum < least) { least = sum; best = cl; }
   }
-  return tiles > 0 && (double)(padded - tiles) / tiles <= 0.2 ? 2 : 1;
+  return best;
 }
 
 // The mode triplet of every job's V in the FP64 or double-float form: the ordered elements

@@ -3,10 +3,20 @@
 // split error-free into short integer digits whose products the tensor cores sum exactly.
 //
 // The contraction is the complex GEMM of the other tensor-core forms,
-//   C[(d1,d2)][(p,d3)] = sum_k A[(d1,d2)][k] Bop[k][(p,d3)],   k = (site, spin pair, colour),
-// A the diquark (q1_alpha x q2_beta)_c(x) and Bop = e^{-i p.x} q3_(alpha beta)[x][c][d3], built
-// here from the double-float fields and phases (about 48 significant bits) of the
-// double-float projection.
+//   C[(d1,d2)][(p,d3)] = sum_k A[(d1,d2)][k] Bop[k][(p,d3)],   k = (site, spin group, colour),
+// A the diquark sum over the group's terms (the spin triples sharing a quark spin) of
+// (q_alpha x q_beta)_c(x), and Bop = e^{-i p.x} q3_gamma[x][c][d3], built here from the
+// double-float fields and phases (about 48 significant bits) of the double-float projection.
+//
+// Row-factored units (RF): the columns are (n0, d3) for the distinct components n0 of the momenta
+// along one axis, Bop = w^{n0 x0} q3, and the epilogue multiplies each lattice row's sum by
+// w^{n1 x1 + n2 x2} into one double-float running sum per momentum. 9 momenta have 3 or so
+// distinct n0, so the MMAs and the third quark's digits fall by that ratio; a row's last stage
+// is padded with zeros and its epilogue costs 2 double-float products per momentum and element,
+// beside the next row's MMAs. L = 32, 9 momenta, 4 triples in 2 groups, jobs of N_dil 48 and 32,
+// contraction: 148 ms with (p, d3) columns per spin pair, 57 ms grouped and row-factored, 42.6 ms
+// with the producers' element runs and digits as rolled loops (9.9 -> 7.7, 44 -> 32 and
+// 78 -> 60.6 ms for one job of N_dil 32, 48, 64).
 //
 // * Scales. Every row m = (d1, d2) of A gets, per site slab, a power of two 2^eA bounding
 //   |Re| and |Im| of its entries: |(u_b v_c - u_c v_b)| <= |u_b||v_c| + |u_c||v_b|
@@ -107,13 +117,8 @@ template <int C> struct OzRoles {
 };
 __host__ __device__ constexpr int group_begin(int r, int C) { return (kOzM / 8) * r / C; }
 
-// 1.5 * 2^(16 - 8 i): adding and subtracting it rounds |v| < 2^(15 - 8 i) to the nearest
-// multiple of 2^(-7 - 8 i).
-__device__ __forceinline__ float round_const(int i) {
-  constexpr float r[kDigits] = {0x1.8p16f, 0x1.8p8f, 0x1.8p0f, 0x1.8p-8f, 0x1.8p-16f,
-                                0x1.8p-24f, 0x1.8p-32f};
-  return r[i];
-}
+// A digit's rounding constant is 1.5 * 2^(16 - 8 i): adding and subtracting it rounds
+// |v| < 2^(15 - 8 i) to the nearest multiple of 2^(-7 - 8 i).
 
 // Packed (re, im) FP32 arithmetic; a - b as fma(-1, b, a) rounds exactly like a subtraction.
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) {
@@ -147,18 +152,6 @@ __device__ __forceinline__ int exp_a(float M, float u, float v) {
   return ceil_log2(__fmul_rn(__fmaf_rn(0x1p-19f * u, v, M), 1.f + 0x1p-20f));
 }
 __device__ __forceinline__ int exp_b(float w) { return ceil_log2(__fmul_rn(w, 1.f + 0x1p-18f)); }
-
-// acc = a * b (double-float, three leading partial products)
-__device__ __forceinline__ dfloat df_prod(dfloat a, dfloat b) {
-  const float p = __fmul_rn(a.h, b.h);
-  float e = fmaf(a.h, b.h, -p);
-  e = fmaf(a.h, b.l, e);
-  e = fmaf(a.l, b.h, e);
-  return dfloat{p, e};
-}
-__device__ __forceinline__ dfloat df_neg(dfloat a) { return dfloat{-a.h, -a.l}; }
-__device__ __forceinline__ dfloat dre(float4 z) { return dfloat{z.x, z.y}; }
-__device__ __forceinline__ dfloat dim(float4 z) { return dfloat{z.z, z.w}; }
 
 // Packed double-float products, (re, im) in the two lanes: acc = a * b and acc += a * b with
 // a = (ah, al), b = (bh, bl) pairs of FP32x2 (the three leading partial products; the low
@@ -378,20 +371,23 @@ __device__ __forceinline__ void oz_produce(const ContractParams& prm, const OzSh
         // G = (E + 4) / 3 (site, group) pairs; the loads of a batch of elements (4 diquark
         // elements of one term, 8 third-quark ones) are all issued before its arithmetic, so
         // that their latencies overlap.
-        constexpr int G = (E + 4) / 3;
-        constexpr int LB = A ? 4 : 8;
-        int gg[G], xg[G];
+        // The runs of 4 elements of an 8-element thread and the digits are rolled loops: with
+        // three roles of straight-line code in flight on an SM, instruction fetch was the
+        // largest stall (2.7 of 11 cycles an issue).
+        constexpr int LB = 4, G = 2;
+        int hc = c0, hg = g0, hx = x0, hk = kk0;
+#pragma unroll 1
+        for (int h = 0; h < E / LB; ++h) {
+          int gg[G], xg[G];
 #pragma unroll
-        for (int k = 0; k < G; ++k) {
-          int g = g0 + k, xx = x0;
-          while (g >= ng) { g -= ng; ++xx; }
-          gg[k] = g;
-          xg[k] = xx;
-        }
-        float2 va[E], vb[E];   // scaled entries (re, im): high parts, low parts
-        int c = c0, gi = 0, kk = kk0;
-#pragma unroll
-        for (int b0 = 0; b0 < E; b0 += LB) {
+          for (int k = 0; k < G; ++k) {
+            int g = hg + k, xx = hx;
+            while (g >= ng) { g -= ng; ++xx; }
+            gg[k] = g;
+            xg[k] = xx;
+          }
+          float2 va[LB], vb[LB];   // scaled entries (re, im): high parts, low parts
+          int c = hc, gi = 0, kk = hk;
           bool vld[LB];
           int eg[LB], ex[LB], ec[LB];   // group, site and colour of the batch's elements
 #pragma unroll
@@ -472,42 +468,50 @@ __device__ __forceinline__ void oz_produce(const ContractParams& prm, const OzSh
           for (int jj = 0; jj < LB; ++jj) {
             // elements past the run's K or of an unused row are zero
             const float sv = vld[jj] ? sc : 0.f;
-            va[b0 + jj] = __fmul2_rn(v[jj].h, make_float2(sv, sv));
-            vb[b0 + jj] = __fmul2_rn(v[jj].l, make_float2(sv, sv));
+            va[jj] = __fmul2_rn(v[jj].h, make_float2(sv, sv));
+            vb[jj] = __fmul2_rn(v[jj].l, make_float2(sv, sv));
           }
-        }
-        // digits, most significant first; each digit's E values are one K run of the row
+          // digits, most significant first; each digit's 4 values are one K run of the row
+          uint8_t* dp = sh.smem + (uint32_t)(slot * kStageBytes) + (A ? a_row : (uint32_t)kAStage + b_row) + h * 8;
+          float Rc = 0x1.8p16f;   // 1.5 * 2^(16 - 8 i)
+#pragma unroll 1
+          for (int i = 0; i < kDigits; ++i) {
+            const float2 R2 = make_float2(Rc, Rc);
+            float2 d[LB];
 #pragma unroll
-        for (int i = 0; i < kDigits; ++i) {
-          const float Rc = round_const(i);
-          const float2 R2 = make_float2(Rc, Rc);
-          float2 d[E];
+            for (int j = 0; j < LB; ++j) {
+              if (i == 2 || i == 4) two_sum2(va[j], vb[j], va[j], vb[j]);
+              d[j] = sub2(__fadd2_rn(va[j], R2), R2);
+              va[j] = sub2(va[j], d[j]);
+            }
+            uint32_t wr[LB / 2], wi[LB / 2];
 #pragma unroll
-          for (int j = 0; j < E; ++j) {
-            if (i == 2 || i == 4) two_sum2(va[j], vb[j], va[j], vb[j]);
-            d[j] = sub2(__fadd2_rn(va[j], R2), R2);
-            va[j] = sub2(va[j], d[j]);
+            for (int q = 0; q < LB / 2; ++q) {
+              wr[q] = pack_bf16(d[2 * q].x, d[2 * q + 1].x);
+              wi[q] = pack_bf16(d[2 * q].y, d[2 * q + 1].y);
+            }
+            if (A) {
+              store_run<LB>(dp, wr);
+              store_run<LB>(dp + 256, wi);
+              dp += 512;
+            } else {
+              uint32_t wn[LB / 2];
+#pragma unroll
+              for (int q = 0; q < LB / 2; ++q) wn[q] = wi[q] ^ 0x80008000u;
+              // third-quark digit i, planes -Bi, Br, Bi (NC rows each, adjacent)
+              store_run<LB>(dp, wn);
+              store_run<LB>(dp + NC * kK * 2, wr);
+              store_run<LB>(dp + 2 * NC * kK * 2, wi);
+              dp += 3 * kBPlaneMax;
+            }
+            Rc *= 0x1p-8f;
           }
-          uint32_t wr[E / 2], wi[E / 2];
-#pragma unroll
-          for (int q = 0; q < E / 2; ++q) {
-            wr[q] = pack_bf16(d[2 * q].x, d[2 * q + 1].x);
-            wi[q] = pack_bf16(d[2 * q].y, d[2 * q + 1].y);
-          }
-          const uint32_t stage = (uint32_t)(slot * kStageBytes);
-          if (A) {
-            store_run<E>(sh.smem + stage + (uint32_t)((i * 2 + 0) * 256) + a_row, wr);
-            store_run<E>(sh.smem + stage + (uint32_t)((i * 2 + 1) * 256) + a_row, wi);
-          } else {
-            uint32_t wn[E / 2];
-#pragma unroll
-            for (int q = 0; q < E / 2; ++q) wn[q] = wi[q] ^ 0x80008000u;
-            // third-quark digit i, planes -Bi, Br, Bi (NC rows each, adjacent)
-            uint8_t* bp = sh.smem + stage + kAStage + (uint32_t)(i * 3 * kBPlaneMax) + b_row;
-            store_run<E>(bp, wn);
-            store_run<E>(bp + NC * kK * 2, wr);
-            store_run<E>(bp + 2 * NC * kK * 2, wi);
-          }
+          // the next 4 elements: one group and one colour on
+          int groups = 1;
+          if (++hc == 3) { hc = 0; ++groups; }
+          hg += groups;
+          while (hg >= ng) { hg -= ng; ++hx; }
+          hk += LB;
         }
       }
       // every lane's stores are made visible to the async proxy; then one lane acts for the
@@ -765,7 +769,7 @@ k_contract_oz(const __grid_constant__ ContractParams prm) {
             const bool last = ch == n_chunks - 1;
             float4* const part = reinterpret_cast<float4*>(J.partial) +
                                  (size_t)w.slab * prm.P_total * nd3 * M + m;
-            constexpr int UB = 8;   // updates whose loads are in flight together
+            constexpr int UB = 4;   // updates whose loads are in flight together
             for (int b = 0; b < n_upd; b += UB) {
               float4 run[UB], ts[UB], *at[UB];
               int mom[UB], d3s[UB];
