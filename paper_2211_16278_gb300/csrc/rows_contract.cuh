@@ -19,7 +19,9 @@
 //     and 4 for every +-n0 class: e^{-ip.x} = w^{n0 x0} w^{n1 x1 + n2 x2}, a lattice row is
 //     summed over x0 against each class first. With e = c + i s the four real sums c Sr, s Si,
 //     c Si, s Sr give both signs: (c Sr -+ s Si) + i (c Si +- s Sr). Without a class
-//     (RowPlan picks the axis with the fewest) k1..k3 run on over the whole row, unrecombined;
+//     (RowPlan picks the axis with the fewest) k1..k3 run on over the whole row, unrecombined
+//     (FP64; in double-float the longer sums of the larger k's cost accuracy, 4.2e-14 against
+//     2.7e-14 at L = 24, so each site is recombined, 4 operations);
 //   * 4 per momentum and row at the row's end, into the unit's partial block, which stays in
 //     L2 (the read-modify-write is below 3 % of the L2 rate in the FP64 form).
 // (A singlet per spin pair and a phase product per momentum and site take 9 n_pairs + 2 + 4 P:
@@ -51,6 +53,7 @@ __device__ __forceinline__ int find_job(const ContractJob* jobs, int n_jobs, lon
 
 // IEEE double on the FP64 pipe. T: a number, Cx: a complex number, Z: its 16 bytes in memory.
 struct ArithF64 {
+  static constexpr bool kEachSite = false;   // recombine k1..k3 at each site also without a class
   using T = double;
   struct Cx { double re, im; };
   using Z = double2;
@@ -69,6 +72,7 @@ struct ArithF64 {
 // Double-float pairs on the FP32 pipe (12 instructions per multiply-add), low parts collected
 // lazily: norm() brings them back below ulp(h) / 2.
 struct ArithDf {
+  static constexpr bool kEachSite = true;
   using T = dfloat;
   using Cx = dcomplex;
   using Z = float4;
@@ -239,6 +243,16 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
                 A::fma_add(k3[i][j], ai[i], be[j]);
               }
           }
+          if (NCLS == 0 && A::kEachSite) {
+#pragma unroll
+            for (int i = 0; i < RM; ++i)
+#pragma unroll
+              for (int j = 0; j < ACT; ++j) {
+                zr[i][j] = A::add(zr[i][j], A::sub(k1[i][j], k3[i][j]));
+                zi[i][j] = A::add(zi[i][j], A::add(k1[i][j], k2[i][j]));
+                k1[i][j] = k2[i][j] = k3[i][j] = A::zero();
+              }
+          }
           if (NCLS > 0) {
             Cx e[NC];
 #pragma unroll
@@ -326,11 +340,6 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
         for (int i = 0; i < RM; ++i)
 #pragma unroll
           for (int j = 0; j < RN; ++j) {
-            if (NCLS == 0) {
-              k1[i][j] = A::norm(k1[i][j]);
-              k2[i][j] = A::norm(k2[i][j]);
-              k3[i][j] = A::norm(k3[i][j]);
-            }
             zr[i][j] = A::norm(zr[i][j]);
             zi[i][j] = A::norm(zi[i][j]);
 #pragma unroll
@@ -349,7 +358,7 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
       for (int i = 0; i < RM; ++i)
 #pragma unroll
         for (int j = 0; j < RN; ++j)
-          if (NCLS == 0) {
+          if (NCLS == 0 && !A::kEachSite) {
             zr[i][j] = A::norm(A::sub(k1[i][j], k3[i][j]));
             zi[i][j] = A::norm(A::add(k1[i][j], k2[i][j]));
           }
