@@ -139,6 +139,7 @@ struct ContractParams {
   int b_slot[kMaxPairs];         // term -> line-2 field
   // FP64 and double-float forms: lattice extent, rows (of L^2) per slab, sites of a row staged at a time
   int L, rows_per_slab, xc;
+  int row_parts;                 // above 1: a slab is one of row_parts runs of sites of one row
   RowPlan rows;
   const double2* phase;          // w^k = e^{-2 pi i k / L}, k = 0..L-1
   int p0;                        // Ozaki form: first momentum of this launch

@@ -44,6 +44,7 @@ struct NoallocParams {
 // the spin coefficients folded while the tile is staged, and w^k by sincospi.
 struct NoallocSource {
   using Cx = rowsc::ArithF64::Cx;
+  static constexpr bool kRowParts = true;
   const NoallocParams* np;
   __device__ const ContractJob& job(long long) const { return np->job; }
   __device__ static double2 fold(const NaFold& f, const double2* q, size_t spin_stride, size_t at) {
@@ -84,21 +85,44 @@ k_contract_fp64_noalloc(const __grid_constant__ NoallocParams prm) {
   rowsc::contract_rows<rowsc::ArithF64, NCLS, kRowRM, RN>(prm.base, NoallocSource{&prm});
 }
 
-// B[e] = sum over slabs of partial[slab][e], slabs in index order.
+// B[e] = sum over slabs of partial[slab][e]: LANES threads per element take runs of the slabs, in
+// index order, with the loads of 8 in flight, then their sums in order. A small call has many slabs
+// of few elements, one long chain of loads at one thread per element (L = 6, N_dil 14, 11, 9, 5
+// momenta, 72 slabs: the call takes 72.3 us with 1 thread, 62.6 with 8).
+template <int LANES>
 __global__ void k_reduce_noalloc(const double2* __restrict__ partial, double2* __restrict__ B,
                                  long long per, int n_slab) {
-  for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < per;
-       e += (long long)gridDim.x * blockDim.x) {
-    double2 s = partial[e];
-    for (int sl = 1; sl < n_slab; ++sl) {
-      const double2 v = partial[(size_t)sl * per + e];
-      s.x += v.x;
-      s.y += v.y;
+  constexpr int E = kThreads / LANES;   // elements of a block at a time
+  __shared__ double2 sums[LANES][E];
+  const int le = threadIdx.x % E, lane = threadIdx.x / E;
+  const int run = (n_slab + LANES - 1) / LANES;
+  const int s0 = min(n_slab, lane * run), s1 = min(n_slab, s0 + run);
+  for (long long e0 = blockIdx.x * (long long)E; e0 < per; e0 += (long long)gridDim.x * E) {
+    const long long e = e0 + le;
+    double2 s = make_double2(0.0, 0.0);
+    if (e < per) {
+#pragma unroll 8
+      for (int sl = s0; sl < s1; ++sl) {
+        const double2 v = partial[(size_t)sl * per + e];
+        s.x += v.x;
+        s.y += v.y;
+      }
     }
-    B[e] = s;
+    if (LANES > 1) {
+      sums[lane][le] = s;
+      __syncthreads();
+      if (lane == 0) {
+#pragma unroll
+        for (int k = 1; k < LANES; ++k) {
+          s.x += sums[k][le].x;
+          s.y += sums[k][le].y;
+        }
+      }
+      __syncthreads();
+    }
+    if (lane == 0 && e < per) B[e] = s;
   }
 }
-
 
 template <int NCLS, int RN>
 cudaError_t na_launch(const NoallocParams& prm, int grid, cudaStream_t s) {
@@ -310,23 +334,39 @@ extern "C" int bblock_contract_noalloc(int L, const void* q1, const void* q2, co
     return na_fail(err, err_len, BBLOCK_ERR_CUDA, "device query failed");
   }
   const long long tiles = (long long)job.m_tiles * job.n_tiles;
-  // Slabs of lattice rows, at most what the scratch holds: the count with the fewest rows on the
-  // busiest SM (the FP64 pipe is shared by an SM's CTAs, so only its units count). With 12 slabs
-  // allowed and 32 tiles (L = 16, N_dil = 32, 5 momenta) 12 would put 3 units of 22 rows on some
-  // SMs, 9 put 2 of 29: 9.64 -> 8.36 ms.
+  // Slabs of lattice rows, at most what the scratch holds: the count with the least work on the
+  // busiest SM (the FP64 pipe is shared by an SM's CTAs, so only its units count), in operations
+  // of the contraction per output: 9 per group and 4 per class of a site, 6 per momentum of a
+  // row's end. With 12 slabs allowed and 32 tiles (L = 16, N_dil = 32, 5 momenta) 12 would put 3
+  // units of 22 rows on some SMs, 9 put 2 of 29: 9.64 -> 8.36 ms. Where single rows are too coarse
+  // for the SMs, rows are divided into runs of sites, each with a row's end of its own (L = 6,
+  // N_dil 14, 11, 9, 5 momenta: contraction 63.5 -> 57.8 us).
+  // Among equals, the count with the least work one after another: an SM's resident CTAs take the
+  // latencies side by side.
   const int n_rows = L * L;
-  long long best = -1;
-  for (long long n = 1; n <= (long long)max_slabs_fit && n <= n_rows; ++n) {
-    const long long rps = (n_rows + n - 1) / n, slabs = (n_rows + rps - 1) / rps;
-    const long long cost = (tiles * slabs + num_sms - 1) / num_sms * rps;
-    if (best < 0 || cost < best) {
+  const long long resident = (long long)rows_ctas_per_sm(n_cls, rn) * num_sms;
+  const long long site_ops = 9 * base.n_groups + 4 + 4 * n_cls, row_ops = 6 * n_mom;
+  long long best = -1, best_chain = 0;
+  auto consider = [&](int rps, int parts) {
+    const long long slabs = (n_rows + rps - 1) / rps * (long long)parts;
+    const long long work = rps * ((L + parts - 1) / parts * site_ops + row_ops);
+    const long long cost = (tiles * slabs + num_sms - 1) / num_sms * work;
+    const long long chain = (tiles * slabs + resident - 1) / resident * work;
+    if (best < 0 || cost < best || (cost == best && chain < best_chain)) {
       best = cost;
-      base.rows_per_slab = (int)rps;
+      best_chain = chain;
+      base.rows_per_slab = rps;
+      base.row_parts = parts;
+      base.n_slab = (int)slabs;
     }
-    if (slabs * tiles >= 8LL * num_sms) break;   // finer slabs gain nothing more
-  }
+    return slabs * tiles < 8LL * num_sms;   // finer slabs gain nothing more
+  };
+  bool finer = true;
+  for (long long n = 1; finer && n <= (long long)max_slabs_fit && n <= n_rows; ++n)
+    finer = consider((int)((n_rows + n - 1) / n), 1);
+  for (int parts = 2; finer && parts <= L && (long long)n_rows * parts <= (long long)max_slabs_fit; ++parts)
+    finer = consider(1, parts);
   base.sites_per_slab = base.rows_per_slab * L;
-  base.n_slab = (n_rows + base.rows_per_slab - 1) / base.rows_per_slab;
   base.total_units = tiles * base.n_slab;
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -338,10 +378,11 @@ extern "C" int bblock_contract_noalloc(int L, const void* q1, const void* q2, co
     e = na_dispatch(prm, rn, (int)(base.total_units < cap ? base.total_units : cap), s);
   }
   if (e == cudaSuccess) {
-    long long bx = ((long long)per + kThreads - 1) / kThreads;
+    const int lanes = base.n_slab >= 16 ? 8 : 1;
+    long long bx = ((long long)per * lanes + kThreads - 1) / kThreads;
     if (bx > 4096) bx = 4096;
-    k_reduce_noalloc<<<(unsigned)bx, kThreads, 0, s>>>(job.partial, static_cast<double2*>(B_out),
-                                                       (long long)per, base.n_slab);
+    (lanes == 8 ? k_reduce_noalloc<8> : k_reduce_noalloc<1>)<<<(unsigned)bx, kThreads, 0, s>>>(
+        job.partial, static_cast<double2*>(B_out), (long long)per, base.n_slab);
     note_launch();
     e = cudaGetLastError();
   }

@@ -118,6 +118,7 @@ __device__ __forceinline__ void cross_add(typename A::Cx& acc, typename A::Cx a,
 template <class A> struct TableSource {
   using Cx = typename A::Cx;
   using Z = typename A::Z;
+  static constexpr bool kRowParts = false;   // slabs are whole rows
   const ContractParams* prm;
   __device__ const ContractJob& job(long long u) const {
     return prm->jobs[find_job(prm->jobs, prm->n_jobs, u)];
@@ -184,8 +185,16 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
     // the 16-column blocks that hold an l3 > l2 of the tile's first row are needed
     const int col0 = (J.tri ? (tri_l2(mt * MT) + 1) / 16 * 16 : 0) + nt * NT;
     if (col0 >= nd3) continue;
-    const int row_begin = slab * prm.rows_per_slab;
-    const int row_end = min(L * L, row_begin + prm.rows_per_slab);
+    // a slab of rows, or, of small lattices, one run of sites of a row
+    int row_begin = slab * prm.rows_per_slab, row_end = min(L * L, row_begin + prm.rows_per_slab);
+    int x_begin = 0, x_end = L;
+    if (Src::kRowParts && prm.row_parts > 1) {
+      const int len = (L + prm.row_parts - 1) / prm.row_parts;
+      row_begin = slab / prm.row_parts;
+      row_end = row_begin + 1;
+      x_begin = min(L, (slab - row_begin * prm.row_parts) * len);
+      x_end = min(L, x_begin + len);
+    }
     const int ms = mt * MT + ml;
     const bool m_ok = ms < M;
     int d1 = 0, d2 = 0;
@@ -279,8 +288,8 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
         }
       };
 
-      for (int x0 = 0; x0 < L; x0 += XC) {
-        const int nx = min(XC, L - x0);
+      for (int x0 = x_begin; x0 < x_end; x0 += XC) {   // [0, L) without parts
+        const int nx = min(XC, x_end - x0);
         // --- diquark tile: A[(xc, group, c)][m], the group's terms summed
         for (int xc = tid / MT; xc < nx; xc += kThreads / MT) {
           const int x = base + (x0 + xc) * sx;
