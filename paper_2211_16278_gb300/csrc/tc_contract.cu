@@ -563,6 +563,41 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
         }
       }
     };
+    // The same with the role's plane offsets in registers, one copy of the code for both roles: they
+    // run side by side, and instruction fetch is what a second copy costs (3.2 instead of 2.0
+    // cycles an issue). Contraction with two copies and with one: TF32, L = 7, N_dil = 42, one
+    // pair 223 -> 190 us; BF16 3 products, L = 24, N_dil = 42 1.41 -> 1.35 ms; row-factored
+    // clusters, L = 32, six jobs of N_dil 32 to 64 49.0 -> 47.5 ms, L = 48 47.6 -> 46.5. The short
+    // FP16 split of plain row-factored CTAs keeps two (L = 7, N_dil = 16: 38.5, one copy 39.0 us).
+    const uint32_t run_step = is_a ? (kSets ? 768u : 2u * kAPlaneBytes) : (uint32_t)(kBPlanes * Lay::kBPlaneB);
+    const uint32_t run_re = is_a ? 0u : (uint32_t)Lay::kBr * b_plane_bytes;
+    const uint32_t run_im = is_a ? (kSets ? 384u : (uint32_t)kAPlaneBytes) : (uint32_t)Lay::kBi * b_plane_bytes;
+    const uint32_t run_c = kSets && is_a ? 128u : 256u;
+    auto store_run_any = [&](float (&re)[3][8], float (&im)[3][8], auto kNG, int slot) {
+      [[maybe_unused]] constexpr int NGc = decltype(kNG)::value;
+      uint8_t* const run = smem + (uint32_t)(slot * STAGE_BYTES) + run_ofs;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        uint8_t* dr[LEVELS];
+        uint8_t* di[LEVELS];
+        uint8_t* dn[LEVELS];
+#pragma unroll
+        for (int l = 0; l < LEVELS; ++l) {
+          uint8_t* const q = run + c * run_c + l * run_step;
+          dr[l] = q + run_re;
+          di[l] = q + run_im;
+          dn[l] = q;
+        }
+        uint8_t* const* neg = (is_a || !kTwoMma) ? nullptr : dn;
+        if constexpr (F16) {
+          split_store8_f16<NGc>(re[c], dr, nullptr);
+          split_store8_f16<NGc>(im[c], di, neg);
+        } else {
+          split_store8<TF32, LEVELS, TF32 ? 8 : NGc>(re[c], dr, nullptr);
+          split_store8<TF32, LEVELS, TF32 ? 8 : NGc>(im[c], di, neg);
+        }
+      }
+    };
     // a stage's first group (site g_xl of the slab or, row-factored, of the stage's lattice row,
     // and pair g_pr) and the row-factored phase index (n0 x0) mod L advance incrementally from
     // stage to stage, with no division in the stage loop: each stage moves G groups on
@@ -720,12 +755,13 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
             // (Tried without gain: packed FP32 pairs; the next run's loads issued ahead of the
             // split and the wait, 15.5 against 14.6 ms row-factored; row sums in registers with
             // setmaxnreg, 17.4.)
+            constexpr bool kOneStore = (!F16 || kSets) && R::kBGroups == kAG;
+            float re[3][8], im[3][8];
             auto build = [&](auto kNG, auto kIsA) {
               constexpr int NGc = decltype(kNG)::value;
               constexpr bool Ac = decltype(kIsA)::value;
               constexpr int LR = Ac ? (kLoadRun < NGc ? kLoadRun : NGc) : (CHECKS ? 4 : NGc);
               constexpr int NV = Ac ? 6 : 4;
-              float re[3][8], im[3][8];
               uint32_t vmask = 0;   // groups of this run that lie inside the slab and a used row
               int xl = g_xl, pr = g_pr;
               [[maybe_unused]] int ph = rf_ph;
@@ -805,10 +841,11 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
                     re[2][jj] = 0.f; im[2][jj] = 0.f;
                   }
               }
-              store_run(re, im, kNG, kIsA, slot);
+              if constexpr (!kOneStore) store_run(re, im, kNG, kIsA, slot);
             };
             if (is_a) build(std::integral_constant<int, kAG>{}, std::true_type{});
             else build(std::integral_constant<int, R::kBGroups>{}, std::false_type{});
+            if constexpr (kOneStore) store_run_any(re, im, std::integral_constant<int, kAG>{}, slot);
           }
         }
         // every lane's core-matrix stores are made visible to the tensor core's (async)
