@@ -151,27 +151,41 @@ def projection_flops(X, n_ev, nd, n_alpha, n_beta, pairs):
     return 8.0 * 3 * X * n_ev * (n_alpha * nd[0] + n_beta * nd[1] + pairs * nd[2])
 
 
-def folded_gemm_flops(X, nd, P, pairs):
+def third_quark_groups(spins):
+    """Groups of spin terms the FP64-accurate forms sum: one per (alpha, beta) pair, or one per
+    gamma where those are fewer (the benchmarked operators)."""
+    s3 = {tuple(int(v) for v in s) for s in np.asarray(spins).reshape(-1, 3)}
+    return min(len({s[:2] for s in s3}), len({s[2] for s in s3}))
+
+
+def folded_gemm_flops(X, nd, P, groups):
     """Useful flops of the folded contraction run on the tensor cores: one complex GEMM
-    of M = d1 d2, N = P d3, K = 3 pairs X, 8 M N K (phase and colour sum folded in). With
-    the row-factored phase P is the number of distinct n0 of the momenta instead."""
-    return 8.0 * nd[0] * nd[1] * (P * nd[2]) * (3 * pairs * X)
+    of M = d1 d2, N = P d3, K = 3 groups X, 8 M N K (phase and colour sum folded in): groups are
+    the (alpha, beta) pairs, or third_quark_groups in the Ozaki form. With the row-factored
+    phase P is the number of distinct n0 of the momenta instead."""
+    return 8.0 * nd[0] * nd[1] * (P * nd[2]) * (3 * groups * X)
 
 
 def phase_columns(path, L, momenta):
     """Phase columns per d3 of the tensor-core GEMM: every momentum, or (row-factored
-    path) the distinct x-components n0 mod L."""
+    path) the distinct x-components n0 mod L; in the Ozaki form (row-factored on the
+    benchmarked workloads) those along the axis with the fewest."""
     mom = np.asarray(momenta).reshape(-1, 3)
-    return len({int(m[0]) % L for m in mom}) if path.startswith("tc_rows") else len(mom)
+    distinct = [len({int(m[a]) % L for m in mom}) for a in range(3)]
+    return distinct[0] if path.startswith("tc_rows") else min(distinct) if path == "ozaki" else len(mom)
 
 
-def contraction_df_inst(X, nd, P, pairs):
+def contraction_df_inst(X, nd, momenta, spins):
     """FP32 instructions of the double-float contraction's inner loops per (time slice,
     noise triple): 12 per double-float FMA (exact product error, TwoSum, lazy error sum),
-    three per (pair, colour) in the singlet, four per momentum, 16 for the singlet's real and
-    imaginary parts; per (d1, d2, d3, x)."""
+    three per (group, colour) in the singlet, 16 for its real and imaginary parts, 16 for the
+    momenta of n0 = 0 and four FMAs per class of +-n0 along the axis with the fewest, and four
+    per momentum and lattice row; per (d1, d2, d3, x)."""
     d1, d2, d3 = nd
-    return (108.0 * pairs + 16.0 + 48.0 * P) * d1 * d2 * d3 * X
+    L = round(X ** (1 / 3))
+    mom = np.asarray(momenta).reshape(-1, 3)
+    classes = min(len({min(int(m[a]) % L, -int(m[a]) % L) for m in mom} - {0}) for a in range(3))
+    return (108.0 * third_quark_groups(spins) + 32.0 + 48.0 * (classes + len(mom) / L)) * d1 * d2 * d3 * X
 
 
 # ------------------------------------------------------------------ clocks
@@ -520,8 +534,9 @@ def fp64_roofline(prof, alg_flops, steps, traffic, traffic_rec):
             "traffic": traffic,
             "traffic_capture": traffic_rec.get("captured_workload") if traffic_rec else None,
             "peak_source": FP64_PEAK["source"],
-            "flops": "paper-ordering complex count (cmul 6, complex FMA 8); the kernel "
-                     "executes about 80/96 of it (three-multiplication complex products)",
+            "flops": "paper-ordering complex count (cmul 6, complex FMA 8); the kernel executes "
+                     "a third to a half of it (spin terms grouped by third quark, momenta summed "
+                     "along lattice rows, three-multiplication complex products)",
             "flops_per_launch": alg_flops * steps / n_c,
             "launches": n_c, "avg_launch_ms": ms_c / n_c}
 
@@ -815,9 +830,11 @@ def fp64_form_per_size(R, w, inp, V, phis, head_ms_per_step, blocks_per_step, ch
         if form == "fp64":
             roof = fp64_roofline(pr, alg, 2, None, None)
         elif form == "df64":
-            roof = df_roofline(pr, contraction_df_inst(w.X, nd, P, pairs), alg, 2)
+            roof = df_roofline(pr, contraction_df_inst(w.X, nd, inp.momenta, inp.spins), alg, 2)
         else:
-            roof = tensor_roofline(form, pr, folded_gemm_flops(w.X, nd, P, pairs), alg, 2,
+            cols = phase_columns(bb.bblock_last_path(c), w.L, inp.momenta)
+            groups = third_quark_groups(inp.spins) if form == "ozaki" else pairs
+            roof = tensor_roofline(form, pr, folded_gemm_flops(w.X, nd, cols, groups), alg, 2,
                                    None, None, bb.bblock_last_path(c))
         per_size[nd[0]] = {"noise": k, "ms_per_job": t_ms / 2, "blocks_per_s": 2 * P / (t_ms / 1e3),
                            "roofline": roof, "kernels": kernel_table(pr, t_ms)}
@@ -931,13 +948,14 @@ def run_single(args, R, w, rank, head, clk, steps, warmup, extras=True):
     value = job_throughput(R.world, blocks_per_step, steps, ms / 1e3)
 
     def gemm_of(c):
-        return n_t * folded_gemm_flops(w.X, nd, phase_columns(bb.bblock_last_path(c), w.L,
-                                                              inp.momenta), pairs)
+        path = bb.bblock_last_path(c)
+        return n_t * folded_gemm_flops(w.X, nd, phase_columns(path, w.L, inp.momenta),
+                                       third_quark_groups(inp.spins) if path == "ozaki" else pairs)
     if head == "fp64":
         traffic, trec = load_traffic(f"k_contract_fp64/fp64/{w.name}") if full_shape else (None, None)
         roofline = fp64_roofline(prof, contract_alg, steps, traffic, trec)
     elif head == "df64":
-        roofline = df_roofline(prof, n_t * contraction_df_inst(w.X, nd, P, pairs), contract_alg,
+        roofline = df_roofline(prof, n_t * contraction_df_inst(w.X, nd, inp.momenta, inp.spins), contract_alg,
                                steps)
     else:
         path = bb.bblock_last_path(ctx)
@@ -961,7 +979,7 @@ def run_single(args, R, w, rank, head, clk, steps, warmup, extras=True):
                    f"speedup_vs_{head}_form": ms / t_ms,
                    "kernels": kernel_table(pr, t_ms)}
             if name == "df64":
-                ent["alu_roofline"] = df_roofline(pr, n_t * contraction_df_inst(w.X, nd, P, pairs),
+                ent["alu_roofline"] = df_roofline(pr, n_t * contraction_df_inst(w.X, nd, inp.momenta, inp.spins),
                                                   contract_alg, steps)
             elif name == "fp64":
                 ent["alu_roofline"] = fp64_roofline(pr, contract_alg, steps, None, None)
