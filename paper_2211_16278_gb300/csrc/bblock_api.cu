@@ -22,8 +22,9 @@ struct bblock_ctx {
   std::string err;
   cudaStream_t last_stream = nullptr;
   int* d_status = nullptr;
-  // phase cache
+  // phase cache: phase_mom and omega_ready are set once the table they stand for is filled
   std::vector<int32_t> phase_mom;
+  bool omega_ready = false;       // FP64 and double-float forms: d_phase holds w^k
   double2* d_phase = nullptr;     // FP64 phases [n_mom][X], then their FP32 copy
   float2* d_phase_f = nullptr;
   float4* d_phase_df = nullptr;    // Ozaki form: the phases as double-float float4
@@ -185,6 +186,7 @@ int fail(bblock_ctx* c, int code, const char* fmt, ...) {
 }
 
 int cuda_fail(bblock_ctx* c, cudaError_t e, const char* what) {
+  cudaGetLastError();   // reported here: not again by the next call's first launch
   return fail(c, BBLOCK_ERR_CUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
@@ -419,16 +421,18 @@ GroupPlan plan_groups(const SpinPlan& sp, bool may_group, const std::vector<JobI
 int ensure_phase(bblock_ctx* c, const int32_t* momenta, int n_mom, cudaStream_t s) {
   if (c->cfg.precision == BBLOCK_FP64 || c->cfg.precision == BBLOCK_DF64) {
     // these contractions need w^k = e^{-2 pi i k / L} only, whatever the momenta
-    if (c->d_phase) return BBLOCK_OK;
+    if (c->omega_ready) return BBLOCK_OK;
     int rc = grow_device(c, reinterpret_cast<char**>(&c->d_phase), &c->phase_cap,
                          sizeof(double2) * c->cfg.L);
     if (rc) return rc;
     CK(c, timed_launch(c, K_PHASE, s, [&] { return launch_omega_table(c->cfg.L, c->d_phase, s); }));
     CK(c, cudaStreamSynchronize(s));   // later calls may come on another stream
+    c->omega_ready = true;
     return BBLOCK_OK;
   }
   std::vector<int32_t> key(momenta, momenta + 3 * n_mom);
   if (c->d_phase && key == c->phase_mom) return BBLOCK_OK;
+  c->phase_mom.clear();   // until this call's table is filled, none is
   const size_t n_ph = (size_t)c->X * n_mom;
   const bool oz = c->cfg.precision == BBLOCK_OZAKI;
   const size_t df_ofs = align_up((sizeof(double2) + sizeof(float2)) * n_ph, 256);
