@@ -114,29 +114,31 @@ __global__ void k_tri_fill(const TriSlice* __restrict__ slices, int n, int n_mom
   }
 }
 
-// Complex GEMMs of the three mode products, FP64. Bound by the FP64 pipe: three-multiplication
-// complex products (re = k1 - k3, im = k1 + k2; the operand sums formed once per staged element)
-// take 3 instead of 4 operations per multiply-add, and the row tile is the one that wastes fewer
-// rows: 64 (T x3 phi3, thousands of rows), or 32 (the products over N_dil rows, half of a 64-row
-// tile idle at N_dil = 32). L = 24, N_ev = 96, N_dil = 32, 3 momenta, 3 pairs / 2 gammas, all
-// products of one time slice: 3.61 -> 1.67 ms (1.4 ms of FP64 operations).
+// Complex GEMMs of the three mode products, FP64, bound by the FP64 pipe. Four multiplications to a
+// complex one: the form with three (re = k1 - k3, im = k1 + k2) takes 1.74 instead of 2.12 ms for the
+// case below, but leaves each part accurate to the modulus only, and over three products in a row
+// the error grew from 1.13e-15 to 1.32e-15. The products of a list are summed from zero each and
+// then added, 9.8e-16 (in one chain 1.18e-15). The row tile is the one that wastes fewer rows:
+// 64 (T x3 phi3, thousands of rows), or 32 (the products over N_dil rows, half of a 64-row tile
+// idle at N_dil = 32). L = 24, N_ev = 96, N_dil = 32, 3 momenta, 3 pairs / 2 gammas, all products of
+// one time slice: 3.63 ms with a product per pair, 2.12 with one per group (1.8 of FP64 operations).
 constexpr int ZBK = 16, ZRN = 4, ZBN = 8 * ZRN;
 
-template <int RM>
+template <int RM, bool SUM>
 __global__ void __launch_bounds__(kThreads) k_zgemm(const __grid_constant__ ZgemmParams p) {
   constexpr int BM = 32 * RM;
-  __shared__ double Ar[ZBK][BM], Ai[ZBK][BM], As[ZBK][BM];
-  __shared__ double Bc[ZBK][ZBN], Bd[ZBK][ZBN], Be[ZBK][ZBN];
+  __shared__ double2 As[ZBK][BM], Bs[ZBK][ZBN];
   const int m0 = blockIdx.x * BM, n0 = blockIdx.y * ZBN;
   const long long bt = blockIdx.z % p.batch;
-  const int l0 = p.sum_list ? 0 : (int)(blockIdx.z / p.batch), l1 = p.sum_list ? p.n_list : l0 + 1;
-  double2* __restrict__ C = p.C[p.sum_list ? 0 : l0] + bt * p.c_b;
+  const int l0 = SUM ? 0 : (int)(blockIdx.z / p.batch), l1 = SUM ? p.n_list : l0 + 1;
+  double2* __restrict__ C = p.C[l0] + bt * p.c_b;
   const int tid = threadIdx.x, tn = tid % 8, tm = tid / 8;
-  double k1[RM][ZRN], k2[RM][ZRN], k3[RM][ZRN];
+  double re[RM][ZRN], im[RM][ZRN];
+  double sr[RM][ZRN], si[RM][ZRN];   // SUM: of the list's products, each summed from zero
 #pragma unroll
   for (int i = 0; i < RM; ++i)
 #pragma unroll
-    for (int j = 0; j < ZRN; ++j) k1[i][j] = k2[i][j] = k3[i][j] = 0.0;
+    for (int j = 0; j < ZRN; ++j) re[i][j] = im[i][j] = sr[i][j] = si[i][j] = 0.0;
 
   for (int l = l0; l < l1; ++l) {
     const double2* __restrict__ A = p.A[l] + bt * p.a_b;
@@ -148,46 +150,43 @@ __global__ void __launch_bounds__(kThreads) k_zgemm(const __grid_constant__ Zgem
         const int m = m0 + r, k = k0 + kk;
         double2 v = make_double2(0.0, 0.0);
         if (m < p.M && k < p.K) v = A[(long long)m * p.a_m + (long long)k * p.a_k];
-        Ar[kk][r] = v.x;
-        Ai[kk][r] = v.y;
-        As[kk][r] = v.x + v.y;
+        As[kk][r] = v;
       }
       for (int idx = tid; idx < ZBK * ZBN; idx += kThreads) {
         const int c = idx % ZBN, kk = idx / ZBN;
         const int n = n0 + c, k = k0 + kk;
         double2 v = make_double2(0.0, 0.0);
         if (n < p.N && k < p.K) v = B[(long long)k * p.b_k + (long long)n * p.b_n];
-        Bc[kk][c] = v.x;
-        Bd[kk][c] = v.y - v.x;
-        Be[kk][c] = v.x + v.y;
+        Bs[kk][c] = v;
       }
       __syncthreads();
       const int kn = min(ZBK, p.K - k0);
 #pragma unroll 4
       for (int kk = 0; kk < kn; ++kk) {
-        double ar[RM], ai[RM], as[RM], bc[ZRN], bd[ZRN], be[ZRN];
+        double2 a[RM], b[ZRN];
 #pragma unroll
-        for (int i = 0; i < RM; ++i) {
-          ar[i] = Ar[kk][tm + 32 * i];
-          ai[i] = Ai[kk][tm + 32 * i];
-          as[i] = As[kk][tm + 32 * i];
-        }
+        for (int i = 0; i < RM; ++i) a[i] = As[kk][tm + 32 * i];
 #pragma unroll
-        for (int j = 0; j < ZRN; ++j) {
-          bc[j] = Bc[kk][tn + 8 * j];
-          bd[j] = Bd[kk][tn + 8 * j];
-          be[j] = Be[kk][tn + 8 * j];
-        }
+        for (int j = 0; j < ZRN; ++j) b[j] = Bs[kk][tn + 8 * j];
 #pragma unroll
         for (int i = 0; i < RM; ++i)
 #pragma unroll
           for (int j = 0; j < ZRN; ++j) {
-            k1[i][j] = fma(bc[j], as[i], k1[i][j]);
-            k2[i][j] = fma(ar[i], bd[j], k2[i][j]);
-            k3[i][j] = fma(ai[i], be[j], k3[i][j]);
+            re[i][j] = fma(a[i].x, b[j].x, fma(-a[i].y, b[j].y, re[i][j]));
+            im[i][j] = fma(a[i].x, b[j].y, fma(a[i].y, b[j].x, im[i][j]));
           }
       }
       __syncthreads();
+    }
+    if (SUM) {
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < ZRN; ++j) {
+          sr[i][j] += re[i][j];
+          si[i][j] += im[i][j];
+          re[i][j] = im[i][j] = 0.0;
+        }
     }
   }
 #pragma unroll
@@ -199,7 +198,7 @@ __global__ void __launch_bounds__(kThreads) k_zgemm(const __grid_constant__ Zgem
       const int n = n0 + tn + 8 * j;
       if (n >= p.N) continue;
       double2& c = C[(long long)m * p.c_m + (long long)n * p.c_n];
-      double2 r = make_double2(k1[i][j] - k3[i][j], k1[i][j] + k2[i][j]);
+      double2 r = SUM ? make_double2(sr[i][j], si[i][j]) : make_double2(re[i][j], im[i][j]);
       if (p.accumulate) { r.x += c.x; r.y += c.y; }
       c = r;
     }
@@ -269,8 +268,8 @@ cudaError_t launch_zgemm(const ZgemmParams& p, cudaStream_t s) {
     q.batch = (int)(p.batch - b0 < step ? p.batch - b0 : step);
     const int bm = half ? 32 : 64;
     const dim3 grid((p.M + bm - 1) / bm, (p.N + ZBN - 1) / ZBN, q.batch * per);
-    if (half) k_zgemm<1><<<grid, kThreads, 0, s>>>(q);
-    else k_zgemm<2><<<grid, kThreads, 0, s>>>(q);
+    (p.sum_list ? half ? k_zgemm<1, true> : k_zgemm<2, true>
+                : half ? k_zgemm<1, false> : k_zgemm<2, false>)<<<grid, kThreads, 0, s>>>(q);
     note_launch();
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
