@@ -1191,6 +1191,58 @@ int oz_cluster_for(const bblock_ctx* c, const std::vector<JobIn>& jobs, size_t b
   return best;
 }
 
+// Slabs of an FP64 or double-float contraction: of whole lattice rows, or of staged chunks of sites
+// where the momenta have a phase per site.
+struct RowSlabs { int n, rows, sites, xc; };   // xc: sites of a chunk (a phase per site)
+RowSlabs row_slabs(const bblock_ctx* c, const RowPlan& r, int rn, int groups, long long tiles, int want) {
+  const int L = c->cfg.L, grid = rows_ctas_per_sm(r, rn) * c->num_sms, max_slabs = 64;
+  RowSlabs s{};
+  if (r.per_site) {
+    const int X = c->X, xc = s.xc = site_chunk(L, groups, tiles, grid);
+    const int n = want > 0 ? std::min(want, (X + xc - 1) / xc) : choose_slabs(tiles, grid, X, xc, max_slabs);
+    s.sites = ((X + n - 1) / n + xc - 1) / xc * xc;
+    s.n = (X + s.sites - 1) / s.sites;
+  } else {
+    const int n = want > 0 ? std::min(want, L * L) : choose_slabs(tiles, grid, L * L, 1, max_slabs);
+    s.rows = (L * L + n - 1) / n;
+    s.sites = s.rows * L;
+    s.n = (L * L + s.rows - 1) / s.rows;
+  }
+  return s;
+}
+
+// Spin groups, row plans (per-momentum coefficients: one plan per momentum) and d3 tile of an FP64 or
+// double-float call. The groups are planned for the widest tile, then once more for the one the
+// momenta leave: with narrow tiles a term's diquark is built more often.
+struct RowCall {
+  GroupPlan groups;
+  std::vector<RowPlan> plans;
+  int rn = 1;
+};
+RowCall plan_row_call(const bblock_ctx* c, const SpinPlan& sp, const int32_t* momenta, int n_mom,
+                      int per_mom, const std::vector<JobIn>& jobs) {
+  const int L = c->cfg.L;
+  const bool df = c->cfg.precision == BBLOCK_DF64;
+  int nd3 = 1;
+  for (const JobIn& j : jobs) nd3 = std::max(nd3, j.nd[2]);
+  RowCall r;
+  r.groups = plan_groups(sp, true, jobs, c->cfg.n_ev, 64);
+  const int G = r.groups.n_groups, T = r.groups.n_terms;
+  if (per_mom) {
+    r.plans.resize(n_mom);
+    for (int p = 0; p < n_mom; ++p) {
+      plan_rows(L, momenta + 3 * p, 1, G, T, nd3, df, &r.plans[p], 1);
+      r.plans[p].mom[0].p = p;
+    }
+  } else {
+    r.plans.resize(plan_rows(L, momenta, n_mom, G, T, nd3, df, nullptr, 0));
+    plan_rows(L, momenta, n_mom, G, T, nd3, df, r.plans.data(), (int)r.plans.size());
+  }
+  r.rn = rows_rn_for(r.plans.data(), (int)r.plans.size(), nd3);
+  if (r.rn < 4) r.groups = plan_groups(sp, true, jobs, c->cfg.n_ev, 16 * r.rn);
+  return r;
+}
+
 // The mode triplet of every job's V in the FP64 or double-float form: the ordered elements
 // l1 < l2 < l3 by the row-factored contraction, then T by its antisymmetry.
 int run_triplet(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momenta, int n_mom,
@@ -1198,11 +1250,9 @@ int run_triplet(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* mo
   const int L = c->cfg.L, rows = c->rows, n = c->cfg.n_ev, X = c->X;
   const bool df = c->cfg.precision == BBLOCK_DF64;
   const int M = n * (n - 1) / 2;
-  std::vector<RowPlan> rplans(plan_rows(L, momenta, n_mom, nullptr, 0));
-  plan_rows(L, momenta, n_mom, rplans.data(), (int)rplans.size());
-  int r_cls = 0;
-  for (const RowPlan& r : rplans) r_cls = std::max(r_cls, r.n_cls);
-  const int rn = rows_rn_for(r_cls, n);
+  std::vector<RowPlan> rplans(plan_rows(L, momenta, n_mom, 1, 1, n, df, nullptr, 0));
+  plan_rows(L, momenta, n_mom, 1, 1, n, df, rplans.data(), (int)rplans.size());
+  const int rn = rows_rn_for(rplans.data(), (int)rplans.size(), n);
   const int m_tiles = (M + 16 * kRowRM - 1) / (16 * kRowRM), n_tiles = (n + 16 * rn - 1) / (16 * rn);
   const int max_slabs = 64;
   const size_t f_bytes = align_up((size_t)rows * n * sizeof(double2), 256);
@@ -1217,11 +1267,8 @@ int run_triplet(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* mo
     const int nj = (int)(end - job_idx);
     ++c->last_waves;
     const long long tiles = std::max(1LL, (long long)nj * m_tiles * n_tiles);
-    int n_slab = c->opt_slabs > 0 ? std::min(c->opt_slabs, L * L)
-                                  : choose_slabs(tiles, rows_ctas_per_sm(rplans[0].n_cls, rn) * c->num_sms,
-                                                 L * L, 1, max_slabs);
-    const int per_slab = (L * L + n_slab - 1) / n_slab;
-    n_slab = (L * L + per_slab - 1) / per_slab;
+    const RowSlabs rs = row_slabs(c, rplans[0], rn, 1, tiles, c->opt_slabs);
+    const int n_slab = rs.n;
     int rc = grow_device(c, &c->d_ws, &c->ws_cap, nj * job_bytes(n_slab));
     if (rc) return rc;
     std::vector<ContractJob> cjobs(nj);
@@ -1266,19 +1313,19 @@ int run_triplet(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* mo
     prm.total_units = (long long)nj * m_tiles * n_tiles * n_slab;
     prm.X = X;
     prm.n_slab = n_slab;
-    prm.sites_per_slab = per_slab * L;
+    prm.sites_per_slab = rs.sites;
     prm.n_groups = prm.n_terms = 1;
     prm.tbeg[1] = 1;
     prm.L = L;
-    prm.rows_per_slab = per_slab;
+    prm.rows_per_slab = rs.rows;
     prm.phase = c->d_phase;
     prm.P_total = n_mom;
     prm.status = c->d_status;
     for (const RowPlan& r : rplans) {
       prm.rows = r;
-      prm.xc = rows_sites_per_chunk(L, r.n_cls, rn, 1);
+      prm.xc = r.per_site ? rs.xc : rows_sites_per_chunk(L, r, rn, 1);
       const int grid = (int)std::min<long long>(prm.total_units,
-                                                (long long)rows_ctas_per_sm(r.n_cls, rn) * c->num_sms);
+                                                (long long)rows_ctas_per_sm(r, rn) * c->num_sms);
       CK(c, timed_launch(c, K_CONTRACT, s, [&] {
         return df ? launch_contract_df(prm, rn, grid, s) : launch_contract_fp64(prm, rn, grid, s);
       }));
@@ -1318,9 +1365,11 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
 
   const int X = c->X, rows = c->rows, n_ev = c->cfg.n_ev, L = c->cfg.L;
   const bool rowf = !oz;   // FP64 and double-float: the row-factored contraction
-  int max_nd3_all = 1;
-  for (const JobIn& j : jobs) max_nd3_all = std::max(max_nd3_all, j.nd[2]);
-  const GroupPlan gp = plan_groups(sp, true, jobs, n_ev, rowf ? 64 : 32);
+  RowCall rc_rows;
+  if (rowf) rc_rows = plan_row_call(c, sp, momenta, n_mom, per_mom, jobs);
+  const GroupPlan gp = rowf ? rc_rows.groups : plan_groups(sp, true, jobs, n_ev, 32);
+  const std::vector<RowPlan>& rplans = rc_rows.plans;
+  const int row_rn = rc_rows.rn;
   OzRows ozr{};
   if (oz) ozr = plan_oz_rows(c, momenta, n_mom, per_mom, gp.n_groups);
   for (int g = 0; g < gp.n_groups; ++g)
@@ -1328,27 +1377,10 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
   ozr.max_terms = (float)ozr.max_terms_i;
   const size_t oz_scratch = ozr.on ? (size_t)c->num_sms * kOzMaxNC * kOzM * sizeof(float4) : 0;
   const int n2_fields = (int)gp.f2.size(), n3_fields = gp.n_groups * sp.n_coef_sets;
-  // the momenta in row plans (per-momentum coefficients: one plan per momentum)
-  std::vector<RowPlan> rplans;
-  int r_cls = 0;
-  if (rowf) {
-    if (per_mom) {
-      rplans.resize(n_mom);
-      for (int p = 0; p < n_mom; ++p) {
-        plan_rows(L, momenta + 3 * p, 1, &rplans[p], 1);
-        rplans[p].mom[0].p = p;
-      }
-    } else {
-      rplans.resize(plan_rows(L, momenta, n_mom, nullptr, 0));
-      plan_rows(L, momenta, n_mom, rplans.data(), (int)rplans.size());
-    }
-    for (const RowPlan& r : rplans) r_cls = std::max(r_cls, r.n_cls);
-  }
-  const int row_rn = rows_rn_for(r_cls, max_nd3_all);
   // Ozaki form: N columns per d3 of a launch, the momenta or their distinct n0
   const int P_cols = ozr.on ? ozr.nidx : per_mom ? 1 : n_mom;
   // Ozaki form: units run one per CTA (clusters: one per cluster of oz_cl CTAs)
-  const int ctas = (oz ? 1 : rows_ctas_per_sm(rplans[0].n_cls, row_rn)) * c->num_sms;
+  const int ctas = (oz ? 1 : rows_ctas_per_sm(rplans[0], row_rn)) * c->num_sms;
   const int max_slabs = 64;
   const int oz_nc = c->opt_tc_nc > 0 && c->opt_tc_nc <= kOzMaxNC ? c->opt_tc_nc : kOzMaxNC;
   int oz_cl = 1;   // Ozaki form: CTAs per cluster of the current wave
@@ -1412,15 +1444,24 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
       max_elems = std::max(max_elems, (long long)n_mom * j.nd[0] * j.nd[1] * j.nd[2]);
     }
     const int unit_slots = oz ? ctas / oz_cl : ctas;
-    // slabs are ranges of lattice rows (Ozaki form with momentum columns: of sites)
-    const bool row_slabs = rowf || ozr.on;
-    const int parts = row_slabs ? L * L : X;
-    int n_slab = c->opt_slabs > 0 ? std::min(c->opt_slabs, parts)
-                                   : choose_slabs(tiles, unit_slots, parts, 1, max_slabs);
-    const int per_slab = (parts + n_slab - 1) / n_slab;
-    n_slab = (parts + per_slab - 1) / per_slab;
-    const int sites_per_slab = row_slabs ? per_slab * L : per_slab;
-    ozr.slabs.per_slab = per_slab;
+    // slabs are ranges of lattice rows or (see row_slabs; Ozaki form with momentum columns) of sites
+    int n_slab, rows_per_slab, sites_per_slab, site_xc = 1;
+    if (rowf) {
+      const RowSlabs rs = row_slabs(c, rplans[0], row_rn, gp.n_groups, tiles, c->opt_slabs);
+      n_slab = rs.n;
+      rows_per_slab = rs.rows;
+      sites_per_slab = rs.sites;
+      site_xc = rs.xc;
+    } else {
+      const int parts = ozr.on ? L * L : X;
+      n_slab = c->opt_slabs > 0 ? std::min(c->opt_slabs, parts)
+                                : choose_slabs(tiles, unit_slots, parts, 1, max_slabs);
+      const int per_slab = (parts + n_slab - 1) / n_slab;
+      n_slab = (parts + per_slab - 1) / per_slab;
+      rows_per_slab = per_slab;
+      sites_per_slab = ozr.on ? per_slab * L : per_slab;
+      ozr.slabs.per_slab = per_slab;
+    }
 
     size_t ws_need = oz_scratch, oz_need = 0;
     for (size_t k = job_idx; k < end; ++k) {
@@ -1612,7 +1653,7 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
     memcpy(prm.a_slot, gp.a_slot, sizeof(prm.a_slot));
     memcpy(prm.b_slot, gp.b_slot, sizeof(prm.b_slot));
     prm.L = L;
-    prm.rows_per_slab = per_slab;
+    prm.rows_per_slab = rows_per_slab;
     prm.phase = c->d_phase;
     prm.P_total = n_mom;
     prm.status = c->d_status;
@@ -1642,9 +1683,9 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
       for (size_t k = 0; k < rplans.size(); ++k) {
         prm.jobs = reinterpret_cast<const ContractJob*>(c->d_tab + fbytes + jbytes * (per_mom ? k : 0));
         prm.rows = rplans[k];
-        prm.xc = rows_sites_per_chunk(L, prm.rows.n_cls, row_rn, gp.n_groups);
+        prm.xc = prm.rows.per_site ? site_xc : rows_sites_per_chunk(L, prm.rows, row_rn, gp.n_groups);
         const int grid = (int)std::min<long long>(
-            unit, (long long)rows_ctas_per_sm(prm.rows.n_cls, row_rn) * c->num_sms);
+            unit, (long long)rows_ctas_per_sm(prm.rows, row_rn) * c->num_sms);
         CK(c, timed_launch(c, K_CONTRACT, s, [&] {
           return df ? launch_contract_df(prm, row_rn, grid, s) : launch_contract_fp64(prm, row_rn, grid, s);
         }));
@@ -1811,12 +1852,14 @@ CallPlan plan_call(const bblock_ctx* c, int n_t, const int nd[3], int n_mom, int
     return pl;
   }
   if (fp64_like(c->cfg)) {
-    const int rn = rows_rn_for(1, nd[2]);
+    RowPlan one_class{};
+    one_class.n_cls = 1;
+    const int rn = rows_rn_for(&one_class, 1, nd[2]);
     const int parts = c->cfg.L * c->cfg.L;   // slabs of lattice rows
     const long long tiles = (long long)n_t * ((nd[0] * nd[1] + 16 * kRowRM - 1) / (16 * kRowRM)) *
                             ((nd[2] + 16 * rn - 1) / (16 * rn));
     const int ns = slabs_opt > 0 ? std::min(slabs_opt, parts)
-                                 : choose_slabs(tiles, rows_ctas_per_sm(1, rn) * c->num_sms, parts, 1, 64);
+                                 : choose_slabs(tiles, rows_ctas_per_sm(one_class, rn) * c->num_sms, parts, 1, 64);
     const int sps = (parts + ns - 1) / ns;
     pl.n_slab = (parts + sps - 1) / sps;
     pl.units = tiles * pl.n_slab;

@@ -13,9 +13,12 @@ constexpr int kMaxPairs = 16;   // distinct (alpha, beta) spin pairs
 constexpr int kMaxRfP = 16;
 constexpr int kMaxRfIdx = 8;
 constexpr int kMaxRfL = 128;    // lattice extent (the w^k table follows the stage buffers)
-// Row-factored FP64 and double-float contractions: momenta and +-n0 classes of one launch.
+// FP64 and double-float contractions: momenta and +-n0 classes of a row-factored launch, momenta of a
+// launch with a phase per site (as many as the accumulators fit: 10 in FP64, 8 in double-float).
 constexpr int kMaxRowP = 32;
 constexpr int kMaxRowCls = 3;
+constexpr int kMaxSiteP = 10;
+constexpr int kMaxSitePDf = 8;
 constexpr int kThreads = 256;   // threads per CTA of the FP64 kernels
 constexpr int kSmHint = 152;    // SMs of a GB300: where small launches take smaller tiles
 
@@ -91,13 +94,14 @@ __host__ __device__ inline int tri_l2(int m) {
   return l;
 }
 
-// A momentum of a row-factored launch: p = index in the call's list, n1 and n2 = its
-// components along the two axes that are not summed (ascending, reduced to [0, L)), sel = 0
-// where its component n0 along the summed axis is 0 mod L, +(c + 1) where n0 = cls_n0[c] and
-// -(c + 1) where n0 = -cls_n0[c] mod L.
+// A momentum of a launch: p = index in the call's list, n1 and n2 = its components along the two
+// axes that a row does not run along (ascending, reduced to [0, L)). sel: row-factored, 0 where its
+// component n0 along the row is 0 mod L, +(c + 1) where n0 = cls_n0[c] and -(c + 1) where
+// n0 = -cls_n0[c] mod L; with a phase per site, n0 in [0, L).
 struct RowMom { int p, n1, n2, sel; };
 struct RowPlan {
-  int axis;                      // the lattice axis whose sites a row sums
+  int axis;                      // the lattice axis along which rows run
+  int per_site;                  // 1: a phase per momentum and site, 0: row-factored
   int n_cls, cls_n0[kMaxRowCls]; // classes of +-n0, n0 in [1, L / 2]
   int has_zero;                  // a momentum has n0 = 0
   int n_mom;
@@ -137,7 +141,8 @@ struct ContractParams {
   int tbeg[kMaxPairs + 1];
   int a_slot[kMaxPairs];         // term -> line-1 slot
   int b_slot[kMaxPairs];         // term -> line-2 field
-  // FP64 and double-float forms: lattice extent, rows (of L^2) per slab, sites of a row staged at a time
+  // FP64 and double-float forms: lattice extent, rows (of L^2) per slab (with a phase per site:
+  // sites_per_slab), sites staged at a time
   int L, rows_per_slab, xc;
   int row_parts;                 // above 1: a slab is one of row_parts runs of sites of one row
   RowPlan rows;
@@ -155,38 +160,61 @@ struct ContractParams {
   long long wait_limit;
 };
 
-// Tiles of the row-factored FP64 and double-float contractions: 16 kRowRM (d1, d2) pairs by 16 rn d3 columns.
-// A wider d3 tile shares each diquark among more outputs; the row sums of the launch's classes
-// limit it (registers). One CTA per SM for the tiles that need more than 128 registers.
+// Tiles of the FP64 and double-float contractions: 16 kRowRM (d1, d2) pairs by 16 rn d3 columns.
+// A wider d3 tile shares each diquark among more outputs; the sums of the launch's classes or
+// momenta limit it (registers). One CTA per SM for the tiles that need more than 128 registers.
 constexpr int kRowRM = 2;
-inline int rows_max_rn(int n_cls) { return n_cls <= 1 ? 4 : 2; }
-inline int rows_ctas_per_sm(int n_cls, int rn) { return rn == 4 || n_cls >= 2 ? 1 : 2; }
-// rn for a launch sequence of at most n_cls classes over jobs of at most nd3 columns
-inline int rows_rn_for(int n_cls, int nd3) {
-  const int want = nd3 <= 16 ? 1 : nd3 <= 32 ? 2 : 4, most = rows_max_rn(n_cls);
-  return want < most ? want : most;
+constexpr int kSitePNarrow = 4;   // momenta of the per-site launches with two d3 columns a thread
+inline int rows_max_rn(const RowPlan& r) {
+  if (r.per_site) return r.n_mom > kSitePNarrow ? 1 : 2;
+  return r.n_cls <= 1 ? 4 : 2;
+}
+inline int rows_ctas_per_sm(const RowPlan& r, int rn) {
+  return rn == 4 || r.n_cls >= 2 ? 1 : 2;
+}
+// rn for a launch sequence of these plans over jobs of at most nd3 columns
+inline int rows_rn_for(const RowPlan* plans, int n_plans, int nd3) {
+  int rn = nd3 <= 16 ? 1 : nd3 <= 32 ? 2 : 4;
+  for (int k = 0; k < n_plans; ++k)
+    if (rows_max_rn(plans[k]) < rn) rn = rows_max_rn(plans[k]);
+  return rn;
+}
+// w^k of each staged site a launch keeps in shared memory
+inline int rows_phases(const RowPlan& r) {
+  if (r.per_site) return r.n_mom > kSitePNarrow ? kMaxSiteP : kSitePNarrow;
+  return r.n_cls > 0 ? r.n_cls : 1;
 }
 // Sites of a row staged at a time (KC = xc * groups * 3 operand rows of 24 (16 kRowRM + 16 rn)
 // bytes): as many as fit the CTA's share of the shared memory, in chunks of equal size.
-inline size_t rows_smem_bytes(int L, int n_cls, int rn, int n_groups, int xc) {
+inline size_t rows_smem_bytes(int L, const RowPlan& r, int rn, int n_groups, int xc) {
   return (size_t)24 * (16 * kRowRM + 16 * rn) * 3 * n_groups * xc +
-         16 * ((size_t)xc * (n_cls > 0 ? n_cls : 1) + L);
+         16 * ((size_t)xc * rows_phases(r) + L);
 }
-inline int rows_sites_per_chunk(int L, int n_cls, int rn, int n_groups) {
-  const size_t budget = (size_t)(rows_ctas_per_sm(n_cls, rn) == 1 ? 220 : 108) * 1024;
+inline int rows_sites_per_chunk(int L, const RowPlan& r, int rn, int n_groups) {
+  const size_t budget = (size_t)(rows_ctas_per_sm(r, rn) == 1 ? 220 : 108) * 1024;
   int xc = L < 16 ? L : 16;
-  while (xc > 1 && rows_smem_bytes(L, n_cls, rn, n_groups, xc) > budget) --xc;
+  while (xc > 1 && rows_smem_bytes(L, r, rn, n_groups, xc) > budget) --xc;
   const int chunks = (L + xc - 1) / xc;
   return (L + chunks - 1) / chunks;
 }
+// The same for a phase per site, where a slab is a number of chunks: 48 operand rows, fewer where the
+// units (tiles by chunks) would leave most of `slots` empty.
+inline int site_chunk(int L, int n_groups, long long tiles, long long slots) {
+  const int X = L * L * L, most = 16 / n_groups > 1 ? 16 / n_groups : 1;
+  int xc = most < X ? most : X;
+  while (xc > 2 && tiles * ((X + xc - 1) / xc) < slots / 4) xc = (xc + 1) / 2;
+  return xc;
+}
 // Whether the tile of the most groups a call can have fits the shared memory of a CTA.
-static_assert((size_t)24 * (16 * kRowRM + 64) * 3 * kMaxPairs + 16 * (kMaxRowCls + 128) <= 227 * 1024,
+static_assert((size_t)24 * (16 * kRowRM + 64) * 3 * kMaxPairs + 16 * (kMaxSiteP + 128) <= 227 * 1024,
               "one site of kMaxPairs groups fits");
-// The momenta of a call, each in one RowPlan: `axis` is the one with the fewest +-n0 classes
-// (the last on a tie), and a plan takes at most kMaxRowCls classes and kMaxRowP momenta.
+// The momenta of a call, each in one RowPlan: row-factored (at most kMaxRowP momenta and kMaxRowCls
+// classes each) or with a phase per site, whichever takes fewer operations (see fp64_kernels.cu).
+// groups, terms: of the spin sum; nd3: the widest job's d3 columns; df: double-float.
 // Returns the number of plans written to `out` (at most max_out), or the number needed where
 // out is null.
-int plan_rows(int L, const int32_t* momenta, int n_mom, RowPlan* out, int max_out);
+int plan_rows(int L, const int32_t* momenta, int n_mom, int groups, int terms, int nd3, bool df,
+              RowPlan* out, int max_out);
 
 // ---------------------------------------------------------------- tensor-core forms
 

@@ -79,10 +79,10 @@ struct NoallocSource {
   }
 };
 
-template <int NCLS, int RN>
+template <int NCLS, int NP, int RN>
 __global__ void __launch_bounds__(kThreads, RN == 4 || NCLS >= 2 ? 1 : 2)
 k_contract_fp64_noalloc(const __grid_constant__ NoallocParams prm) {
-  rowsc::contract_rows<rowsc::ArithF64, NCLS, kRowRM, RN>(prm.base, NoallocSource{&prm});
+  rowsc::contract_rows<rowsc::ArithF64, NCLS, NP, kRowRM, RN>(prm.base, NoallocSource{&prm});
 }
 
 // B[e] = sum over slabs of partial[slab][e]: LANES threads per element take runs of the slabs, in
@@ -124,32 +124,18 @@ __global__ void k_reduce_noalloc(const double2* __restrict__ partial, double2* _
   }
 }
 
-template <int NCLS, int RN>
-cudaError_t na_launch(const NoallocParams& prm, int grid, cudaStream_t s) {
-  const size_t smem = rows_smem_bytes(prm.base.L, NCLS, RN, prm.base.n_groups, prm.base.xc);
-  cudaError_t e = cudaFuncSetAttribute(k_contract_fp64_noalloc<NCLS, RN>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_contract_fp64_noalloc<NCLS, RN><<<grid, kThreads, smem, s>>>(prm);
-  note_launch();
-  return cudaGetLastError();
-}
-
-cudaError_t na_dispatch(const NoallocParams& prm, int rn, int grid, cudaStream_t s) {
-  switch (prm.base.rows.n_cls * 8 + rn) {
-    case 0 + 1: return na_launch<0, 1>(prm, grid, s);
-    case 0 + 2: return na_launch<0, 2>(prm, grid, s);
-    case 0 + 4: return na_launch<0, 4>(prm, grid, s);
-    case 8 + 1: return na_launch<1, 1>(prm, grid, s);
-    case 8 + 2: return na_launch<1, 2>(prm, grid, s);
-    case 8 + 4: return na_launch<1, 4>(prm, grid, s);
-    case 16 + 1: return na_launch<2, 1>(prm, grid, s);
-    case 16 + 2: return na_launch<2, 2>(prm, grid, s);
-    case 24 + 1: return na_launch<3, 1>(prm, grid, s);
-    case 24 + 2: return na_launch<3, 2>(prm, grid, s);
-    default: return cudaErrorInvalidValue;
+template <int NCLS, int NP, int RN>
+struct RowsNoalloc {
+  static cudaError_t launch(const NoallocParams& prm, int grid, cudaStream_t s) {
+    const size_t smem = rows_smem_bytes(prm.base.L, prm.base.rows, RN, prm.base.n_groups, prm.base.xc);
+    cudaError_t e = cudaFuncSetAttribute(k_contract_fp64_noalloc<NCLS, NP, RN>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_contract_fp64_noalloc<NCLS, NP, RN><<<grid, kThreads, smem, s>>>(prm);
+    note_launch();
+    return cudaGetLastError();
   }
-}
+};
 
 // Per-device device address of g_noalloc_scratch. In host code the array's name stands
 // for a host-side shadow, not device memory, so the address must be looked up with
@@ -244,10 +230,6 @@ extern "C" int bblock_contract_noalloc(int L, const void* q1, const void* q2, co
   base.X = X;
   base.n_jobs = 1;
   base.P_total = n_mom;
-  RowPlan plans[kNaMaxP];
-  const int n_plans = plan_rows(L, momenta, n_mom, plans, kNaMaxP);
-  int n_cls = 0;
-  for (int k = 0; k < n_plans; ++k) n_cls = plans[k].n_cls > n_cls ? plans[k].n_cls : n_cls;
   // spin triples -> coefficients by (alpha, beta, gamma), then the groups: one per
   // (alpha, beta) pair with the coefficients in its third quark, or, where that makes fewer,
   // one per gamma with a term per alpha and the coefficients in its line-2 element
@@ -301,7 +283,9 @@ extern "C" int bblock_contract_noalloc(int L, const void* q1, const void* q2, co
       }
   }
 
-  const int rn = rows_rn_for(n_cls, nd3);
+  RowPlan plans[kNaMaxP];
+  const int n_plans = plan_rows(L, momenta, n_mom, base.n_groups, base.n_terms, nd3, false, plans, kNaMaxP);
+  const int rn = rows_rn_for(plans, n_plans, nd3);
   job.m_tiles = (nd1 * nd2 + 16 * kRowRM - 1) / (16 * kRowRM);
   job.n_tiles = (nd3 + 16 * rn - 1) / (16 * rn);
   const size_t per = (size_t)n_mom * nd1 * nd2 * nd3;
@@ -344,38 +328,57 @@ extern "C" int bblock_contract_noalloc(int L, const void* q1, const void* q2, co
   // Among equals, the count with the least work one after another: an SM's resident CTAs take the
   // latencies side by side.
   const int n_rows = L * L;
-  const long long resident = (long long)rows_ctas_per_sm(n_cls, rn) * num_sms;
-  const long long site_ops = 9 * base.n_groups + 4 + 4 * n_cls, row_ops = 6 * n_mom;
+  const long long resident = (long long)rows_ctas_per_sm(plans[0], rn) * num_sms;
+  const int per_mom = plans[0].per_site ? plans[0].n_mom : plans[0].n_cls;
+  const long long site_ops = 9 * base.n_groups + 4 + 4 * per_mom, row_ops = 6 * n_mom;
   long long best = -1, best_chain = 0;
-  auto consider = [&](int rps, int parts) {
-    const long long slabs = (n_rows + rps - 1) / rps * (long long)parts;
-    const long long work = rps * ((L + parts - 1) / parts * site_ops + row_ops);
-    const long long cost = (tiles * slabs + num_sms - 1) / num_sms * work;
+  auto consider = [&](long long slabs, long long cost, long long work, int rps, int parts, int sites) {
     const long long chain = (tiles * slabs + resident - 1) / resident * work;
     if (best < 0 || cost < best || (cost == best && chain < best_chain)) {
       best = cost;
       best_chain = chain;
       base.rows_per_slab = rps;
       base.row_parts = parts;
+      base.sites_per_slab = sites;
       base.n_slab = (int)slabs;
     }
     return slabs * tiles < 8LL * num_sms;   // finer slabs gain nothing more
   };
+  auto on_busiest = [&](long long slabs) { return (tiles * slabs + num_sms - 1) / num_sms; };
+  const long long most = (long long)max_slabs_fit;
   bool finer = true;
-  for (long long n = 1; finer && n <= (long long)max_slabs_fit && n <= n_rows; ++n)
-    finer = consider((int)((n_rows + n - 1) / n), 1);
-  for (int parts = 2; finer && parts <= L && (long long)n_rows * parts <= (long long)max_slabs_fit; ++parts)
-    finer = consider(1, parts);
-  base.sites_per_slab = base.rows_per_slab * L;
+  const int xc = site_chunk(L, base.n_groups, tiles, resident);
+  if (plans[0].per_site) {
+    // slabs of staged chunks of sites; a unit's start and end cost about 4 sites, and an uneven last
+    // round leaves some SMs with a unit more than others (measured: L = 12, N_dil = 32, 6 momenta,
+    // one pair, 448 units on 304 CTAs 11 % slower than 576)
+    const int chunks = (X + xc - 1) / xc;
+    for (long long n = 1; finer && n <= most && n <= chunks; ++n) {
+      const int sites = (int)((chunks + n - 1) / n) * xc;
+      const long long slabs = (X + sites - 1) / sites, work = (sites + 4) * site_ops;
+      const long long rounds = (tiles * slabs + resident - 1) / resident;
+      finer = consider(slabs, (3 * on_busiest(slabs) + resident / num_sms * rounds) * work, work, 0, 1, sites);
+    }
+  } else {
+    for (long long n = 1; finer && n <= most && n <= n_rows; ++n) {
+      const int rps = (int)((n_rows + n - 1) / n);
+      const long long slabs = (n_rows + rps - 1) / rps, work = rps * (L * site_ops + row_ops);
+      finer = consider(slabs, on_busiest(slabs) * work, work, rps, 1, rps * L);
+    }
+    for (int parts = 2; finer && parts <= L && (long long)n_rows * parts <= most; ++parts) {
+      const long long slabs = (long long)n_rows * parts, work = (L + parts - 1) / parts * site_ops + row_ops;
+      finer = consider(slabs, on_busiest(slabs) * work, work, 1, parts, L);
+    }
+  }
   base.total_units = tiles * base.n_slab;
 
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   cudaError_t e = cudaSuccess;
   for (int k = 0; k < n_plans && e == cudaSuccess; ++k) {
     base.rows = plans[k];
-    base.xc = rows_sites_per_chunk(L, plans[k].n_cls, rn, base.n_groups);
-    const long long cap = (long long)rows_ctas_per_sm(plans[k].n_cls, rn) * num_sms;
-    e = na_dispatch(prm, rn, (int)(base.total_units < cap ? base.total_units : cap), s);
+    base.xc = plans[k].per_site ? xc : rows_sites_per_chunk(L, plans[k], rn, base.n_groups);
+    const long long cap = (long long)rows_ctas_per_sm(plans[k], rn) * num_sms;
+    e = rowsc::launch_plan<RowsNoalloc, kNaMaxP>(plans[k], rn, prm, (int)(base.total_units < cap ? base.total_units : cap), s);
   }
   if (e == cudaSuccess) {
     const int lanes = base.n_slab >= 16 ? 8 : 1;

@@ -15,40 +15,30 @@
 namespace bb {
 namespace {
 
-template <int NCLS, int RN>
+template <int NCLS, int NP, int RN>
 __global__ void __launch_bounds__(kThreads, RN == 4 || NCLS >= 2 ? 1 : 2)
 k_contract_df(const __grid_constant__ ContractParams prm) {
-  rowsc::contract_rows<rowsc::ArithDf, NCLS, kRowRM, RN>(prm, rowsc::TableSource<rowsc::ArithDf>{&prm});
+  rowsc::contract_rows<rowsc::ArithDf, NCLS, NP, kRowRM, RN>(prm, rowsc::TableSource<rowsc::ArithDf>{&prm});
 }
 
-template <int NCLS, int RN>
-cudaError_t launch_df_c(const ContractParams& prm, int grid, cudaStream_t s) {
-  const size_t smem = rows_smem_bytes(prm.L, NCLS, RN, prm.n_groups, prm.xc);
-  cudaError_t e = cudaFuncSetAttribute(k_contract_df<NCLS, RN>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_contract_df<NCLS, RN><<<grid, kThreads, smem, s>>>(prm);
-  note_launch();
-  return cudaGetLastError();
-}
+template <int NCLS, int NP, int RN>
+struct RowsDf {
+  static cudaError_t launch(const ContractParams& prm, int grid, cudaStream_t s) {
+    const size_t smem = rows_smem_bytes(prm.L, prm.rows, RN, prm.n_groups, prm.xc);
+    cudaError_t e = cudaFuncSetAttribute(k_contract_df<NCLS, NP, RN>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_contract_df<NCLS, NP, RN><<<grid, kThreads, smem, s>>>(prm);
+    note_launch();
+    return cudaGetLastError();
+  }
+};
 
 }  // namespace
 
 cudaError_t launch_contract_df(const ContractParams& prm, int rn, int grid, cudaStream_t s) {
   if (prm.total_units == 0 || prm.rows.n_mom == 0) return cudaSuccess;
-  switch (prm.rows.n_cls * 8 + rn) {
-    case 0 + 1: return launch_df_c<0, 1>(prm, grid, s);
-    case 0 + 2: return launch_df_c<0, 2>(prm, grid, s);
-    case 0 + 4: return launch_df_c<0, 4>(prm, grid, s);
-    case 8 + 1: return launch_df_c<1, 1>(prm, grid, s);
-    case 8 + 2: return launch_df_c<1, 2>(prm, grid, s);
-    case 8 + 4: return launch_df_c<1, 4>(prm, grid, s);
-    case 16 + 1: return launch_df_c<2, 1>(prm, grid, s);
-    case 16 + 2: return launch_df_c<2, 2>(prm, grid, s);
-    case 24 + 1: return launch_df_c<3, 1>(prm, grid, s);
-    case 24 + 2: return launch_df_c<3, 2>(prm, grid, s);
-    default: return cudaErrorInvalidValue;
-  }
+  return rowsc::launch_plan<RowsDf, kMaxSitePDf>(prm.rows, rn, prm, grid, s);
 }
 
 }  // namespace bb

@@ -201,32 +201,26 @@ cudaError_t launch_omega_table(int L, double2* om, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-int plan_rows(int L, const int32_t* momenta, int n_mom, RowPlan* out, int max_out) {
-  auto md = [L](int v) { const int m = v % L; return m < 0 ? m + L : m; };
-  auto cls = [&](int p, int axis) {   // |n0| in [0, L / 2]
-    const int n = md(momenta[3 * p + axis]);
+namespace {
+
+int mod_l(int v, int L) { const int m = v % L; return m < 0 ? m + L : m; }
+
+// The row-factored plans along one axis: classes in order of appearance, kMaxRowCls to a plan;
+// the momenta of n0 = 0 join the first plan; a plan that is full of momenta continues in another.
+int row_plans(int L, const int32_t* momenta, int n_mom, int axis, RowPlan* out, int max_out) {
+  auto cls = [&](int p) {   // |n0| in [0, L / 2]
+    const int n = mod_l(momenta[3 * p + axis], L);
     return n < L - n ? n : L - n;
   };
-  int axis = 2, fewest = 1 << 30;
-  for (int a = 2; a >= 0; --a) {
-    bool seen[65] = {};               // |n0| <= L / 2 <= 64
-    int n = 0;
-    for (int p = 0; p < n_mom; ++p) {
-      const int k = cls(p, a) % 65;
-      if (k && !seen[k]) { seen[k] = true; ++n; }
-    }
-    if (n < fewest) { fewest = n; axis = a; }
-  }
-  int n_plans = 0;
-  // plan of each class: classes in order of appearance, kMaxRowCls to a plan; the momenta of
-  // class 0 join the first plan; a plan that is full of momenta continues in another
-  int order[65], n_order = 0;
+  int order[65], n_order = 0;   // L / 2 <= 64
   for (int p = 0; p < n_mom; ++p) {
-    const int k = cls(p, axis);
+    const int k = cls(p);
     bool have = k == 0;
     for (int i = 0; i < n_order; ++i) have = have || order[i] == k;
     if (!have && n_order < 65) order[n_order++] = k;
   }
+  const int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
+  int n_plans = 0;
   for (int first = 0; first == 0 || first < n_order; first += kMaxRowCls) {
     RowPlan pl{};
     auto start = [&] {
@@ -239,19 +233,18 @@ int plan_rows(int L, const int32_t* momenta, int n_mom, RowPlan* out, int max_ou
       ++n_plans;
     };
     start();
-    const int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
     for (int p = 0; p < n_mom; ++p) {
-      const int k = cls(p, axis);
+      const int k = cls(p);
       int sel = 0;
       if (k == 0) {
         if (first != 0) continue;
       } else {
         for (int c = 0; c < pl.n_cls; ++c)
-          if (pl.cls_n0[c] == k) sel = md(momenta[3 * p + axis]) == k ? c + 1 : -(c + 1);
+          if (pl.cls_n0[c] == k) sel = mod_l(momenta[3 * p + axis], L) == k ? c + 1 : -(c + 1);
         if (sel == 0) continue;
       }
       if (pl.n_mom == kMaxRowP) { flush(); start(); }
-      pl.mom[pl.n_mom++] = RowMom{p, md(momenta[3 * p + a1]), md(momenta[3 * p + a2]), sel};
+      pl.mom[pl.n_mom++] = RowMom{p, mod_l(momenta[3 * p + a1], L), mod_l(momenta[3 * p + a2], L), sel};
       if (sel == 0) pl.has_zero = 1;
     }
     if (pl.n_mom > 0) flush();
@@ -259,38 +252,87 @@ int plan_rows(int L, const int32_t* momenta, int n_mom, RowPlan* out, int max_ou
   return n_plans;
 }
 
-template <int NCLS, int RN>
-__global__ void __launch_bounds__(kThreads, RN == 4 || NCLS >= 2 ? 1 : 2)
-k_contract_fp64(const __grid_constant__ ContractParams prm) {
-  rowsc::contract_rows<rowsc::ArithF64, NCLS, kRowRM, RN>(prm, rowsc::TableSource<rowsc::ArithF64>{&prm});
+// The plans with a phase per site, at most cap momenta each, as evenly as possible.
+int site_plans(int L, const int32_t* momenta, int n_mom, int cap, RowPlan* out, int max_out) {
+  const int parts = (n_mom + cap - 1) / cap, step = (n_mom + parts - 1) / parts;
+  int n_plans = 0;
+  for (int first = 0; first < n_mom; first += step, ++n_plans) {
+    if (!out || n_plans >= max_out) continue;
+    RowPlan pl{};
+    pl.per_site = 1;
+    for (int p = first; p < n_mom && p < first + step; ++p)
+      pl.mom[pl.n_mom++] = RowMom{p, mod_l(momenta[3 * p + 1], L), mod_l(momenta[3 * p + 2], L),
+                                  mod_l(momenta[3 * p], L)};
+    out[n_plans] = pl;
+  }
+  return n_plans;
 }
 
-template <int NCLS, int RN>
-static cudaError_t launch_rows_c(const ContractParams& prm, int grid, cudaStream_t s) {
-  const size_t smem = rows_smem_bytes(prm.L, NCLS, RN, prm.n_groups, prm.xc);
-  cudaError_t e = cudaFuncSetAttribute(k_contract_fp64<NCLS, RN>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  k_contract_fp64<NCLS, RN><<<grid, kThreads, smem, s>>>(prm);
-  note_launch();
-  return cudaGetLastError();
+}  // namespace
+
+// Row-factored along the axis with the fewest classes (the last on a tie), or a phase per site, by
+// the operations per output and site (rows_contract.cuh) of all launches: each of them repeats the
+// singlet and the diquarks, so lists with more classes than a launch takes, and whose momenta
+// hardly share a class, are the second kind's. Beside the operations, as measured (L = 2 to 24,
+// N_dil 16 and 32, 1 to 4 pairs): a row's end costs 8 (16 in double-float: the partial block's
+// latency) per momentum after the first, and launches of two or three classes, one CTA an SM, a
+// tenth more. L = 16, N_dil = 32, one pair, momenta (k, k, k), FP64 / double-float, ms row-factored
+// and per site: k < 2  4.72 / 1.40 and 4.91 / 1.44; k < 4  6.86 / 2.18 and 6.72 / 1.88;
+// k < 8  16.7 / 5.23 and 10.5 / 2.81; -3 <= k <= 3  7.07 / 2.40 and 9.6 / 2.59.
+int plan_rows(int L, const int32_t* momenta, int n_mom, int groups, int terms, int nd3, bool df,
+              RowPlan* out, int max_out) {
+  if (n_mom < 1) return 0;
+  int axis = 2, fewest = 1 << 30;
+  for (int a = 2; a >= 0; --a) {
+    bool seen[65] = {};
+    int n = 0;
+    for (int p = 0; p < n_mom; ++p) {
+      const int n0 = mod_l(momenta[3 * p + a], L), k = n0 < L - n0 ? n0 : L - n0;
+      if (k && !seen[k]) { seen[k] = true; ++n; }
+    }
+    if (n < fewest) { fewest = n; axis = a; }
+  }
+  const int cap = df ? kMaxSitePDf : kMaxSiteP;
+  auto singlet_ops = [&](const RowPlan& shape) {   // of a launch, with the diquarks
+    const int tile = 16 * rows_rn_for(&shape, 1, nd3);
+    return 9.0 * groups + 24.0 * terms / (tile < nd3 ? tile : nd3);
+  };
+  RowPlan shape{};
+  shape.n_cls = fewest < kMaxRowCls ? fewest : kMaxRowCls;
+  const double site_ops = fewest > 0 ? 4.0 : df ? 4.0 : 0.0;   // recombined, and n0 = 0 (ArithF64::kEachSite)
+  double by_row = row_plans(L, momenta, n_mom, axis, nullptr, 0) * (singlet_ops(shape) + site_ops) +
+                  4.0 * fewest + (df ? 16.0 : 8.0) * (n_mom - 1) / L;
+  if (shape.n_cls >= 2) by_row *= 1.1;
+  shape = RowPlan{};
+  shape.per_site = 1;
+  shape.n_mom = n_mom < cap ? n_mom : cap;
+  const double by_site = (n_mom + cap - 1) / cap * (singlet_ops(shape) + 2.0) + 4.0 * n_mom;
+  if (by_site < 0.97 * by_row) return site_plans(L, momenta, n_mom, cap, out, max_out);
+  return row_plans(L, momenta, n_mom, axis, out, max_out);
 }
+
+template <int NCLS, int NP, int RN>
+__global__ void __launch_bounds__(kThreads, RN == 4 || NCLS >= 2 ? 1 : 2)
+k_contract_fp64(const __grid_constant__ ContractParams prm) {
+  rowsc::contract_rows<rowsc::ArithF64, NCLS, NP, kRowRM, RN>(prm, rowsc::TableSource<rowsc::ArithF64>{&prm});
+}
+
+template <int NCLS, int NP, int RN>
+struct RowsF64 {
+  static cudaError_t launch(const ContractParams& prm, int grid, cudaStream_t s) {
+    const size_t smem = rows_smem_bytes(prm.L, prm.rows, RN, prm.n_groups, prm.xc);
+    cudaError_t e = cudaFuncSetAttribute(k_contract_fp64<NCLS, NP, RN>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_contract_fp64<NCLS, NP, RN><<<grid, kThreads, smem, s>>>(prm);
+    note_launch();
+    return cudaGetLastError();
+  }
+};
 
 cudaError_t launch_contract_fp64(const ContractParams& prm, int rn, int grid, cudaStream_t s) {
   if (prm.total_units == 0 || prm.rows.n_mom == 0) return cudaSuccess;
-  switch (prm.rows.n_cls * 8 + rn) {
-    case 0 + 1: return launch_rows_c<0, 1>(prm, grid, s);
-    case 0 + 2: return launch_rows_c<0, 2>(prm, grid, s);
-    case 0 + 4: return launch_rows_c<0, 4>(prm, grid, s);
-    case 8 + 1: return launch_rows_c<1, 1>(prm, grid, s);
-    case 8 + 2: return launch_rows_c<1, 2>(prm, grid, s);
-    case 8 + 4: return launch_rows_c<1, 4>(prm, grid, s);
-    case 16 + 1: return launch_rows_c<2, 1>(prm, grid, s);
-    case 16 + 2: return launch_rows_c<2, 2>(prm, grid, s);
-    case 24 + 1: return launch_rows_c<3, 1>(prm, grid, s);
-    case 24 + 2: return launch_rows_c<3, 2>(prm, grid, s);
-    default: return cudaErrorInvalidValue;
-  }
+  return rowsc::launch_plan<RowsF64, kMaxSiteP>(prm.rows, rn, prm, grid, s);
 }
 
 // ------------------------------------------------------------------ slab reduction

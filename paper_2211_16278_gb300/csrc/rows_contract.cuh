@@ -23,7 +23,10 @@
 //     (FP64; in double-float the longer sums of the larger k's cost accuracy, 4.2e-14 against
 //     2.7e-14 at L = 24, so each site is recombined, 4 operations);
 //   * 4 per momentum and row at the row's end, into the unit's partial block, which stays in
-//     L2 (the read-modify-write is below 3 % of the L2 rate in the FP64 form).
+//     L2 (the read-modify-write is below 3 % of the L2 rate in the FP64 form);
+//   * or, for lists whose momenta hardly share an n0 (plan_rows), a phase per momentum and site
+//     (NP of them): 2 to recombine, then 4 for every momentum, into sums that stay in registers
+//     over the unit's rows.
 // (A singlet per spin pair and a phase product per momentum and site take 9 n_pairs + 2 + 4 P:
 // 74 instead of 26 at 4 pairs, 2 groups and 9 momenta of n0 = 0, +-1.) Times: k_contract_fp64,
 // k_contract_df.
@@ -54,6 +57,7 @@ __device__ __forceinline__ int find_job(const ContractJob* jobs, int n_jobs, lon
 // IEEE double on the FP64 pipe. T: a number, Cx: a complex number, Z: its 16 bytes in memory.
 struct ArithF64 {
   static constexpr bool kEachSite = false;   // recombine k1..k3 at each site also without a class
+  static constexpr bool kExactP = false;     // a site loop of its own for each momentum count (NP)
   using T = double;
   struct Cx { double re, im; };
   using Z = double2;
@@ -73,6 +77,7 @@ struct ArithF64 {
 // lazily: norm() brings them back below ulp(h) / 2.
 struct ArithDf {
   static constexpr bool kEachSite = true;
+  static constexpr bool kExactP = true;
   using T = dfloat;
   using Cx = dcomplex;
   using Z = float4;
@@ -139,10 +144,23 @@ template <class A> struct TableSource {
   __device__ Cx omega(int k) const { return A::cx(prm->phase[k]); }
 };
 
-template <class A, int NCLS, int RM, int RN, class Src>
+// f(integral_constant n), n in [LO, HI]
+template <int LO, int HI, class F> __device__ __forceinline__ void with_count(int n, F&& f) {
+  if constexpr (LO < HI) {
+    if (n <= LO) f(std::integral_constant<int, LO>{});
+    else with_count<LO + 1, HI>(n, f);
+  } else {
+    f(std::integral_constant<int, HI>{});
+  }
+}
+
+template <class A, int NCLS, int NP, int RM, int RN, class Src>
 __device__ __forceinline__ void contract_rows(const ContractParams& prm, const Src& src) {
+  static_assert(NCLS == 0 || NP == 0, "row-factored or a phase per site");
   constexpr int MT = 16 * RM, NT = 16 * RN;
   constexpr int NC = NCLS > 0 ? NCLS : 1;
+  constexpr int NPS = NP > 0 ? NP : 1;
+  constexpr int NPH = NCLS + NP > 0 ? NCLS + NP : 1;   // phases of a site
   using T = typename A::T;
   using Cx = typename A::Cx;
   using Z = typename A::Z;
@@ -159,12 +177,12 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
   T* __restrict__ Bd = Bc + KC * NT;
   T* __restrict__ Be = Bd + KC * NT;
   Z* __restrict__ ph = reinterpret_cast<Z*>(Be + KC * NT);
-  Z* __restrict__ om = ph + XC * NC;
+  Z* __restrict__ om = ph + XC * (NP > kSitePNarrow ? kMaxSiteP : NPH);
 
   const int tid = threadIdx.x, tn = tid % 16, tm = tid / 16;
   const int ml = tid % MT;   // the diquark row this thread stages
   // sites of a row: base + x0 * sx along the summed axis
-  const int sx = rp.axis == 0 ? 1 : rp.axis == 1 ? L : L * L;
+  const int sx = NP > 0 || rp.axis == 0 ? 1 : rp.axis == 1 ? L : L * L;
   for (int k = tid; k < L; k += kThreads) A::store(om + k, src.omega(k));
   __syncthreads();
 
@@ -188,7 +206,12 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
     // a slab of rows, or, of small lattices, one run of sites of a row
     int row_begin = slab * prm.rows_per_slab, row_end = min(L * L, row_begin + prm.rows_per_slab);
     int x_begin = 0, x_end = L;
-    if (Src::kRowParts && prm.row_parts > 1) {
+    if (NP > 0) {   // a phase per site: a slab of sites, in the lattice's own order
+      row_begin = 0;
+      row_end = 1;
+      x_begin = slab * prm.sites_per_slab;
+      x_end = min(prm.X, x_begin + prm.sites_per_slab);
+    } else if (Src::kRowParts && prm.row_parts > 1) {
       const int len = (L + prm.row_parts - 1) / prm.row_parts;
       row_begin = slab / prm.row_parts;
       row_end = row_begin + 1;
@@ -209,9 +232,17 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
     const int act_n = min(RN, (nd3 - col0 + 15) / 16);
     const int n_cols = act_n * 16;
 
+    T wr[RM][RN][NPS], wi[RM][RN][NPS];   // the unit's sums of each momentum (a phase per site)
+#pragma unroll
+    for (int i = 0; i < RM; ++i)
+#pragma unroll
+      for (int j = 0; j < RN; ++j)
+#pragma unroll
+        for (int c = 0; c < NPS; ++c) wr[i][j][c] = wi[i][j][c] = A::zero();
+
     for (int row = row_begin; row < row_end; ++row) {
       const int ra = row % L, rb = row / L;   // the other two coordinates, ascending
-      const int base = rp.axis == 0 ? L * row : rp.axis == 1 ? ra + L * L * rb : row;
+      const int base = NP > 0 ? 0 : rp.axis == 0 ? L * row : rp.axis == 1 ? ra + L * L * rb : row;
       T k1[RM][RN], k2[RM][RN], k3[RM][RN];
       T zr[RM][RN], zi[RM][RN];                                          // n0 = 0
       T cr[RM][RN][NC], si_[RM][RN][NC], ci[RM][RN][NC], sr_[RM][RN][NC];   // +-n0 classes
@@ -224,8 +255,8 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
           for (int c = 0; c < NC; ++c) cr[i][j][c] = si_[i][j][c] = ci[i][j][c] = sr_[i][j][c] = A::zero();
         }
 
-      auto add_sites = [&](auto act, int nx) {
-        constexpr int ACT = decltype(act)::value;
+      auto add_sites = [&](auto act, auto n_site, int nx) {
+        constexpr int ACT = decltype(act)::value, NS = decltype(n_site)::value;   // NS: of NP
         for (int xc = 0; xc < nx; ++xc) {
           const int kbeg = xc * G * 3, kend = kbeg + G * 3;
 #pragma unroll 3
@@ -252,7 +283,7 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
                 A::fma_add(k3[i][j], ai[i], be[j]);
               }
           }
-          if (NCLS == 0 && A::kEachSite) {
+          if (NCLS == 0 && NP == 0 && A::kEachSite) {
 #pragma unroll
             for (int i = 0; i < RM; ++i)
 #pragma unroll
@@ -261,6 +292,34 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
                 zi[i][j] = A::add(zi[i][j], A::add(k1[i][j], k2[i][j]));
                 k1[i][j] = k2[i][j] = k3[i][j] = A::zero();
               }
+          }
+          if (NP > 0) {
+#pragma unroll
+            for (int i = 0; i < RM; ++i)
+#pragma unroll
+              for (int j = 0; j < ACT; ++j) {
+                const T sr = A::sub(k1[i][j], k3[i][j]);
+                k2[i][j] = A::add(k1[i][j], k2[i][j]);
+                k1[i][j] = sr;
+              }
+#pragma unroll
+            for (int c = 0; c < NS; ++c) {
+              if (!A::kExactP && c >= rp.n_mom) break;
+              const Cx e = A::load(ph + xc * NPH + c);
+#pragma unroll
+              for (int i = 0; i < RM; ++i)
+#pragma unroll
+                for (int j = 0; j < ACT; ++j) {
+                  Cx w{wr[i][j][c], wi[i][j][c]};
+                  cmul_add<A>(w, e, Cx{k1[i][j], k2[i][j]});
+                  wr[i][j][c] = w.re;
+                  wi[i][j][c] = w.im;
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < RM; ++i)
+#pragma unroll
+              for (int j = 0; j < ACT; ++j) k1[i][j] = k2[i][j] = k3[i][j] = A::zero();
           }
           if (NCLS > 0) {
             Cx e[NC];
@@ -288,7 +347,7 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
         }
       };
 
-      for (int x0 = x_begin; x0 < x_end; x0 += XC) {   // [0, L) without parts
+      for (int x0 = x_begin; x0 < x_end; x0 += XC) {   // a row: [0, L) without parts
         const int nx = min(XC, x_end - x0);
         // --- diquark tile: A[(xc, group, c)][m], the group's terms summed
         for (int xc = tid / MT; xc < nx; xc += kThreads / MT) {
@@ -334,16 +393,24 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
             const int c = idx % NC, xc = idx / NC;
             ph[idx] = om[(rp.cls_n0[c] * (x0 + xc)) % L];
           }
+        if (NP > 0)
+          for (int idx = tid; idx < nx * NP; idx += kThreads) {
+            const int c = idx % NPS, xc = idx / NPS;
+            if (c >= rp.n_mom) continue;
+            const RowMom mo = rp.mom[c];
+            const int x = x0 + xc, xr = x / L;
+            ph[idx] = om[(mo.sel * (x - xr * L) + mo.n1 * (xr % L) + mo.n2 * (xr / L)) % L];
+          }
         __syncthreads();
 
         // the staged sites into the sums, by the tile's 16-column blocks in use: a block that is
         // only predicated off still takes the FP64 pipe (measured: 96 columns cost 128)
-        switch (act_n) {
-          case 1: add_sites(std::integral_constant<int, 1>{}, nx); break;
-          case 2: add_sites(std::integral_constant<int, RN < 2 ? RN : 2>{}, nx); break;
-          case 3: add_sites(std::integral_constant<int, RN < 3 ? RN : 3>{}, nx); break;
-          default: add_sites(std::integral_constant<int, RN>{}, nx); break;
-        }
+        with_count<1, RN>(act_n, [&](auto act) {
+          if constexpr (NP > 0 && A::kExactP)
+            with_count<(NP > kSitePNarrow ? kSitePNarrow + 1 : 1), NP>(rp.n_mom, [&](auto n) { add_sites(act, n, nx); });
+          else
+            add_sites(act, std::integral_constant<int, NP>{}, nx);
+        });
         // renormalise once per chunk of sites
 #pragma unroll
         for (int i = 0; i < RM; ++i)
@@ -358,6 +425,11 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
               ci[i][j][c] = A::norm(ci[i][j][c]);
               sr_[i][j][c] = A::norm(sr_[i][j][c]);
             }
+#pragma unroll
+            for (int c = 0; c < NP; ++c) {
+              wr[i][j][c] = A::norm(wr[i][j][c]);
+              wi[i][j][c] = A::norm(wi[i][j][c]);
+            }
           }
         __syncthreads();
       }
@@ -367,11 +439,11 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
       for (int i = 0; i < RM; ++i)
 #pragma unroll
         for (int j = 0; j < RN; ++j)
-          if (NCLS == 0 && !A::kEachSite) {
+          if (NCLS == 0 && NP == 0 && !A::kEachSite) {
             zr[i][j] = A::norm(A::sub(k1[i][j], k3[i][j]));
             zi[i][j] = A::norm(A::add(k1[i][j], k2[i][j]));
           }
-      for (int q = 0; q < rp.n_mom; ++q) {
+      for (int q = 0; NP == 0 && q < rp.n_mom; ++q) {
         const RowMom mo = rp.mom[q];
         const Cx e = A::load(om + (mo.n1 * ra + mo.n2 * rb) % L);
         // the unit's own sums until its last row, which leaves them in FP64
@@ -410,6 +482,44 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
         }
       }
     }
+    // --- a phase per site: the unit's sums are its partial block
+#pragma unroll
+    for (int c = 0; c < NP; ++c) {
+      if (c >= rp.n_mom) break;
+      double2* __restrict__ out = J.partial + ((size_t)slab * prm.P_total + rp.mom[c].p) * M * nd3;
+#pragma unroll
+      for (int i = 0; i < RM; ++i)
+#pragma unroll
+        for (int j = 0; j < RN; ++j) {
+          const int m = mt * MT + tm + 16 * i, n = col0 + tn + 16 * j;
+          if (m < M && n < nd3) out[(size_t)m * nd3 + n] = A::to_double2(Cx{wr[i][j][c], wi[i][j][c]});
+        }
+    }
+  }
+}
+
+// The launch of Kernel<NCLS, NP, RN> for a plan; WIDE: momenta of the widest per-site launch.
+template <template <int, int, int> class Kernel, int WIDE, class Params>
+cudaError_t launch_plan(const RowPlan& r, int rn, const Params& prm, int grid, cudaStream_t s) {
+  if (rn > rows_max_rn(r)) return cudaErrorInvalidValue;
+  if (r.per_site) {
+    if (r.n_mom > WIDE) return cudaErrorInvalidValue;
+    if (r.n_mom > kSitePNarrow) return Kernel<0, WIDE, 1>::launch(prm, grid, s);
+    return rn == 1 ? Kernel<0, kSitePNarrow, 1>::launch(prm, grid, s)
+                   : Kernel<0, kSitePNarrow, 2>::launch(prm, grid, s);
+  }
+  switch (r.n_cls * 8 + rn) {
+    case 0 + 1: return Kernel<0, 0, 1>::launch(prm, grid, s);
+    case 0 + 2: return Kernel<0, 0, 2>::launch(prm, grid, s);
+    case 0 + 4: return Kernel<0, 0, 4>::launch(prm, grid, s);
+    case 8 + 1: return Kernel<1, 0, 1>::launch(prm, grid, s);
+    case 8 + 2: return Kernel<1, 0, 2>::launch(prm, grid, s);
+    case 8 + 4: return Kernel<1, 0, 4>::launch(prm, grid, s);
+    case 16 + 1: return Kernel<2, 0, 1>::launch(prm, grid, s);
+    case 16 + 2: return Kernel<2, 0, 2>::launch(prm, grid, s);
+    case 24 + 1: return Kernel<3, 0, 1>::launch(prm, grid, s);
+    case 24 + 2: return Kernel<3, 0, 2>::launch(prm, grid, s);
+    default: return cudaErrorInvalidValue;
   }
 }
 
