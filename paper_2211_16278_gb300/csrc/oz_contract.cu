@@ -371,10 +371,13 @@ __device__ __forceinline__ void oz_produce(const ContractParams& prm, const OzSh
         // G = (E + 4) / 3 (site, group) pairs; the loads of a batch of elements (4 diquark
         // elements of one term, 8 third-quark ones) are all issued before its arithmetic, so
         // that their latencies overlap.
-        // The runs of 4 elements of an 8-element thread and the digits are rolled loops: with
-        // three roles of straight-line code in flight on an SM, instruction fetch was the
-        // largest stall (2.7 of 11 cycles an issue).
-        constexpr int LB = 4, G = 2;
+        // The runs of 4 elements of an 8-element thread and, in clusters, the digits are rolled loops:
+        // with three roles of straight-line code in flight on an SM, instruction fetch was the
+        // largest stall (2.7 of 11 cycles an issue). Plain CTAs keep the digits unrolled, and groups
+        // of one term skip the term table. Contraction of plain CTAs against straight-line code per
+        // spin pair, 144 shapes of L = 6 to 20, N_dil 8 to 64: one pair 1.10 with rolled digits, 0.95
+        // so; three pairs in two groups 1.03 and 0.89 (220 and 32 bytes of spills).
+        constexpr int LB = 4, G = 2, kDigitUnroll = C == 1 ? kDigits : 1;
         int hc = c0, hg = g0, hx = x0, hk = kk0;
 #pragma unroll 1
         for (int h = 0; h < E / LB; ++h) {
@@ -411,9 +414,13 @@ __device__ __forceinline__ void oz_produce(const ContractParams& prm, const OzSh
               bool has[LB];
 #pragma unroll
               for (int jj = 0; jj < LB; ++jj) {
-                int t = prm.tbeg[eg[jj]] + tt;
-                has[jj] = t < prm.tbeg[eg[jj] + 1];
-                if (!has[jj]) t = 0;
+                int t = eg[jj];
+                has[jj] = true;
+                if (prm.oz.max_terms_i > 1) {
+                  t = prm.tbeg[eg[jj]] + tt;
+                  has[jj] = t < prm.tbeg[eg[jj] + 1];
+                  if (!has[jj]) t = 0;
+                }
                 const int cc = ec[jj];
                 const int c1 = cc == 2 ? 0 : cc + 1, c2 = cc == 0 ? 2 : cc - 1;
                 const int x = base + ex[jj] * sx;
@@ -474,7 +481,7 @@ __device__ __forceinline__ void oz_produce(const ContractParams& prm, const OzSh
           // digits, most significant first; each digit's 4 values are one K run of the row
           uint8_t* dp = sh.smem + (uint32_t)(slot * kStageBytes) + (A ? a_row : (uint32_t)kAStage + b_row) + h * 8;
           float Rc = 0x1.8p16f;   // 1.5 * 2^(16 - 8 i)
-#pragma unroll 1
+#pragma unroll kDigitUnroll
           for (int i = 0; i < kDigits; ++i) {
             const float2 R2 = make_float2(Rc, Rc);
             float2 d[LB];
