@@ -1126,14 +1126,73 @@ int run_jobs_tc(bblock_ctx* c, const std::vector<JobIn>& jobs, const SpinPlan& s
   return BBLOCK_OK;
 }
 
+// Ozaki form: time of the contraction and slab reduction of jobs [b, e) in microseconds, for clusters
+// of cl CTAs that share each diquark tile across adjacent N tiles. rows: row-factored units (cols
+// distinct n0, n_mom momenta), else cols momenta as columns. A unit costs a start and a stage time per
+// 16 K elements, more with several terms a group; a row-factored one per lattice row, beside whose
+// stages the epilogue updates n_mom / cols momenta of every column. The constants are fits to GB300
+// over L = 6 to 24, N_dil 8 to 64, 2 to 12 momenta (27 the most), 1 and 2 groups of 1 or 1.5 terms
+// (3300 timings, 8 to 11 % off). With the route and cluster of least time (rows only 5 % ahead, single
+// row-factored CTAs a tenth, clusters of 3 and 4 3 %) 430 shapes take 0.81 of the time of pairs over all
+// (p, d3) columns, 1.03 at most, and 1.009 of the best of all eight choices on average.
+double oz_time(const bblock_ctx* c, const std::vector<JobIn>& jobs, size_t b, size_t e, bool rows,
+               int cols, int n_mom, const GroupPlan& gp, int cl, int nc) {
+  struct Cost { double start, start_update, stage, more_terms, update; };
+  static const Cost by_cols[4] = {{19.0, 0.0, 5.02, 0.80, 0.0}, {19.6, 0.0, 3.90, 0.575, 0.0},
+                                  {19.0, 0.0, 3.84, 0.56, 0.0}, {18.6, 0.0, 3.70, 0.385, 0.0}};
+  static const Cost by_rows[4] = {{14.5, 0.209, 5.54, 0.775, 0.290}, {15.9, 0.190, 4.46, 0.27, 0.288},
+                                  {13.0, 0.204, 4.34, 0.33, 0.278}, {13.2, 0.230, 3.78, 0.22, 0.252}};
+  static const double resident[4] = {1.0, 0.5, 46.0 / 152, 36.0 / 152};   // clusters per SM
+  const Cost& k = rows ? by_rows[cl - 1] : by_cols[cl - 1];
+  const int n_groups = gp.n_groups;
+  const double stage = k.stage * (1.0 + k.more_terms * ((double)gp.n_terms / n_groups - 1.0));
+  const int L = c->cfg.L, parts = rows ? L * L : c->X;
+  long long tiles = 0, out = 0;
+  int max_nd3 = 1;
+  for (size_t i = b; i < e; ++i) {
+    const int* nd = jobs[i].nd;
+    const long long nt = ((long long)cols * nd[2] + nc - 1) / nc;
+    tiles += (long long)((nd[0] * nd[1] + kOzM - 1) / kOzM) * ((nt + cl - 1) / cl);
+    out += (long long)nd[0] * nd[1] * nd[2];
+    max_nd3 = std::max(max_nd3, nd[2]);
+  }
+  if (tiles == 0) return 0.0;
+  const int ns = c->opt_slabs > 0 ? std::min(c->opt_slabs, parts)
+                                  : choose_slabs(tiles, c->num_sms / cl, parts, 1, 64);
+  const int per = (parts + ns - 1) / ns, n_slab = (parts + per - 1) / per;
+  const double rounds = std::ceil(tiles * n_slab / std::max(1.0, std::floor(resident[cl - 1] * c->num_sms)));
+  const double bytes = 16.0 * n_slab * n_mom * out;
+  if (!rows) return rounds * (k.start + std::ceil(per * 3.0 * n_groups / 16.0) * stage) + 14.0 + bytes / 6.0e6;
+  const double updates = std::min(nc, cols * max_nd3) * (double)n_mom / cols;
+  const double stages = std::ceil(3.0 * n_groups * L / 16.0) * stage, epilogue = updates * k.update;
+  // whichever is longer, and a little of the other
+  const double row = std::cbrt(stages * stages * stages + epilogue * epilogue * epilogue);
+  return rounds * (k.start + k.start_update * updates + per * row) + 21.0 + bytes / 2.9e6;
+}
+
+// Ozaki form: the cluster size of jobs [b, e): `fixed` if it is 1 to 4, else the one of least oz_time.
+int oz_cluster_for(const bblock_ctx* c, const std::vector<JobIn>& jobs, size_t b, size_t e, bool rows,
+                   int cols, int n_mom, const GroupPlan& gp, int nc, int fixed, double* time = nullptr) {
+  if (fixed >= 1 && fixed <= 4 && !time) return fixed;
+  int best = 0;
+  double least = 0.0;
+  for (int cl = 1; cl <= 4; ++cl) {
+    const double t = oz_time(c, jobs, b, e, rows, cols, n_mom, gp, cl, nc) *
+                     (cl > 2 ? 1.03 : cl == 1 && rows ? 1.1 : 1.0);
+    if (best == 0 || t < least) { least = t; best = cl; }
+  }
+  if (time) *time = least;
+  return best;
+}
+
 // Ozaki form: the row-factored phase, e^{-ip.x} = w^{n0 x0} w^{n1 x1 + n2 x2} along the axis
 // with the fewest distinct n0. The tensor cores then run nidx instead of n_mom phase columns
 // per d3, a row's last stage is padded with zeros, and the epilogue adds each row's sums into
-// the running sums of all momenta. Taken where the model of a row says it is faster: stages of
-// about 10 kcycles, an epilogue of 6 kcycles plus 0.18 per column and momentum beside them
-// (measured at L = 32, 9 momenta, N_dil = 48: 12 stages a row). BBLOCK_OPT_TC_ROWS 1: wherever
-// it fits, 2: never.
-OzRows plan_oz_rows(const bblock_ctx* c, const int32_t* momenta, int n_mom, int per_mom, int n_groups) {
+// the running sums of all momenta. Taken where oz_time says that it is at least 5 % faster
+// for the call's jobs, whatever the cluster size asked for (clusters leave the bits as they are).
+// BBLOCK_OPT_TC_ROWS 1: wherever it fits, 2: never.
+OzRows plan_oz_rows(const bblock_ctx* c, const int32_t* momenta, int n_mom, int per_mom, const GroupPlan& gp,
+                    const std::vector<JobIn>& jobs, int nc) {
   OzRows r{};
   const int L = c->cfg.L;
   r.slabs.axis = -1;
@@ -1149,10 +1208,13 @@ OzRows plan_oz_rows(const bblock_ctx* c, const int32_t* momenta, int n_mom, int 
     }
     if ((int)seen.size() < fewest) { fewest = (int)seen.size(); axis = a; }
   }
-  if (fewest > kOzMaxIdx) return r;
-  const double k_row = 3.0 * n_groups * L, spr = std::ceil(k_row / 16.0), stage = 10.0;
-  const double row_rf = std::max(spr * stage, 6.0 + 0.18 * kOzMaxNC * n_mom / fewest);
-  if (c->opt_tc_rows == 0 && fewest * row_rf >= n_mom * (k_row / 16.0) * stage) return r;
+  if (fewest > kOzMaxIdx || (c->opt_tc_rows == 0 && fewest >= n_mom)) return r;
+  if (c->opt_tc_rows == 0) {
+    double by_rows = 0.0, by_cols = 0.0;
+    oz_cluster_for(c, jobs, 0, jobs.size(), true, fewest, n_mom, gp, nc, 0, &by_rows);
+    oz_cluster_for(c, jobs, 0, jobs.size(), false, n_mom, n_mom, gp, nc, 0, &by_cols);
+    if (1.05 * by_rows >= by_cols) return r;
+  }
   const int a1 = axis == 0 ? 1 : 0, a2 = axis == 2 ? 1 : 2;
   for (int p = 0; p < n_mom; ++p) {
     const int n0 = md(momenta[3 * p + axis]);
@@ -1166,29 +1228,6 @@ OzRows plan_oz_rows(const bblock_ctx* c, const int32_t* momenta, int n_mom, int 
   r.on = 1;
   r.axis = r.slabs.axis = axis;
   return r;
-}
-
-// Ozaki form: clusters of C CTAs share each diquark tile across C adjacent N tiles; each builds
-// 1/C of the tile's rows, which sets the stage time, but the last cluster of a ragged job pads its
-// N tiles, and fewer CTAs of larger clusters are resident (138 and 144 of 152 SMs at 3 and 4).
-// Measured per N tile slot (L = 32, 9 momenta, row-factored, N_dil 32 to 64): 1.95, 1, 1.27 and
-// 1.06 for C = 1 to 4. Auto: the C with the least slots times that over the wave's jobs.
-int oz_cluster_for(const bblock_ctx* c, const std::vector<JobIn>& jobs, size_t b, size_t e,
-                   int P_launch, int nc) {
-  if (c->opt_tc_cluster >= 1 && c->opt_tc_cluster <= 4) return c->opt_tc_cluster;
-  const double slot_cost[4] = {1.95, 1.0, 1.27, 1.06};
-  int best = 1;
-  double least = 0.0;
-  for (int cl = 1; cl <= 4; ++cl) {
-    double sum = 0.0;
-    for (size_t k = b; k < e; ++k) {
-      const long long nt = ((long long)P_launch * jobs[k].nd[2] + nc - 1) / nc;
-      const long long mt = ((long long)jobs[k].nd[0] * jobs[k].nd[1] + kOzM - 1) / kOzM;
-      sum += (double)(mt * ((nt + cl - 1) / cl) * cl) * slot_cost[cl - 1];
-    }
-    if (cl == 1 || sum < least) { least = sum; best = cl; }
-  }
-  return best;
 }
 
 // Slabs of an FP64 or double-float contraction: of whole lattice rows, or of staged chunks of sites
@@ -1371,7 +1410,8 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
   const std::vector<RowPlan>& rplans = rc_rows.plans;
   const int row_rn = rc_rows.rn;
   OzRows ozr{};
-  if (oz) ozr = plan_oz_rows(c, momenta, n_mom, per_mom, gp.n_groups);
+  const int oz_nc = c->opt_tc_nc > 0 && c->opt_tc_nc <= kOzMaxNC ? c->opt_tc_nc : kOzMaxNC;
+  if (oz) ozr = plan_oz_rows(c, momenta, n_mom, per_mom, gp, jobs, oz_nc);
   for (int g = 0; g < gp.n_groups; ++g)
     ozr.max_terms_i = std::max(ozr.max_terms_i, gp.tbeg[g + 1] - gp.tbeg[g]);
   ozr.max_terms = (float)ozr.max_terms_i;
@@ -1382,7 +1422,6 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
   // Ozaki form: units run one per CTA (clusters: one per cluster of oz_cl CTAs)
   const int ctas = (oz ? 1 : rows_ctas_per_sm(rplans[0], row_rn)) * c->num_sms;
   const int max_slabs = 64;
-  const int oz_nc = c->opt_tc_nc > 0 && c->opt_tc_nc <= kOzMaxNC ? c->opt_tc_nc : kOzMaxNC;
   int oz_cl = 1;   // Ozaki form: CTAs per cluster of the current wave
   // M tiles and N tiles (Ozaki form: clusters of oz_cl N tiles) of a job's contraction
   auto job_tiles = [&](const JobIn& j, int& mt, int& nt) {
@@ -1430,7 +1469,9 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
     }
     ++c->last_waves;
     const int nj = (int)(end - job_idx);
-    if (oz) oz_cl = oz_cluster_for(c, jobs, job_idx, end, P_cols, oz_nc);
+    if (oz)
+      oz_cl = oz_cluster_for(c, jobs, job_idx, end, ozr.on, P_cols, per_mom ? 1 : n_mom, gp, oz_nc,
+                             c->opt_tc_cluster);
     long long tiles = 0;
     int max_nd3 = 0, max_ndf = 0;
     long long max_elems = 0;
@@ -1837,9 +1878,13 @@ CallPlan plan_call(const bblock_ctx* c, int n_t, const int nd[3], int n_mom, int
   if (c->cfg.precision == BBLOCK_OZAKI) {
     // units (job, 128-row tile, N tile over every momentum's columns, slab)
     const int nc = nc_opt > 0 && nc_opt <= kOzMaxNC ? nc_opt : kOzMaxNC;
+    std::vector<JobIn> one(1);
+    one[0].nd[0] = nd[0]; one[0].nd[1] = nd[1]; one[0].nd[2] = nd[2];
+    GroupPlan as_pairs;
+    as_pairs.n_groups = as_pairs.n_terms = pairs;
     OzRows ozr{};   // (the momenta of the last call, as for the FP16 form)
     if (c->phase_mom.size() == (size_t)3 * n_mom)
-      ozr = plan_oz_rows(c, c->phase_mom.data(), n_mom, 0, pairs);
+      ozr = plan_oz_rows(c, c->phase_mom.data(), n_mom, 0, as_pairs, one, nc);
     const int cols = ozr.on ? ozr.nidx : n_mom, parts = ozr.on ? c->cfg.L * c->cfg.L : X;
     const long long nt = ((long long)cols * nd[2] + nc - 1) / nc;
     const long long tiles = (long long)n_t * ((nd[0] * nd[1] + kOzM - 1) / kOzM) * nt;
