@@ -2236,7 +2236,7 @@ int bblock_from_triplet(bblock_ctx* c, int n_t, const void* T, const void* phi1,
   for (int g = 0; g < gp.n_groups; ++g)
     for (int t = gp.tbeg[g]; t < gp.tbeg[g + 1]; ++t) group_of[t] = g;
   // intermediates for the momenta of one coefficient set, for as many terms at a time as fit
-  // 1 GiB (one at least)
+  // 1 GiB and the caller's workspace limit (one at least), or as can be had
   const int P_set = coeff_per_mom ? 1 : n_mom;
   const size_t f3_bytes = align_up(sizeof(double2) * (size_t)n_ev * nd3, 256);
   const size_t f2_bytes = align_up(sizeof(double2) * (size_t)n_ev * nd2, 256);
@@ -2246,16 +2246,24 @@ int bblock_from_triplet(bblock_ctx* c, int n_t, const void* T, const void* phi1,
   auto bytes_of = [&](int t0, int t1) {
     return groups_in(t0, t1) * (f3_bytes + u1_bytes) + (t1 - t0) * (f2_bytes + u2_bytes);
   };
-  std::vector<int> cut{0};   // the chunks of terms
-  size_t need = 0;
-  while (cut.back() < gp.n_terms) {
-    int t1 = cut.back() + 1;
-    while (t1 < gp.n_terms && bytes_of(cut.back(), t1 + 1) <= ((size_t)1 << 30)) ++t1;
-    need = std::max(need, bytes_of(cut.back(), t1));
-    cut.push_back(t1);
+  std::vector<int> cut;   // the chunks of terms
+  for (size_t limit = std::min((size_t)1 << 30, wave_budget(c));;) {
+    size_t need = 0, longest = 0;
+    cut.assign(1, 0);
+    while (cut.back() < gp.n_terms) {
+      const int t0 = cut.back();
+      int t1 = t0 + 1;
+      while (t1 < gp.n_terms && bytes_of(t0, t1 + 1) <= limit) ++t1;
+      need = std::max(need, bytes_of(t0, t1));
+      longest = std::max(longest, (size_t)(t1 - t0));
+      cut.push_back(t1);
+    }
+    rc = grow_device(c, &c->d_tri, &c->tri_cap, need);
+    if (rc != BBLOCK_ERR_OOM || longest == 1) break;
+    limit = std::min(limit, need) / 2;   // shorter chunks
   }
-  rc = grow_device(c, &c->d_tri, &c->tri_cap, need);
   if (rc) return rc;
+  c->err.clear();
   const long long launches0 = t_kernel_launches;
   for (int t = 0; t < n_t; ++t) {
     const double2* Tt = static_cast<const double2*>(T) + t * tstride;
@@ -2428,7 +2436,7 @@ int bblock_compute_host(bblock_ctx* c, int n_t, const void* V, const void* phi1,
 
 size_t bblock_workspace_bytes(const bblock_ctx* c) {
   if (!c) return 0;
-  return c->ws_cap + c->phase_cap + c->mom_cap + c->tab_cap + c->io_cap + sizeof(int);
+  return c->ws_cap + c->phase_cap + c->mom_cap + c->tab_cap + c->io_cap + c->tri_cap + sizeof(int);
 }
 
 int bblock_last_launch_count(const bblock_ctx* c) { return c ? c->last_launches : 0; }
