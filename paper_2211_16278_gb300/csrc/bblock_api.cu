@@ -1460,7 +1460,7 @@ int run_jobs(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* momen
   size_t job_idx = 0;
   while (job_idx < jobs.size()) {
     // wave of jobs whose workspace fits the budget
-    size_t end = job_idx, need = 0;
+    size_t end = job_idx, need = oz_scratch;
     while (end < jobs.size()) {
       size_t b = job_bytes(jobs[end], max_slabs);
       if (end > job_idx && need + b > wave_budget(c)) break;
