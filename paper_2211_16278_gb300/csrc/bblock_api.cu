@@ -1871,42 +1871,35 @@ struct CallPlan {
   double pad = 0.0;  // padded / actual columns - 1
 };
 
-CallPlan plan_call(const bblock_ctx* c, int n_t, const int nd[3], int n_mom, int pairs,
-                   int nc_opt, int chunk_opt, int slabs_opt) {
+CallPlan plan_call(const bblock_ctx* c, int n_t, const int nd[3], const int32_t* momenta, int n_mom,
+                   const SpinPlan& sp, int nc_opt, int chunk_opt, int slabs_opt) {
   CallPlan pl;
-  const int X = c->X;
+  const int X = c->X, pairs = sp.n_pairs;
+  JobIn shape{};
+  for (int i = 0; i < 3; ++i) shape.nd[i] = nd[i];
   if (c->cfg.precision == BBLOCK_OZAKI) {
-    // units (job, 128-row tile, N tile over every momentum's columns, slab)
+    // units (job, 128-row tile, cluster of N tiles over the momenta or their distinct n0, slab)
+    const std::vector<JobIn> jobs(n_t, shape);
     const int nc = nc_opt > 0 && nc_opt <= kOzMaxNC ? nc_opt : kOzMaxNC;
-    std::vector<JobIn> one(1);
-    one[0].nd[0] = nd[0]; one[0].nd[1] = nd[1]; one[0].nd[2] = nd[2];
-    GroupPlan as_pairs;
-    as_pairs.n_groups = as_pairs.n_terms = pairs;
-    OzRows ozr{};   // (the momenta of the last call, as for the FP16 form)
-    if (c->phase_mom.size() == (size_t)3 * n_mom)
-      ozr = plan_oz_rows(c, c->phase_mom.data(), n_mom, 0, as_pairs, one, nc);
+    const GroupPlan gp = plan_groups(sp, true, jobs, c->cfg.n_ev, 32);
+    const OzRows ozr = plan_oz_rows(c, momenta, n_mom, 0, gp, jobs, nc);
     const int cols = ozr.on ? ozr.nidx : n_mom, parts = ozr.on ? c->cfg.L * c->cfg.L : X;
-    const long long nt = ((long long)cols * nd[2] + nc - 1) / nc;
+    const int cl = oz_cluster_for(c, jobs, 0, jobs.size(), ozr.on, cols, n_mom, gp, nc, c->opt_tc_cluster);
+    const long long nt = (((long long)cols * nd[2] + nc - 1) / nc + cl - 1) / cl;
     const long long tiles = (long long)n_t * ((nd[0] * nd[1] + kOzM - 1) / kOzM) * nt;
     pl.nc = nc;
-    pl.n_slab = slabs_opt > 0 ? std::min(slabs_opt, parts) : choose_slabs(tiles, c->num_sms, parts, 1, 64);
+    pl.n_slab = slabs_opt > 0 ? std::min(slabs_opt, parts) : choose_slabs(tiles, c->num_sms / cl, parts, 1, 64);
     const int sps = (parts + pl.n_slab - 1) / pl.n_slab;
     pl.n_slab = (parts + sps - 1) / sps;
-    pl.units = tiles * pl.n_slab;
-    pl.pad = (double)(nt * nc) / ((double)cols * nd[2]) - 1.0;
+    pl.units = tiles * pl.n_slab * cl;
+    pl.pad = (double)(nt * cl * nc) / ((double)cols * nd[2]) - 1.0;
     return pl;
   }
   if (fp64_like(c->cfg)) {
-    RowPlan one_class{};
-    one_class.n_cls = 1;
-    const int rn = rows_rn_for(&one_class, 1, nd[2]);
-    const int parts = c->cfg.L * c->cfg.L;   // slabs of lattice rows
+    const RowCall rc = plan_row_call(c, sp, momenta, n_mom, 0, {shape});
     const long long tiles = (long long)n_t * ((nd[0] * nd[1] + 16 * kRowRM - 1) / (16 * kRowRM)) *
-                            ((nd[2] + 16 * rn - 1) / (16 * rn));
-    const int ns = slabs_opt > 0 ? std::min(slabs_opt, parts)
-                                 : choose_slabs(tiles, rows_ctas_per_sm(one_class, rn) * c->num_sms, parts, 1, 64);
-    const int sps = (parts + ns - 1) / ns;
-    pl.n_slab = (parts + sps - 1) / sps;
+                            ((nd[2] + 16 * rc.rn - 1) / (16 * rc.rn));
+    pl.n_slab = row_slabs(c, rc.plans[0], rc.rn, rc.groups.n_groups, tiles, slabs_opt).n;
     pl.units = tiles * pl.n_slab;
     pl.pad = (double)((nd[2] + 15) / 16 * 16) / nd[2] - 1.0;   // idle 16-column blocks are skipped
     return pl;
@@ -1916,8 +1909,7 @@ CallPlan plan_call(const bblock_ctx* c, int n_t, const int nd[3], int n_mom, int
   const long long max_groups_per_unit = 256LL * pl.chunk * G;
   const int min_slabs = (int)std::min<long long>(X, ((long long)X * pairs + max_groups_per_unit - 1) / max_groups_per_unit);
   const int max_slabs = std::max(64, min_slabs);
-  std::vector<JobIn> one(1);
-  one[0].nd[0] = nd[0]; one[0].nd[1] = nd[1]; one[0].nd[2] = nd[2];
+  const std::vector<JobIn> one(1, shape);
   const RfPlan rp = plan_rf(c, n_mom, 0, tc_form_of(c->cfg), pairs, G, nc_opt);
   if (rp.on) {   // row-factored: units over d3 tiles and slabs of lattice rows
     const int L = c->cfg.L, n_rows = L * L;
@@ -2461,7 +2453,15 @@ int bblock_autotune(bblock_ctx* c, int n_t, const void* V, const void* phi1, con
   const int nd[3] = {nd1, nd2, nd3};
   // candidate option sets
   std::vector<std::array<int, 3>> cand;
-  const CallPlan base = plan_call(c, n_t, nd, n_mom, sp.n_pairs, 0, 0, 0);
+  // the options that the plans read are the candidate's; the caller's are put back below
+  const int saved[4] = {c->opt_graphs, c->opt_tc_nc, c->opt_tc_chunk, c->opt_slabs};
+  auto set_tiles = [&](int nc, int chunk, int slabs) {
+    c->opt_tc_nc = nc;
+    c->opt_tc_chunk = chunk;
+    c->opt_slabs = slabs;
+  };
+  set_tiles(0, 0, 0);
+  const CallPlan base = plan_call(c, n_t, nd, momenta, n_mom, sp, 0, 0, 0);
   const int a = std::max(1, base.n_slab);
   const int slab_choices[4] = {0, std::max(1, a / 2), 2 * a, 4 * a};
   if (fp64_like(c->cfg)) {
@@ -2485,7 +2485,8 @@ int bblock_autotune(bblock_ctx* c, int n_t, const void* V, const void* phi1, con
     ent[i].nc = cand[i][0];
     ent[i].chunk = cand[i][1];
     ent[i].slabs = cand[i][2];
-    const CallPlan pl = plan_call(c, n_t, nd, n_mom, sp.n_pairs, cand[i][0], cand[i][1], cand[i][2]);
+    set_tiles(cand[i][0], cand[i][1], cand[i][2]);
+    const CallPlan pl = plan_call(c, n_t, nd, momenta, n_mom, sp, cand[i][0], cand[i][1], cand[i][2]);
     tune_features(c, n_t, nd, n_mom, sp.n_pairs, pl, ent[i].features);
     std::copy(ent[i].features, ent[i].features + BBLOCK_TUNE_FEATURES, feat.begin() + (size_t)i * BBLOCK_TUNE_FEATURES);
     ent[i].predicted = 0.f;
@@ -2497,13 +2498,15 @@ int bblock_autotune(bblock_ctx* c, int n_t, const void* V, const void* phi1, con
   if (model) {
     std::vector<float> pred(n_c);
     rc = bblock_costmodel_predict(model, feat.data(), n_c, pred.data());
-    if (rc) return fail(c, rc, "cost-model prediction failed");
+    if (rc) {
+      set_tiles(saved[1], saved[2], saved[3]);
+      return fail(c, rc, "cost-model prediction failed");
+    }
     for (int i = 0; i < n_c; ++i) ent[i].predicted = pred[i];
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return pred[x] < pred[y]; });
     n_time = std::min(top_k, n_c);
   }
   // time the chosen candidates with plain launches
-  const int saved[4] = {c->opt_graphs, c->opt_tc_nc, c->opt_tc_chunk, c->opt_slabs};
   const bool saved_prof = c->prof;
   c->opt_graphs = 0;
   c->prof = false;
@@ -2516,9 +2519,7 @@ int bblock_autotune(bblock_ctx* c, int n_t, const void* V, const void* phi1, con
   int best = -1;
   for (int r = 0; r < n_time && rc == BBLOCK_OK; ++r) {
     const int i = order[r];
-    c->opt_tc_nc = cand[i][0];
-    c->opt_tc_chunk = cand[i][1];
-    c->opt_slabs = cand[i][2];
+    set_tiles(cand[i][0], cand[i][1], cand[i][2]);
     std::vector<float> t;
     for (int k = 0; k <= repeats && rc == BBLOCK_OK; ++k) {
       if (k > 0) cudaEventRecord(e0, s);
@@ -2544,13 +2545,9 @@ int bblock_autotune(bblock_ctx* c, int n_t, const void* V, const void* phi1, con
   c->opt_graphs = saved[0];
   c->prof = saved_prof;
   if (rc == BBLOCK_OK && best >= 0) {
-    c->opt_tc_nc = cand[best][0];
-    c->opt_tc_chunk = cand[best][1];
-    c->opt_slabs = cand[best][2];
+    set_tiles(cand[best][0], cand[best][1], cand[best][2]);
   } else {
-    c->opt_tc_nc = saved[1];
-    c->opt_tc_chunk = saved[2];
-    c->opt_slabs = saved[3];
+    set_tiles(saved[1], saved[2], saved[3]);
   }
   drop_graph(c);
   c->last_sig.clear();
