@@ -99,9 +99,9 @@ struct bblock_ctx {
 namespace {
 // bblock_compute_host moves its time slices in at most this many chunks
 constexpr int kHostChunks = 8;
-enum KernelKind { K_PHASE = 0, K_PROJECT, K_CONTRACT, K_REDUCE, K_CONVERT, K_CANARY, K_COUNT };
+enum KernelKind { K_PHASE = 0, K_PROJECT, K_CONTRACT, K_REDUCE, K_CONVERT, K_CANARY, K_TABLES, K_COUNT };
 const char* const kKernelNames[K_COUNT] = {"phase", "project", "contract", "reduce", "convert",
-                                           "canary"};
+                                           "canary", "tables"};
 static_assert(K_COUNT <= 8, "graph launch-time slots");
 
 cudaEvent_t take_event(bblock_ctx* c) {
@@ -489,7 +489,7 @@ int upload_tables(bblock_ctx* c, const void* src, size_t bytes, cudaStream_t s) 
       return fail(c, BBLOCK_ERR_UNSUPPORTED, "table growth during graph capture");
     char* h = c->h_graph_tab + c->graph_tab_off;
     memcpy(h, src, bytes);
-    CK(c, copy_tables(c->d_tab, h, bytes, s));
+    CK(c, timed_launch(c, K_TABLES, s, [&] { return copy_tables(c->d_tab, h, bytes, s); }));
     c->graph_tab_off += slot;
     return BBLOCK_OK;
   }
@@ -507,7 +507,7 @@ int upload_tables(bblock_ctx* c, const void* src, size_t bytes, cudaStream_t s) 
   int rc = grow_device(c, &c->d_tab, &c->tab_cap, slot);
   if (rc) return rc;
   memcpy(c->h_tab, src, bytes);
-  CK(c, copy_tables(c->d_tab, c->h_tab, bytes, s));
+  CK(c, timed_launch(c, K_TABLES, s, [&] { return copy_tables(c->d_tab, c->h_tab, bytes, s); }));
   CK(c, cudaEventRecord(c->tab_free, s));
   return BBLOCK_OK;
 }
