@@ -560,7 +560,7 @@ int validate_job(bblock_ctx* c, const JobIn& j, int idx, bool device, int n_mom 
                            sz * 4 * c->cfg.n_ev * j.nd[1], sz * 4 * c->cfg.n_ev * j.nd[2],
                            sz * n_mom * j.nd[0] * j.nd[1] * j.nd[2]};
     for (int k = 0; k < 5; ++k)
-      if (ext[k] && !within_allocation(ptrs[k], ext[k]))
+      if (ext[k] && !(j.tri && k >= 1 && k <= 3) && !within_allocation(ptrs[k], ext[k]))
         return fail(c, BBLOCK_ERR_INVALID_ARG, "job %d: %s does not hold %zu bytes", idx,
                     names[k], ext[k]);
   }
@@ -2150,14 +2150,22 @@ int bblock_mode_triplet(bblock_ctx* c, int n_t, const void* V, const int32_t* mo
   if (n_t == 0 || n_mom == 0) { c->last_launches = 0; c->last_waves = 0; return BBLOCK_OK; }
   CK(c, cudaSetDevice(c->cfg.device));
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (!c->d_ident) {
-    if (c->capturing) return fail(c, BBLOCK_ERR_UNSUPPORTED, "allocation during graph capture");
-    if (cudaMalloc(&c->d_ident, sizeof(double2) * 4 * (size_t)n_ev * n_ev) != cudaSuccess) {
+  // FP64 and double-float without checks sum the ordered elements of V itself (run_triplet); the
+  // other routes contract fields of identity coefficients
+  const bool tri = !c->opt_checks && (c->cfg.precision == BBLOCK_FP64 || c->cfg.precision == BBLOCK_DF64);
+  if (!tri && !c->d_ident) {
+    double2* ident = nullptr;
+    if (cudaMalloc(&ident, sizeof(double2) * 4 * (size_t)n_ev * n_ev) != cudaSuccess) {
       cudaGetLastError();
-      c->d_ident = nullptr;
       return fail(c, BBLOCK_ERR_OOM, "identity coefficients");
     }
-    CK(c, launch_fill_identity(c->d_ident, n_ev, s));
+    cudaError_t e = launch_fill_identity(ident, n_ev, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // later calls may come on another stream
+    if (e != cudaSuccess) {
+      cudaFree(ident);
+      return cuda_fail(c, e, "identity coefficients");
+    }
+    c->d_ident = ident;
   }
   const size_t vstride = (size_t)n_ev * c->rows;
   const size_t tstride = (size_t)n_mom * n_ev * n_ev * n_ev;
@@ -2165,10 +2173,10 @@ int bblock_mode_triplet(bblock_ctx* c, int n_t, const void* V, const int32_t* mo
   for (int t = 0; t < n_t; ++t) {
     JobIn& j = jobs[t];
     j.V = static_cast<const double2*>(V) + t * vstride;
-    j.phi[0] = j.phi[1] = j.phi[2] = c->d_ident;
+    j.phi[0] = j.phi[1] = j.phi[2] = tri ? j.V : c->d_ident;
     j.nd[0] = j.nd[1] = j.nd[2] = n_ev;
     j.B = static_cast<double2*>(T_out) + t * tstride;
-    j.tri = !c->opt_checks && (c->cfg.precision == BBLOCK_FP64 || c->cfg.precision == BBLOCK_DF64);
+    j.tri = tri;
     rc = validate_job(c, j, t, true, n_mom);
     if (rc) return rc;
   }
