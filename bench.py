@@ -23,7 +23,8 @@ The same line reports, on the same inputs:
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
                   [--workload NAME] [--form FORM]
 
-Prints one JSON line (rank 0). Under torchrun every rank computes its own independent
+Prints one JSON line (rank 0) and, on stderr, one with the details (rooflines, step times, errors, the
+other forms). Under torchrun every rank computes its own independent
 inputs (weak scaling, no data-path collective); the timed region is bracketed by a barrier
 and the maximum over ranks is reported.
 """
@@ -552,6 +553,18 @@ def df_roofline(prof, inst, alg_flops, steps):
             "flops": "modelled FP32 instructions of the double-float inner loops",
             "complex_count_tflops": alg_flops * steps / (msc / 1e3) / 1e12, "launches": nc,
             "avg_launch_ms": msc / nc}
+
+
+RESULT_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+               "scaling", "vs_baseline", "dtype", "data", "config", "e2e", "gpu_launches", "clocks",
+               "speedup_vs_fp64_form")
+
+
+def result_and_detail(line):
+    """The result line (stdout), short enough that a reader who keeps the last 1500 characters of the
+    output has all of it, and the rest (stderr): rooflines, step times, errors, the other forms."""
+    return ({k: line[k] for k in RESULT_KEYS if k in line},
+            {"detail": {k: v for k, v in line.items() if k not in RESULT_KEYS}})
 
 
 def kernel_table(prof, ms):
@@ -1160,7 +1173,9 @@ def run_ours(args):
         line["cpu_baseline"] = cpu
         line["clocks"] = clk.summary()
         line["secondary"] = secondary
-        print(json.dumps(line), flush=True)
+        result, detail = result_and_detail(line)
+        print(json.dumps(detail), file=sys.stderr, flush=True)
+        print(json.dumps(result), flush=True)
     if world > 1:
         dist.destroy_process_group()
     return 0
