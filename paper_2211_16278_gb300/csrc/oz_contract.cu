@@ -514,8 +514,9 @@ __device__ __forceinline__ void oz_produce(const ContractParams& prm, const OzSh
             Rc *= 0x1p-8f;
           }
           // the next 4 elements: one group and one colour on
-          int groups = 1;
-          if (++hc == 3) { hc = 0; ++groups; }
+          int groups = LB / 3;
+          hc += LB % 3;
+          if (hc >= 3) { hc -= 3; ++groups; }
           hg += groups;
           while (hg >= ng) { hg -= ng; ++hx; }
           hk += LB;
