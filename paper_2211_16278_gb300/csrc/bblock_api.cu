@@ -1268,14 +1268,20 @@ RowCall plan_row_call(const bblock_ctx* c, const SpinPlan& sp, const int32_t* mo
   r.groups = plan_groups(sp, true, jobs, c->cfg.n_ev, 64);
   const int G = r.groups.n_groups, T = r.groups.n_terms;
   if (per_mom) {
+    // one kind for all: the launches share slabs, of rows or of sites
     r.plans.resize(n_mom);
+    bool all_site = true;
     for (int p = 0; p < n_mom; ++p) {
-      plan_rows(L, momenta + 3 * p, 1, G, T, nd3, df, &r.plans[p], 1);
+      plan_rows(L, momenta + 3 * p, 1, G, T, nd3, df, ROWS_AUTO, &r.plans[p], 1);
+      all_site = all_site && r.plans[p].per_site;
+    }
+    for (int p = 0; p < n_mom; ++p) {
+      if (!all_site) plan_rows(L, momenta + 3 * p, 1, G, T, nd3, df, ROWS_FACTORED, &r.plans[p], 1);
       r.plans[p].mom[0].p = p;
     }
   } else {
-    r.plans.resize(plan_rows(L, momenta, n_mom, G, T, nd3, df, nullptr, 0));
-    plan_rows(L, momenta, n_mom, G, T, nd3, df, r.plans.data(), (int)r.plans.size());
+    r.plans.resize(plan_rows(L, momenta, n_mom, G, T, nd3, df, ROWS_AUTO, nullptr, 0));
+    plan_rows(L, momenta, n_mom, G, T, nd3, df, ROWS_AUTO, r.plans.data(), (int)r.plans.size());
   }
   r.rn = rows_rn_for(r.plans.data(), (int)r.plans.size(), nd3);
   if (r.rn < 4) r.groups = plan_groups(sp, true, jobs, c->cfg.n_ev, 16 * r.rn);
@@ -1289,8 +1295,8 @@ int run_triplet(bblock_ctx* c, const std::vector<JobIn>& jobs, const int32_t* mo
   const int L = c->cfg.L, rows = c->rows, n = c->cfg.n_ev, X = c->X;
   const bool df = c->cfg.precision == BBLOCK_DF64;
   const int M = n * (n - 1) / 2;
-  std::vector<RowPlan> rplans(plan_rows(L, momenta, n_mom, 1, 1, n, df, nullptr, 0));
-  plan_rows(L, momenta, n_mom, 1, 1, n, df, rplans.data(), (int)rplans.size());
+  std::vector<RowPlan> rplans(plan_rows(L, momenta, n_mom, 1, 1, n, df, ROWS_AUTO, nullptr, 0));
+  plan_rows(L, momenta, n_mom, 1, 1, n, df, ROWS_AUTO, rplans.data(), (int)rplans.size());
   const int rn = rows_rn_for(rplans.data(), (int)rplans.size(), n);
   const int m_tiles = (M + 16 * kRowRM - 1) / (16 * kRowRM), n_tiles = (n + 16 * rn - 1) / (16 * rn);
   const int max_slabs = 64;

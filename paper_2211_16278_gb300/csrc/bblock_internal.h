@@ -213,8 +213,10 @@ static_assert((size_t)24 * (16 * kRowRM + 64) * 3 * kMaxPairs + 16 * (kMaxSiteP 
 // groups, terms: of the spin sum; nd3: the widest job's d3 columns; df: double-float.
 // Returns the number of plans written to `out` (at most max_out), or the number needed where
 // out is null.
+// All plans of a call are of one kind: they share the call's slabs.
+enum RowKind { ROWS_AUTO, ROWS_FACTORED };
 int plan_rows(int L, const int32_t* momenta, int n_mom, int groups, int terms, int nd3, bool df,
-              RowPlan* out, int max_out);
+              RowKind kind, RowPlan* out, int max_out);
 
 // ---------------------------------------------------------------- tensor-core forms
 

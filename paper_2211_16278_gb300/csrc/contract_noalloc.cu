@@ -284,7 +284,7 @@ extern "C" int bblock_contract_noalloc(int L, const void* q1, const void* q2, co
   }
 
   RowPlan plans[kNaMaxP];
-  const int n_plans = plan_rows(L, momenta, n_mom, base.n_groups, base.n_terms, nd3, false, plans, kNaMaxP);
+  const int n_plans = plan_rows(L, momenta, n_mom, base.n_groups, base.n_terms, nd3, false, ROWS_AUTO, plans, kNaMaxP);
   const int rn = rows_rn_for(plans, n_plans, nd3);
   job.m_tiles = (nd1 * nd2 + 16 * kRowRM - 1) / (16 * kRowRM);
   job.n_tiles = (nd3 + 16 * rn - 1) / (16 * rn);
@@ -378,7 +378,7 @@ extern "C" int bblock_contract_noalloc(int L, const void* q1, const void* q2, co
     base.rows = plans[k];
     base.xc = plans[k].per_site ? xc : rows_sites_per_chunk(L, plans[k], rn, base.n_groups);
     const long long cap = (long long)rows_ctas_per_sm(plans[k], rn) * num_sms;
-    e = rowsc::launch_plan<RowsNoalloc, kNaMaxP>(plans[k], rn, prm, (int)(base.total_units < cap ? base.total_units : cap), s);
+    e = rowsc::launch_plan<RowsNoalloc, kNaMaxP>(base, rn, prm, (int)(base.total_units < cap ? base.total_units : cap), s);
   }
   if (e == cudaSuccess) {
     const int lanes = base.n_slab >= 16 ? 8 : 1;

@@ -38,7 +38,7 @@ struct RowsDf {
 
 cudaError_t launch_contract_df(const ContractParams& prm, int rn, int grid, cudaStream_t s) {
   if (prm.total_units == 0 || prm.rows.n_mom == 0) return cudaSuccess;
-  return rowsc::launch_plan<RowsDf, kMaxSitePDf>(prm.rows, rn, prm, grid, s);
+  return rowsc::launch_plan<RowsDf, kMaxSitePDf>(prm, rn, prm, grid, s);
 }
 
 }  // namespace bb

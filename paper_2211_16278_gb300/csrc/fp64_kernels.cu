@@ -280,7 +280,7 @@ int site_plans(int L, const int32_t* momenta, int n_mom, int cap, RowPlan* out, 
 // and per site: k < 2  4.72 / 1.40 and 4.91 / 1.44; k < 4  6.86 / 2.18 and 6.72 / 1.88;
 // k < 8  16.7 / 5.23 and 10.5 / 2.81; -3 <= k <= 3  7.07 / 2.40 and 9.6 / 2.59.
 int plan_rows(int L, const int32_t* momenta, int n_mom, int groups, int terms, int nd3, bool df,
-              RowPlan* out, int max_out) {
+              RowKind kind, RowPlan* out, int max_out) {
   if (n_mom < 1) return 0;
   int axis = 2, fewest = 1 << 30;
   for (int a = 2; a >= 0; --a) {
@@ -307,7 +307,7 @@ int plan_rows(int L, const int32_t* momenta, int n_mom, int groups, int terms, i
   shape.per_site = 1;
   shape.n_mom = n_mom < cap ? n_mom : cap;
   const double by_site = (n_mom + cap - 1) / cap * (singlet_ops(shape) + 2.0) + 4.0 * n_mom;
-  if (by_site < 0.97 * by_row) return site_plans(L, momenta, n_mom, cap, out, max_out);
+  if (kind == ROWS_AUTO && by_site < 0.97 * by_row) return site_plans(L, momenta, n_mom, cap, out, max_out);
   return row_plans(L, momenta, n_mom, axis, out, max_out);
 }
 
@@ -332,7 +332,7 @@ struct RowsF64 {
 
 cudaError_t launch_contract_fp64(const ContractParams& prm, int rn, int grid, cudaStream_t s) {
   if (prm.total_units == 0 || prm.rows.n_mom == 0) return cudaSuccess;
-  return rowsc::launch_plan<RowsF64, kMaxSiteP>(prm.rows, rn, prm, grid, s);
+  return rowsc::launch_plan<RowsF64, kMaxSiteP>(prm, rn, prm, grid, s);
 }
 
 // ------------------------------------------------------------------ slab reduction

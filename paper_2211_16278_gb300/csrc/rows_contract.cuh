@@ -500,8 +500,11 @@ __device__ __forceinline__ void contract_rows(const ContractParams& prm, const S
 
 // The launch of Kernel<NCLS, NP, RN> for a plan; WIDE: momenta of the widest per-site launch.
 template <template <int, int, int> class Kernel, int WIDE, class Params>
-cudaError_t launch_plan(const RowPlan& r, int rn, const Params& prm, int grid, cudaStream_t s) {
-  if (rn > rows_max_rn(r)) return cudaErrorInvalidValue;
+cudaError_t launch_plan(const ContractParams& c, int rn, const Params& prm, int grid, cudaStream_t s) {
+  const RowPlan& r = c.rows;
+  // a chunk and a slab of the plan's kind, and tiles that it has
+  if (c.xc < 1 || (r.per_site ? c.sites_per_slab : c.rows_per_slab) < 1 || rn > rows_max_rn(r))
+    return cudaErrorInvalidValue;
   if (r.per_site) {
     if (r.n_mom > WIDE) return cudaErrorInvalidValue;
     if (r.n_mom > kSitePNarrow) return Kernel<0, WIDE, 1>::launch(prm, grid, s);

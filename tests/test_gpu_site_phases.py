@@ -110,3 +110,27 @@ def test_mode_triplet(env, form):
     bb.bblock_destroy(ctx)
     ref = oracle.mode_triplet(L, inp.V[0], mom)
     assert np.linalg.norm(T - ref) <= TOL * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("form", ["fp64", "df64"])
+@pytest.mark.parametrize("mom", [[(0, 0, 0), (1, 1, 1), (1, 0, 0)], [(2, 1, 1), (1, 1, 3), (-1, 1, 2)]])
+@pytest.mark.parametrize("nd", [(3, 4, 16), (5, 6, 40)])
+def test_a_coefficient_set_for_each_momentum(env, form, mom, nd):
+    """A launch per momentum, all of one kind: some momenta alone would be row-factored, some not."""
+    torch, bb = env
+    L, n_ev = 9, 4
+    spins, coeffs = SPINS["three"]
+    per_mom = np.array([[c * (1 + p) for c in coeffs] for p in range(len(mom))], np.complex128)
+    inp = workloads.custom(L, n_ev, nd, 2, mom, spins, coeffs, seed=9600)
+    dev = torch.device("cuda:0")
+    ctx = bb.bblock_create(L, n_ev, max(nd), form)
+    B = bb.bblock_compute(ctx, torch.from_numpy(inp.V).to(dev),
+                          *[torch.from_numpy(inp.phi[0][i]).to(dev) for i in range(3)],
+                          inp.momenta, inp.spins, per_mom)
+    bb.bblock_status(ctx)
+    for t in range(2):
+        for p in range(len(mom)):
+            ref = oracle.bblock(L, inp.V[t], *[inp.phi[0][i][t] for i in range(3)], inp.momenta[p:p + 1],
+                                inp.spins, per_mom[p])
+            assert np.linalg.norm(B[t, p].cpu().numpy() - ref[0]) <= TOL * np.linalg.norm(ref), (t, p)
+    bb.bblock_destroy(ctx)
