@@ -689,219 +689,219 @@ __device__ __forceinline__ void tc_body(const TcParams& prm) {
       for (int st = 0; st < w.n_stages; ++st, ++s_g) {
         const int slot = (int)(s_g % STAGES);
         if (!kSets || !is_a || (int)(s_g & 1) == pt / 128) {
-        bool ok = !abort_flag;
-        if (ok && s_g >= STAGES)
-          ok = wait_bounded(smem_u32(&bar_empty[slot]), (uint32_t)(((s_g / STAGES) + 1) & 1),
-                            &abort_flag, prm.status, prm.wait_limit);
-        // a warp either fills its rows of this stage or (after an abort) none of them
-        ok = __all_sync(0xffffffffu, ok);
-        if (ok && row_used) {
-          if constexpr (PROJ) {
-            float re[3][8], im[3][8];
-            // element (colour c, group g0 + j) of this stage is eigenvector index l
-            const int rows = prm.p_rows, n_ev = prm.p_n_ev;
-            if (is_a) {
-              float2 v[3][8];
+          bool ok = !abort_flag;
+          if (ok && s_g >= STAGES)
+            ok = wait_bounded(smem_u32(&bar_empty[slot]), (uint32_t)(((s_g / STAGES) + 1) & 1),
+                              &abort_flag, prm.status, prm.wait_limit);
+          // a warp either fills its rows of this stage or (after an abort) none of them
+          ok = __all_sync(0xffffffffu, ok);
+          if (ok && row_used) {
+            if constexpr (PROJ) {
+              float re[3][8], im[3][8];
+              // element (colour c, group g0 + j) of this stage is eigenvector index l
+              const int rows = prm.p_rows, n_ev = prm.p_n_ev;
+              if (is_a) {
+                float2 v[3][8];
 #pragma unroll
-              for (int c = 0; c < 3; ++c)
+                for (int c = 0; c < 3; ++c)
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                  const int l = st * 3 * G + c * G + g0 + j;
-                  v[c][j] = (j < NG && row_ok && l < n_ev) ? p_src[(size_t)l * rows]
-                                                           : make_float2(0.f, 0.f);
-                }
+                  for (int j = 0; j < 8; ++j) {
+                    const int l = st * 3 * G + c * G + g0 + j;
+                    v[c][j] = (j < NG && row_ok && l < n_ev) ? p_src[(size_t)l * rows]
+                                                             : make_float2(0.f, 0.f);
+                  }
 #pragma unroll
-              for (int c = 0; c < 3; ++c)
+                for (int c = 0; c < 3; ++c)
 #pragma unroll
-                for (int j = 0; j < 8; ++j) { re[c][j] = v[c][j].x; im[c][j] = v[c][j].y; }
+                  for (int j = 0; j < 8; ++j) { re[c][j] = v[c][j].x; im[c][j] = v[c][j].y; }
+              } else {
+#pragma unroll
+                for (int c = 0; c < 3; ++c)
+#pragma unroll
+                  for (int j = 0; j < 8; ++j) {
+                    const int l = st * 3 * G + c * G + g0 + j;
+                    float2 b = make_float2(0.f, 0.f);
+                    if (j < NG && row_ok && l < n_ev) {
+#pragma unroll
+                      for (int t = 0; t < kMaxTerms; ++t)
+                        if (t < p_terms) {
+                          const float2 f = p_src[(size_t)p_off[t] + (size_t)l * p_nd];
+                          b.x = fmaf(p_w[t].x, f.x, fmaf(-p_w[t].y, f.y, b.x));
+                          b.y = fmaf(p_w[t].x, f.y, fmaf(p_w[t].y, f.x, b.y));
+                        }
+                    }
+                    re[c][j] = b.x;
+                    im[c][j] = b.y;
+                  }
+              }
+              if (is_a) store_run(re, im, std::integral_constant<int, 8>{}, std::true_type{}, slot);
+              else store_run(re, im, std::integral_constant<int, 8>{}, std::false_type{}, slot);
             } else {
+              // the stage's sites [sx0, sx1): the slab's, or (row-factored) the stage's row, whose
+              // groups count from its first site; this thread's first group of its run of NG is
+              // (site sx0 + g_xl, pair g_pr)
+              const int sx0 = RF ? (w.x_begin + rf_row) * prm.L : w.x_begin;
+              const int sx1 = RF ? sx0 + prm.L : w.x_end;
+              // One role's groups, with their group count and loads per group known at compile
+              // time, so that each role's load buffers take only its own registers: the
+              // diquark side loads 6 values per group in rounds of kLoadRun groups, the
+              // third-quark side 4 per group, all of its groups in one round (unchecked). Then
+              // the run is split into pieces and stored. The producers' instructions bound the
+              // stage (half of its issue slots at 55 % issue activity), so offsets are 32-bit (a
+              // field has 3 X nd < 2^31 elements) and stores take one address per thread with
+              // constant plane offsets. Measured against 64-bit offsets and per-plane pointers,
+              // contraction of one time slice, L = 32, N_dil = 64: BF16 6 products, 5 momenta
+              // 34.9 -> 31.4 ms, TF32 46.7 -> 40.0, FP16 pairs, 9 momenta 38.3 -> 34.0.
+              // (Tried without gain: packed FP32 pairs; the next run's loads issued ahead of the
+              // split and the wait, 15.5 against 14.6 ms row-factored; row sums in registers with
+              // setmaxnreg, 17.4.)
+              constexpr bool kOneStore = (!F16 || kSets) && R::kBGroups == kAG;
+              float re[3][8], im[3][8];
+              auto build = [&](auto kNG, auto kIsA) {
+                constexpr int NGc = decltype(kNG)::value;
+                constexpr bool Ac = decltype(kIsA)::value;
+                constexpr int LR = Ac ? (kLoadRun < NGc ? kLoadRun : NGc) : (CHECKS ? 4 : NGc);
+                constexpr int NV = Ac ? 6 : 4;
+                uint32_t vmask = 0;   // groups of this run that lie inside the slab and a used row
+                int xl = g_xl, pr = g_pr;
+                [[maybe_unused]] int ph = rf_ph;
+                const int s1x3 = 3 * s1, s2x3 = 3 * s2;
 #pragma unroll
-              for (int c = 0; c < 3; ++c)
+                for (int half = 0; half < NGc / LR; ++half) {
+                  // LR groups: issue every load first, then compute
+                  float2 ld[LR][NV];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                  const int l = st * 3 * G + c * G + g0 + j;
-                  float2 b = make_float2(0.f, 0.f);
-                  if (j < NG && row_ok && l < n_ev) {
-#pragma unroll
-                    for (int t = 0; t < kMaxTerms; ++t)
-                      if (t < p_terms) {
-                        const float2 f = p_src[(size_t)p_off[t] + (size_t)l * p_nd];
-                        b.x = fmaf(p_w[t].x, f.x, fmaf(-p_w[t].y, f.y, b.x));
-                        b.y = fmaf(p_w[t].x, f.y, fmaf(p_w[t].y, f.x, b.y));
+                  for (int j = 0; j < LR; ++j) {
+                    const int x = sx0 + xl;
+                    bool vld = row_ok && x < sx1;
+                    int xs = x < sx1 ? x : sx0;
+                    if (CHECKS) {
+                      const long long fl = 3LL * prm.X * s1;            // elements of a field
+                      bool good = idx_ok(prm, (long long)xs * 3 * s1 + off1 + 2LL * s1, fl, Ac ? 1 : 3, w.job) &&
+                                  idx_ok(prm, pr, np, 6, w.job);
+                      if (Ac) good = good && idx_ok(prm, (long long)xs * 3 * s2 + off2 + 2LL * s2, 3LL * prm.X * s2, 2, w.job);
+                      else good = good && idx_ok(prm, (long long)pidx * prm.X + xs, (long long)prm.P * prm.X, 4, w.job);
+                      if (!good) { vld = false; xs = 0; pr = 0; }
+                    }
+                    vmask |= (uint32_t)vld << (half * LR + j);
+                    const uint32_t ou = (uint32_t)(xs * s1x3 + off1);
+                    if constexpr (Ac) {
+                      const float2* const uf = s_q1[pr];
+                      const float2* const vf = s_q2[pr];
+                      const uint32_t ov = (uint32_t)(xs * s2x3 + off2);
+                      ld[j][0] = uf[ou]; ld[j][1] = uf[ou + s1]; ld[j][2] = uf[ou + 2 * s1];
+                      ld[j][3] = vf[ov]; ld[j][4] = vf[ov + s2]; ld[j][5] = vf[ov + 2 * s2];
+                    } else {
+                      const float2* const qf = s_q3[pr];
+                      ld[j][0] = qf[ou]; ld[j][1] = qf[ou + s1]; ld[j][2] = qf[ou + 2 * s1];
+                      if constexpr (RF) ld[j][3] = s_omega[ph];
+                      else ld[j][3] = phase_p[xs];
+                    }
+                    if (++pr == np) {
+                      pr = 0;
+                      ++xl;
+                      if constexpr (RF) {
+                        ph += pidx;
+                        if (ph >= prm.L) ph -= prm.L;
                       }
-                  }
-                  re[c][j] = b.x;
-                  im[c][j] = b.y;
-                }
-            }
-            if (is_a) store_run(re, im, std::integral_constant<int, 8>{}, std::true_type{}, slot);
-            else store_run(re, im, std::integral_constant<int, 8>{}, std::false_type{}, slot);
-          } else {
-            // the stage's sites [sx0, sx1): the slab's, or (row-factored) the stage's row, whose
-            // groups count from its first site; this thread's first group of its run of NG is
-            // (site sx0 + g_xl, pair g_pr)
-            const int sx0 = RF ? (w.x_begin + rf_row) * prm.L : w.x_begin;
-            const int sx1 = RF ? sx0 + prm.L : w.x_end;
-            // One role's groups, with their group count and loads per group known at compile
-            // time, so that each role's load buffers take only its own registers: the
-            // diquark side loads 6 values per group in rounds of kLoadRun groups, the
-            // third-quark side 4 per group, all of its groups in one round (unchecked). Then
-            // the run is split into pieces and stored. The producers' instructions bound the
-            // stage (half of its issue slots at 55 % issue activity), so offsets are 32-bit (a
-            // field has 3 X nd < 2^31 elements) and stores take one address per thread with
-            // constant plane offsets. Measured against 64-bit offsets and per-plane pointers,
-            // contraction of one time slice, L = 32, N_dil = 64: BF16 6 products, 5 momenta
-            // 34.9 -> 31.4 ms, TF32 46.7 -> 40.0, FP16 pairs, 9 momenta 38.3 -> 34.0.
-            // (Tried without gain: packed FP32 pairs; the next run's loads issued ahead of the
-            // split and the wait, 15.5 against 14.6 ms row-factored; row sums in registers with
-            // setmaxnreg, 17.4.)
-            constexpr bool kOneStore = (!F16 || kSets) && R::kBGroups == kAG;
-            float re[3][8], im[3][8];
-            auto build = [&](auto kNG, auto kIsA) {
-              constexpr int NGc = decltype(kNG)::value;
-              constexpr bool Ac = decltype(kIsA)::value;
-              constexpr int LR = Ac ? (kLoadRun < NGc ? kLoadRun : NGc) : (CHECKS ? 4 : NGc);
-              constexpr int NV = Ac ? 6 : 4;
-              uint32_t vmask = 0;   // groups of this run that lie inside the slab and a used row
-              int xl = g_xl, pr = g_pr;
-              [[maybe_unused]] int ph = rf_ph;
-              const int s1x3 = 3 * s1, s2x3 = 3 * s2;
-#pragma unroll
-              for (int half = 0; half < NGc / LR; ++half) {
-                // LR groups: issue every load first, then compute
-                float2 ld[LR][NV];
-#pragma unroll
-                for (int j = 0; j < LR; ++j) {
-                  const int x = sx0 + xl;
-                  bool vld = row_ok && x < sx1;
-                  int xs = x < sx1 ? x : sx0;
-                  if (CHECKS) {
-                    const long long fl = 3LL * prm.X * s1;            // elements of a field
-                    bool good = idx_ok(prm, (long long)xs * 3 * s1 + off1 + 2LL * s1, fl, Ac ? 1 : 3, w.job) &&
-                                idx_ok(prm, pr, np, 6, w.job);
-                    if (Ac) good = good && idx_ok(prm, (long long)xs * 3 * s2 + off2 + 2LL * s2, 3LL * prm.X * s2, 2, w.job);
-                    else good = good && idx_ok(prm, (long long)pidx * prm.X + xs, (long long)prm.P * prm.X, 4, w.job);
-                    if (!good) { vld = false; xs = 0; pr = 0; }
-                  }
-                  vmask |= (uint32_t)vld << (half * LR + j);
-                  const uint32_t ou = (uint32_t)(xs * s1x3 + off1);
-                  if constexpr (Ac) {
-                    const float2* const uf = s_q1[pr];
-                    const float2* const vf = s_q2[pr];
-                    const uint32_t ov = (uint32_t)(xs * s2x3 + off2);
-                    ld[j][0] = uf[ou]; ld[j][1] = uf[ou + s1]; ld[j][2] = uf[ou + 2 * s1];
-                    ld[j][3] = vf[ov]; ld[j][4] = vf[ov + s2]; ld[j][5] = vf[ov + 2 * s2];
-                  } else {
-                    const float2* const qf = s_q3[pr];
-                    ld[j][0] = qf[ou]; ld[j][1] = qf[ou + s1]; ld[j][2] = qf[ou + 2 * s1];
-                    if constexpr (RF) ld[j][3] = s_omega[ph];
-                    else ld[j][3] = phase_p[xs];
-                  }
-                  if (++pr == np) {
-                    pr = 0;
-                    ++xl;
-                    if constexpr (RF) {
-                      ph += pidx;
-                      if (ph >= prm.L) ph -= prm.L;
                     }
                   }
-                }
 #pragma unroll
-                for (int j = 0; j < LR; ++j) {
-                  float2 c[3];
-                  if constexpr (Ac) {
-                    const float2 u0 = ld[j][0], u1 = ld[j][1], u2 = ld[j][2];
-                    const float2 v0 = ld[j][3], v1 = ld[j][4], v2 = ld[j][5];
-                    c[0] = sub2f(cmulf(u1, v2), cmulf(u2, v1));
-                    c[1] = sub2f(cmulf(u2, v0), cmulf(u0, v2));
-                    c[2] = sub2f(cmulf(u0, v1), cmulf(u1, v0));
-                    if constexpr (F16) {
+                  for (int j = 0; j < LR; ++j) {
+                    float2 c[3];
+                    if constexpr (Ac) {
+                      const float2 u0 = ld[j][0], u1 = ld[j][1], u2 = ld[j][2];
+                      const float2 v0 = ld[j][3], v1 = ld[j][4], v2 = ld[j][5];
+                      c[0] = sub2f(cmulf(u1, v2), cmulf(u2, v1));
+                      c[1] = sub2f(cmulf(u2, v0), cmulf(u0, v2));
+                      c[2] = sub2f(cmulf(u0, v1), cmulf(u1, v0));
+                      if constexpr (F16) {
 #pragma unroll
-                      for (int k = 0; k < 3; ++k) { c[k].x *= f16s; c[k].y *= f16s; }
+                        for (int k = 0; k < 3; ++k) { c[k].x *= f16s; c[k].y *= f16s; }
+                      }
+                    } else {
+                      float2 phv = ld[j][3];
+                      if constexpr (F16) { phv.x *= f16s; phv.y *= f16s; }
+#pragma unroll
+                      for (int k = 0; k < 3; ++k) c[k] = cmulf(phv, ld[j][k]);
                     }
-                  } else {
-                    float2 phv = ld[j][3];
-                    if constexpr (F16) { phv.x *= f16s; phv.y *= f16s; }
+                    const int jj = half * LR + j;
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) c[k] = cmulf(phv, ld[j][k]);
+                    for (int k = 0; k < 3; ++k) { re[k][jj] = c[k].x; im[k][jj] = c[k].y; }
                   }
-                  const int jj = half * LR + j;
-#pragma unroll
-                  for (int k = 0; k < 3; ++k) { re[k][jj] = c[k].x; im[k][jj] = c[k].y; }
                 }
-              }
-              // groups past the slab's end or of an unused row (their loads read a valid site)
-              // contribute zeros; this branch is taken only at ragged edges
-              if (vmask != (1u << NGc) - 1u) {
+                // groups past the slab's end or of an unused row (their loads read a valid site)
+                // contribute zeros; this branch is taken only at ragged edges
+                if (vmask != (1u << NGc) - 1u) {
 #pragma unroll
-                for (int jj = 0; jj < NGc; ++jj)
-                  if (!((vmask >> jj) & 1u)) {
-                    re[0][jj] = 0.f; im[0][jj] = 0.f;
-                    re[1][jj] = 0.f; im[1][jj] = 0.f;
-                    re[2][jj] = 0.f; im[2][jj] = 0.f;
-                  }
-              }
-              if constexpr (!kOneStore) store_run(re, im, kNG, kIsA, slot);
-            };
-            if (is_a) build(std::integral_constant<int, kAG>{}, std::true_type{});
-            else build(std::integral_constant<int, R::kBGroups>{}, std::false_type{});
-            if constexpr (kOneStore) store_run_any(re, im, std::integral_constant<int, kAG>{}, slot);
-          }
-        }
-        // every lane's core-matrix stores are made visible to the tensor core's (async)
-        // proxy; once the whole warp has fenced, one lane acts for the warp
-        fence_async_smem();
-        __syncwarp();
-        if (lane == 0) {
-          if (SHB && is_b && ok) {
-            // this warp's third-quark row groups (16 rows of this CTA's share) of every
-            // plane go to the peer, at the same offsets of its stage
-            const uint32_t peer = rank ^ 1u;
-            const uint32_t mbar = map_to_rank(smem_u32(&bar_full[slot]), peer);
-            const int lr0 = ((pt - R::kAThreads) / 32) * 16;
-#pragma unroll
-            for (int gq = 0; gq < 2; ++gq) {
-              if (lr0 + 8 * gq >= NC / 2) break;
-              const uint32_t rg = (uint32_t)(((int)rank * (NC / 2) + lr0 + 8 * gq) >> 3);
-#pragma unroll
-              for (int l = 0; l < LEVELS; ++l)
-#pragma unroll
-                for (int pl = 0; pl < kBPlanes; ++pl) {
-                  const uint32_t src = smem_base + b_plane(slot, l, pl) + rg * 768u;
-                  copy_to_peer(map_to_rank(src, peer), src, 768u, mbar);
+                  for (int jj = 0; jj < NGc; ++jj)
+                    if (!((vmask >> jj) & 1u)) {
+                      re[0][jj] = 0.f; im[0][jj] = 0.f;
+                      re[1][jj] = 0.f; im[1][jj] = 0.f;
+                      re[2][jj] = 0.f; im[2][jj] = 0.f;
+                    }
                 }
+                if constexpr (!kOneStore) store_run(re, im, kNG, kIsA, slot);
+              };
+              if (is_a) build(std::integral_constant<int, kAG>{}, std::true_type{});
+              else build(std::integral_constant<int, R::kBGroups>{}, std::false_type{});
+              if constexpr (kOneStore) store_run_any(re, im, std::integral_constant<int, kAG>{}, slot);
             }
           }
-          if (kSets && is_a && ok) {
-            // this warp's 32 diquark rows and K half of every plane go to the peer
-            const uint32_t src = smem_base + (uint32_t)(slot * STAGE_BYTES) +
-                                 (uint32_t)(g0 / 8) * kSetHalf + (uint32_t)(rr >> 3) * kSetGroup;
-            const uint32_t peer = rank ^ 1u;
-            copy_to_peer(map_to_rank(src, peer), src, 4 * kSetGroup,
-                         map_to_rank(smem_u32(&bar_full[slot]), peer));
-          }
-          if (kShareA && !kSets && is_a && ok) {
-            // this warp's 8 diquark rows (one row group) of every plane go to every peer
-            const uint32_t rg = (uint32_t)(rr >> 3);
-            const uint32_t full_local = smem_u32(&bar_full[slot]);
-            for (uint32_t q = 0; q < (uint32_t)C; ++q) {
-              if (q == rank) continue;
-              const uint32_t mbar = map_to_rank(full_local, q);
+          // every lane's core-matrix stores are made visible to the tensor core's (async)
+          // proxy; once the whole warp has fenced, one lane acts for the warp
+          fence_async_smem();
+          __syncwarp();
+          if (lane == 0) {
+            if (SHB && is_b && ok) {
+              // this warp's third-quark row groups (16 rows of this CTA's share) of every
+              // plane go to the peer, at the same offsets of its stage
+              const uint32_t peer = rank ^ 1u;
+              const uint32_t mbar = map_to_rank(smem_u32(&bar_full[slot]), peer);
+              const int lr0 = ((pt - R::kAThreads) / 32) * 16;
 #pragma unroll
-              for (int l = 0; l < LEVELS; ++l)
+              for (int gq = 0; gq < 2; ++gq) {
+                if (lr0 + 8 * gq >= NC / 2) break;
+                const uint32_t rg = (uint32_t)(((int)rank * (NC / 2) + lr0 + 8 * gq) >> 3);
 #pragma unroll
-                for (int pl = 0; pl < 2; ++pl) {
-                  const uint32_t src = smem_base + a_plane(slot, l, pl) + rg * 768u;
-                  copy_to_peer(map_to_rank(src, q), src, 768u, mbar);
-                }
+                for (int l = 0; l < LEVELS; ++l)
+#pragma unroll
+                  for (int pl = 0; pl < kBPlanes; ++pl) {
+                    const uint32_t src = smem_base + b_plane(slot, l, pl) + rg * 768u;
+                    copy_to_peer(map_to_rank(src, peer), src, 768u, mbar);
+                  }
+              }
             }
+            if (kSets && is_a && ok) {
+              // this warp's 32 diquark rows and K half of every plane go to the peer
+              const uint32_t src = smem_base + (uint32_t)(slot * STAGE_BYTES) +
+                                   (uint32_t)(g0 / 8) * kSetHalf + (uint32_t)(rr >> 3) * kSetGroup;
+              const uint32_t peer = rank ^ 1u;
+              copy_to_peer(map_to_rank(src, peer), src, 4 * kSetGroup,
+                           map_to_rank(smem_u32(&bar_full[slot]), peer));
+            }
+            if (kShareA && !kSets && is_a && ok) {
+              // this warp's 8 diquark rows (one row group) of every plane go to every peer
+              const uint32_t rg = (uint32_t)(rr >> 3);
+              const uint32_t full_local = smem_u32(&bar_full[slot]);
+              for (uint32_t q = 0; q < (uint32_t)C; ++q) {
+                if (q == rank) continue;
+                const uint32_t mbar = map_to_rank(full_local, q);
+#pragma unroll
+                for (int l = 0; l < LEVELS; ++l)
+#pragma unroll
+                  for (int pl = 0; pl < 2; ++pl) {
+                    const uint32_t src = smem_base + a_plane(slot, l, pl) + rg * 768u;
+                    copy_to_peer(map_to_rank(src, q), src, 768u, mbar);
+                  }
+              }
+            }
+            if (C > 1 && (pt == 0 || (kSets && pt == 128)))
+              mbar_arrive_expect_tx(smem_u32(&bar_full[slot]), peer_tx);
+            else
+              mbar_arrive(smem_u32(&bar_full[slot]));
           }
-          if (C > 1 && (pt == 0 || (kSets && pt == 128)))
-            mbar_arrive_expect_tx(smem_u32(&bar_full[slot]), peer_tx);
-          else
-            mbar_arrive(smem_u32(&bar_full[slot]));
-        }
-        __syncwarp();
+          __syncwarp();
         }
         if constexpr (!PROJ) {
           // the next stage's first group: G groups on, or the next row's first
