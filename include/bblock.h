@@ -165,8 +165,9 @@ int bblock_compute_batch(bblock_ctx* ctx, const bblock_job* jobs, int n_jobs,
  * serves every noise triple and spin operator of a run.
  *
  * bblock_mode_triplet: T[t][p][l1][l2][l3] = sum_x e^{-i p.x} eps_abc V[l1][x][a]
- * V[l2][x][b] V[l3][x][c] for every time slice, computed by the context's form (it is the
- * contraction with identity coefficients). V as in bblock_compute (device); T_out device,
+ * V[l2][x][b] V[l3][x][c] for every time slice, computed by the context's form: FP64 and
+ * double-float sum the elements l1 < l2 < l3 and complete T by its antisymmetry (general
+ * contraction with BBLOCK_OPT_CHECKS), the other forms contract identity coefficients. V as in bblock_compute (device); T_out device,
  * complex128 [n_t][n_mom][n_ev][n_ev][n_ev], l3 fastest, caller-owned. Requires
  * max_ndil >= n_ev (BBLOCK_ERR_INVALID_ARG otherwise). Asynchronous on `stream`. */
 int bblock_mode_triplet(bblock_ctx* ctx, int n_t, const void* V, const int32_t* momenta,
@@ -174,8 +175,11 @@ int bblock_mode_triplet(bblock_ctx* ctx, int n_t, const void* V, const int32_t* 
 
 /* bblock_from_triplet: B[t][p][d1][d2][d3] = sum_s c_s sum_{l1 l2 l3} T[t][p][l1][l2][l3]
  * phi1[t][alpha_s n_ev + l1][d1] phi2[t][beta_s n_ev + l2][d2] phi3[t][gamma_s n_ev + l3][d3]
- * as three batched complex mode products in FP64 (per time slice and (alpha, beta) pair:
- * T x3 folded phi3, then x2 phi2, then x1 phi1). T as written by bblock_mode_triplet; phi_i,
+ * as three batched complex mode products in FP64 (per time slice: T x3 phi3 for each group of
+ * spin terms that share it, x2 phi2 and x1 phi1 for each term; four multiplications to a complex
+ * one, so each part of a block is accurate to its own size). The intermediates of as many terms
+ * as fit 1 GiB and the wave budget are held at a time, fewer where the device cannot hold
+ * them. T as written by bblock_mode_triplet; phi_i,
  * B_out, spins and coefficients as in bblock_compute (device buffers; the momenta
  * themselves are not needed, only their number). Asynchronous on `stream`. */
 int bblock_from_triplet(bblock_ctx* ctx, int n_t, const void* T, const void* phi1,
@@ -186,7 +190,7 @@ int bblock_from_triplet(bblock_ctx* ctx, int n_t, const void* T, const void* phi
 /* Device bytes the context holds right now (workspace + caches). */
 size_t bblock_workspace_bytes(const bblock_ctx* ctx);
 
-/* Number of kernel launches enqueued by the last compute call. */
+/* Number of kernel launches enqueued by the last compute call, table copies included. */
 int bblock_last_launch_count(const bblock_ctx* ctx);
 
 /* Contraction path of the last compute call (for reporting executed work; the blocks do
@@ -301,7 +305,7 @@ int bblock_get_option(const bblock_ctx* ctx, int option);
  * and of the fields plus the projection kernel) is bracketed by two CUDA events recorded
  * on the launching stream. */
 typedef struct {
-  char name[32];    /* "phase", "project", "contract", "reduce", ... */
+  char name[32];    /* "phase", "project", "contract", "reduce", "tables", ... */
   int launches;     /* kernel launches of the steps timed since the last read */
   double total_ms;  /* summed event-to-event durations of those steps */
 } bblock_kernel_stat;

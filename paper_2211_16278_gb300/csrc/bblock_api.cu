@@ -45,8 +45,8 @@ struct bblock_ctx {
   char* d_io = nullptr;
   size_t io_cap = 0;
   cudaStream_t copy_stream = nullptr;
-  // mode-triplet ordering: identity coefficients [4 n_ev][n_ev] and the mode-product
-  // intermediates (folded phi3, T x3 phi3', then x2 phi2)
+  // mode-triplet ordering: identity coefficients [4 n_ev][n_ev] (forms that contract them) and the
+  // mode products' intermediates (folded phi3 and phi2, T x3 phi3', then x2 phi2')
   double2* d_ident = nullptr;
   char* d_tri = nullptr;
   size_t tri_cap = 0;
@@ -2139,8 +2139,9 @@ int bblock_compute_batch(bblock_ctx* c, const bblock_job* jobs_in, int n_jobs,
                   static_cast<cudaStream_t>(stream));
 }
 
-// Eq. (4): T[t][p] is the contraction with q_i = V, i.e. identity coefficients and the
-// single spin triple (0, 0, 0), computed by the context's form for every time slice.
+// Eq. (4): T[t][p] is the contraction with q_i = V and the single spin triple (0, 0, 0), computed by
+// the context's form for every time slice: the ordered elements of V (run_triplet), or identity
+// coefficients through the general path.
 int bblock_mode_triplet(bblock_ctx* c, int n_t, const void* V, const int32_t* momenta, int n_mom,
                         void* T_out, void* stream) {
   if (!c) return BBLOCK_ERR_INVALID_ARG;
@@ -2189,10 +2190,11 @@ int bblock_mode_triplet(bblock_ctx* c, int n_t, const void* V, const int32_t* mo
   return run_jobs_cached(c, jobs, momenta, n_mom, spin, one, 1, 0, s);
 }
 
-// Eq. (3) through the mode triplet: for every time slice and (alpha, beta) pair,
-//   U1 = T x3 phi3'   (phi3' = the pair's folded line-3 coefficients),
-//   U2 = U1 x2 phi2[beta],  B += U2 x1 phi1[alpha],
-// three batched complex GEMMs in FP64.
+// Eq. (3) through the mode triplet: for every time slice,
+//   U1_g = T x3 phi3'_g            for each group g of spin terms (plan_groups),
+//   U2_t = U1_g(t) x2 phi2'_t      for each term t,
+//   B = sum_t U2_t x1 phi1[alpha_t],
+// three lists of batched complex GEMMs in FP64.
 int bblock_from_triplet(bblock_ctx* c, int n_t, const void* T, const void* phi1, const void* phi2,
                         const void* phi3, int nd1, int nd2, int nd3, int n_mom,
                         const int32_t* spin_idx, const double* spin_coeffs, int n_spin,

@@ -36,9 +36,9 @@ constexpr int kCanaryBytes = 256;   // canary after every workspace block (check
 
 // One reconstructed field of Eq. (2):
 //   q[r][d] = sum_l V[l][r] * Phi[l][d],   Phi[l][d] = sum_t w[t] * phi[row_off[t] + l][d],
-// r = 3x + a running over the 3X (site, colour) rows. Lines 1 and 2 use one term
-// (row_off = alpha * n_ev, w = 1); line 3 folds the spin coefficients of every
-// triple that shares an (alpha, beta) pair into one field (Eq. 1 is linear in q3).
+// r = 3x + a running over the 3X (site, colour) rows. Line 1 uses one term (row_off = alpha * n_ev,
+// w = 1). The spin coefficients are folded into line 3, one field per (alpha, beta) pair, or into
+// line 2, one field per (alpha, gamma) (Eq. 1 is linear in each line).
 struct ProjField {
   const double2* V;     // [n_ev][3X]
   const double2* phi;   // [4 n_ev][nd]

@@ -26,13 +26,13 @@
 //     L2 (the read-modify-write is below 3 % of the L2 rate in the FP64 form);
 //   * or, for lists whose momenta hardly share an n0 (plan_rows), a phase per momentum and site
 //     (NP of them): 2 to recombine, then 4 for every momentum, into sums that stay in registers
-//     over the unit's rows.
+//     over the unit's sites.
 // (A singlet per spin pair and a phase product per momentum and site take 9 n_pairs + 2 + 4 P:
 // 74 instead of 26 at 4 pairs, 2 groups and 9 momenta of n0 = 0, +-1.) Times: k_contract_fp64,
 // k_contract_df.
 //
-// Work unit = (job, slab of lattice rows, 16 RM (d1, d2) pairs, 16 RN d3 columns). Per chunk
-// of XC sites of a row the CTA stages A[k][m] = diquark and B[k][n] = third quark with
+// Work unit = (job, slab of lattice rows or, with a phase per site, of sites, 16 RM (d1, d2) pairs,
+// 16 RN d3 columns). Per chunk of XC sites the CTA stages A[k][m] = diquark and B[k][n] = third quark with
 // k = (site, group, colour); each thread owns RM x RN outputs. A wide d3 tile matters: the
 // diquark costs 24 operations per term, pair and site for all of the tile's columns.
 #pragma once
