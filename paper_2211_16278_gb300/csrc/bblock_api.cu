@@ -1268,15 +1268,10 @@ RowCall plan_row_call(const bblock_ctx* c, const SpinPlan& sp, const int32_t* mo
   r.groups = plan_groups(sp, true, jobs, c->cfg.n_ev, 64);
   const int G = r.groups.n_groups, T = r.groups.n_terms;
   if (per_mom) {
-    // one kind for all: the launches share slabs, of rows or of sites
+    // one kind for all, since the launches share slabs; a momentum by itself is cheaper by rows
     r.plans.resize(n_mom);
-    bool all_site = true;
     for (int p = 0; p < n_mom; ++p) {
-      plan_rows(L, momenta + 3 * p, 1, G, T, nd3, df, ROWS_AUTO, &r.plans[p], 1);
-      all_site = all_site && r.plans[p].per_site;
-    }
-    for (int p = 0; p < n_mom; ++p) {
-      if (!all_site) plan_rows(L, momenta + 3 * p, 1, G, T, nd3, df, ROWS_FACTORED, &r.plans[p], 1);
+      plan_rows(L, momenta + 3 * p, 1, G, T, nd3, df, ROWS_FACTORED, &r.plans[p], 1);
       r.plans[p].mom[0].p = p;
     }
   } else {

@@ -209,7 +209,8 @@ inline int site_chunk(int L, int n_groups, long long tiles, long long slots) {
 static_assert((size_t)24 * (16 * kRowRM + 64) * 3 * kMaxPairs + 16 * (kMaxSiteP + 128) <= 227 * 1024,
               "one site of kMaxPairs groups fits");
 // The momenta of a call, each in one RowPlan: row-factored (at most kMaxRowP momenta and kMaxRowCls
-// classes each) or with a phase per site, whichever takes fewer operations (see fp64_kernels.cu).
+// classes each) or, unless `kind` forbids it, with a phase per site, whichever takes fewer operations
+// (see fp64_kernels.cu).
 // groups, terms: of the spin sum; nd3: the widest job's d3 columns; df: double-float.
 // Returns the number of plans written to `out` (at most max_out), or the number needed where
 // out is null.

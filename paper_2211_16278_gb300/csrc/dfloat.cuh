@@ -36,6 +36,13 @@ __device__ __forceinline__ dfloat df_norm(dfloat a) {
   return dfloat{s, t};
 }
 
+// The same in half the instructions: exact while |h| >= |l|, else off by at most ulp(l), which is
+// the size of the roundings that l holds already.
+__device__ __forceinline__ dfloat df_norm_quick(dfloat a) {
+  const float s = __fadd_rn(a.h, a.l);
+  return dfloat{s, __fsub_rn(a.l, __fsub_rn(s, a.h))};
+}
+
 // Exact conversion from a double's leading 48 bits (the rest is rounded into l).
 __device__ __forceinline__ dfloat df_from_double(double x) {
   const float h = __double2float_rn(x);
@@ -55,6 +62,15 @@ __device__ __forceinline__ dfloat df_sub(dfloat a, dfloat b) {
   float s, t;
   two_sum(a.h, -b.h, s, t);
   return dfloat{s, __fadd_rn(t, __fsub_rn(a.l, b.l))};
+}
+
+// a * b (lazily normalised).
+__device__ __forceinline__ dfloat df_mul(dfloat a, dfloat b) {
+  const float p = __fmul_rn(a.h, b.h);
+  float e = fmaf(a.h, b.h, -p);   // exact error of p
+  e = fmaf(a.h, b.l, e);
+  e = fmaf(a.l, b.h, e);
+  return dfloat{p, e};
 }
 
 // acc += a * b (lazily normalised).

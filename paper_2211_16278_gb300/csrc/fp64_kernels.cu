@@ -276,9 +276,12 @@ int site_plans(int L, const int32_t* momenta, int n_mom, int cap, RowPlan* out, 
 // hardly share a class, are the second kind's. Beside the operations, as measured (L = 2 to 24,
 // N_dil 16 and 32, 1 to 4 pairs): a row's end costs 8 (16 in double-float: the partial block's
 // latency) per momentum after the first, and launches of two or three classes, one CTA an SM, a
-// tenth more. L = 16, N_dil = 32, one pair, momenta (k, k, k), FP64 / double-float, ms row-factored
-// and per site: k < 2  4.72 / 1.40 and 4.91 / 1.44; k < 4  6.86 / 2.18 and 6.72 / 1.88;
-// k < 8  16.7 / 5.23 and 10.5 / 2.81; -3 <= k <= 3  7.07 / 2.40 and 9.6 / 2.59.
+// tenth more; a phase per site costs a tenth more too (spills, its runs' ends, the shorter
+// renormalisation of double-float), so that a single momentum, or lists of one class from L = 4 on,
+// go by rows. L = 16, N_dil = 32, one pair, momenta (k, k, k), FP64 / double-float, ms row-factored
+// and per site: k < 4  6.83 / 2.17 and 6.70 / 2.13; k < 5  10.7 / 3.34 and 7.96 / 2.51;
+// k < 8  16.7 / 5.21 and 10.8 / 3.28; k < 16 in double-float 6.12 and 6.4;
+// -3 <= k <= 3  7.06 / 2.39 and 9.6 / 2.6.
 int plan_rows(int L, const int32_t* momenta, int n_mom, int groups, int terms, int nd3, bool df,
               RowKind kind, RowPlan* out, int max_out) {
   if (n_mom < 1) return 0;
@@ -306,7 +309,7 @@ int plan_rows(int L, const int32_t* momenta, int n_mom, int groups, int terms, i
   shape = RowPlan{};
   shape.per_site = 1;
   shape.n_mom = n_mom < cap ? n_mom : cap;
-  const double by_site = (n_mom + cap - 1) / cap * (singlet_ops(shape) + 2.0) + 4.0 * n_mom;
+  const double by_site = 1.1 * ((n_mom + cap - 1) / cap * (singlet_ops(shape) + 2.0) + 4.0 * n_mom);
   if (kind == ROWS_AUTO && by_site < 0.97 * by_row) return site_plans(L, momenta, n_mom, cap, out, max_out);
   return row_plans(L, momenta, n_mom, axis, out, max_out);
 }
